@@ -214,7 +214,8 @@ const char *lskum_last_error(const lskum_ctx *ctx)
 struct HostPrep {
     std::vector<int32_t> slice_off, deg, enb;
     std::vector<uint8_t> emb, fl_i;
-    std::vector<double> edx, edy, ew1, ew2, egx, egy, geo_i, wnx, wny;
+    std::vector<uint2> ew1, ew2;  // residual weights, integer and remainder in units of G_WSC
+    std::vector<double> edx, edy, egx, egy, geo_i, wnx, wny;
     std::vector<double> exx, exy, eyx, eyy;  // wgx dx, wgx dy, wgy dx, wgy dy per slot
     // LU-SGS lower / upper slot lists (CSR, internal order) and level orders
     std::vector<int32_t> lo_off, lo_nbr, up_off, up_nbr, sw_fwd, sw_bwd;
@@ -235,6 +236,15 @@ struct HostPrep {
     std::vector<double> lp_w1[2], lp_w2[2];
 };
 static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &hp);
+
+// A residual weight w in units of `unit` (a power of two, 0 where the point
+// has none): the nearest integer and the remainder in units of 2^-24.
+static uint2 split_weight(double w, double unit)
+{
+    if (!(unit > 0.0)) return uint2{0, 0};
+    const double v = w / unit, r = std::nearbyint(v);
+    return uint2{(uint32_t)(int32_t)r, (uint32_t)(int32_t)std::nearbyint(std::ldexp(v - r, 24))};
+}
 
 // Is point p (caller order of the union) an unknown of the iteration?  Outer
 // points are only under the kinetic far field.
@@ -690,6 +700,14 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
                 geo[(G_ABS_0 + s) * n + p] += std::fabs(w);
             }
         }
+        // unit of the residual's weights: a power of two such that the integer
+        // weights of the point's slots (rounded, in their two sub-stencils)
+        // add up to less than 2^30 in magnitude
+        double wsum = 0.0;
+        for (int s = 0; s < 4; s++) wsum += geo[(G_ABS_0 + s) * n + p];
+        int wexp = 0;
+        std::frexp(wsum, &wexp);  // wsum < 2^wexp
+        geo[G_WSC * n + p] = std::ldexp(1.0, wexp - 29);
         if (kouter) {  // the mirrored free-stream ghosts
             geo[G_LS1_3 * n + p] = -geo[G_LS1_2 * n + p];
             geo[G_ABS_3 * n + p] = geo[G_ABS_2 * n + p];
@@ -796,10 +814,13 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
     const size_t esz = std::max<int64_t>(ell, 1);
     std::vector<int32_t> &enb = hp.enb;
     std::vector<uint8_t> &emb = hp.emb;
-    std::vector<double> &edx = hp.edx, &edy = hp.edy, &ew1 = hp.ew1, &ew2 = hp.ew2, &egx = hp.egx, &egy = hp.egy;
+    std::vector<double> &edx = hp.edx, &edy = hp.edy, &egx = hp.egx, &egy = hp.egy;
+    std::vector<uint2> &ew1 = hp.ew1, &ew2 = hp.ew2;
+    ew1.assign(esz, uint2{0, 0});
+    ew2.assign(esz, uint2{0, 0});
     enb.assign(esz, 0);
     emb.assign(esz, 0);
-    for (auto *v : {&edx, &edy, &ew1, &ew2, &egx, &egy, &hp.exx, &hp.exy, &hp.eyx, &hp.eyy}) v->assign(esz, 0.0);
+    for (auto *v : {&edx, &edy, &egx, &egy, &hp.exx, &hp.exy, &hp.eyx, &hp.eyy}) v->assign(esz, 0.0);
     for (int32_t k = 0; k < n; k++) {
         const int32_t p = c->perm[k];
         deg[k] = off[p + 1] - off[p];
@@ -812,8 +833,8 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
             emb[t] = smb[e];
             edx[t] = 0.5 * sdx[e];  // half offsets (exact): the residual's reconstruction
             edy[t] = 0.5 * sdy[e];  // steps q - (dx, dy)/2 . grad q
-            ew1[t] = sw1[e];
-            ew2[t] = sw2[e];
+            ew1[t] = split_weight(sw1[e], geo[(size_t)G_WSC * n + p]);
+            ew2[t] = split_weight(sw2[e], geo[(size_t)G_WSC * n + p]);
             egx[t] = swgx[e];
             egy[t] = swgy[e];
             hp.exx[t] = swgx[e] * sdx[e];
@@ -1014,7 +1035,8 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     const int32_t n = c->n, ld = c->ld, nsl = ld / 32;
     std::vector<int32_t> &slice_off = hp.slice_off, &deg = hp.deg, &enb = hp.enb;
     std::vector<uint8_t> &emb = hp.emb, &fl_i = hp.fl_i;
-    std::vector<double> &edx = hp.edx, &edy = hp.edy, &ew1 = hp.ew1, &ew2 = hp.ew2, &egx = hp.egx, &egy = hp.egy;
+    std::vector<double> &edx = hp.edx, &edy = hp.edy, &egx = hp.egx, &egy = hp.egy;
+    std::vector<uint2> &ew1 = hp.ew1, &ew2 = hp.ew2;
     std::vector<double> &geo_i = hp.geo_i, &wnx = hp.wnx, &wny = hp.wny;
     // ---- device memory ----
     cudaError_t e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
@@ -1036,7 +1058,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     int32_t *dso = A.alloc<int32_t>(nsl + 1), *ddeg = A.alloc<int32_t>(n), *dnb = A.alloc<int32_t>(enb.size());
     uint8_t *dmb = A.alloc<uint8_t>(emb.size());
     double *ddx = A.alloc<double>(edx.size()), *ddy = A.alloc<double>(edx.size());
-    double *dw1 = A.alloc<double>(edx.size()), *dw2 = A.alloc<double>(edx.size());
+    uint2 *dw1 = A.alloc<uint2>(edx.size()), *dw2 = A.alloc<uint2>(edx.size());
     double *dgx = A.alloc<double>(edx.size()), *dgy = A.alloc<double>(edx.size());
     double *dxx = A.alloc<double>(edx.size()), *dxy = A.alloc<double>(edx.size());
     double *dyx = A.alloc<double>(edx.size()), *dyy = A.alloc<double>(edx.size());
@@ -1163,7 +1185,10 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     d.dUs = A.alloc<double>(4 * (size_t)ld);
     d.dU = A.alloc<double>(4 * (size_t)ld);
     // launch shape: enough threads per point to fill the GPU on small clouds
-    c->launch.res_block = 128;
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
+    if (e != cudaSuccess) return cuda_fail(c, e, "cudaDeviceGetAttribute");
+    c->launch.res_blocks = 2 * std::max(sms, 1);
     c->launch.tpp = n >= 100000 ? 1 : (n >= 50000 ? 2 : (n >= 25000 ? 4 : 8));
     c->launch.sweep_lanes = 4;
     d.n_blk = (int32_t)hp.blk_case.size();
@@ -1195,8 +1220,8 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     d.memb = dmb;
     d.nhx = ddx;
     d.nhy = ddy;
-    d.w1 = dw1;
-    d.w2 = dw2;
+    d.wq1 = dw1;
+    d.wq2 = dw2;
     d.wgx = dgx;
     d.wgy = dgy;
     d.gxx = dxx;
@@ -1257,8 +1282,8 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     up(dmb, emb.data(), emb.size());
     up(ddx, edx.data(), edx.size() * sizeof(double));
     up(ddy, edy.data(), edy.size() * sizeof(double));
-    up(dw1, ew1.data(), ew1.size() * sizeof(double));
-    up(dw2, ew2.data(), ew2.size() * sizeof(double));
+    up(dw1, ew1.data(), ew1.size() * sizeof(uint2));
+    up(dw2, ew2.data(), ew2.size() * sizeof(uint2));
     up(dgx, egx.data(), egx.size() * sizeof(double));
     up(dgy, egy.data(), egy.size() * sizeof(double));
     up(dxx, hp.exx.data(), hp.exx.size() * sizeof(double));

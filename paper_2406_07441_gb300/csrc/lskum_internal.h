@@ -56,6 +56,7 @@ enum GeoField {
                                          // outer points: LS_3(1) = -LS_2(1), the ghosts)
     G_ABS_0, G_ABS_1, G_ABS_2, G_ABS_3,  // sum_i |w_i| of each split sub-stencil
     G_DMIN,                              // min_i |r_i - r_0|
+    G_WSC,                               // unit of the residual's weights (a power of two)
     G_SXX, G_SXY, G_SYX, G_SYY,          // sums over the stencil of wgx dx, wgx dy, wgy dx, wgy dy
     G_NFIELDS
 };
@@ -99,7 +100,10 @@ struct Dev {
     const int32_t *nbr;       // neighbour (internal index)
     const uint8_t *memb;      // bits 0/1: e1 sub-stencil +/-, bits 2/3: e2 sub-stencil +/-
     const double *nhx, *nhy;  // (x_i - x_0)/2, (y_i - y_0)/2
-    const double *w1, *w2;    // LS weight of the slot in its e1 / e2 split sub-stencil (0 if none)
+    // LS weight of the slot in its e1 / e2 split sub-stencil (0 if none), in
+    // units of the point's G_WSC: x the nearest integer (int32; the sum of a
+    // point's |x| is below 2^30), y the remainder in units of 2^-24 (int32)
+    const uint2 *wq1, *wq2;
     const double *wgx, *wgy;  // full-stencil LS weights of d/dx and d/dy (Eq. 10, 16)
     const double *gxx, *gxy, *gyx, *gyy;  // wgx dx, wgx dy, wgy dx, wgy dy (inner iterations)
     // iteration buffers
@@ -189,7 +193,7 @@ struct Dev {
 // this iteration; the update writes set 1 - cur.
 struct Launch {
     int tpp;          // threads per point of the gradient and residual kernels (1, 2, 4, 8)
-    int res_block;    // threads per block of the residual kernel
+    int res_blocks;   // blocks of the residual kernel resident at once (its persistent grid)
     int sweep_lanes;  // lanes per point of the sweep kernels (2, 4, 8), or 32: the packed form
     const int32_t *pk_lw[2];  // packed form: host arrays [n_levels + 1], first framed-point warp of each level
     const int32_t *lp_lg[2];  // packed form: host arrays [n_levels + 1], first interior group of each level

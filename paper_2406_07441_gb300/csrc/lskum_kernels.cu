@@ -33,6 +33,8 @@
 #include <cstdint>
 
 #include "lskum_fastmath.cuh"
+#include "lskum_fixflux.cuh"
+#include "lskum_fluxtable.h"
 
 namespace lskum {
 
@@ -472,19 +474,18 @@ __global__ void __launch_bounds__(256) k_grad(Dev d, const double *__restrict__ 
 // ---------------------------------------------------------------------------
 // flux residual, time step, diagonal, norm partials
 // ---------------------------------------------------------------------------
-// R += y with Kahan's compensated summation (W. Kahan, "Further remarks on
-// reducing truncation errors", CACM 8(1), 1965): c carries the negated
-// rounding error of the running sum into the next term.  The caller forms y
-// as the terms of a group of four slots less c, the weighted flux
-// differences of their split sub-stencils folded in by FMAs, so one
-// compensated addition serves the group (a quarter of the per-slot
-// additions' FP64 instructions; R changed by at most 6e-17 relative).  The
-// final sum is R - c.
-__device__ __forceinline__ void comp_add(double &R, double &c, double y)
+// The frame of point k: (1,0), (0,1), or (t, n) at wall and kinetic outer points.
+__device__ __forceinline__ void point_frame(const Dev &d, int k, bool framed, double &e1x, double &e1y, double &e2x,
+                                            double &e2y)
 {
-    const double t = R + y;
-    c = (t - R) - y;  // what the addition lost (negated)
-    R = t;
+    e1x = 1.0, e1y = 0.0, e2x = 0.0, e2y = 1.0;
+    if (framed) {
+        const int ld = d.ld;
+        e1x = d.geo[G_E1X * ld + k];
+        e1y = d.geo[G_E1Y * ld + k];
+        e2x = d.geo[G_E2X * ld + k];
+        e2y = d.geo[G_E2Y * ld + k];
+    }
 }
 
 // The sign of x with magnitude 0 (what 0 * x gives), on the integer pipe.
@@ -493,165 +494,265 @@ __device__ __forceinline__ double zero_like(double x)
     return __hiloint2double(__double2hiint(x) & (int)0x80000000, 0);
 }
 
-template <int TPP, bool COMP>
-// Blocks of the residual kept resident per SM: 4 x 128 threads caps it at
-// 128 registers without spills (5 spills and runs slower; with no cap the
-// integer multiplies take it to 139 registers and 3 blocks).
-#ifndef LSKUM_RES_MIN_BLOCKS
-#define LSKUM_RES_MIN_BLOCKS 4
-#endif
-__global__ void __launch_bounds__(128, LSKUM_RES_MIN_BLOCKS) k_residual(Dev d, StateSet st, const double *__restrict__ g)
+// The modified q-variables of a slot (Eq. 15): neighbour i's and the point's
+// own, reconstructed over half the offset (hdx, hdy).
+__device__ __forceinline__ void reconstruct(const double *__restrict__ q, const double *__restrict__ g, int ld, int i,
+                                            const double q0[4], const double gx0[4], const double gy0[4], double hdx,
+                                            double hdy, double qi[4], double q0t[4])
 {
-    __shared__ MathTables T;
+    const double2 *gr = reinterpret_cast<const double2 *>(g + 8 * (size_t)i);
+    const double2 x01 = gr[0], x23 = gr[1], y01 = gr[2], y23 = gr[3];
+    const double gxi[4] = {x01.x, x01.y, x23.x, x23.y}, gyi[4] = {y01.x, y01.y, y23.x, y23.y};
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        qi[c] = fma(-hdx, gxi[c], fma(-hdy, gyi[c], q[c * ld + i]));
+        q0t[c] = fma(-hdx, gx0[c], fma(-hdy, gy0[c], q0[c]));
+    }
+}
+
+// The slots sub, sub + TPP, ... of point k in FP64, for points of which a
+// state lies outside the fixed-point ranges (hypersonic, very hot or very
+// dense states, non-finite ones); the group's lanes add their sums.
+template <int TPP>
+__device__ __noinline__ void residual_fp64(const Dev &d, const double *__restrict__ q, const double *__restrict__ g,
+                                           int k, int sub, bool second, double R[4])
+{
+    const MathTables &T = g_math;
+    const int ld = d.ld;
+    const bool framed = d.flag[k] != kInterior;
+    const double e1x = d.geo[G_E1X * ld + k], e1y = d.geo[G_E1Y * ld + k];
+    const double e2x = d.geo[G_E2X * ld + k], e2y = d.geo[G_E2Y * ld + k];
+    const double wsc = d.geo[G_WSC * ld + k];
+    double q0[4], gx0[4], gy0[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        q0[c] = q[c * ld + k];
+        gx0[c] = g[8 * (size_t)k + c];
+        gy0[c] = g[8 * (size_t)k + 4 + c];
+        R[c] = 0.0;
+    }
+    const int deg = d.deg[k];
+    const int base = d.slice_off[k >> 5] + (k & 31);
+    for (int j = sub; j < deg; j += TPP) {
+        const int e = base + 32 * j;
+        const int mb = d.memb[e];
+        if (!mb) continue;
+        const double hx = d.nhx[e], hy = d.nhy[e];
+        double qi[4], q0t[4];
+        reconstruct(q, g, ld, d.nbr[e], q0, gx0, gy0, second ? hx : zero_like(hx), second ? hy : zero_like(hy), qi,
+                    q0t);
+        const Prim Pi = q_to_prim(T, qi);
+        const Prim P0 = q_to_prim(T, q0t);
+#pragma unroll 1
+        for (int sb = 0; sb < 2; sb++) {
+            const int m = sb == 0 ? (mb & 3) : (mb >> 2);
+            if (!m) continue;
+            const bool pos = m & 1, xdir = sb == 0;
+            const uint2 wq = xdir ? d.wq1[e] : d.wq2[e];
+            const double w = fma((double)(int)wq.y, 0x1p-24, (double)(int)wq.x) * wsc;
+            const double dx = xdir ? e1x : e2x, dy = xdir ? e1y : e2y;
+            double Gi[4], G0[4];
+            split_flux(T, Pi, framed, xdir, dx, dy, pos, Gi);
+            split_flux(T, P0, framed, xdir, dx, dy, pos, G0);
+#pragma unroll
+            for (int c = 0; c < 4; c++) R[c] = fma(w, Gi[c] - G0[c], R[c]);
+        }
+    }
+}
+
+// A point's residual complete (the ghost term of kinetic outer points added)
+// and stored, with its local time step and scalar diagonal.
+__device__ __forceinline__ void residual_point(const Dev &d, const StateSet &st, int k, int fl, double cfl, double e1x,
+                                               double e1y, double e2x, double e2y, double R[4])
+{
+    const int ld = d.ld;
+    if (fl == kOuter) {
+        // kinetic far field: the n- side is free-stream ghosts at the mirror
+        // images of the inside neighbours, LS_3(1) (G_n^-(U_inf) - G_n^-(U_0))
+        // with LS_3(1) = -LS_2(1); first order (the point's own state)
+        const double *ui = d.case_uinf + 4 * d.case_of[k];
+        double U0[4], Ui[4];
+        bool same = true;
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            U0[c] = st.U[c * ld + k];
+            Ui[c] = ui[c];
+            same = same && U0[c] == Ui[c];
+        }
+        if (!same) {  // (equal states give exactly 0)
+            double Gi[4], G0[4];
+            flux_cons(g_math, Ui, e2x, e2y, false, Gi);
+            flux_cons(g_math, U0, e2x, e2y, false, G0);
+            const double l3 = d.geo[G_LS1_3 * ld + k];
+#pragma unroll
+            for (int c = 0; c < 4; c++) R[c] = fma(l3, Gi[c] - G0[c], R[c]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; c++) d.R[c * ld + k] = R[c];
+    // local time step (reading: CFL min_i|dr| / (|u| + a)) and the scalar
+    // diagonal of Eq. 26 with the spectral radii of Eq. 34, kept at least
+    // sum_s rho_s sum_i |w_i| so that it bounds the off-diagonal blocks
+    const double *pr = st.prim + (size_t)k * kPrimStride;
+    const double u = pr[P_U], v = pr[P_V];
+    const double a = sqrt(1.4 * pr[P_P] * pr[P_IRHO]);
+    const double dt = cfl * d.geo[G_DMIN * ld + k] / (sqrt(u * u + v * v) + a);
+    // D and 1/D: the sweeps multiply by 1/D (one division per point here
+    // instead of one per point in each sweep)
+    if (d.scheme == 1) {  // explicit: D = 1/dt, the step is -dt R
+        d.D[k] = 1.0 / dt;
+        d.iD[k] = dt;
+        return;
+    }
+    if (d.lusgs == 1) {  // revised LU-SGS: Jameson's splitting, rho(A_d) = |u_d| + a
+        const double u1 = fabs(u * e1x + v * e1y) + a, u2 = fabs(u * e2x + v * e2y) + a;
+        const double Dm = 1.0 / dt +
+                          0.5 * (u1 * (fabs(d.geo[G_LS1_0 * ld + k]) + fabs(d.geo[G_LS1_1 * ld + k])) +
+                                 u2 * (fabs(d.geo[G_LS1_2 * ld + k]) + fabs(d.geo[G_LS1_3 * ld + k])));
+        d.D[k] = Dm;
+        d.iD[k] = 1.0 / Dm;
+        return;
+    }
+    double Dp = 1.0 / dt, Ddom = 0.0;
+    const double u1 = u * e1x + v * e1y, u2 = u * e2x + v * e2y;
+    const double r0 = fmax(u1 + a, 0.0), r1 = fmax(a - u1, 0.0);
+    const double r2 = fmax(u2 + a, 0.0), r3 = fmax(a - u2, 0.0);
+    Dp -= r0 * d.geo[G_LS1_0 * ld + k];
+    Dp += r1 * d.geo[G_LS1_1 * ld + k];
+    Dp -= r2 * d.geo[G_LS1_2 * ld + k];
+    Dp += r3 * d.geo[G_LS1_3 * ld + k];
+    Ddom = r0 * d.geo[G_ABS_0 * ld + k] + r1 * d.geo[G_ABS_1 * ld + k] + r2 * d.geo[G_ABS_2 * ld + k]
+         + r3 * d.geo[G_ABS_3 * ld + k];
+    const double Da = Dp > Ddom ? Dp : Ddom;
+    d.D[k] = Da;
+    d.iD[k] = 1.0 / Da;
+}
+
+// Threads per block of the residual (two blocks per SM share its registers).
+constexpr int kResBlock = 256;
+
+// Flux residual, local time step and scalar diagonal; TPP lanes per point
+// over its slots, persistent blocks (a warp takes every W-th group of 32/TPP
+// points, so a block loads the 46 KB of tables once).
+// The reconstruction (16 FMAs per slot) runs on the FP64 unit; the inverse of
+// Eq. 14, the four split fluxes of a slot and the weighted sums run in 64-bit
+// fixed point on the integer pipes (lskum_fixflux.cuh), beside it.  The sums
+// are exact integers, so R does not depend on the order of the slots or on
+// TPP, and needs no compensation.  A framed point's velocities are rotated
+// into its frame, where every split flux is along an axis, and the sum's
+// momentum back out of it.  Measured on the 147,584-point cloud (1 lane per
+// point): 0.649 ms with the fluxes in FP64 and integer-pipe multiplies, 0.693
+// ms with compensated sums; 0.266 ms like this, FMA-heavy pipe 57 % and FP64
+// unit 55 % busy, the rest latency (4 warps per scheduler: 128 registers).
+template <int TPP>
+__global__ void __launch_bounds__(kResBlock, 2) k_residual(Dev d, StateSet st, const double *__restrict__ g)
+{
+    __shared__ __align__(16) uint64_t T[kFluxTableWords];
     if (halted(d.ctrl)) return;
-    load_math_tables(T);
+    static_assert(kFluxTableR == kFluxRows && kFluxTableExp == kFluxExpRows && kFluxTableWords % 2 == 0, "tables");
+    for (int i = threadIdx.x; i < kFluxTableWords / 2; i += kResBlock)
+        reinterpret_cast<ulonglong2 *>(T)[i] = reinterpret_cast<const ulonglong2 *>(kFluxTable)[i];
     __syncthreads();
     const int n1 = ((const volatile Ctrl *)d.ctrl)->it;  // this iteration, counted by k_begin
     const double cfl = (d.ramp > 0.0 && (double)n1 < d.ramp) ? d.cfl * ((double)n1 / d.ramp) : d.cfl;
     const bool second = n1 > d.first_order;  // first-order start: q~ = q
-    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = gt / TPP, sub = gt % TPP;
-    const bool active = k < d.n;
-    const int kk = active ? k : d.n - 1;
     const int ld = d.ld;
-    const int fl = d.flag[kk];
-    const bool work = active && (fl != kOuter || d.farfield == 1) && !frozen(d, kk);
-    const bool framed = fl != kInterior;  // (t, n) frame: wall and kinetic outer points
     const double *__restrict__ q = st.q;
-    double R[4] = {0.0, 0.0, 0.0, 0.0};
-    double Rc[4] = {0.0, 0.0, 0.0, 0.0};  // compensation terms (COMP)
-    const double e1x = d.geo[G_E1X * ld + kk], e1y = d.geo[G_E1Y * ld + kk];
-    const double e2x = d.geo[G_E2X * ld + kk], e2y = d.geo[G_E2Y * ld + kk];
-    if (work) {
-        double q0[4], gx0[4], gy0[4];
+    constexpr int kPts = 32 / TPP;
+    const int lane = threadIdx.x & 31, sub = lane % TPP;
+    const int tasks = (d.n + kPts - 1) / kPts;
+    for (int task = (blockIdx.x * kResBlock + threadIdx.x) / 32; task < tasks; task += gridDim.x * (kResBlock / 32)) {
+        const int k = task * kPts + lane / TPP;
+        const bool active = k < d.n;
+        const int kk = active ? k : d.n - 1;
+        const int fl = d.flag[kk];
+        const bool work = active && (fl != kOuter || d.farfield == 1) && !frozen(d, kk);
+        const bool framed = fl != kInterior;  // (t, n) frame: wall and kinetic outer points
+        double e1x, e1y, e2x, e2y;
+        point_frame(d, kk, framed, e1x, e1y, e2x, e2y);
+        FxSum acc[4] = {};
+        uint32_t bad = 0;
+        if (work) {
+            double q0[4], gx0[4], gy0[4];
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                q0[c] = q[c * ld + kk];
+                gx0[c] = g[8 * (size_t)kk + c];
+                gy0[c] = g[8 * (size_t)kk + 4 + c];
+            }
+            const int deg = d.deg[kk];
+            const int base = d.slice_off[kk >> 5] + (kk & 31);
+            for (int j = sub; j < deg; j += TPP) {
+                const int e = base + 32 * j;
+                const int mb = d.memb[e];
+                if (!mb) continue;
+                const double hx = d.nhx[e], hy = d.nhy[e];  // half offsets
+                double qi[4], q0t[4];
+                reconstruct(q, g, ld, d.nbr[e], q0, gx0, gy0, second ? hx : zero_like(hx),
+                            second ? hy : zero_like(hy), qi, q0t);
+                if (framed) {
+                    const double a = qi[1], b = q0t[1];
+                    qi[1] = fma(a, e1x, qi[2] * e1y);
+                    qi[2] = fma(a, e2x, qi[2] * e2y);
+                    q0t[1] = fma(b, e1x, q0t[2] * e1y);
+                    q0t[2] = fma(b, e2x, q0t[2] * e2y);
+                }
+                FxState si, s0;
+                fx_state(T, qi[0], qi[1], qi[2], qi[3], si, bad);
+                fx_state(T, q0t[0], q0t[1], q0t[2], q0t[3], s0, bad);
+                if (mb & 3) {
+                    const uint2 w = d.wq1[e];
+                    const bool pos = mb & 1;
+                    FxFlux Gi, G0;
+                    fx_flux(T, si, si.u, si.su, si.v, si.sv, pos, Gi, bad);
+                    fx_flux(T, s0, s0.u, s0.su, s0.v, s0.sv, pos, G0, bad);
+                    const int wh = (int)w.x, wl = (int)w.y, sh = pos ? wh : -wh, sl = pos ? wl : -wl;
+                    fx_add(acc[0], sh, sl, Gi.rm, G0.rm);
+                    fx_add(acc[1], wh, wl, Gi.ga, G0.ga);
+                    fx_add(acc[2], sh, sl, Gi.go, G0.go);
+                    fx_add(acc[3], sh, sl, Gi.g3, G0.g3);
+                }
+                if (mb & 12) {
+                    const uint2 w = d.wq2[e];
+                    const bool pos = mb & 4;
+                    FxFlux Gi, G0;
+                    fx_flux(T, si, si.v, si.sv, si.u, si.su, pos, Gi, bad);
+                    fx_flux(T, s0, s0.v, s0.sv, s0.u, s0.su, pos, G0, bad);
+                    const int wh = (int)w.x, wl = (int)w.y, sh = pos ? wh : -wh, sl = pos ? wl : -wl;
+                    fx_add(acc[0], sh, sl, Gi.rm, G0.rm);
+                    fx_add(acc[2], wh, wl, Gi.ga, G0.ga);
+                    fx_add(acc[1], sh, sl, Gi.go, G0.go);
+                    fx_add(acc[3], sh, sl, Gi.g3, G0.g3);
+                }
+            }
+        }
+        double R[4];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            q0[c] = q[c * ld + kk];
-            gx0[c] = g[8 * (size_t)kk + c];
-            gy0[c] = g[8 * (size_t)kk + 4 + c];
+            acc[c].hh = group_sum<TPP>(acc[c].hh);
+            acc[c].l = group_sum<TPP>(acc[c].l);
+            acc[c].r = group_sum<TPP>(acc[c].r);
         }
-        const int deg = d.deg[kk];
-        const int base = d.slice_off[kk >> 5] + (kk & 31);
-        // (COMP) the terms of a group of four slots are summed by FMAs into y,
-        // which starts as the negated carried error; each group then enters R
-        // by one compensated addition, and a last partial group after the loop
-        double y[4] = {0.0, 0.0, 0.0, 0.0};
-        int ng = 0;  // (COMP) slots in the current group
-        for (int j = sub; j < deg; j += TPP) {
-            const int e = base + 32 * j;
-            const int mb = d.memb[e];
-            if (!mb) continue;
-            const int i = d.nbr[e];
-            const double hx = d.nhx[e], hy = d.nhy[e];  // half offsets
-            double qi[4], q0t[4];
-            const double2 *gr = reinterpret_cast<const double2 *>(g + 8 * (size_t)i);
-            const double2 x01 = gr[0], x23 = gr[1], y01 = gr[2], y23 = gr[3];
-            const double gxi[4] = {x01.x, x01.y, x23.x, x23.y}, gyi[4] = {y01.x, y01.y, y23.x, y23.y};
-            const double hdx = second ? hx : zero_like(hx), hdy = second ? hy : zero_like(hy);
+        const double wsc = d.geo[G_WSC * ld + kk];
+        R[0] = fx_total(acc[0]) * (wsc * 0x1p-27);
+        R[3] = fx_total(acc[3]) * (wsc * 0x1p-23);
+        const double Ra = fx_total(acc[1]) * (wsc * 0x1p-25), Ro = fx_total(acc[2]) * (wsc * 0x1p-25);
+        R[1] = framed ? fma(Ra, e1x, Ro * e2x) : Ra;
+        R[2] = framed ? fma(Ra, e1y, Ro * e2y) : Ro;
+        // (work is the same for the lanes of a group; the whole warp takes part in the sums)
+        bool slow = (bad >> 31) != 0;
+#pragma unroll
+        for (int o = TPP / 2; o > 0; o >>= 1) slow |= __shfl_xor_sync(kFull, (int)slow, o) != 0;
+        if (__any_sync(kFull, slow)) {
+            double Rs[4] = {0.0, 0.0, 0.0, 0.0};
+            if (slow) residual_fp64<TPP>(d, q, g, kk, sub, second, Rs);
 #pragma unroll
             for (int c = 0; c < 4; c++) {
-                qi[c] = fma(-hdx, gxi[c], fma(-hdy, gyi[c], q[c * ld + i]));
-                q0t[c] = fma(-hdx, gx0[c], fma(-hdy, gy0[c], q0[c]));
-            }
-            const Prim Pi = q_to_prim(T, qi);
-            const Prim P0 = q_to_prim(T, q0t);
-            // the slot's sub-stencils (x then y, or t then n): one loop body
-#pragma unroll 1
-            for (int sb = 0; sb < 2; sb++) {
-                const int m = sb == 0 ? (mb & 3) : (mb >> 2);
-                if (!m) continue;
-                const bool pos = m & 1, xdir = sb == 0;
-                const double w = xdir ? d.w1[e] : d.w2[e];
-                const double dx = xdir ? e1x : e2x, dy = xdir ? e1y : e2y;
-                double Gi[4], G0[4];
-                split_flux(T, Pi, framed, xdir, dx, dy, pos, Gi);
-                split_flux(T, P0, framed, xdir, dx, dy, pos, G0);
-#pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    if (COMP) y[c] = fma(w, Gi[c] - G0[c], y[c]);
-                    else R[c] = fma(w, Gi[c] - G0[c], R[c]);
-                }
-            }
-            if (COMP && ++ng == 4) {
-#pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    comp_add(R[c], Rc[c], y[c]);
-                    y[c] = -Rc[c];
-                }
-                ng = 0;
+                Rs[c] = group_sum<TPP>(Rs[c]);
+                if (slow) R[c] = Rs[c];
             }
         }
-        if (COMP && ng > 0) {
-#pragma unroll
-            for (int c = 0; c < 4; c++) comp_add(R[c], Rc[c], y[c]);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        if (COMP) R[c] -= Rc[c];
-        R[c] = group_sum<TPP>(R[c]);
-    }
-    if (work && sub == 0) {
-        if (fl == kOuter) {
-            // kinetic far field: the n- side is free-stream ghosts at the mirror
-            // images of the inside neighbours, LS_3(1) (G_n^-(U_inf) - G_n^-(U_0))
-            // with LS_3(1) = -LS_2(1); first order (the point's own state)
-            const double *ui = d.case_uinf + 4 * d.case_of[k];
-            double U0[4], Ui[4];
-            bool same = true;
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                U0[c] = st.U[c * ld + k];
-                Ui[c] = ui[c];
-                same = same && U0[c] == Ui[c];
-            }
-            if (!same) {  // (equal states give exactly 0)
-                double Gi[4], G0[4];
-                flux_cons(T, Ui, e2x, e2y, false, Gi);
-                flux_cons(T, U0, e2x, e2y, false, G0);
-                const double l3 = d.geo[G_LS1_3 * ld + k];
-#pragma unroll
-                for (int c = 0; c < 4; c++) R[c] = fma(l3, Gi[c] - G0[c], R[c]);
-            }
-        }
-#pragma unroll
-        for (int c = 0; c < 4; c++) d.R[c * ld + k] = R[c];
-        // local time step (reading: CFL min_i|dr| / (|u| + a)) and the scalar
-        // diagonal of Eq. 26 with the spectral radii of Eq. 34, kept at least
-        // sum_s rho_s sum_i |w_i| so that it bounds the off-diagonal blocks
-        const double *pr = st.prim + (size_t)k * kPrimStride;
-        const double u = pr[P_U], v = pr[P_V];
-        const double a = sqrt(1.4 * pr[P_P] * pr[P_IRHO]);
-        const double dt = cfl * d.geo[G_DMIN * ld + k] / (sqrt(u * u + v * v) + a);
-        // D and 1/D: the sweeps multiply by 1/D (one division per point here
-        // instead of one per point in each sweep)
-        if (d.scheme == 1) {  // explicit: D = 1/dt, the step is -dt R
-            d.D[k] = 1.0 / dt;
-            d.iD[k] = dt;
-            return;
-        }
-        if (d.lusgs == 1) {  // revised LU-SGS: Jameson's splitting, rho(A_d) = |u_d| + a
-            const double u1 = fabs(u * e1x + v * e1y) + a, u2 = fabs(u * e2x + v * e2y) + a;
-            const double Dm = 1.0 / dt +
-                              0.5 * (u1 * (fabs(d.geo[G_LS1_0 * ld + k]) + fabs(d.geo[G_LS1_1 * ld + k])) +
-                                     u2 * (fabs(d.geo[G_LS1_2 * ld + k]) + fabs(d.geo[G_LS1_3 * ld + k])));
-            d.D[k] = Dm;
-            d.iD[k] = 1.0 / Dm;
-            return;
-        }
-        double Dp = 1.0 / dt, Ddom = 0.0;
-        const double u1 = u * e1x + v * e1y, u2 = u * e2x + v * e2y;
-        const double r0 = fmax(u1 + a, 0.0), r1 = fmax(a - u1, 0.0);
-        const double r2 = fmax(u2 + a, 0.0), r3 = fmax(a - u2, 0.0);
-        Dp -= r0 * d.geo[G_LS1_0 * ld + k];
-        Dp += r1 * d.geo[G_LS1_1 * ld + k];
-        Dp -= r2 * d.geo[G_LS1_2 * ld + k];
-        Dp += r3 * d.geo[G_LS1_3 * ld + k];
-        Ddom = r0 * d.geo[G_ABS_0 * ld + k] + r1 * d.geo[G_ABS_1 * ld + k] + r2 * d.geo[G_ABS_2 * ld + k]
-             + r3 * d.geo[G_ABS_3 * ld + k];
-        const double Da = Dp > Ddom ? Dp : Ddom;
-        d.D[k] = Da;
-        d.iD[k] = 1.0 / Da;
+        if (work && sub == 0) residual_point(d, st, k, fl, cfl, e1x, e1y, e2x, e2y, R);
     }
 }
 
@@ -904,20 +1005,6 @@ __device__ __forceinline__ void sweep_point(const Dev &d, const StateSet &st, co
     T *out = FWD ? sb.dUs : sb.dU;
 #pragma unroll
     for (int c = 0; c < 4; c++) out[4 * k + c] = w[c];
-}
-
-// The frame of point k: (1,0), (0,1), or (t, n) at wall and kinetic outer points.
-__device__ __forceinline__ void point_frame(const Dev &d, int k, bool framed, double &e1x, double &e1y, double &e2x,
-                                            double &e2y)
-{
-    e1x = 1.0, e1y = 0.0, e2x = 0.0, e2y = 1.0;
-    if (framed) {
-        const int ld = d.ld;
-        e1x = d.geo[G_E1X * ld + k];
-        e1y = d.geo[G_E1Y * ld + k];
-        e2x = d.geo[G_E2X * ld + k];
-        e2y = d.geo[G_E2Y * ld + k];
-    }
 }
 
 // G lanes per point over the point's list, butterfly reduction.
@@ -1491,9 +1578,8 @@ template <int TPP>
 cudaError_t enqueue_res(const Dev &d, const Launch &L, int cur, cudaStream_t s, int *launches)
 {
     const int fin = d.K & 1;
-    const int rb = (d.n * TPP + L.res_block - 1) / L.res_block;
-    if (d.precision) k_residual<TPP, true><<<rb, L.res_block, 0, s>>>(d, d.set[cur], d.gq[fin]);
-    else k_residual<TPP, false><<<rb, L.res_block, 0, s>>>(d, d.set[cur], d.gq[fin]);
+    const int want = (d.n * TPP + kResBlock - 1) / kResBlock;
+    k_residual<TPP><<<want < L.res_blocks ? want : L.res_blocks, kResBlock, 0, s>>>(d, d.set[cur], d.gq[fin]);
     (*launches)++;
     return cudaGetLastError();
 }
