@@ -18,6 +18,7 @@
 // |S| < 2.5 and a mass moment below 4 along each axis.  They hold for subsonic to moderately supersonic flow; a state
 // outside (or not finite) is reported and its point is evaluated in FP64.
 #pragma once
+#include <cmath>
 #include <cstdint>
 
 #include "lskum_fixmath.cuh"
@@ -229,11 +230,11 @@ LSKUM_HD void fx_add(FxSum &s, int32_t wh, int32_t wl, uint64_t Gi, uint64_t G0)
 }
 
 // The sum as a double, in units of 2^32 of the flux's unit times the weight's
-// (wl's products with the differences' low words, below 2^-24 of a unit of
-// the flux each, are left out).
+// (left out: 8 bits of l, 2^-24 of a unit of the flux in all, and wl's
+// products with the differences' low words, below that unit each).
 LSKUM_HD double fx_total(const FxSum &s)
 {
-    return (double)s.hh + ((double)s.l * 0x1p-32 + (double)s.r * 0x1p-24);
+    return fma((double)((s.l >> 8) + s.r), 0x1p-24, (double)s.hh);  // |l >> 8| + |r| < 2^63
 }
 
 }  // namespace lskum

@@ -214,8 +214,9 @@ const char *lskum_last_error(const lskum_ctx *ctx)
 struct HostPrep {
     std::vector<int32_t> slice_off, deg, enb;
     std::vector<uint8_t> emb, fl_i;
-    std::vector<uint2> ew1, ew2;  // residual weights, integer and remainder in units of G_WSC
-    std::vector<double> edx, edy, egx, egy, geo_i, wnx, wny;
+    std::vector<uint4> ewq;       // residual weights, integers and remainders in units of G_WSC
+    std::vector<double2> ehxy;    // half offsets
+    std::vector<double> egx, egy, geo_i, wnx, wny;
     std::vector<double> exx, exy, eyx, eyy;  // wgx dx, wgx dy, wgy dx, wgy dy per slot
     // LU-SGS lower / upper slot lists (CSR, internal order) and level orders
     std::vector<int32_t> lo_off, lo_nbr, up_off, up_nbr, sw_fwd, sw_bwd;
@@ -679,7 +680,7 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
             geo[G_SYX * n + p] += swgy[e] * sdx[e];
             geo[G_SYY * n + p] += swgy[e] * sdy[e];
         }
-        geo[G_DMIN * n + p] = dmin;
+        geo[G_IDMIN * n + p] = 1.0 / dmin;
         if (!swept(c, p)) continue;
         double det[4];
         for (int s = 0; s < 4; s++) {
@@ -814,13 +815,12 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
     const size_t esz = std::max<int64_t>(ell, 1);
     std::vector<int32_t> &enb = hp.enb;
     std::vector<uint8_t> &emb = hp.emb;
-    std::vector<double> &edx = hp.edx, &edy = hp.edy, &egx = hp.egx, &egy = hp.egy;
-    std::vector<uint2> &ew1 = hp.ew1, &ew2 = hp.ew2;
-    ew1.assign(esz, uint2{0, 0});
-    ew2.assign(esz, uint2{0, 0});
+    std::vector<double> &egx = hp.egx, &egy = hp.egy;
+    hp.ewq.assign(esz, uint4{0, 0, 0, 0});
+    hp.ehxy.assign(esz, double2{0.0, 0.0});
     enb.assign(esz, 0);
     emb.assign(esz, 0);
-    for (auto *v : {&edx, &edy, &egx, &egy, &hp.exx, &hp.exy, &hp.eyx, &hp.eyy}) v->assign(esz, 0.0);
+    for (auto *v : {&egx, &egy, &hp.exx, &hp.exy, &hp.eyx, &hp.eyy}) v->assign(esz, 0.0);
     for (int32_t k = 0; k < n; k++) {
         const int32_t p = c->perm[k];
         deg[k] = off[p + 1] - off[p];
@@ -831,10 +831,12 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
             const int64_t e = off[p] + j, t = base + 32 * j;
             enb[t] = c->inv[idx[e]];
             emb[t] = smb[e];
-            edx[t] = 0.5 * sdx[e];  // half offsets (exact): the residual's reconstruction
-            edy[t] = 0.5 * sdy[e];  // steps q - (dx, dy)/2 . grad q
-            ew1[t] = split_weight(sw1[e], geo[(size_t)G_WSC * n + p]);
-            ew2[t] = split_weight(sw2[e], geo[(size_t)G_WSC * n + p]);
+            // half offsets (exact): the residual's reconstruction steps
+            // q - (dx, dy)/2 . grad q
+            hp.ehxy[t] = double2{0.5 * sdx[e], 0.5 * sdy[e]};
+            const uint2 wa = split_weight(sw1[e], geo[(size_t)G_WSC * n + p]);
+            const uint2 wb = split_weight(sw2[e], geo[(size_t)G_WSC * n + p]);
+            hp.ewq[t] = uint4{wa.x, wa.y, wb.x, wb.y};
             egx[t] = swgx[e];
             egy[t] = swgy[e];
             hp.exx[t] = swgx[e] * sdx[e];
@@ -1035,8 +1037,8 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     const int32_t n = c->n, ld = c->ld, nsl = ld / 32;
     std::vector<int32_t> &slice_off = hp.slice_off, &deg = hp.deg, &enb = hp.enb;
     std::vector<uint8_t> &emb = hp.emb, &fl_i = hp.fl_i;
-    std::vector<double> &edx = hp.edx, &edy = hp.edy, &egx = hp.egx, &egy = hp.egy;
-    std::vector<uint2> &ew1 = hp.ew1, &ew2 = hp.ew2;
+    std::vector<double> &egx = hp.egx, &egy = hp.egy;
+    const size_t esz = egx.size();
     std::vector<double> &geo_i = hp.geo_i, &wnx = hp.wnx, &wny = hp.wny;
     // ---- device memory ----
     cudaError_t e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
@@ -1057,11 +1059,11 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     double *dgeo = A.alloc<double>((size_t)G_NFIELDS * ld);
     int32_t *dso = A.alloc<int32_t>(nsl + 1), *ddeg = A.alloc<int32_t>(n), *dnb = A.alloc<int32_t>(enb.size());
     uint8_t *dmb = A.alloc<uint8_t>(emb.size());
-    double *ddx = A.alloc<double>(edx.size()), *ddy = A.alloc<double>(edx.size());
-    uint2 *dw1 = A.alloc<uint2>(edx.size()), *dw2 = A.alloc<uint2>(edx.size());
-    double *dgx = A.alloc<double>(edx.size()), *dgy = A.alloc<double>(edx.size());
-    double *dxx = A.alloc<double>(edx.size()), *dxy = A.alloc<double>(edx.size());
-    double *dyx = A.alloc<double>(edx.size()), *dyy = A.alloc<double>(edx.size());
+    double2 *dhxy = A.alloc<double2>(esz);
+    uint4 *dwq = A.alloc<uint4>(esz);
+    double *dgx = A.alloc<double>(esz), *dgy = A.alloc<double>(esz);
+    double *dxx = A.alloc<double>(esz), *dxy = A.alloc<double>(esz);
+    double *dyx = A.alloc<double>(esz), *dyy = A.alloc<double>(esz);
     for (int s = 0; s < 2; s++) {
         d.set[s].U = A.alloc<double>(4 * (size_t)ld);
         d.set[s].q = A.alloc<double>(4 * (size_t)ld);
@@ -1188,7 +1190,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaDeviceGetAttribute");
-    c->launch.res_blocks = 2 * std::max(sms, 1);
+    c->launch.sms = std::max(sms, 1);
     c->launch.tpp = n >= 100000 ? 1 : (n >= 50000 ? 2 : (n >= 25000 ? 4 : 8));
     c->launch.sweep_lanes = 4;
     d.n_blk = (int32_t)hp.blk_case.size();
@@ -1218,10 +1220,8 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     d.deg = ddeg;
     d.nbr = dnb;
     d.memb = dmb;
-    d.nhx = ddx;
-    d.nhy = ddy;
-    d.wq1 = dw1;
-    d.wq2 = dw2;
+    d.hxy = dhxy;
+    d.wq = dwq;
     d.wgx = dgx;
     d.wgy = dgy;
     d.gxx = dxx;
@@ -1280,10 +1280,8 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     up(ddeg, deg.data(), n * sizeof(int32_t));
     up(dnb, enb.data(), enb.size() * sizeof(int32_t));
     up(dmb, emb.data(), emb.size());
-    up(ddx, edx.data(), edx.size() * sizeof(double));
-    up(ddy, edy.data(), edy.size() * sizeof(double));
-    up(dw1, ew1.data(), ew1.size() * sizeof(uint2));
-    up(dw2, ew2.data(), ew2.size() * sizeof(uint2));
+    up(dhxy, hp.ehxy.data(), esz * sizeof(double2));
+    up(dwq, hp.ewq.data(), esz * sizeof(uint4));
     up(dgx, egx.data(), egx.size() * sizeof(double));
     up(dgy, egy.data(), egy.size() * sizeof(double));
     up(dxx, hp.exx.data(), hp.exx.size() * sizeof(double));
@@ -1747,7 +1745,7 @@ lskum_status lskum_get_field(lskum_ctx *c, int32_t field, double *out)
     int comps = 4, stride = 0;
     switch (field) {
     case LSKUM_FIELD_U: src = d.set[c->cur].U; break;
-    case LSKUM_FIELD_Q: src = d.set[c->cur].q; break;
+    case LSKUM_FIELD_Q: src = d.set[c->cur].q; stride = 4; break;
     case LSKUM_FIELD_QX: src = d.gq[K]; stride = 8; break;
     case LSKUM_FIELD_QY: src = d.gq[K] + 4; stride = 8; break;
     case LSKUM_FIELD_R: src = d.R; break;
@@ -1781,7 +1779,7 @@ lskum_status lskum_get_field_dev(lskum_ctx *c, int32_t field, double *out_dev, v
     int comps = 4, stride = 0;
     switch (field) {
     case LSKUM_FIELD_U: src = d.set[c->cur].U; break;
-    case LSKUM_FIELD_Q: src = d.set[c->cur].q; break;
+    case LSKUM_FIELD_Q: src = d.set[c->cur].q; stride = 4; break;
     case LSKUM_FIELD_QX: src = d.gq[K]; stride = 8; break;
     case LSKUM_FIELD_QY: src = d.gq[K] + 4; stride = 8; break;
     case LSKUM_FIELD_R: src = d.R; break;

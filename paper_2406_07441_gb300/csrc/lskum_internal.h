@@ -55,7 +55,7 @@ enum GeoField {
     G_LS1_0, G_LS1_1, G_LS1_2, G_LS1_3,  // LS_s(1) of the four split sub-stencils (kinetic
                                          // outer points: LS_3(1) = -LS_2(1), the ghosts)
     G_ABS_0, G_ABS_1, G_ABS_2, G_ABS_3,  // sum_i |w_i| of each split sub-stencil
-    G_DMIN,                              // min_i |r_i - r_0|
+    G_IDMIN,                             // 1 / min_i |r_i - r_0|
     G_WSC,                               // unit of the residual's weights (a power of two)
     G_SXX, G_SXY, G_SYX, G_SYY,          // sums over the stencil of wgx dx, wgx dy, wgy dx, wgy dy
     G_NFIELDS
@@ -83,7 +83,7 @@ static_assert(P_NFIELDS <= kPrimStride, "prim record too small");
 
 struct StateSet {
     double *U;     // [4][ld] conserved variables
-    double *q;     // [4][ld] q-variables
+    double *q;     // [ld][4] q-variables (a neighbour's are one 32-byte gather)
     double *prim;  // [ld][kPrimStride]
     float *primf;  // [ld][kPrimStride] FP32 copy (mixed precision only, else null)
 };
@@ -99,11 +99,12 @@ struct Dev {
     const int32_t *deg;       // [n]
     const int32_t *nbr;       // neighbour (internal index)
     const uint8_t *memb;      // bits 0/1: e1 sub-stencil +/-, bits 2/3: e2 sub-stencil +/-
-    const double *nhx, *nhy;  // (x_i - x_0)/2, (y_i - y_0)/2
-    // LS weight of the slot in its e1 / e2 split sub-stencil (0 if none), in
-    // units of the point's G_WSC: x the nearest integer (int32; the sum of a
-    // point's |x| is below 2^30), y the remainder in units of 2^-24 (int32)
-    const uint2 *wq1, *wq2;
+    const double2 *hxy;       // (x_i - x_0)/2, (y_i - y_0)/2
+    // LS weights of the slot in its e1 / e2 split sub-stencils (0 if none), in
+    // units of the point's G_WSC: x, z the nearest integers (int32; the sum of
+    // a point's magnitudes is below 2^30), y, w the remainders in units of
+    // 2^-24 (int32)
+    const uint4 *wq;
     const double *wgx, *wgy;  // full-stencil LS weights of d/dx and d/dy (Eq. 10, 16)
     const double *gxx, *gxy, *gyx, *gyy;  // wgx dx, wgx dy, wgy dx, wgy dy (inner iterations)
     // iteration buffers
@@ -193,14 +194,15 @@ struct Dev {
 // this iteration; the update writes set 1 - cur.
 struct Launch {
     int tpp;          // threads per point of the gradient and residual kernels (1, 2, 4, 8)
-    int res_blocks;   // blocks of the residual kernel resident at once (its persistent grid)
+    int sms;          // multiprocessors (the residual's persistent grid)
     int sweep_lanes;  // lanes per point of the sweep kernels (2, 4, 8), or 32: the packed form
     const int32_t *pk_lw[2];  // packed form: host arrays [n_levels + 1], first framed-point warp of each level
     const int32_t *lp_lg[2];  // packed form: host arrays [n_levels + 1], first interior group of each level
-    // optional side branch of a captured iteration: the framed points'
-    // Jacobians (k_framed_jac) run on `side` between the `fork` after k_begin
-    // and the `join` before the forward sweep, beside the q-derivatives and
-    // the residual; null: inline, before the forward sweep
+    // optional side branch of a captured iteration: what depends only on the
+    // state (the framed points' Jacobians, the diagonals of the shapes with
+    // several residual lanes per point) runs on `side` between the `fork`
+    // after k_begin and the `join` before the forward sweep or explicit step,
+    // beside the q-derivatives and the residual; null: inline
     cudaStream_t side;
     cudaEvent_t fork, join;
 };

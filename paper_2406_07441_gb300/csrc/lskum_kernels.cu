@@ -391,6 +391,28 @@ __device__ __forceinline__ T group_sum(T v)
     return v;
 }
 
+// Four consecutive values from 16-byte-aligned storage (one point's product).
+__device__ __forceinline__ void load4(const double *__restrict__ p, double v[4])
+{
+    const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
+    v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
+__device__ __forceinline__ void load4(const float *__restrict__ p, float v[4])
+{
+    const float4 a = *reinterpret_cast<const float4 *>(p);
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+}
+
+__device__ __forceinline__ void store4(double *p, const double v[4])
+{
+    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
+}
+__device__ __forceinline__ void store4(float *p, const float v[4])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+}
+
 // ---------------------------------------------------------------------------
 // q-derivatives: first order (Eq. 10), then Jacobi inner iterations of Eq. 16
 // ---------------------------------------------------------------------------
@@ -415,7 +437,7 @@ __global__ void __launch_bounds__(256) k_grad(Dev d, const double *__restrict__ 
     double q0[4], sx[4], sy[4];
 #pragma unroll
     for (int c = 0; c < 4; c++) {
-        if (!CORR) q0[c] = q[c * ld + kk];
+        if (!CORR) q0[c] = q[4 * (size_t)kk + c];
         sx[c] = 0.0;
         sy[c] = 0.0;
     }
@@ -426,9 +448,11 @@ __global__ void __launch_bounds__(256) k_grad(Dev d, const double *__restrict__ 
         const int i = d.nbr[e];
         if (!CORR) {
             const double wx = d.wgx[e], wy = d.wgy[e];
+            double qi[4];
+            load4(q + 4 * (size_t)i, qi);
 #pragma unroll
             for (int c = 0; c < 4; c++) {
-                const double dq = q[c * ld + i] - q0[c];
+                const double dq = qi[c] - q0[c];
                 sx[c] = fma(wx, dq, sx[c]);
                 sy[c] = fma(wy, dq, sy[c]);
             }
@@ -494,18 +518,15 @@ __device__ __forceinline__ double zero_like(double x)
     return __hiloint2double(__double2hiint(x) & (int)0x80000000, 0);
 }
 
-// The modified q-variables of a slot (Eq. 15): neighbour i's and the point's
-// own, reconstructed over half the offset (hdx, hdy).
-__device__ __forceinline__ void reconstruct(const double *__restrict__ q, const double *__restrict__ g, int ld, int i,
+// The modified q-variables of a slot (Eq. 15): neighbour i's (q-variables q,
+// q-derivatives x and y) and the point's own, over half the offset (hdx, hdy).
+__device__ __forceinline__ void reconstruct(const double q[4], const double x[4], const double y[4],
                                             const double q0[4], const double gx0[4], const double gy0[4], double hdx,
                                             double hdy, double qi[4], double q0t[4])
 {
-    const double2 *gr = reinterpret_cast<const double2 *>(g + 8 * (size_t)i);
-    const double2 x01 = gr[0], x23 = gr[1], y01 = gr[2], y23 = gr[3];
-    const double gxi[4] = {x01.x, x01.y, x23.x, x23.y}, gyi[4] = {y01.x, y01.y, y23.x, y23.y};
 #pragma unroll
     for (int c = 0; c < 4; c++) {
-        qi[c] = fma(-hdx, gxi[c], fma(-hdy, gyi[c], q[c * ld + i]));
+        qi[c] = fma(-hdx, x[c], fma(-hdy, y[c], q[c]));
         q0t[c] = fma(-hdx, gx0[c], fma(-hdy, gy0[c], q0[c]));
     }
 }
@@ -524,23 +545,24 @@ __device__ __noinline__ void residual_fp64(const Dev &d, const double *__restric
     const double e2x = d.geo[G_E2X * ld + k], e2y = d.geo[G_E2Y * ld + k];
     const double wsc = d.geo[G_WSC * ld + k];
     double q0[4], gx0[4], gy0[4];
+    load4(q + 4 * (size_t)k, q0);
+    load4(g + 8 * (size_t)k, gx0);
+    load4(g + 8 * (size_t)k + 4, gy0);
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-        q0[c] = q[c * ld + k];
-        gx0[c] = g[8 * (size_t)k + c];
-        gy0[c] = g[8 * (size_t)k + 4 + c];
-        R[c] = 0.0;
-    }
+    for (int c = 0; c < 4; c++) R[c] = 0.0;
     const int deg = d.deg[k];
     const int base = d.slice_off[k >> 5] + (k & 31);
     for (int j = sub; j < deg; j += TPP) {
         const int e = base + 32 * j;
         const int mb = d.memb[e];
         if (!mb) continue;
-        const double hx = d.nhx[e], hy = d.nhy[e];
-        double qi[4], q0t[4];
-        reconstruct(q, g, ld, d.nbr[e], q0, gx0, gy0, second ? hx : zero_like(hx), second ? hy : zero_like(hy), qi,
-                    q0t);
+        const int i = d.nbr[e];
+        const double hx = d.hxy[e].x, hy = d.hxy[e].y;
+        double qn[4], xn[4], yn[4], qi[4], q0t[4];
+        load4(q + 4 * (size_t)i, qn);
+        load4(g + 8 * (size_t)i, xn);
+        load4(g + 8 * (size_t)i + 4, yn);
+        reconstruct(qn, xn, yn, q0, gx0, gy0, second ? hx : zero_like(hx), second ? hy : zero_like(hy), qi, q0t);
         const Prim Pi = q_to_prim(T, qi);
         const Prim P0 = q_to_prim(T, q0t);
 #pragma unroll 1
@@ -548,8 +570,8 @@ __device__ __noinline__ void residual_fp64(const Dev &d, const double *__restric
             const int m = sb == 0 ? (mb & 3) : (mb >> 2);
             if (!m) continue;
             const bool pos = m & 1, xdir = sb == 0;
-            const uint2 wq = xdir ? d.wq1[e] : d.wq2[e];
-            const double w = fma((double)(int)wq.y, 0x1p-24, (double)(int)wq.x) * wsc;
+            const uint4 wq = d.wq[e];
+            const double w = fma((double)(int)(xdir ? wq.y : wq.w), 0x1p-24, (double)(int)(xdir ? wq.x : wq.z)) * wsc;
             const double dx = xdir ? e1x : e2x, dy = xdir ? e1y : e2y;
             double Gi[4], G0[4];
             split_flux(T, Pi, framed, xdir, dx, dy, pos, Gi);
@@ -560,76 +582,107 @@ __device__ __noinline__ void residual_fp64(const Dev &d, const double *__restric
     }
 }
 
-// A point's residual complete (the ghost term of kinetic outer points added)
-// and stored, with its local time step and scalar diagonal.
-__device__ __forceinline__ void residual_point(const Dev &d, const StateSet &st, int k, int fl, double cfl, double e1x,
-                                               double e1y, double e2x, double e2y, double R[4])
+// The ghost term of a kinetic outer point: the n- side is free-stream ghosts
+// at the mirror images of the inside neighbours, LS_3(1) (G_n^-(U_inf) -
+// G_n^-(U_0)) with LS_3(1) = -LS_2(1); first order (the point's own state).
+__device__ __noinline__ void add_ghosts(const Dev &d, const double *__restrict__ U, int k, double e2x, double e2y,
+                                        double R[4])
 {
     const int ld = d.ld;
-    if (fl == kOuter) {
-        // kinetic far field: the n- side is free-stream ghosts at the mirror
-        // images of the inside neighbours, LS_3(1) (G_n^-(U_inf) - G_n^-(U_0))
-        // with LS_3(1) = -LS_2(1); first order (the point's own state)
-        const double *ui = d.case_uinf + 4 * d.case_of[k];
-        double U0[4], Ui[4];
-        bool same = true;
+    const double *ui = d.case_uinf + 4 * d.case_of[k];
+    double U0[4], Ui[4];
+    bool same = true;
 #pragma unroll
-        for (int c = 0; c < 4; c++) {
-            U0[c] = st.U[c * ld + k];
-            Ui[c] = ui[c];
-            same = same && U0[c] == Ui[c];
-        }
-        if (!same) {  // (equal states give exactly 0)
-            double Gi[4], G0[4];
-            flux_cons(g_math, Ui, e2x, e2y, false, Gi);
-            flux_cons(g_math, U0, e2x, e2y, false, G0);
-            const double l3 = d.geo[G_LS1_3 * ld + k];
+    for (int c = 0; c < 4; c++) {
+        U0[c] = U[c * ld + k];
+        Ui[c] = ui[c];
+        same = same && U0[c] == Ui[c];
+    }
+    if (same) return;  // (equal states give exactly 0)
+    double Gi[4], G0[4];
+    flux_cons(g_math, Ui, e2x, e2y, false, Gi);
+    flux_cons(g_math, U0, e2x, e2y, false, G0);
+    const double l3 = d.geo[G_LS1_3 * ld + k];
 #pragma unroll
-            for (int c = 0; c < 4; c++) R[c] = fma(l3, Gi[c] - G0[c], R[c]);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; c++) d.R[c * ld + k] = R[c];
-    // local time step (reading: CFL min_i|dr| / (|u| + a)) and the scalar
-    // diagonal of Eq. 26 with the spectral radii of Eq. 34, kept at least
-    // sum_s rho_s sum_i |w_i| so that it bounds the off-diagonal blocks
-    const double *pr = st.prim + (size_t)k * kPrimStride;
-    const double u = pr[P_U], v = pr[P_V];
-    const double a = sqrt(1.4 * pr[P_P] * pr[P_IRHO]);
-    const double dt = cfl * d.geo[G_DMIN * ld + k] / (sqrt(u * u + v * v) + a);
-    // D and 1/D: the sweeps multiply by 1/D (one division per point here
-    // instead of one per point in each sweep)
-    if (d.scheme == 1) {  // explicit: D = 1/dt, the step is -dt R
-        d.D[k] = 1.0 / dt;
-        d.iD[k] = dt;
-        return;
-    }
-    if (d.lusgs == 1) {  // revised LU-SGS: Jameson's splitting, rho(A_d) = |u_d| + a
-        const double u1 = fabs(u * e1x + v * e1y) + a, u2 = fabs(u * e2x + v * e2y) + a;
-        const double Dm = 1.0 / dt +
-                          0.5 * (u1 * (fabs(d.geo[G_LS1_0 * ld + k]) + fabs(d.geo[G_LS1_1 * ld + k])) +
-                                 u2 * (fabs(d.geo[G_LS1_2 * ld + k]) + fabs(d.geo[G_LS1_3 * ld + k])));
-        d.D[k] = Dm;
-        d.iD[k] = 1.0 / Dm;
-        return;
-    }
-    double Dp = 1.0 / dt, Ddom = 0.0;
-    const double u1 = u * e1x + v * e1y, u2 = u * e2x + v * e2y;
-    const double r0 = fmax(u1 + a, 0.0), r1 = fmax(a - u1, 0.0);
-    const double r2 = fmax(u2 + a, 0.0), r3 = fmax(a - u2, 0.0);
-    Dp -= r0 * d.geo[G_LS1_0 * ld + k];
-    Dp += r1 * d.geo[G_LS1_1 * ld + k];
-    Dp -= r2 * d.geo[G_LS1_2 * ld + k];
-    Dp += r3 * d.geo[G_LS1_3 * ld + k];
-    Ddom = r0 * d.geo[G_ABS_0 * ld + k] + r1 * d.geo[G_ABS_1 * ld + k] + r2 * d.geo[G_ABS_2 * ld + k]
-         + r3 * d.geo[G_ABS_3 * ld + k];
-    const double Da = Dp > Ddom ? Dp : Ddom;
-    d.D[k] = Da;
-    d.iD[k] = 1.0 / Da;
+    for (int c = 0; c < 4; c++) R[c] = fma(l3, Gi[c] - G0[c], R[c]);
 }
 
-// Threads per block of the residual (two blocks per SM share its registers).
-constexpr int kResBlock = 256;
+// x, or 0 where x is negative, on the integer pipe.
+__device__ __forceinline__ double positive_part(double x)
+{
+    const int m = ~(__double2hiint(x) >> 31);
+    return __hiloint2double(__double2hiint(x) & m, __double2loint(x) & m);
+}
+
+// Local time step (reading: CFL min_i|dr| / (|u| + a)) and scalar diagonal of
+// point k: Eq. 26 with the spectral radii of Eq. 34, kept at least sum_s
+// rho_s sum_i |w_i| so that it bounds the off-diagonal blocks.  D and 1/D are
+// stored (the sweeps multiply by 1/D).  One square root and one division: a
+// from the record's 1/sqrt(beta) (a^2 = 0.7/beta), 1/min|dr| stored.
+__device__ __forceinline__ void diag_point(const Dev &d, const StateSet &st, int k, double cfl, double e1x, double e1y,
+                                           double e2x, double e2y)
+{
+    const int ld = d.ld;
+    const double *pr = st.prim + (size_t)k * kPrimStride;
+    const double u = pr[P_U], v = pr[P_V];
+    const double a = 0.83666002653407554798 * pr[P_ISB];  // sqrt(0.7 / beta)
+    const double idt = (sqrt(pr[P_Q2]) + a) * d.geo[G_IDMIN * ld + k] * (1.0 / cfl);
+    if (d.scheme == 1) {  // explicit: D = 1/dt, the step is -dt R
+        d.D[k] = idt;
+        d.iD[k] = 1.0 / idt;
+        return;
+    }
+    const double u1 = u * e1x + v * e1y, u2 = u * e2x + v * e2y;
+    double D = idt;
+    if (d.lusgs == 1) {  // revised LU-SGS: Jameson's splitting, rho(A_d) = |u_d| + a
+        const double s1 = fabs(u1) + a, s2 = fabs(u2) + a;
+        D += 0.5 * (s1 * (fabs(d.geo[G_LS1_0 * ld + k]) + fabs(d.geo[G_LS1_1 * ld + k])) +
+                    s2 * (fabs(d.geo[G_LS1_2 * ld + k]) + fabs(d.geo[G_LS1_3 * ld + k])));
+    } else {
+        const double r0 = positive_part(u1 + a), r1 = positive_part(a - u1);
+        const double r2 = positive_part(u2 + a), r3 = positive_part(a - u2);
+        D -= r0 * d.geo[G_LS1_0 * ld + k];
+        D += r1 * d.geo[G_LS1_1 * ld + k];
+        D -= r2 * d.geo[G_LS1_2 * ld + k];
+        D += r3 * d.geo[G_LS1_3 * ld + k];
+        const double dom = r0 * d.geo[G_ABS_0 * ld + k] + r1 * d.geo[G_ABS_1 * ld + k] + r2 * d.geo[G_ABS_2 * ld + k] +
+                           r3 * d.geo[G_ABS_3 * ld + k];
+        D = D > dom ? D : dom;
+    }
+    d.D[k] = D;
+    d.iD[k] = 1.0 / D;
+}
+
+// The CFL number of this iteration (counted by k_begin).
+__device__ __forceinline__ double cfl_now(const Dev &d, int n1)
+{
+    return (d.ramp > 0.0 && (double)n1 < d.ramp) ? d.cfl * ((double)n1 / d.ramp) : d.cfl;
+}
+
+// Diagonals of all swept points, a thread per point, for the launch shapes
+// with several lanes per point in the residual: there a warp holds few
+// points, and its FP64 sequence per point (about 45 instructions) would cost
+// more than the fluxes it follows.  It needs only the state, so a captured
+// iteration runs it beside the q-derivatives and the residual.
+__global__ void __launch_bounds__(256) k_diag(Dev d, StateSet st)
+{
+    if (halted(d.ctrl)) return;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= d.n) return;
+    const int fl = d.flag[k];
+    if ((fl == kOuter && d.farfield != 1) || frozen(d, k)) return;
+    double e1x, e1y, e2x, e2y;
+    point_frame(d, k, fl != kInterior, e1x, e1y, e2x, e2y);
+    diag_point(d, st, k, cfl_now(d, ((const volatile Ctrl *)d.ctrl)->it), e1x, e1y, e2x, e2y);
+}
+
+// Threads per block of the residual: 512 threads share an SM's registers and
+// one copy of the tables (one lane per point: 0.229 ms on 147,584 points
+// against 0.237 with two blocks of 256); with several lanes per point, the
+// shapes of small clouds, two blocks of 256 spread the work over more SMs
+// (10,240 points, two lanes: 0.032 ms against 0.038).
+template <int TPP>
+constexpr int kResBlock = TPP == 1 ? 512 : 256;
 
 // Flux residual, local time step and scalar diagonal; TPP lanes per point
 // over its slots, persistent blocks (a warp takes every W-th group of 32/TPP
@@ -642,55 +695,71 @@ constexpr int kResBlock = 256;
 // into its frame, where every split flux is along an axis, and the sum's
 // momentum back out of it.  Measured on the 147,584-point cloud (1 lane per
 // point): 0.649 ms with the fluxes in FP64 and integer-pipe multiplies, 0.693
-// ms with compensated sums; 0.266 ms like this, FMA-heavy pipe 57 % and FP64
-// unit 55 % busy, the rest latency (4 warps per scheduler: 128 registers).
+// ms with compensated sums; 0.229 ms like this (41,194 points, four lanes:
+// 0.235 -> 0.097 ms).  The FMA-heavy pipe, which runs the 32-bit multiplies,
+// is about 60 % busy; four warps per scheduler (128 registers) do not hide
+// the rest of the chains' latency.  Staging the next slot's records in shared
+// memory, prefetching them, and a lane per state with more warps were slower.
 template <int TPP>
-__global__ void __launch_bounds__(kResBlock, 2) k_residual(Dev d, StateSet st, const double *__restrict__ g)
+__global__ void __launch_bounds__(kResBlock<TPP>, 512 / kResBlock<TPP>)
+    k_residual(Dev d, StateSet st, const double *__restrict__ g)
 {
     __shared__ __align__(16) uint64_t T[kFluxTableWords];
     if (halted(d.ctrl)) return;
     static_assert(kFluxTableR == kFluxRows && kFluxTableExp == kFluxExpRows && kFluxTableWords % 2 == 0, "tables");
-    for (int i = threadIdx.x; i < kFluxTableWords / 2; i += kResBlock)
+    for (int i = threadIdx.x; i < kFluxTableWords / 2; i += kResBlock<TPP>)
         reinterpret_cast<ulonglong2 *>(T)[i] = reinterpret_cast<const ulonglong2 *>(kFluxTable)[i];
     __syncthreads();
     const int n1 = ((const volatile Ctrl *)d.ctrl)->it;  // this iteration, counted by k_begin
-    const double cfl = (d.ramp > 0.0 && (double)n1 < d.ramp) ? d.cfl * ((double)n1 / d.ramp) : d.cfl;
     const bool second = n1 > d.first_order;  // first-order start: q~ = q
     const int ld = d.ld;
     const double *__restrict__ q = st.q;
     constexpr int kPts = 32 / TPP;
     const int lane = threadIdx.x & 31, sub = lane % TPP;
     const int tasks = (d.n + kPts - 1) / kPts;
-    for (int task = (blockIdx.x * kResBlock + threadIdx.x) / 32; task < tasks; task += gridDim.x * (kResBlock / 32)) {
+    for (int task = (blockIdx.x * kResBlock<TPP> + threadIdx.x) / 32; task < tasks;
+         task += gridDim.x * (kResBlock<TPP> / 32)) {
         const int k = task * kPts + lane / TPP;
         const bool active = k < d.n;
         const int kk = active ? k : d.n - 1;
         const int fl = d.flag[kk];
         const bool work = active && (fl != kOuter || d.farfield == 1) && !frozen(d, kk);
         const bool framed = fl != kInterior;  // (t, n) frame: wall and kinetic outer points
-        double e1x, e1y, e2x, e2y;
-        point_frame(d, kk, framed, e1x, e1y, e2x, e2y);
         FxSum acc[4] = {};
         uint32_t bad = 0;
         if (work) {
             double q0[4], gx0[4], gy0[4];
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                q0[c] = q[c * ld + kk];
-                gx0[c] = g[8 * (size_t)kk + c];
-                gy0[c] = g[8 * (size_t)kk + 4 + c];
-            }
+            load4(q + 4 * (size_t)kk, q0);
+            load4(g + 8 * (size_t)kk, gx0);
+            load4(g + 8 * (size_t)kk + 4, gy0);
             const int deg = d.deg[kk];
-            const int base = d.slice_off[kk >> 5] + (kk & 31);
-            for (int j = sub; j < deg; j += TPP) {
-                const int e = base + 32 * j;
-                const int mb = d.memb[e];
-                if (!mb) continue;
-                const double hx = d.nhx[e], hy = d.nhy[e];  // half offsets
-                double qi[4], q0t[4];
-                reconstruct(q, g, ld, d.nbr[e], q0, gx0, gy0, second ? hx : zero_like(hx),
-                            second ? hy : zero_like(hy), qi, q0t);
-                if (framed) {
+            int e = d.slice_off[kk >> 5] + (kk & 31) + 32 * sub;
+            int in = kk, mn = 0;
+            if (sub < deg) {
+                in = d.nbr[e];
+                mn = d.memb[e];
+            }
+            for (int j = sub; j < deg; j += TPP, e += 32 * TPP) {
+                const int i = in, m = mn;
+                if (j + TPP < deg) {  // the next slot's index before this slot's work
+                    in = d.nbr[e + 32 * TPP];
+                    mn = d.memb[e + 32 * TPP];
+                }
+                if (!m) continue;
+                double qn[4], xn[4], yn[4], qi[4], q0t[4];
+                load4(q + 4 * (size_t)i, qn);
+                load4(g + 8 * (size_t)i, xn);
+                load4(g + 8 * (size_t)i + 4, yn);
+                const double2 h = d.hxy[e];  // half offsets
+                const uint4 wq = d.wq[e];
+                reconstruct(qn, xn, yn, q0, gx0, gy0, second ? h.x : zero_like(h.x),
+                            second ? h.y : zero_like(h.y), qi, q0t);
+                // (a loop of at most one pass: as a predicated sequence this would
+                // occupy the FP64 unit at every interior point too)
+#pragma unroll 1
+                for (int r = 0; r < (int)framed; r++) {
+                    const double e1x = d.geo[G_E1X * ld + kk], e1y = d.geo[G_E1Y * ld + kk];
+                    const double e2x = d.geo[G_E2X * ld + kk], e2y = d.geo[G_E2Y * ld + kk];
                     const double a = qi[1], b = q0t[1];
                     qi[1] = fma(a, e1x, qi[2] * e1y);
                     qi[2] = fma(a, e2x, qi[2] * e2y);
@@ -700,25 +769,23 @@ __global__ void __launch_bounds__(kResBlock, 2) k_residual(Dev d, StateSet st, c
                 FxState si, s0;
                 fx_state(T, qi[0], qi[1], qi[2], qi[3], si, bad);
                 fx_state(T, q0t[0], q0t[1], q0t[2], q0t[3], s0, bad);
-                if (mb & 3) {
-                    const uint2 w = d.wq1[e];
-                    const bool pos = mb & 1;
+                if (m & 3) {
+                    const bool pos = m & 1;
                     FxFlux Gi, G0;
                     fx_flux(T, si, si.u, si.su, si.v, si.sv, pos, Gi, bad);
                     fx_flux(T, s0, s0.u, s0.su, s0.v, s0.sv, pos, G0, bad);
-                    const int wh = (int)w.x, wl = (int)w.y, sh = pos ? wh : -wh, sl = pos ? wl : -wl;
+                    const int wh = (int)wq.x, wl = (int)wq.y, sh = pos ? wh : -wh, sl = pos ? wl : -wl;
                     fx_add(acc[0], sh, sl, Gi.rm, G0.rm);
                     fx_add(acc[1], wh, wl, Gi.ga, G0.ga);
                     fx_add(acc[2], sh, sl, Gi.go, G0.go);
                     fx_add(acc[3], sh, sl, Gi.g3, G0.g3);
                 }
-                if (mb & 12) {
-                    const uint2 w = d.wq2[e];
-                    const bool pos = mb & 4;
+                if (m & 12) {
+                    const bool pos = m & 4;
                     FxFlux Gi, G0;
                     fx_flux(T, si, si.v, si.sv, si.u, si.su, pos, Gi, bad);
                     fx_flux(T, s0, s0.v, s0.sv, s0.u, s0.su, pos, G0, bad);
-                    const int wh = (int)w.x, wl = (int)w.y, sh = pos ? wh : -wh, sl = pos ? wl : -wl;
+                    const int wh = (int)wq.z, wl = (int)wq.w, sh = pos ? wh : -wh, sl = pos ? wl : -wl;
                     fx_add(acc[0], sh, sl, Gi.rm, G0.rm);
                     fx_add(acc[2], wh, wl, Gi.ga, G0.ga);
                     fx_add(acc[1], sh, sl, Gi.go, G0.go);
@@ -726,6 +793,8 @@ __global__ void __launch_bounds__(kResBlock, 2) k_residual(Dev d, StateSet st, c
                 }
             }
         }
+        double e1x, e1y, e2x, e2y;
+        point_frame(d, kk, framed, e1x, e1y, e2x, e2y);
         double R[4];
 #pragma unroll
         for (int c = 0; c < 4; c++) {
@@ -752,7 +821,12 @@ __global__ void __launch_bounds__(kResBlock, 2) k_residual(Dev d, StateSet st, c
                 if (slow) R[c] = Rs[c];
             }
         }
-        if (work && sub == 0) residual_point(d, st, k, fl, cfl, e1x, e1y, e2x, e2y, R);
+        if (work && sub == 0) {
+            if (fl == kOuter) add_ghosts(d, st.U, k, e2x, e2y, R);
+#pragma unroll
+            for (int c = 0; c < 4; c++) d.R[c * ld + k] = R[c];
+            if (TPP == 1) diag_point(d, st, k, cfl_now(d, n1), e1x, e1y, e2x, e2y);  // else k_diag
+        }
     }
 }
 
@@ -1038,28 +1112,6 @@ __global__ void __launch_bounds__(256) k_sweep(Dev d, StateSet st, int lb, int l
     for (int c = 0; c < 4; c++) acc[c] = group_sum<G>(acc[c]);
     T w[4];
     if (live && sub == 0) sweep_point<FWD, T>(d, st, sb, k, wall, e1x, e1y, e2x, e2y, acc, w);
-}
-
-// Four consecutive values from 16-byte-aligned storage (one point's product).
-__device__ __forceinline__ void load4(const double *__restrict__ p, double v[4])
-{
-    const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
-    v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
-}
-__device__ __forceinline__ void load4(const float *__restrict__ p, float v[4])
-{
-    const float4 a = *reinterpret_cast<const float4 *>(p);
-    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
-}
-
-__device__ __forceinline__ void store4(double *p, const double v[4])
-{
-    reinterpret_cast<double2 *>(p)[0] = make_double2(v[0], v[1]);
-    reinterpret_cast<double2 *>(p)[1] = make_double2(v[2], v[3]);
-}
-__device__ __forceinline__ void store4(float *p, const float v[4])
-{
-    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
 }
 
 // Axis product cb (0: x+, 1: x-, 2: y+, 3: y-) of point k's new increment w
@@ -1444,10 +1496,12 @@ __global__ void __launch_bounds__(256) k_update(Dev d, int cur, bool inc, bool p
 #pragma unroll
     for (int c = 0; c < 4; c++) dst.U[c * ld + k] = U[c];
     // q1 = ln rho + 2.5 ln beta - beta |u|^2 with one logarithm: ln(rho beta^2 sqrt(beta))
-    dst.q[0 * ld + k] = fma(-P.beta, P.q2, log(mul_i(mul_i(P.rho, mul_i(P.beta, P.beta)), P.sb)));
-    dst.q[1 * ld + k] = mul_i(twice(P.beta), P.u);
-    dst.q[2 * ld + k] = mul_i(twice(P.beta), P.v);
-    dst.q[3 * ld + k] = signed_by(twice(P.beta), false);
+    double qn[4];
+    qn[0] = fma(-P.beta, P.q2, log(mul_i(mul_i(P.rho, mul_i(P.beta, P.beta)), P.sb)));
+    qn[1] = mul_i(twice(P.beta), P.u);
+    qn[2] = mul_i(twice(P.beta), P.v);
+    qn[3] = signed_by(twice(P.beta), false);
+    store4(dst.q + 4 * (size_t)k, qn);
     // the per-point record, assembled in registers and stored as 16-byte
     // vectors (and, in mixed precision, its FP32 copy from the same registers)
     double rec[P_NFIELDS];
@@ -1533,7 +1587,7 @@ __global__ void __launch_bounds__(256) k_repair(Dev d, int cur)
 #pragma unroll
     for (int c = 0; c < 4; c++) {
         dst.U[c * ld + k] = src.U[c * ld + k];
-        dst.q[c * ld + k] = src.q[c * ld + k];
+        dst.q[4 * (size_t)k + c] = src.q[4 * (size_t)k + c];
     }
     for (int f = 0; f < kPrimStride; f++) dst.prim[(size_t)k * kPrimStride + f] = src.prim[(size_t)k * kPrimStride + f];
     if (src.primf)
@@ -1578,8 +1632,9 @@ template <int TPP>
 cudaError_t enqueue_res(const Dev &d, const Launch &L, int cur, cudaStream_t s, int *launches)
 {
     const int fin = d.K & 1;
-    const int want = (d.n * TPP + kResBlock - 1) / kResBlock;
-    k_residual<TPP><<<want < L.res_blocks ? want : L.res_blocks, kResBlock, 0, s>>>(d, d.set[cur], d.gq[fin]);
+    constexpr int block = kResBlock<TPP>;
+    const int want = (d.n * TPP + block - 1) / block, most = L.sms * (512 / block);
+    k_residual<TPP><<<want < most ? want : most, block, 0, s>>>(d, d.set[cur], d.gq[fin]);
     (*launches)++;
     return cudaGetLastError();
 }
@@ -1648,15 +1703,18 @@ void enqueue_framed_jac(const Dev &d, int cur, cudaStream_t s, int *launches)
     (*launches)++;
 }
 
+void enqueue_diag(const Dev &d, int cur, cudaStream_t s, int *launches)
+{
+    k_diag<<<(d.n + 255) / 256, 256, 0, s>>>(d, d.set[cur]);
+    (*launches)++;
+}
+
 template <int JVP>
 void enqueue_sweeps_packed(const Dev &d, const Launch &L, int cur, int n_levels, cudaStream_t s, int *launches,
                            bool fwd, bool bwd)
 {
     const StateSet st = d.set[cur];
-    if (fwd && needs_framed_jac(d, L)) {
-        if (L.side) cudaStreamWaitEvent(s, L.join, 0);  // formed on the side branch
-        else enqueue_framed_jac(d, cur, s, launches);
-    }
+    if (fwd && !L.side && needs_framed_jac(d, L)) enqueue_framed_jac(d, cur, s, launches);
     for (int l = 0; fwd && l < n_levels; l++) {
         const int wb = L.pk_lw[0][l], wf = L.pk_lw[0][l + 1] - wb;
         const int g0 = L.lp_lg[0][l], ng = L.lp_lg[0][l + 1] - g0;
@@ -1699,22 +1757,26 @@ cudaError_t enqueue_sweeps(const Dev &d, const Launch &L, int cur, int n_levels,
 cudaError_t enqueue_phase(const Dev &d, const Launch &L, int cur, int ph, int n_levels, const int32_t *lvl_beg,
                           const int32_t *lvl_act_end, const int32_t *lvl_end, cudaStream_t s, int *launches)
 {
+    const bool side = L.side && (needs_framed_jac(d, L) || L.tpp > 1);
     switch (ph) {
     case 0:
         k_begin<<<1, 1, 0, s>>>(d.ctrl);
         (*launches)++;
-        if (L.side && needs_framed_jac(d, L)) {
-            // the framed points' Jacobians depend only on the state: a side
-            // branch beside the q-derivatives and the residual
+        if (side) {
+            // what depends only on the state: a side branch beside the
+            // q-derivatives and the residual
             cudaError_t e = cudaEventRecord(L.fork, s);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(L.side, L.fork, 0);
             if (e != cudaSuccess) return e;
-            enqueue_framed_jac(d, cur, L.side, launches);
+            if (needs_framed_jac(d, L)) enqueue_framed_jac(d, cur, L.side, launches);
+            if (L.tpp > 1) enqueue_diag(d, cur, L.side, launches);
             e = cudaEventRecord(L.join, L.side);
             if (e != cudaSuccess) return e;
         }
         return enqueue_grad_res(d, L, cur, s, launches, true, false);
-    case 1: return enqueue_grad_res(d, L, cur, s, launches, false, true);
+    case 1:
+        if (!side && L.tpp > 1) enqueue_diag(d, cur, s, launches);
+        return enqueue_grad_res(d, L, cur, s, launches, false, true);
     case 2:
         k_norm_partials<<<d.n_blk, 256, 0, s>>>(d);
         k_norm_cases<<<d.n_cases, 256, 0, s>>>(d);
@@ -1722,6 +1784,10 @@ cudaError_t enqueue_phase(const Dev &d, const Launch &L, int cur, int ph, int n_
         return cudaGetLastError();
     case 3:
     case 4:
+        if (ph == 3 && side) {
+            cudaError_t e = cudaStreamWaitEvent(s, L.join, 0);
+            if (e != cudaSuccess) return e;
+        }
         if (d.scheme == 1) {  // explicit: one step kernel instead of the two sweeps
             if (ph == 3) {
                 k_explicit<<<(d.n + 255) / 256, 256, 0, s>>>(d);
