@@ -64,6 +64,7 @@ struct lskum_ctx {
     std::vector<int32_t> lvl_beg, lvl_act_end, lvl_end;
     std::vector<int32_t> pk_lw[2];      // packed sweeps: first framed-point warp of each level (+ total), per direction
     std::vector<int32_t> lp_lg[2];      // packed sweeps: first interior group of each level (+ total), per direction
+    std::vector<int32_t> lvl_lanes;     // packed sweeps: lanes per interior point of each level (2 or 4)
     bool pk_ok = false;                 // packed sweeps available (every list <= 32 slots)
     // device
     Arena arena;
@@ -229,12 +230,11 @@ struct HostPrep {
     std::vector<int32_t> pk_pt[2], pk_nbr[2];
     std::vector<uint8_t> pk_mb[2], pk_steps[2];
     std::vector<double> pk_w1[2], pk_w2[2];
-    // interior points in lane-per-point groups of 32 (thread t of group g:
-    // point lp_k[32 g + t], -1 for none, with lp_len[32 g + t] slots at
-    // lp_goff[g] + 32 j + t)
-    std::vector<int32_t> lp_k[2], lp_len[2], lp_goff[2], lp_nbr[2];
-    std::vector<uint8_t> lp_mb[2];
-    std::vector<double> lp_w1[2], lp_w2[2];
+    std::vector<int32_t> pk_k[2];
+    // interior points in groups (lskum_internal.h: lp_k, ...)
+    std::vector<int32_t> lp_k[2], lp_len[2], lp_goff[2];
+    std::vector<uint32_t> lp_nm[2];
+    std::vector<double2> lp_w[2];
 };
 static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &hp);
 
@@ -425,11 +425,12 @@ static lskum_status verify_layout(lskum_ctx *c, const lskum_cloud *cl, const Hos
         }
         // interior groups: sizes, and every lane's list inside its group's slots
         const std::vector<int32_t> &lg = c->lp_lg[dir], &lk = hp.lp_k[dir], &ll = hp.lp_len[dir];
-        const std::vector<int32_t> &go = hp.lp_goff[dir], &lnb = hp.lp_nbr[dir];
-        if ((int32_t)lg.size() != c->n_levels + 1 || lg[0] != 0 || (size_t)lg.back() * kPointsPerWarp != lk.size() ||
+        const std::vector<int32_t> &go = hp.lp_goff[dir];
+        const std::vector<uint32_t> &lnm = hp.lp_nm[dir];
+        if ((int32_t)lg.size() != c->n_levels + 1 || lg[0] != 0 || (size_t)lg.back() * kGroupPoints != lk.size() ||
+            (int32_t)c->lvl_lanes.size() != c->n_levels ||
             ll.size() != lk.size() || go.size() != (size_t)lg.back() + 1 || go[0] != 0 ||
-            (size_t)go.back() != lnb.size() || hp.lp_mb[dir].size() != lnb.size() ||
-            hp.lp_w1[dir].size() != lnb.size() || hp.lp_w2[dir].size() != lnb.size())
+            (size_t)go.back() != lnm.size() || hp.lp_w[dir].size() != lnm.size() || hp.pk_k[dir].size() != pt.size())
             return fail(c, LSKUM_ERR_ARG, "layout: interior groups size");
         std::vector<int32_t> pos_of(n, -1);  // sweep position of each swept point
         for (int32_t l = 0; l < c->n_levels; l++)
@@ -439,6 +440,8 @@ static lskum_status verify_layout(lskum_ctx *c, const lskum_cloud *cl, const Hos
         for (int32_t l = 0; l < c->n_levels; l++) {
             for (int64_t t = (int64_t)lw[l] * 32; t < (int64_t)lw[l + 1] * 32; t++) {
                 const int32_t pos = pt[t];
+                if (hp.pk_k[dir][t] != (pos < 0 ? -1 : so[pos]))
+                    return fail(c, LSKUM_ERR_ARG, "layout: packed slot %lld", (long long)t);
                 if (pos < 0) continue;
                 if (pos < c->lvl_beg[l] || pos >= c->lvl_act_end[l] || nb[t] < 0 || nb[t] >= n)
                     return fail(c, LSKUM_ERR_ARG, "layout: packed slot %lld", (long long)t);
@@ -457,20 +460,22 @@ static lskum_status verify_layout(lskum_ctx *c, const lskum_cloud *cl, const Hos
                 if (go[g + 1] < go[g] || (go[g + 1] - go[g]) % 32 != 0)
                     return fail(c, LSKUM_ERR_ARG, "layout: interior group %lld", (long long)g);
                 const int32_t width = (go[g + 1] - go[g]) / 32;
-                constexpr int L = kLanesPerPoint;
-                for (int32_t t = 0; t < kPointsPerWarp; t++) {
-                    const int32_t k = lk[(int64_t)kPointsPerWarp * g + t];
+                const int L = c->lvl_lanes[l];
+                if (L != 2 && L != 4) return fail(c, LSKUM_ERR_ARG, "layout: lanes of level %d", l);
+                for (int32_t t = 0; t < kGroupPoints; t++) {
+                    const int32_t k = lk[(int64_t)kGroupPoints * g + t];
                     if (k < 0) continue;
-                    if (k >= n || c->flag[c->perm[k]] != LSKUM_INTERIOR)
+                    if (t >= 32 / L || k >= n || c->flag[c->perm[k]] != LSKUM_INTERIOR)
                         return fail(c, LSKUM_ERR_ARG, "layout: interior group %lld", (long long)g);
                     const int32_t pos = pos_of[k], len = loff[k + 1] - loff[k];
                     if (pos < c->lvl_beg[l] || pos >= c->lvl_act_end[l] || seen_pos[pos]++)
                         return fail(c, LSKUM_ERR_ARG, "layout: interior point %d", k);
-                    if (ll[(int64_t)kPointsPerWarp * g + t] != len || (len + L - 1) / L > width)
+                    if (ll[(int64_t)kGroupPoints * g + t] != len || (len + L - 1) / L > width)
                         return fail(c, LSKUM_ERR_ARG, "layout: interior list of point %d", k);
                     for (int32_t j = 0; j < len; j++) {
                         const int64_t e = go[g] + 32 * (int64_t)(j / L) + L * t + j % L;
-                        if (lnb[e] != lnbr[loff[k] + j] || lnb[e] < 0 || lnb[e] >= n)
+                        const int32_t i = (int32_t)(lnm[e] & 0x0fffffffu);
+                        if (i != lnbr[loff[k] + j] || i >= n || lnm[e] >> 28 == 0)
                             return fail(c, LSKUM_ERR_ARG, "layout: interior list of point %d", k);
                     }
                 }
@@ -886,13 +891,20 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
     //   point with an empty list takes one slot with membership 0), a point
     //   never straddling two warps;
     // - interior points, which gather their neighbours' stored axis products:
-    //   kLanesPerPoint lanes per point, in groups of kPointsPerWarp points in
-    //   sweep order (decreasing list length), each group's lists in ELL
-    //   layout (slot j of point p at lp_goff[g] + 32 (j / L) + L p + j % L,
-    //   L = kLanesPerPoint).
-    c->pk_ok = true;
+    //   L lanes per point (lvl_lanes), in groups of 32 / L points in sweep order
+    //   (decreasing list length), each group's lists in ELL layout (slot j of
+    //   point p at lp_goff[g] + 32 (j / L) + L p + j % L).
+    // the packed entries hold a point's index in 28 bits (2^28 points would not
+    // fit the GPU's memory)
+    c->pk_ok = n < (1 << 28);
     for (int32_t k = 0; k < n; k++)
         if (hp.lo_off[k + 1] - hp.lo_off[k] > 32 || hp.up_off[k + 1] - hp.up_off[k] > 32) c->pk_ok = false;
+    c->lvl_lanes.assign(c->n_levels, 4);
+    for (int32_t l = 0; l < c->n_levels; l++) {
+        int32_t inner = 0;
+        for (int32_t k = c->lvl_beg[l]; k < c->lvl_act_end[l]; k++) inner += c->flag[c->perm[k]] == LSKUM_INTERIOR;
+        if (inner > kWideLevel) c->lvl_lanes[l] = 2;
+    }
     for (int dir = 0; dir < 2 && c->pk_ok; dir++) {
         const std::vector<int32_t> &so = dir == 0 ? hp.sw_fwd : hp.sw_bwd;
         const std::vector<int32_t> &loff = dir == 0 ? hp.lo_off : hp.up_off;
@@ -965,12 +977,13 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
             }
             nw += (int32_t)members.size();
             lw.push_back(nw);
-            // interior points: groups of kPointsPerWarp points, ELL lists
-            constexpr int L = kLanesPerPoint;
-            for (size_t g0 = 0; g0 < inner.size(); g0 += kPointsPerWarp) {
+            // interior points: groups of 32 / L points, ELL lists
+            const int L = c->lvl_lanes[l];
+            const size_t per = 32 / L;
+            for (size_t g0 = 0; g0 < inner.size(); g0 += per) {
                 int32_t width = 0;  // rows of 32 slots
-                for (size_t t = 0; t < (size_t)kPointsPerWarp; t++) {
-                    const int32_t k = g0 + t < inner.size() ? inner[g0 + t] : -1;
+                for (size_t t = 0; t < (size_t)kGroupPoints; t++) {
+                    const int32_t k = t < per && g0 + t < inner.size() ? inner[g0 + t] : -1;
                     const int32_t len = k >= 0 ? loff[k + 1] - loff[k] : 0;
                     hp.lp_k[dir].push_back(k);
                     hp.lp_len[dir].push_back(len);
@@ -978,18 +991,14 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
                 }
                 const int32_t base = hp.lp_goff[dir].back();
                 hp.lp_goff[dir].push_back(base + 32 * width);
-                hp.lp_nbr[dir].resize((size_t)base + 32 * width, 0);
-                hp.lp_mb[dir].resize((size_t)base + 32 * width, 0);
-                hp.lp_w1[dir].resize((size_t)base + 32 * width, 0.0);
-                hp.lp_w2[dir].resize((size_t)base + 32 * width, 0.0);
-                for (size_t t = 0; t < (size_t)kPointsPerWarp && g0 + t < inner.size(); t++) {
+                hp.lp_nm[dir].resize((size_t)base + 32 * width, 0);
+                hp.lp_w[dir].resize((size_t)base + 32 * width, double2{0.0, 0.0});
+                for (size_t t = 0; t < per && g0 + t < inner.size(); t++) {
                     const int32_t k = inner[g0 + t];
                     for (int32_t j = 0; j < loff[k + 1] - loff[k]; j++) {
                         const size_t e = (size_t)base + 32 * (size_t)(j / L) + L * t + j % L;
-                        hp.lp_nbr[dir][e] = lnbr[loff[k] + j];
-                        hp.lp_mb[dir][e] = lmb[loff[k] + j];
-                        hp.lp_w1[dir][e] = lw1[loff[k] + j];
-                        hp.lp_w2[dir][e] = lw2[loff[k] + j];
+                        hp.lp_nm[dir][e] = (uint32_t)lnbr[loff[k] + j] | (uint32_t)lmb[loff[k] + j] << 28;
+                        hp.lp_w[dir][e] = double2{lw1[loff[k] + j], lw2[loff[k] + j]};
                     }
                 }
                 ng++;
@@ -997,6 +1006,8 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
             lg.push_back(ng);
         }
     }
+    for (int dir = 0; dir < 2 && c->pk_ok; dir++)
+        for (int32_t pos : hp.pk_pt[dir]) hp.pk_k[dir].push_back(pos < 0 ? -1 : (dir == 0 ? hp.sw_fwd : hp.sw_bwd)[pos]);
     for (auto *v : {&hp.lo_nbr, &hp.up_nbr}) if (v->empty()) v->push_back(0);
     for (auto *v : {&hp.lo_mb, &hp.up_mb}) if (v->empty()) v->push_back(0);
     for (auto *v : {&hp.lo_w1, &hp.lo_w2, &hp.up_w1, &hp.up_w2}) if (v->empty()) v->push_back(0.0);
@@ -1096,17 +1107,24 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     }
     // packed sweep form (arrays of at least one element, so that a level set
     // without framed points, or without interior points, still has them)
-    std::vector<float> pkf[2][2], lpf[2][2];
+    std::vector<float> pkf[2][2];
+    std::vector<float2> lpf[2];
+    d.lvl_lanes = nullptr;
+    if (c->pk_ok) d.lvl_lanes = A.alloc<int32_t>(std::max<size_t>(c->lvl_lanes.size(), 1));
     for (int dir = 0; dir < 2; dir++) {
         d.pk_pt[dir] = d.pk_nbr[dir] = nullptr;
         d.pk_mb[dir] = d.pk_steps[dir] = nullptr;
         d.pk_w1[dir] = d.pk_w2[dir] = nullptr;
         d.pk_w1f[dir] = d.pk_w2f[dir] = nullptr;
-        d.lp_k[dir] = d.lp_len[dir] = d.lp_goff[dir] = d.lp_nbr[dir] = nullptr;
-        d.lp_mb[dir] = nullptr;
-        d.lp_w1[dir] = d.lp_w2[dir] = nullptr;
-        d.lp_w1f[dir] = d.lp_w2f[dir] = nullptr;
+        d.pk_k[dir] = d.pk_f[dir] = nullptr;
+        d.lp_k[dir] = d.lp_len[dir] = d.lp_goff[dir] = nullptr;
+        d.lp_nm[dir] = nullptr;
+        d.lp_w[dir] = nullptr;
+        d.lp_wf[dir] = nullptr;
+        d.lvl_fw[dir] = d.lvl_in[dir] = nullptr;
         if (!c->pk_ok) continue;
+        d.lvl_fw[dir] = A.alloc<int32_t>(c->pk_lw[dir].size());
+        d.lvl_in[dir] = A.alloc<int32_t>(c->lp_lg[dir].size());
         const size_t m = std::max<size_t>(hp.pk_pt[dir].size(), 1);
         d.pk_pt[dir] = A.alloc<int32_t>(m);
         d.pk_nbr[dir] = A.alloc<int32_t>(m);
@@ -1114,23 +1132,21 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
         d.pk_steps[dir] = A.alloc<uint8_t>(std::max<size_t>(hp.pk_steps[dir].size(), 1));
         d.pk_w1[dir] = A.alloc<double>(m);
         d.pk_w2[dir] = A.alloc<double>(m);
-        const size_t nk = std::max<size_t>(hp.lp_k[dir].size(), 1), ne = std::max<size_t>(hp.lp_nbr[dir].size(), 1);
+        d.pk_k[dir] = A.alloc<int32_t>(m);
+        d.pk_f[dir] = A.alloc<int32_t>(m);
+        const size_t nk = std::max<size_t>(hp.lp_k[dir].size(), 1), ne = std::max<size_t>(hp.lp_nm[dir].size(), 1);
         d.lp_k[dir] = A.alloc<int32_t>(nk);
         d.lp_len[dir] = A.alloc<int32_t>(nk);
         d.lp_goff[dir] = A.alloc<int32_t>(hp.lp_goff[dir].size());
-        d.lp_nbr[dir] = A.alloc<int32_t>(ne);
-        d.lp_mb[dir] = A.alloc<uint8_t>(ne);
-        d.lp_w1[dir] = A.alloc<double>(ne);
-        d.lp_w2[dir] = A.alloc<double>(ne);
+        d.lp_nm[dir] = A.alloc<uint32_t>(ne);
+        if (!mixed) d.lp_w[dir] = A.alloc<double2>(ne);
         if (mixed) {
             pkf[dir][0].assign(hp.pk_w1[dir].begin(), hp.pk_w1[dir].end());
             pkf[dir][1].assign(hp.pk_w2[dir].begin(), hp.pk_w2[dir].end());
             d.pk_w1f[dir] = A.alloc<float>(m);
             d.pk_w2f[dir] = A.alloc<float>(m);
-            lpf[dir][0].assign(hp.lp_w1[dir].begin(), hp.lp_w1[dir].end());
-            lpf[dir][1].assign(hp.lp_w2[dir].begin(), hp.lp_w2[dir].end());
-            d.lp_w1f[dir] = A.alloc<float>(ne);
-            d.lp_w2f[dir] = A.alloc<float>(ne);
+            for (const double2 &w : hp.lp_w[dir]) lpf[dir].push_back(float2{(float)w.x, (float)w.y});
+            d.lp_wf[dir] = A.alloc<float2>(ne);
         }
     }
     // per-point axis Jacobian products of the packed form (x+, x-, y+, y-)
@@ -1175,10 +1191,6 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
         d.fidx = A.alloc<int32_t>(ld);
         d.fpt = A.alloc<int32_t>(std::max<size_t>(h_fpt.size(), 1));
     }
-    c->launch.pk_lw[0] = c->pk_ok ? c->pk_lw[0].data() : nullptr;
-    c->launch.pk_lw[1] = c->pk_ok ? c->pk_lw[1].data() : nullptr;
-    c->launch.lp_lg[0] = c->pk_ok ? c->lp_lg[0].data() : nullptr;
-    c->launch.lp_lg[1] = c->pk_ok ? c->lp_lg[1].data() : nullptr;
     d.g1x = A.alloc<double>(4 * (size_t)ld);
     d.g1y = A.alloc<double>(4 * (size_t)ld);
     d.R = A.alloc<double>(4 * (size_t)ld);
@@ -1191,6 +1203,14 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device);
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaDeviceGetAttribute");
     c->launch.sms = std::max(sms, 1);
+    // the sweeps' launch: a block per SM (fewer when no level has a warp's
+    // work for each), enough warps for the largest level, at most 8
+    int32_t most = 1;
+    for (int dir = 0; dir < 2 && c->pk_ok; dir++)
+        for (int32_t l = 0; l < c->n_levels; l++)
+            most = std::max(most, c->pk_lw[dir][l + 1] - c->pk_lw[dir][l] + c->lp_lg[dir][l + 1] - c->lp_lg[dir][l]);
+    c->launch.sw_blocks = std::min(c->launch.sms, most);
+    c->launch.sw_threads = 32 * std::min(8, (most + c->launch.sw_blocks - 1) / c->launch.sw_blocks);
     c->launch.tpp = n >= 100000 ? 1 : (n >= 50000 ? 2 : (n >= 25000 ? 4 : 8));
     c->launch.sweep_lanes = 4;
     d.n_blk = (int32_t)hp.blk_case.size();
@@ -1306,9 +1326,21 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     up(dinv, c->inv.data(), n * sizeof(int32_t));
     up(dcase_of, hp.case_of_i.data(), ld * sizeof(int32_t));
     up(dcase_uinf, cuinf.data(), cuinf.size() * sizeof(double));
+    if (d.lvl_lanes) up((void *)d.lvl_lanes, c->lvl_lanes.data(), c->lvl_lanes.size() * sizeof(int32_t));
     for (int dir = 0; dir < 2; dir++) {
         if (!d.pk_pt[dir]) continue;
-        const size_t m = hp.pk_pt[dir].size(), nk = hp.lp_k[dir].size(), ne = hp.lp_nbr[dir].size();
+        const size_t m = hp.pk_pt[dir].size(), nk = hp.lp_k[dir].size(), ne = hp.lp_nm[dir].size();
+        up((void *)d.pk_k[dir], hp.pk_k[dir].data(), m * sizeof(int32_t));
+        if (d.fidx) {  // framed points' numbers of the packed slots
+            std::vector<int32_t> pf(m);
+            for (size_t t = 0; t < m; t++) {
+                const int32_t k = hp.pk_k[dir][t];
+                pf[t] = k < 0 ? 0 : 2 * h_fidx[k] + (c->flag[c->perm[k]] == LSKUM_WALL ? 1 : 0);
+            }
+            up((void *)d.pk_f[dir], pf.data(), m * sizeof(int32_t));
+        }
+        up((void *)d.lvl_fw[dir], c->pk_lw[dir].data(), c->pk_lw[dir].size() * sizeof(int32_t));
+        up((void *)d.lvl_in[dir], c->lp_lg[dir].data(), c->lp_lg[dir].size() * sizeof(int32_t));
         up((void *)d.pk_pt[dir], hp.pk_pt[dir].data(), m * sizeof(int32_t));
         up((void *)d.pk_nbr[dir], hp.pk_nbr[dir].data(), m * sizeof(int32_t));
         up((void *)d.pk_mb[dir], hp.pk_mb[dir].data(), m);
@@ -1318,15 +1350,12 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
         up((void *)d.lp_k[dir], hp.lp_k[dir].data(), nk * sizeof(int32_t));
         up((void *)d.lp_len[dir], hp.lp_len[dir].data(), nk * sizeof(int32_t));
         up((void *)d.lp_goff[dir], hp.lp_goff[dir].data(), hp.lp_goff[dir].size() * sizeof(int32_t));
-        up((void *)d.lp_nbr[dir], hp.lp_nbr[dir].data(), ne * sizeof(int32_t));
-        up((void *)d.lp_mb[dir], hp.lp_mb[dir].data(), ne);
-        up((void *)d.lp_w1[dir], hp.lp_w1[dir].data(), ne * sizeof(double));
-        up((void *)d.lp_w2[dir], hp.lp_w2[dir].data(), ne * sizeof(double));
+        up((void *)d.lp_nm[dir], hp.lp_nm[dir].data(), ne * sizeof(uint32_t));
+        if (d.lp_w[dir]) up((void *)d.lp_w[dir], hp.lp_w[dir].data(), ne * sizeof(double2));
         if (d.pk_w1f[dir]) {
             up((void *)d.pk_w1f[dir], pkf[dir][0].data(), m * sizeof(float));
             up((void *)d.pk_w2f[dir], pkf[dir][1].data(), m * sizeof(float));
-            up((void *)d.lp_w1f[dir], lpf[dir][0].data(), ne * sizeof(float));
-            up((void *)d.lp_w2f[dir], lpf[dir][1].data(), ne * sizeof(float));
+            up((void *)d.lp_wf[dir], lpf[dir].data(), ne * sizeof(float2));
         }
     }
     if (d.fidx) {
@@ -1475,6 +1504,7 @@ lskum_status write_ctrl(lskum_ctx *c, Ctrl &h)
     h.hist = c->hist;
     h.hist4 = c->hist4;
     h.hist_cap = c->hist_cap;
+    h.sweep_bar = 0;
     cudaError_t e = cudaMemcpyAsync(c->ctrl, &h, sizeof(Ctrl), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "writing the control block");
@@ -1693,6 +1723,8 @@ lskum_status lskum_wait(lskum_ctx *c, int32_t *iters_done)
     if (h.error == LSKUM_ERR_DIVERGED)
         return fail(c, LSKUM_ERR_DIVERGED, "residual norm of case %d not finite in iteration %d", -1 - h.bad_point,
                     h.it);
+    if (h.error == LSKUM_ERR_TIMEOUT)
+        return fail(c, LSKUM_ERR_TIMEOUT, "the sweeps' blocks did not meet within their time limit in iteration %d", h.it);
     if (h.error) return fail(c, LSKUM_ERR_CUDA, "device error %d", h.error);
     return LSKUM_OK;
 }
@@ -2071,7 +2103,7 @@ lskum_status lskum_autotune(lskum_ctx *c, int32_t trial_iters, int32_t *tpp, int
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaEventCreate");
     for (int tp : {1, 2, 4, 8}) {
         for (int gl : {2, 4, 8, 32}) {
-            if (gl == 32 && !c->pk_ok) continue;
+            if (c->pk_ok ? gl != 4 && gl != 32 : gl == 32) continue;  // (2, 4 and 8 are one form when packed)
             c->launch.tpp = tp;
             c->launch.sweep_lanes = gl;
             s = build_graphs(c);

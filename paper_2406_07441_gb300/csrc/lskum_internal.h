@@ -38,6 +38,7 @@ struct Ctrl {
     int32_t it_start;    // it when the current run was enqueued
     int32_t hist_cap;    // capacity of each case's history
     int32_t n_cases;
+    uint32_t sweep_bar;  // arrivals at the sweeps' level boundaries; 0 between launches
     double target;       // drop target of the current run (<= 0: none)
     int32_t *case_state; // [n_cases] CaseState; kReachedTarget finishes the
                          // iteration, the next k_begin makes it kStopped
@@ -74,11 +75,15 @@ enum PrimField {
 };
 constexpr int kPrimStride = 24;
 
-// Packed sweep form: lanes per interior point (each takes every kLanesPerPoint-th
-// slot of the point's list and forms one of its four axis products), and so
-// interior points per warp.
-constexpr int kLanesPerPoint = 4;
-constexpr int kPointsPerWarp = 32 / kLanesPerPoint;
+// Packed sweep form: an interior point takes four lanes (each every fourth
+// slot of its list, and one of its four axis products), in levels of more than
+// kWideLevel interior points two (every second slot, both products of one
+// axis: 196 FP64 instructions per 32 points instead of 272, half the warps).
+// The line lies where four lanes give every scheduler of the GPU (152 SMs x 4)
+// a warp: below it two lanes would leave some idle.  Groups hold up to
+// kGroupPoints points.
+constexpr int kGroupPoints = 16;
+constexpr int kWideLevel = 152 * 4 * 8;
 static_assert(P_NFIELDS <= kPrimStride, "prim record too small");
 
 struct StateSet {
@@ -130,6 +135,9 @@ struct Dev {
     // (forward: lower list, backward: upper list), so a warp's groups share a
     // trip count
     const int32_t *sw_fwd, *sw_bwd;
+    // packed sweep form: first framed-point warp and first interior group of
+    // each level, [n_levels + 1] per direction
+    const int32_t *lvl_fw[2], *lvl_in[2];
     // packed sweep form, [0] forward (lower lists), [1] backward (upper
     // lists), for the points in a (t, n) frame: warp w's 32 lanes hold slots
     // 32w .. 32w+31, each with the sweep position of its point (-1: padding),
@@ -140,15 +148,20 @@ struct Dev {
     const uint8_t *pk_steps[2];  // per warp: steps of its segmented sum, ceil(log2(longest list))
     const double *pk_w1[2], *pk_w2[2];
     const float *pk_w1f[2], *pk_w2f[2];
-    // and for the interior points: kLanesPerPoint lanes per point, in groups
-    // of kPointsPerWarp points (by decreasing list length): point p of group g
-    // is lp_k[kPointsPerWarp g + p] (-1: none), with lp_len[...] slots, slot j
-    // at lp_goff[g] + 32 (j / kLanesPerPoint) + kLanesPerPoint p + j % kLanesPerPoint
-    // (lane kLanesPerPoint p + s takes the slots j = s (mod kLanesPerPoint))
-    const int32_t *lp_k[2], *lp_len[2], *lp_goff[2], *lp_nbr[2];
-    const uint8_t *lp_mb[2];
-    const double *lp_w1[2], *lp_w2[2];
-    const float *lp_w1f[2], *lp_w2f[2];
+    // the same slot's point (internal index, -1: padding) and, for the exact
+    // products, 2 x its number among the framed points + (1 at a wall point)
+    const int32_t *pk_k[2], *pk_f[2];
+    // and for the interior points, L = lvl_lanes[level] lanes each (2 or 4), in
+    // groups of 32 / L points (by decreasing list length): point p of group g
+    // is lp_k[kGroupPoints g + p] (-1: none), with lp_len[...] slots, slot j at
+    // lp_goff[g] + 32 (j / L) + L p + j % L (lane L p + s takes the slots j = s
+    // (mod L)): lp_nm its neighbour and (bits 28 up) membership, lp_w / lp_wf
+    // its two weights
+    const int32_t *lvl_lanes;
+    const int32_t *lp_k[2], *lp_len[2], *lp_goff[2];
+    const uint32_t *lp_nm[2];
+    const double2 *lp_w[2];
+    const float2 *lp_wf[2];
     // packed form: per point, the axis split-flux Jacobian products of its
     // latest increment, [ld][4 products: x+, x-, y+, y-][4]: written when the
     // point's increment is formed, gathered by the later levels' interior
@@ -195,9 +208,9 @@ struct Dev {
 struct Launch {
     int tpp;          // threads per point of the gradient and residual kernels (1, 2, 4, 8)
     int sms;          // multiprocessors (the residual's persistent grid)
-    int sweep_lanes;  // lanes per point of the sweep kernels (2, 4, 8), or 32: the packed form
-    const int32_t *pk_lw[2];  // packed form: host arrays [n_levels + 1], first framed-point warp of each level
-    const int32_t *lp_lg[2];  // packed form: host arrays [n_levels + 1], first interior group of each level
+    int sweep_lanes;  // 32: the packed form; 2, 4, 8: lanes per point of the per-slot form where lists are too
+                      // long for it, else the packed form with the framed Jacobians formed in the sweeps' launch
+    int sw_blocks, sw_threads;  // packed form: the sweeps' cooperative launch
     // optional side branch of a captured iteration: what depends only on the
     // state (the framed points' Jacobians, the diagonals of the shapes with
     // several residual lanes per point) runs on `side` between the `fork`

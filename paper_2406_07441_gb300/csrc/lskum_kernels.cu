@@ -345,6 +345,39 @@ __device__ __forceinline__ void jvp_axis_sel(const PrimT<T> &P, const JvpBase<T>
     out[3] = fma(t1, A, fma(ude1, dA, t3));
 }
 
+// Both signs' products along an axis: bit for bit jvp_axis_sel's (the terms
+// that change sign with it are formed once: rounding to nearest is symmetric),
+// 34 FP64 instructions instead of 46.
+template <typename T>
+__device__ __forceinline__ void jvp_axis_pair(const PrimT<T> &P, const JvpBase<T> &b, bool xdir, T Ap, T Am, T ek, T B,
+                                              T B2S, T ude1, T outp[4], T outm[4])
+{
+    const T ud = xdir ? P.u : P.v;
+    const T dud = xdir ? b.du : b.dv;
+    const T dS = fma(dud, P.sb, ud * b.dsb);
+    const T dA = ek * dS;
+    const T dB = fma(B2S, dS, B * b.dsbi);  // minus the tangent of B
+    const T i1 = fma(ud, dA, -dB), pdA = P.p * dA;
+    const T t1 = fma(dud, P.e1, ud * b.de1);
+    const T t3 = fma(b.de2, B, P.e2 * -dB);
+    const T i3 = fma(ude1, dA, t3);
+    const T zero = T(0);
+#pragma unroll
+    for (int m = 0; m < 2; m++) {
+        T *out = m ? outm : outp;
+        const T A = m ? Am : Ap;
+        const T M1 = fma(ud, A, m ? -B : B);
+        const T dM1 = fma(dud, A, m ? -i1 : i1);
+        const T rm = P.rho * M1;
+        const T drm = fma(b.drho, M1, P.rho * dM1);
+        const T pA = fma(b.dp, A, m ? -pdA : pdA);
+        out[0] = drm;
+        out[1] = fma(drm, P.u, fma(rm, b.du, xdir ? pA : zero));
+        out[2] = fma(drm, P.v, fma(rm, b.dv, xdir ? zero : pA));
+        out[3] = fma(t1, A, m ? -i3 : i3);
+    }
+}
+
 // Unsplit Euler-flux Jacobian product A_d(U) dU in direction d = (dx, dy)
 // (the tangent of G_d = (rho u_d, rho u u_d + p dx, rho v u_d + p dy,
 // (E + p) u_d) along dU; the revised LU-SGS's S term).
@@ -400,6 +433,18 @@ __device__ __forceinline__ void load4(const double *__restrict__ p, double v[4])
 __device__ __forceinline__ void load4(const float *__restrict__ p, float v[4])
 {
     const float4 a = *reinterpret_cast<const float4 *>(p);
+    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+}
+
+// The same from L2: values that other blocks write within the launch.
+__device__ __forceinline__ void load4_l2(const double *p, double v[4])
+{
+    const double2 a = __ldcg(reinterpret_cast<const double2 *>(p)), b = __ldcg(reinterpret_cast<const double2 *>(p) + 1);
+    v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+}
+__device__ __forceinline__ void load4_l2(const float *p, float v[4])
+{
+    const float4 a = __ldcg(reinterpret_cast<const float4 *>(p));
     v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
 }
 
@@ -959,13 +1004,12 @@ __device__ __forceinline__ SweepBufs<float> sweep_bufs<float>(const Dev &d, cons
 // split sub-stencils s the slot joins (exact AD or increment products).
 template <int JVP, typename T>
 __device__ __forceinline__ void sweep_slot(const Dev &d, const StateSet &st, const MathTables &Tb,
-                                           const T *__restrict__ dW, const T *__restrict__ pr, bool framed,
+                                           const T *dW, const T *__restrict__ pr, bool framed,
                                            double e1x, double e1y, double e2x, double e2y, int i, int mb, T w1,
                                            T w2, T acc[4])
 {
     T dl[4];
-#pragma unroll
-    for (int c = 0; c < 4; c++) dl[c] = dW[4 * i + c];
+    load4_l2(dW + 4 * (size_t)i, dl);
     if (JVP == 0 && !framed) {
         // interior frame: d = (1,0) or (0,1); A+-, exp(-S^2)/sqrt(pi), B,
         // 2 B S and u_d e1 precomputed per point
@@ -1037,8 +1081,8 @@ __device__ __forceinline__ void sweep_slot(const Dev &d, const StateSet &st, con
 // Point k's new increment from its list sum acc: forward dU*_k = -(R_k (+ S_k)
 // + acc) / D_k, backward dU_k = dU*_k - acc / D_k; normal momentum removed at
 // wall points.  Stored, and returned in w.
-template <bool FWD, typename T>
-__device__ __forceinline__ void sweep_point(const Dev &d, const StateSet &st, const SweepBufs<T> &sb, int k,
+template <typename T>
+__device__ __forceinline__ void sweep_point(bool FWD, const Dev &d, const StateSet &st, const SweepBufs<T> &sb, int k,
                                             bool wall, double e1x, double e1y, double e2x, double e2y,
                                             const T acc[4], T w[4])
 {
@@ -1068,7 +1112,7 @@ __device__ __forceinline__ void sweep_point(const Dev &d, const StateSet &st, co
         for (int c = 0; c < 4; c++) w[c] = -((T)rhs[c] + acc[c]) * iD;
     } else {
 #pragma unroll
-        for (int c = 0; c < 4; c++) w[c] = fma(-acc[c], iD, sb.dUs[4 * k + c]);
+        for (int c = 0; c < 4; c++) w[c] = fma(-acc[c], iD, __ldcg(sb.dUs + 4 * k + c));
     }
     if (wall) {
         const T nx = (T)d.wnx[k], ny = (T)d.wny[k];
@@ -1111,7 +1155,7 @@ __global__ void __launch_bounds__(256) k_sweep(Dev d, StateSet st, int lb, int l
 #pragma unroll
     for (int c = 0; c < 4; c++) acc[c] = group_sum<G>(acc[c]);
     T w[4];
-    if (live && sub == 0) sweep_point<FWD, T>(d, st, sb, k, wall, e1x, e1y, e2x, e2y, acc, w);
+    if (live && sub == 0) sweep_point<T>(FWD, d, st, sb, k, wall, e1x, e1y, e2x, e2y, acc, w);
 }
 
 // Axis product cb (0: x+, 1: x-, 2: y+, 3: y-) of point k's new increment w
@@ -1141,240 +1185,26 @@ __device__ __forceinline__ void store_increment_product(const Dev &d, const Stat
     store4(sb.jc + 16 * (size_t)k + 4 * cb, J);
 }
 
-// Threads per block of the packed sweeps: a level is only a few thousand
-// warps, so small blocks spread them evenly over the SMs (whole blocks of
-// eight warps left half the SMs with one block and half with two).
-#ifndef LSKUM_SWEEP_BLOCK
-#define LSKUM_SWEEP_BLOCK 64
-#endif
-constexpr int kSweepBlock = LSKUM_SWEEP_BLOCK;
-static_assert(kSweepBlock % 32 == 0 && kSweepBlock <= 256, "sweep block");
-
-// Packed form of a level.  A neighbour's Jacobian product along an axis
-// depends only on the neighbour, the axis and the sub-stencil's sign, so a
-// point forms the four axis products of its new increment once, and
-// interior points gather them: 8 FMAs per slot instead of ~70 FP64
-// instructions.  A point's sum depends only on its own list, in a fixed
-// order, so a batch still equals its single solves bit for bit.
-// - wf warps for the points in a (t, n) frame, their slots packed whole into
-//   warps (at create, by best fit; a point with an empty list takes one idle
-//   slot), one lane per slot.  Exact products: the lane applies the slot's
-//   weighted Jacobian, formed for the whole iteration by k_framed_jac (16
-//   FMAs); increments: the split fluxes per slot in the point's frame.  A
-//   segmented suffix sum over the lanes of each point (fixed tree order, no
-//   atomics) leaves the point's sum in its first lane, which finishes the
-//   point; the point's lanes share its four axis products (exact: its
-//   precomputed axis Jacobians).  Packed warps [wb, wb + wf) are the
-//   level's; they are spread evenly over the grid (every S-th warp).
-// - ng warps for the interior points, kLanesPerPoint lanes per point,
-//   kPointsPerWarp points of similar list length per warp (groups
-//   [g0, g0 + ng) are the level's), in the other warp positions in order.
-//   A level is a chain of dependent loads (list, gathers, the point's own
-//   record) and a short FP64 sequence per lane, so the point's own loads
-//   are issued before the gathers, and the x- and y-products of a warp's
-//   lanes share one branch-free FP64 sequence (jvp_axis_sel).
-template <int JVP, bool FWD, typename T>
-__global__ void __launch_bounds__(kSweepBlock) k_sweep_packed(Dev d, StateSet st, int wb, int wf, int g0, int ng)
+// Jacobians of the framed points' products (exact products).  The split-flux
+// Jacobian A_d^+-(U_i) is the derivative of G_d^+- at the state of this
+// iteration and does not depend on the sweeps' increments, so every matrix
+// that the two sweeps apply at the points in a (t, n) frame is formed all in
+// parallel before the forward sweep; inside the levels the framed points'
+// chains are then matrix-vector products.  Item t: one column of pk_jm of a
+// slot lane -- M = w1 A_e1 + w2 A_e2 at the neighbour's state in the point's
+// frame -- or of fj of a framed point and axis product -- A_x+-, A_y+- at the
+// point's own state.  Column j is the forward-mode tangent along the unit
+// vector e_j, evaluated in FP64 by the functions of the per-slot form (stored
+// as T).
+__host__ __device__ inline int framed_jac_items(const Dev &d)
 {
-    const MathTables &Tb = g_math;  // framed points only: no per-block copy
-    if (halted(d.ctrl)) return;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) / 32;
-    if (gw >= wf + ng) return;  // whole warps (blocks are whole warps)
-    const int lane = threadIdx.x & 31;
-    const int dir = FWD ? 0 : 1;
-    const SweepBufs<T> sb = sweep_bufs<T>(d, st);
-    const T *__restrict__ dW = FWD ? sb.dUs : sb.dU;  // earlier levels' increments
-    const T *__restrict__ jn = sb.jc;                 // earlier levels' axis products
-    T acc[4] = {T(0), T(0), T(0), T(0)};
-    T w[4] = {T(0), T(0), T(0), T(0)};
-    const int S = max(1, (wf + ng) / max(wf, 1)), q = gw / S;  // framed warp q at position q S
-    if (wf > 0 && gw % S == 0 && q < wf) {
-        const int fw = wb + q;
-        const size_t e = (size_t)fw * 32 + lane;
-        const int pos = d.pk_pt[dir][e];  // sweep position of the slot's point, -1: padding
-        const int k = pos >= 0 ? (FWD ? d.sw_fwd : d.sw_bwd)[pos] : 0;
-        const bool live = pos >= 0 && !frozen(d, k);
-        const int fk = d.flag[k];
-        const bool wall = fk == kWall, framed = fk != kInterior;
-        double e1x, e1y, e2x, e2y;
-        point_frame(d, k, framed, e1x, e1y, e2x, e2y);
-        const int mb = d.pk_mb[dir][e];
-        if (live && mb) {
-            if (JVP == 0) {
-                // the slot's weighted Jacobian, formed before the sweeps: acc += M dW_i
-                const T *__restrict__ M = (sizeof(T) == 4 ? (const T *)d.pk_jmf[dir] : (const T *)d.pk_jm[dir]) + 16 * e;
-                T dl[4];
-                load4(dW + 4 * (size_t)d.pk_nbr[dir][e], dl);
-#pragma unroll
-                for (int c = 0; c < 4; c++)
-#pragma unroll
-                    for (int j = 0; j < 4; j++) acc[c] = fma(M[4 * c + j], dl[j], acc[c]);
-            } else {
-                const T w1 = sizeof(T) == 4 ? (T)d.pk_w1f[dir][e] : (T)d.pk_w1[dir][e];
-                const T w2 = sizeof(T) == 4 ? (T)d.pk_w2f[dir][e] : (T)d.pk_w2[dir][e];
-                sweep_slot<JVP, T>(d, st, Tb, dW, sb.prim, framed, e1x, e1y, e2x, e2y, d.pk_nbr[dir][e], mb, w1,
-                                   w2, acc);
-            }
-        }
-        // segmented suffix sum: lane l adds lane l + o when both hold the same
-        // point; the warp's longest list bounds the steps (warp-uniform)
-        const int steps = d.pk_steps[dir][fw];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            if (o >= (1 << steps)) break;
-            const int p2 = __shfl_down_sync(kFull, pos, o);
-            T v[4];
-#pragma unroll
-            for (int c = 0; c < 4; c++) v[c] = __shfl_down_sync(kFull, acc[c], o);
-            if (lane + o < 32 && p2 == pos) {
-#pragma unroll
-                for (int c = 0; c < 4; c++) acc[c] += v[c];
-            }
-        }
-        // the point's lanes (consecutive; padding lanes form their own group):
-        // the first finishes the point, then lane r of the point's seg lanes
-        // forms the products r, r + seg, ... of the new increment
-        const unsigned m = __match_any_sync(kFull, pos);
-        const int head = __ffs(m) - 1, seg = __popc(m), r = lane - head;
-        if (live && r == 0) sweep_point<FWD, T>(d, st, sb, k, wall, e1x, e1y, e2x, e2y, acc, w);
-#pragma unroll
-        for (int c = 0; c < 4; c++) w[c] = __shfl_sync(kFull, w[c], head);
-        if (live) {
-            if (JVP == 0) {
-                // the point's axis Jacobians, formed before the sweeps
-                const T *__restrict__ F =
-                    (sizeof(T) == 4 ? (const T *)d.fjf : (const T *)d.fj) + 64 * (size_t)d.fidx[k];
-                for (int cb = r; cb < 4; cb += seg) {
-                    T J[4];
-#pragma unroll
-                    for (int c = 0; c < 4; c++) {
-                        J[c] = F[16 * cb + 4 * c] * w[0];
-#pragma unroll
-                        for (int j = 1; j < 4; j++) J[c] = fma(F[16 * cb + 4 * c + j], w[j], J[c]);
-                    }
-                    store4(sb.jc + 16 * (size_t)k + 4 * cb, J);
-                }
-            } else {
-                for (int cb = r; cb < 4; cb += seg) store_increment_product<T>(d, st, Tb, sb, w, k, cb);
-            }
-        }
-        return;
-    }
-    // interior points: kLanesPerPoint lanes per point, lane s taking the
-    // point's slots j = s (mod kLanesPerPoint) in order; a butterfly over the
-    // point's lanes gives every one of them the same sum (each addition has
-    // the same two operands in either order)
-    const int g = g0 + gw - min(wf, q + 1);  // the framed positions up to gw left out
-    const int p = lane / kLanesPerPoint, s = lane % kLanesPerPoint;
-    const int k = d.lp_k[dir][kPointsPerWarp * g + p];
-    const bool live = k >= 0 && !frozen(d, k);
-    const int len = live ? d.lp_len[dir][kPointsPerWarp * g + p] : 0;
-    const int kk = k >= 0 ? k : 0;  // index for the loads of a slot without a point
-    // loads that depend only on the point, issued before the gathers so that
-    // their latency overlaps theirs: this lane's entries of the point's
-    // primal record (its axis product s: 0 x+, 1 x-, 2 y+, 3 y-) and, in the
-    // point's first lane, the right-hand side (R forward, dU* backward) and 1/D
-    const bool xdir = s < 2, psg = !(s & 1);
-    PrimT<T> P{};
-    T rA = T(0), rEK = T(0), rB = T(0), rBS = T(0), rUE = T(0);
-    if (JVP == 0) {
-        P = load_prim(sb.prim, kk);
-        const T *rec = sb.prim + (size_t)kk * kPrimStride;
-        rA = rec[xdir ? (psg ? P_APX : P_AMX) : (psg ? P_APY : P_AMY)];
-        rEK = rec[xdir ? P_EKX : P_EKY];
-        rB = rec[xdir ? P_BX : P_BY];
-        rBS = rec[xdir ? P_BSX : P_BSY];
-        rUE = rec[xdir ? P_UE1 : P_VE1];
-    }
-    const bool plain = d.lusgs == 0;  // the revised LU-SGS adds its lagged term in sweep_point
-    double rhs[4] = {0.0, 0.0, 0.0, 0.0};
-    T iDk = T(0);
-    if (s == 0 && plain) {
-        iDk = (T)d.iD[kk];
-        if (FWD) {
-            const int ld = d.ld;
-#pragma unroll
-            for (int c = 0; c < 4; c++) rhs[c] = d.R[c * ld + kk];
-        } else {
-            T v[4];
-            load4(sb.dUs + 4 * (size_t)kk, v);
-#pragma unroll
-            for (int c = 0; c < 4; c++) rhs[c] = (double)v[c];
-        }
-    }
-    const size_t base = (size_t)d.lp_goff[dir][g] + lane;
-#pragma unroll 4
-    for (int j = s; j < len; j += kLanesPerPoint) {
-        const size_t e = base + 32 * (size_t)(j / kLanesPerPoint);
-        const int i = d.lp_nbr[dir][e], mb = d.lp_mb[dir][e];
-        T J[4];
-        if (mb & 3) {
-            const T w1 = sizeof(T) == 4 ? (T)d.lp_w1f[dir][e] : (T)d.lp_w1[dir][e];
-            load4(jn + 16 * (size_t)i + ((mb & 1) ? 0 : 4), J);
-#pragma unroll
-            for (int c = 0; c < 4; c++) acc[c] = fma(w1, J[c], acc[c]);
-        }
-        if (mb & 12) {
-            const T w2 = sizeof(T) == 4 ? (T)d.lp_w2f[dir][e] : (T)d.lp_w2[dir][e];
-            load4(jn + 16 * (size_t)i + ((mb & 4) ? 8 : 12), J);
-#pragma unroll
-            for (int c = 0; c < 4; c++) acc[c] = fma(w2, J[c], acc[c]);
-        }
-    }
-#pragma unroll
-    for (int o = 1; o < kLanesPerPoint; o <<= 1) {
-#pragma unroll
-        for (int c = 0; c < 4; c++) acc[c] += __shfl_xor_sync(kFull, acc[c], o);
-    }
-    // the point's first lane finishes it (forward dU* = -(R + acc) / D,
-    // backward dU = dU* - acc / D); each of its lanes then forms one of the
-    // four axis products of the new increment
-#pragma unroll
-    for (int c = 0; c < 4; c++) w[c] = T(0);
-    if (live && s == 0) {
-        if (plain) {
-#pragma unroll
-            for (int c = 0; c < 4; c++) w[c] = FWD ? -((T)rhs[c] + acc[c]) * iDk : fma(-acc[c], iDk, (T)rhs[c]);
-            store4((FWD ? sb.dUs : sb.dU) + 4 * (size_t)k, w);
-        } else {
-            sweep_point<FWD, T>(d, st, sb, k, false, 1.0, 0.0, 0.0, 1.0, acc, w);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; c++) w[c] = __shfl_sync(kFull, w[c], lane - s);
-    if (live) {
-        if (JVP == 0) {
-            const JvpBase<T> jb = jvp_base(P, w);
-            T J[4];
-            jvp_axis_sel<T>(P, jb, xdir, psg, rA, rEK, rB, rBS, rUE, J);
-            store4(sb.jc + 16 * (size_t)k + 4 * s, J);
-        } else {
-            store_increment_product<T>(d, st, Tb, sb, w, k, s);
-        }
-    }
+    return 4 * (d.pk_lanes[0] + d.pk_lanes[1]) + 16 * d.nf;
 }
 
-// Jacobians of the framed points' products for the packed sweeps (exact
-// products).  The split-flux Jacobian A_d^+-(U_i) is the derivative of
-// G_d^+- at the state of this iteration and does not depend on the sweeps'
-// increments, so every matrix that the two sweeps apply at the points in a
-// (t, n) frame is formed here, all in parallel, before the forward sweep;
-// inside the levels the framed points' chains are then matrix-vector
-// products.  One thread per (slot lane, column) of pk_jm -- M = w1 A_e1 +
-// w2 A_e2 at the neighbour's state in the point's frame -- and per (framed
-// point, axis product, column) of fj -- A_x+-, A_y+- at the point's own
-// state.  Column j is the forward-mode tangent along the unit vector e_j,
-// evaluated in FP64 by the functions of the per-slot form (stored as T).
 template <typename T>
-__global__ void __launch_bounds__(256) k_framed_jac(Dev d, StateSet st)
+__device__ __forceinline__ void framed_jac_item(const Dev &d, const StateSet &st, const MathTables &Tb, int t)
 {
-    __shared__ MathTables Tb;
-    if (halted(d.ctrl)) return;
-    load_math_tables(Tb);
-    __syncthreads();
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const int n0 = 4 * d.pk_lanes[0], n1 = 4 * d.pk_lanes[1], nfj = 16 * d.nf;
-    if (t >= n0 + n1 + nfj) return;
+    const int n0 = 4 * d.pk_lanes[0], n1 = 4 * d.pk_lanes[1];
     const int j = t & 3;  // n0 and n1 are multiples of 4
     double dl[4];
 #pragma unroll
@@ -1427,6 +1257,620 @@ __global__ void __launch_bounds__(256) k_framed_jac(Dev d, StateSet st)
     T *F = (sizeof(T) == 4 ? (T *)d.fjf : (T *)d.fj) + 64 * (size_t)f + 16 * cb;
 #pragma unroll
     for (int c = 0; c < 4; c++) F[4 * c + j] = (T)J[c];
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_framed_jac(Dev d, StateSet st)
+{
+    __shared__ MathTables Tb;
+    if (halted(d.ctrl)) return;
+    load_math_tables(Tb);
+    __syncthreads();
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < framed_jac_items(d)) framed_jac_item<T>(d, st, Tb, t);
+}
+
+// Most threads per block of the sweeps' launch: two warps per scheduler keep
+// the FP64 unit busy, and 255 registers hold what is loaded ahead.
+constexpr int kSweepBlock = 256;
+
+// Time limit of the wait at a level boundary, and the status reported past it.
+constexpr uint64_t kSweepWaitNs = 2000000000ull;
+constexpr int kErrTimeout = -6;  // LSKUM_ERR_TIMEOUT
+
+// A level boundary in two halves: every thread of a block arrives, then (after
+// work that needs nothing of the other blocks) waits until all blocks of the
+// launch have arrived with their stores visible (cooperative launch: all
+// blocks are resident).  The arrivals are counted in ctrl->sweep_bar; the
+// launch's last one (number `limit`) wraps it to 0 for the next launch.  The
+// block's last warp arrives and polls for it.  The arrival releases the
+// block's stores to L2; there is no acquiring fence, which would empty L1 of
+// what was loaded ahead: values that other blocks write are read from L2
+// (load4_l2, cp_async16), never from L1.
+__device__ __forceinline__ void boundary_arrive(Ctrl *c, uint32_t limit)
+{
+    __syncthreads();
+    if (threadIdx.x == blockDim.x - 32) {
+        asm volatile("red.release.gpu.global.inc.u32 [%0], %1;" ::"l"(&c->sweep_bar), "r"(limit - 1) : "memory");
+    }
+}
+
+// False past the time limit.
+__device__ __forceinline__ bool boundary_wait(Ctrl *c, uint32_t target, uint32_t limit)
+{
+    __shared__ int reached;
+    if (threadIdx.x == blockDim.x - 32) {
+        const volatile uint32_t *bar = &c->sweep_bar;
+        uint64_t t0 = 0;
+        int ok = 1;
+        for (uint32_t tries = 1;; tries++) {
+            const uint32_t v = *bar;
+            if (target == limit ? v == 0 : v >= target) break;
+            if ((tries & 1023) == 0) {
+                uint64_t now;
+                asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+                if (t0 == 0) t0 = now;
+                if (now - t0 > kSweepWaitNs) {
+                    atomicExch(&c->error, kErrTimeout);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+        reached = ok;
+    }
+    __syncthreads();
+    return reached != 0;
+}
+
+// 16 bytes (8, for float2) of global memory into shared memory; .cg: from L2
+// (values that other blocks write within the launch).
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit()
+{
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+template <typename T>
+struct Pair2;
+template <>
+struct Pair2<double> {
+    using type = double2;
+};
+template <>
+struct Pair2<float> {
+    using type = float2;
+};
+
+// A warp's shared memory: the products of kDepth rows of slots in flight (two
+// of kChunks 16-byte words per lane and row, a warp's lanes apart: conflict-
+// free), and the weights of the first kRows rows.
+constexpr int kDepth = 5, kRows = 10;
+template <typename T>
+constexpr int kChunks = 4 * (int)sizeof(T) / 16;
+template <typename T>
+struct WarpStage {
+    uint4 J[kDepth][2 * kChunks<T>][32];
+    typename Pair2<T>::type w[kRows][32];
+};
+
+// What a lane of an interior point's group reads that no block writes within
+// the launch, loaded while the block waits at the level boundary: the point
+// (-1: none, or frozen), the first kRows slots of its share of the list
+// (their weights into shared memory), its entries of the point's primal
+// record, its components of R and 1/D.
+template <typename T>
+struct LanePre {
+    int k, rows;
+    size_t base;
+    uint32_t nm[kRows];
+    PrimT<T> P;
+    T Ap, Am, EK, B, BS, UE, iD;
+    double R[2];
+};
+
+template <int JVP, int L, typename T>
+__device__ __forceinline__ void lane_load(const Dev &d, const SweepBufs<T> &sb, int dir, int g, int lane,
+                                          WarpStage<T> &ws, LanePre<T> &a)
+{
+    const int p = lane / L, s = lane % L;
+    a.k = d.lp_k[dir][kGroupPoints * g + p];
+    const int len = a.k >= 0 ? d.lp_len[dir][kGroupPoints * g + p] : 0;
+    const int off = d.lp_goff[dir][g];
+    a.rows = (d.lp_goff[dir][g + 1] - off) / 32;  // the same for the warp
+    a.base = (size_t)off + lane;
+    if (a.k >= 0 && frozen(d, a.k)) a.k = -1;
+    const int kk = a.k >= 0 ? a.k : 0;  // index for the loads of a slot without a point
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+        a.nm[r] = 0;
+        if (a.k >= 0 && s + L * r < len) {
+            const size_t e = a.base + 32 * r;
+            a.nm[r] = d.lp_nm[dir][e];
+            if (sizeof(T) == 4) cp_async8(&ws.w[r][lane], d.lp_wf[dir] + e);
+            else cp_async16(&ws.w[r][lane], d.lp_w[dir] + e);
+        }
+    }
+    cp_async_commit();
+    if (JVP == 0) {
+        const bool xdir = L == 2 ? s == 0 : s < 2, psg = !(s & 1);
+        a.P = load_prim(sb.prim, kk);
+        const T *rec = sb.prim + (size_t)kk * kPrimStride;
+        if (L == 2) {
+            a.Ap = rec[xdir ? P_APX : P_APY];
+            a.Am = rec[xdir ? P_AMX : P_AMY];
+        } else {
+            a.Ap = rec[xdir ? (psg ? P_APX : P_AMX) : (psg ? P_APY : P_AMY)];
+        }
+        a.EK = rec[xdir ? P_EKX : P_EKY];
+        a.B = rec[xdir ? P_BX : P_BY];
+        a.BS = rec[xdir ? P_BSX : P_BSY];
+        a.UE = rec[xdir ? P_UE1 : P_VE1];
+    }
+    a.iD = (T)d.iD[kk];
+#pragma unroll
+    for (int c = 0; c < 4 / L; c++) a.R[c] = dir == 0 ? d.R[(4 / L * s + c) * d.ld + kk] : 0.0;
+}
+
+// A slot's products of its neighbour (this sweep's earlier levels) into the stage.
+template <typename T>
+__device__ __forceinline__ void slot_fetch(const T *jc, uint32_t nm, uint4 (*to)[32], int lane)
+{
+    const size_t i = 16 * (size_t)(nm & 0x0fffffffu);
+    const uint32_t mb = nm >> 28;
+    if (mb & 3) {
+        const T *J = jc + i + ((mb & 1) ? 0 : 4);
+#pragma unroll
+        for (int c = 0; c < kChunks<T>; c++) cp_async16(&to[c][lane], J + 16 / sizeof(T) * c);
+    }
+    if (mb & 12) {
+        const T *J = jc + i + ((mb & 4) ? 8 : 12);
+#pragma unroll
+        for (int c = 0; c < kChunks<T>; c++) cp_async16(&to[kChunks<T> + c][lane], J + 16 / sizeof(T) * c);
+    }
+}
+__device__ __forceinline__ void stage_read(const uint4 (*from)[32], int lane, double J[4])
+{
+    const double2 a = *reinterpret_cast<const double2 *>(&from[0][lane]);
+    const double2 b = *reinterpret_cast<const double2 *>(&from[1][lane]);
+    J[0] = a.x, J[1] = a.y, J[2] = b.x, J[3] = b.y;
+}
+__device__ __forceinline__ void stage_read(const uint4 (*from)[32], int lane, float J[4])
+{
+    const float4 a = *reinterpret_cast<const float4 *>(&from[0][lane]);
+    J[0] = a.x, J[1] = a.y, J[2] = a.z, J[3] = a.w;
+}
+
+// A slot's products in the stage, weighted, into acc.
+template <typename T>
+__device__ __forceinline__ void slot_add(uint32_t nm, typename Pair2<T>::type w, const uint4 (*from)[32], int lane,
+                                         T acc[4])
+{
+    T J[4];
+    if ((nm >> 28) & 3) {
+        stage_read(from, lane, J);
+#pragma unroll
+        for (int c = 0; c < 4; c++) acc[c] = fma(w.x, J[c], acc[c]);
+    }
+    if ((nm >> 28) & 12) {
+        stage_read(from + kChunks<T>, lane, J);
+#pragma unroll
+        for (int c = 0; c < 4; c++) acc[c] = fma(w.y, J[c], acc[c]);
+    }
+}
+
+// One group of 32 / L interior points, L lanes each (2 or 4).  Whatever L, a
+// point's sum is (a0 + a1) + (a2 + a3), a_m the sum of its slots j = m (mod 4)
+// in order: with two lanes, lane s keeps a_s and a_{s+2}.
+template <int JVP, int L, typename T>
+__device__ __forceinline__ void sweep_interior(const Dev &d, const StateSet &st, const SweepBufs<T> &sb, int dir,
+                                               int lane, const LanePre<T> &a, WarpStage<T> &ws)
+{
+    constexpr int C = 4 / L;  // components that a lane finishes
+    const int s = lane % L, k = a.k;
+    const bool live = k >= 0;
+    const bool fwd = dir == 0, plain = d.lusgs == 0;  // the revised LU-SGS adds its lagged term in sweep_point
+    T acc[C][4], dus[C];
+#pragma unroll
+    for (int h = 0; h < C; h++) {
+        dus[h] = T(0);
+#pragma unroll
+        for (int c = 0; c < 4; c++) acc[h][c] = T(0);
+    }
+#pragma unroll
+    for (int r = 0; r < kDepth; r++) {
+        slot_fetch(sb.jc, a.nm[r], ws.J[r], lane);
+        cp_async_commit();
+    }
+    if (live && !fwd)
+#pragma unroll
+        for (int c = 0; c < C; c++) dus[c] = __ldcg(sb.dUs + 4 * (size_t)k + C * s + c);
+#pragma unroll
+    for (int r = 0; r < kRows; r++) {
+        if (r >= a.rows) break;
+        cp_async_wait<kDepth - 1>();
+        slot_add(a.nm[r], ws.w[r][lane], ws.J[r % kDepth], lane, acc[r % C]);
+        if (r + kDepth < kRows) slot_fetch(sb.jc, a.nm[r + kDepth], ws.J[r % kDepth], lane);
+        cp_async_commit();
+    }
+#pragma unroll 1
+    for (int r = kRows; r < a.rows; r++) {  // lists longer than kRows L slots (padding has membership 0)
+        const size_t e = a.base + 32 * (size_t)r;
+        const uint32_t nm = live ? d.lp_nm[dir][e] : 0u;
+        typename Pair2<T>::type w;
+        if (sizeof(T) == 4) w.x = (T)d.lp_wf[dir][e].x, w.y = (T)d.lp_wf[dir][e].y;
+        else w.x = (T)d.lp_w[dir][e].x, w.y = (T)d.lp_w[dir][e].y;
+        slot_fetch(sb.jc, nm, ws.J[0], lane);
+        cp_async_commit();
+        cp_async_wait<0>();
+        if (C == 2 && (r & 1)) slot_add(nm, w, ws.J[0], lane, acc[C - 1]);
+        else slot_add(nm, w, ws.J[0], lane, acc[0]);
+    }
+    cp_async_wait<0>();
+    // lane s gets components C s, ... of the lanes' sum
+    T sum[C];
+    if (L == 4) {
+        const bool odd = s & 1, high = s & 2;
+        const T p0 = (odd ? acc[0][1] : acc[0][0]) + __shfl_xor_sync(kFull, odd ? acc[0][0] : acc[0][1], 1);
+        const T p1 = (odd ? acc[0][3] : acc[0][2]) + __shfl_xor_sync(kFull, odd ? acc[0][2] : acc[0][3], 1);
+        sum[0] = (high ? p1 : p0) + __shfl_xor_sync(kFull, high ? p0 : p1, 2);
+    } else {
+#pragma unroll
+        for (int c = 0; c < C; c++) {
+            T pr[C];
+#pragma unroll
+            for (int h = 0; h < C; h++)
+                pr[h] = (s ? acc[h][2 + c] : acc[h][c]) + __shfl_xor_sync(kFull, s ? acc[h][c] : acc[h][2 + c], 1);
+            sum[c] = pr[0] + pr[C - 1];
+        }
+    }
+    T w[4];
+    if (plain) {
+        // forward dU* = -(R + acc) / D, backward dU = dU* - acc / D
+        T *out = (fwd ? sb.dUs : sb.dU) + 4 * (size_t)(live ? k : 0) + C * s;
+        T wn[C];
+#pragma unroll
+        for (int c = 0; c < C; c++) wn[c] = fwd ? -((T)a.R[c] + sum[c]) * a.iD : fma(-sum[c], a.iD, dus[c]);
+        if (live) {
+#pragma unroll
+            for (int c = 0; c < C; c++) out[c] = wn[c];
+        }
+#pragma unroll
+        for (int c = 0; c < 4; c++) w[c] = __shfl_sync(kFull, wn[c % C], lane - s + c / C);
+    } else {
+        T tot[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) tot[c] = __shfl_sync(kFull, sum[c % C], lane - s + c / C), w[c] = T(0);
+        if (live && s == 0) sweep_point<T>(fwd, d, st, sb, k, false, 1.0, 0.0, 0.0, 1.0, tot, w);
+#pragma unroll
+        for (int c = 0; c < 4; c++) w[c] = __shfl_sync(kFull, w[c], lane - s);
+    }
+    if (!live) return;
+    if (JVP == 0) {
+        const JvpBase<T> jb = jvp_base(a.P, w);
+        T J[4];
+        if (L == 4) {
+            jvp_axis_sel<T>(a.P, jb, s < 2, !(s & 1), a.Ap, a.EK, a.B, a.BS, a.UE, J);
+            store4(sb.jc + 16 * (size_t)k + 4 * s, J);
+        } else {
+            T Jm[4];
+            jvp_axis_pair<T>(a.P, jb, s == 0, a.Ap, a.Am, a.EK, a.B, a.BS, a.UE, J, Jm);
+            store4(sb.jc + 16 * (size_t)k + 8 * s, J);
+            store4(sb.jc + 16 * (size_t)k + 8 * s + 4, Jm);
+        }
+    } else {
+#pragma unroll 1
+        for (int c = 0; c < C; c++) store_increment_product<T>(d, st, g_math, sb, w, k, C * s + c);
+    }
+}
+
+// A warp of packed slots of points in a (t, n) frame, exact products: what
+// the level boundary does not change, loaded while the block waits there.
+// The slot's point (-1: none, or frozen), its place among the point's lanes
+// (r of seg, from lane head), the slot's neighbour and weighted Jacobian, the
+// axis Jacobian that the lane applies, and in the point's first lane R, 1/D
+// and the wall normal.
+template <typename T>
+struct FramedPre {
+    int k, f, nb, steps, head, seg, r;
+    bool slot, wall;
+    T M[16], F[16], iD, nx, ny;
+    double R[4];
+};
+
+template <typename T>
+__device__ __forceinline__ const T *axis_jacobians(const Dev &d, int f)
+{
+    return (sizeof(T) == 4 ? (const T *)d.fjf : (const T *)d.fj) + 64 * (size_t)f;
+}
+
+template <typename T>
+__device__ __forceinline__ void framed_load(const Dev &d, int dir, int fw, int lane, FramedPre<T> &a)
+{
+    const size_t e = (size_t)fw * 32 + lane;
+    a.k = d.pk_k[dir][e];
+    const int f2 = d.pk_f[dir][e];
+    a.f = f2 >> 1;
+    a.wall = f2 & 1;
+    a.nb = d.pk_nbr[dir][e];
+    a.slot = d.pk_mb[dir][e] != 0;
+    a.steps = d.pk_steps[dir][fw];
+    const T *M = (sizeof(T) == 4 ? (const T *)d.pk_jmf[dir] : (const T *)d.pk_jm[dir]) + 16 * e;
+#pragma unroll
+    for (int c = 0; c < 4; c++) load4(M + 4 * c, a.M + 4 * c);
+    const unsigned m = __match_any_sync(kFull, a.k);
+    a.head = __ffs(m) - 1;
+    a.seg = __popc(m);
+    a.r = lane - a.head;
+    const int k = a.k;
+    if (k < 0) {
+        a.slot = false;
+        return;
+    }
+    if (a.r < 4) {
+        const T *F = axis_jacobians<T>(d, a.f) + 16 * a.r;
+#pragma unroll
+        for (int c = 0; c < 4; c++) load4(F + 4 * c, a.F + 4 * c);
+    }
+    if (a.r == 0) {
+        a.iD = (T)d.iD[k];
+        if (a.wall) {
+            a.nx = (T)d.wnx[k];
+            a.ny = (T)d.wny[k];
+        }
+#pragma unroll
+        for (int c = 0; c < 4; c++) a.R[c] = dir == 0 ? d.R[c * d.ld + k] : 0.0;
+    }
+    if (frozen(d, k)) a.k = -1, a.slot = false;
+}
+
+template <typename T>
+__device__ __forceinline__ void mat_vec(const T M[16], const T w[4], T J[4])
+{
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        J[c] = M[4 * c] * w[0];
+#pragma unroll
+        for (int j = 1; j < 4; j++) J[c] = fma(M[4 * c + j], w[j], J[c]);
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ void framed_run(const Dev &d, const SweepBufs<T> &sb, int dir, int lane,
+                                           const FramedPre<T> &a)
+{
+    const bool fwd = dir == 0, live = a.k >= 0;
+    const int k = a.k;
+    T acc[4] = {T(0), T(0), T(0), T(0)}, dus[4] = {T(0), T(0), T(0), T(0)}, dl[4] = {T(0), T(0), T(0), T(0)};
+    if (a.slot) load4_l2((fwd ? sb.dUs : sb.dU) + 4 * (size_t)a.nb, dl);  // earlier levels' increments
+    if (live && a.r == 0 && !fwd) load4_l2(sb.dUs + 4 * (size_t)k, dus);
+    if (a.slot) {
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+#pragma unroll
+            for (int j = 0; j < 4; j++) acc[c] = fma(a.M[4 * c + j], dl[j], acc[c]);
+    }
+    // segmented suffix sum: lane l adds lane l + o of the same point; the
+    // warp's longest list bounds the steps (warp-uniform)
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        if (o >= (1 << a.steps)) break;
+        T v[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) v[c] = __shfl_down_sync(kFull, acc[c], o);
+        if (a.r + o < a.seg) {
+#pragma unroll
+            for (int c = 0; c < 4; c++) acc[c] += v[c];
+        }
+    }
+    T w[4] = {T(0), T(0), T(0), T(0)};
+    if (live && a.r == 0) {  // the point's first lane finishes it
+#pragma unroll
+        for (int c = 0; c < 4; c++) w[c] = fwd ? -((T)a.R[c] + acc[c]) * a.iD : fma(-acc[c], a.iD, dus[c]);
+        if (a.wall) {
+            const T mn = w[1] * a.nx + w[2] * a.ny;
+            w[1] -= mn * a.nx;
+            w[2] -= mn * a.ny;
+        }
+        store4((fwd ? sb.dUs : sb.dU) + 4 * (size_t)k, w);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; c++) w[c] = __shfl_sync(kFull, w[c], a.head);
+    if (!live) return;
+    // lane r of the point's seg lanes forms the axis products r, r + seg, ...
+    T J[4];
+    if (a.r < 4) {
+        mat_vec(a.F, w, J);
+        store4(sb.jc + 16 * (size_t)k + 4 * a.r, J);
+    }
+#pragma unroll 1
+    for (int cb = a.r + a.seg; cb < 4; cb += a.seg) {
+        const T *F = axis_jacobians<T>(d, a.f) + 16 * cb;
+        T Fc[16];
+#pragma unroll
+        for (int c = 0; c < 4; c++) load4(F + 4 * c, Fc + 4 * c);
+        mat_vec(Fc, w, J);
+        store4(sb.jc + 16 * (size_t)k + 4 * cb, J);
+    }
+}
+
+// The same for the increment products and for the revised LU-SGS.
+template <int JVP, typename T>
+__device__ __noinline__ void sweep_framed(const Dev &d, const StateSet &st, const SweepBufs<T> &sb, int dir, int fw,
+                                          int lane)
+{
+    const bool fwd = dir == 0;
+    const T *dW = fwd ? sb.dUs : sb.dU;  // earlier levels' increments
+    T acc[4] = {T(0), T(0), T(0), T(0)};
+    T w[4] = {T(0), T(0), T(0), T(0)};
+    const size_t e = (size_t)fw * 32 + lane;
+    const int pos = d.pk_pt[dir][e];  // sweep position of the slot's point, -1: padding
+    const int k = pos >= 0 ? (fwd ? d.sw_fwd : d.sw_bwd)[pos] : 0;
+    const bool live = pos >= 0 && !frozen(d, k);
+    const int fk = d.flag[k];
+    const bool wall = fk == kWall, framed = fk != kInterior;
+    double e1x, e1y, e2x, e2y;
+    point_frame(d, k, framed, e1x, e1y, e2x, e2y);
+    const int mb = d.pk_mb[dir][e];
+    if (live && mb) {
+        if (JVP == 0) {
+            // the slot's weighted Jacobian, formed before the sweeps: acc += M dW_i
+            const T *M = (sizeof(T) == 4 ? (const T *)d.pk_jmf[dir] : (const T *)d.pk_jm[dir]) + 16 * e;
+            T dl[4];
+            load4_l2(dW + 4 * (size_t)d.pk_nbr[dir][e], dl);
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                T Mc[4];
+                load4(M + 4 * c, Mc);
+#pragma unroll
+                for (int j = 0; j < 4; j++) acc[c] = fma(Mc[j], dl[j], acc[c]);
+            }
+        } else {
+            const T w1 = sizeof(T) == 4 ? (T)d.pk_w1f[dir][e] : (T)d.pk_w1[dir][e];
+            const T w2 = sizeof(T) == 4 ? (T)d.pk_w2f[dir][e] : (T)d.pk_w2[dir][e];
+            sweep_slot<JVP, T>(d, st, g_math, dW, sb.prim, framed, e1x, e1y, e2x, e2y, d.pk_nbr[dir][e], mb, w1, w2,
+                               acc);
+        }
+    }
+    // segmented suffix sum: lane l adds lane l + o when both hold the same
+    // point; the warp's longest list bounds the steps (warp-uniform)
+    const int steps = d.pk_steps[dir][fw];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        if (o >= (1 << steps)) break;
+        const int p2 = __shfl_down_sync(kFull, pos, o);
+        T v[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) v[c] = __shfl_down_sync(kFull, acc[c], o);
+        if (lane + o < 32 && p2 == pos) {
+#pragma unroll
+            for (int c = 0; c < 4; c++) acc[c] += v[c];
+        }
+    }
+    // the point's lanes (consecutive; padding lanes form their own group):
+    // the first finishes the point, then lane r of the point's seg lanes
+    // forms the products r, r + seg, ... of the new increment
+    const unsigned m = __match_any_sync(kFull, pos);
+    const int head = __ffs(m) - 1, seg = __popc(m), r = lane - head;
+    if (live && r == 0) sweep_point<T>(fwd, d, st, sb, k, wall, e1x, e1y, e2x, e2y, acc, w);
+#pragma unroll
+    for (int c = 0; c < 4; c++) w[c] = __shfl_sync(kFull, w[c], head);
+    if (!live) return;
+    if (JVP == 0) {
+        // the point's axis Jacobians, formed before the sweeps
+        const T *F = (sizeof(T) == 4 ? (const T *)d.fjf : (const T *)d.fj) + 64 * (size_t)d.fidx[k];
+        for (int cb = r; cb < 4; cb += seg) {
+            T J[4];
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                T Fc[4];
+                load4(F + 16 * cb + 4 * c, Fc);
+                J[c] = Fc[0] * w[0];
+#pragma unroll
+                for (int j = 1; j < 4; j++) J[c] = fma(Fc[j], w[j], J[c]);
+            }
+            store4(sb.jc + 16 * (size_t)k + 4 * cb, J);
+        }
+    } else {
+        for (int cb = r; cb < 4; cb += seg) store_increment_product<T>(d, st, g_math, sb, w, k, cb);
+    }
+}
+
+// The sweeps' levels (dirs: 1 forward, 2 backward, 3 both), one cooperative
+// launch.  A neighbour's Jacobian product along an axis depends only on the
+// neighbour, the axis and the sub-stencil's sign, so a point forms the four
+// axis products of its new increment once, and interior points gather them: 8
+// FMAs per slot instead of ~70 FP64 instructions.  A point's sum depends only
+// on its own list, in a fixed order, so a batch still equals its single
+// solves bit for bit.  A level's tasks are one warp each: first its warps for
+// the points in a (t, n) frame (their slots packed whole into warps at create,
+// by best fit; a point with an empty list takes one idle slot), then its
+// groups of interior points; task t goes to warp t / gridDim of block
+// t % gridDim, so a level spreads over all SMs before it stacks up on one.
+// Between levels all blocks meet; what the next level reads of the cloud and
+// of the iteration's state is loaded while a block waits there, the values
+// other blocks wrote (increments, axis products) after it, from L2.
+// fuse: the framed points' Jacobians are formed here first (else by
+// k_framed_jac beside the q-derivatives).
+template <int JVP, typename T>
+__global__ void __launch_bounds__(kSweepBlock, 1) k_sweeps(Dev d, StateSet st, int n_levels, int dirs, bool fuse)
+{
+    if (halted(d.ctrl)) return;  // the same for every block: set by earlier launches only
+    const int lane = threadIdx.x & 31, t0 = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    const int stride = (blockDim.x >> 5) * gridDim.x;
+    const SweepBufs<T> sb = sweep_bufs<T>(d, st);
+    const int steps = n_levels * (dirs == 3 ? 2 : 1);
+    const uint32_t limit = (uint32_t)(steps - 1 + (fuse ? 1 : 0)) * gridDim.x;
+    uint32_t target = 0;
+    extern __shared__ __align__(16) unsigned char smem[];
+    WarpStage<T> &ws = reinterpret_cast<WarpStage<T> *>(smem)[threadIdx.x >> 5];
+    const bool exact = JVP == 0 && d.lusgs == 0;
+    LanePre<T> pre;
+    FramedPre<T> fpre;
+    bool ready = false;  // pre or fpre holds the warp's first task of the level
+    for (int step = fuse ? -1 : 0; step < steps; step++) {
+        if (step < 0) {
+            for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < framed_jac_items(d); t += gridDim.x * blockDim.x)
+                framed_jac_item<T>(d, st, g_math, t);
+        } else {
+            const int dir = dirs == 3 ? (step < n_levels ? 0 : 1) : dirs - 1;
+            const int l = dir == 0 ? step : steps - 1 - step;
+            const int wb = d.lvl_fw[dir][l], wf = d.lvl_fw[dir][l + 1] - wb;
+            const int g0 = d.lvl_in[dir][l], nt = wf + d.lvl_in[dir][l + 1] - g0;
+            const bool two = d.lvl_lanes[l] == 2;
+            for (int t = t0; t < nt; t += stride) {
+                if (t < wf) {
+                    if (exact) {
+                        if (!ready) framed_load<T>(d, dir, wb + t, lane, fpre);
+                        framed_run<T>(d, sb, dir, lane, fpre);
+                    } else {
+                        sweep_framed<JVP, T>(d, st, sb, dir, wb + t, lane);
+                    }
+                } else if (two) {
+                    if (!ready) lane_load<JVP, 2, T>(d, sb, dir, g0 + t - wf, lane, ws, pre);
+                    sweep_interior<JVP, 2, T>(d, st, sb, dir, lane, pre, ws);
+                } else {
+                    if (!ready) lane_load<JVP, 4, T>(d, sb, dir, g0 + t - wf, lane, ws, pre);
+                    sweep_interior<JVP, 4, T>(d, st, sb, dir, lane, pre, ws);
+                }
+                ready = false;
+            }
+        }
+        if (step + 1 < steps) {
+            boundary_arrive(d.ctrl, limit);
+            const int dir = dirs == 3 ? (step + 1 < n_levels ? 0 : 1) : dirs - 1;
+            const int l = dir == 0 ? step + 1 : steps - 2 - step;
+            const int wb = d.lvl_fw[dir][l], wf = d.lvl_fw[dir][l + 1] - wb;
+            const int g0 = d.lvl_in[dir][l], nt = wf + d.lvl_in[dir][l + 1] - g0;
+            if (t0 < wf) {
+                // (before the first level the matrices may still be being formed)
+                if (exact && step >= 0) {
+                    framed_load<T>(d, dir, wb + t0, lane, fpre);
+                    ready = true;
+                }
+            } else if (t0 < nt) {
+                if (d.lvl_lanes[l] == 2) lane_load<JVP, 2, T>(d, sb, dir, g0 + t0 - wf, lane, ws, pre);
+                else lane_load<JVP, 4, T>(d, sb, dir, g0 + t0 - wf, lane, ws, pre);
+                ready = true;
+            }
+            target += gridDim.x;
+            if (!boundary_wait(d.ctrl, target, limit)) return;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1600,6 +2044,7 @@ __global__ void k_reset_ctrl(Ctrl *c)
     c->stop = 0;
     c->error = 0;
     c->bad_point = 0x7fffffff;
+    c->sweep_bar = 0;
 }
 
 __global__ void k_prep_run(Ctrl *c, double target)
@@ -1607,6 +2052,7 @@ __global__ void k_prep_run(Ctrl *c, double target)
     c->stop = 0;
     c->error = 0;
     c->bad_point = 0x7fffffff;
+    c->sweep_bar = 0;
     c->target = target;
     c->it_start = c->it;
     for (int b = 0; b < c->n_cases; b++)
@@ -1691,13 +2137,12 @@ void enqueue_sweeps_g(const Dev &d, int cur, int n_levels, const int32_t *lvl_be
 // The packed exact sweeps apply precomputed framed-point Jacobians.
 bool needs_framed_jac(const Dev &d, const Launch &L)
 {
-    return d.scheme == 0 && d.jvp == 0 && L.sweep_lanes == 32 && (d.pk_jm[0] || d.pk_jmf[0]) &&
-           4 * (d.pk_lanes[0] + d.pk_lanes[1]) + 16 * d.nf > 0;
+    return d.scheme == 0 && d.jvp == 0 && L.sweep_lanes == 32 && (d.pk_jm[0] || d.pk_jmf[0]) && framed_jac_items(d) > 0;
 }
 
 void enqueue_framed_jac(const Dev &d, int cur, cudaStream_t s, int *launches)
 {
-    const int items = 4 * (d.pk_lanes[0] + d.pk_lanes[1]) + 16 * d.nf;
+    const int items = framed_jac_items(d);
     if (d.precision) k_framed_jac<float><<<(items + 255) / 256, 256, 0, s>>>(d, d.set[cur]);
     else k_framed_jac<double><<<(items + 255) / 256, 256, 0, s>>>(d, d.set[cur]);
     (*launches)++;
@@ -1709,46 +2154,47 @@ void enqueue_diag(const Dev &d, int cur, cudaStream_t s, int *launches)
     (*launches)++;
 }
 
-template <int JVP>
-void enqueue_sweeps_packed(const Dev &d, const Launch &L, int cur, int n_levels, cudaStream_t s, int *launches,
-                           bool fwd, bool bwd)
+template <int JVP, typename T>
+cudaError_t launch_sweeps(const Dev &d, const Launch &L, int cur, int n_levels, int dirs, bool fuse, cudaStream_t s)
 {
-    const StateSet st = d.set[cur];
-    if (fwd && !L.side && needs_framed_jac(d, L)) enqueue_framed_jac(d, cur, s, launches);
-    for (int l = 0; fwd && l < n_levels; l++) {
-        const int wb = L.pk_lw[0][l], wf = L.pk_lw[0][l + 1] - wb;
-        const int g0 = L.lp_lg[0][l], ng = L.lp_lg[0][l + 1] - g0;
-        if (wf + ng <= 0) continue;
-        const int blocks = ((wf + ng) * 32 + kSweepBlock - 1) / kSweepBlock;
-        if (d.precision) k_sweep_packed<JVP, true, float><<<blocks, kSweepBlock, 0, s>>>(d, st, wb, wf, g0, ng);
-        else k_sweep_packed<JVP, true, double><<<blocks, kSweepBlock, 0, s>>>(d, st, wb, wf, g0, ng);
-        (*launches)++;
-    }
-    for (int l = n_levels - 1; bwd && l >= 0; l--) {
-        const int wb = L.pk_lw[1][l], wf = L.pk_lw[1][l + 1] - wb;
-        const int g0 = L.lp_lg[1][l], ng = L.lp_lg[1][l + 1] - g0;
-        if (wf + ng <= 0) continue;
-        const int blocks = ((wf + ng) * 32 + kSweepBlock - 1) / kSweepBlock;
-        if (d.precision) k_sweep_packed<JVP, false, float><<<blocks, kSweepBlock, 0, s>>>(d, st, wb, wf, g0, ng);
-        else k_sweep_packed<JVP, false, double><<<blocks, kSweepBlock, 0, s>>>(d, st, wb, wf, g0, ng);
-        (*launches)++;
-    }
+    Dev dd = d;
+    StateSet st = d.set[cur];
+    void *args[] = {&dd, &st, &n_levels, &dirs, &fuse};
+    const size_t smem = (size_t)(L.sw_threads / 32) * sizeof(WarpStage<T>);
+    const void *kernel = (const void *)k_sweeps<JVP, T>;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return cudaLaunchCooperativeKernel(kernel, dim3(L.sw_blocks), dim3(L.sw_threads), args, smem, s);
 }
 
+template <int JVP>
+cudaError_t enqueue_sweeps_packed(const Dev &d, const Launch &L, int cur, int n_levels, cudaStream_t s, int *launches,
+                                  bool fwd, bool bwd)
+{
+    // the framed points' Jacobians: by k_framed_jac in the packed shape
+    // (beside the q-derivatives when captured), else by the sweeps' launch
+    if (fwd && !L.side && needs_framed_jac(d, L)) enqueue_framed_jac(d, cur, s, launches);
+    const bool fuse = fwd && JVP == 0 && L.sweep_lanes != 32 && framed_jac_items(d) > 0;
+    const int dirs = (fwd ? 1 : 0) + (bwd ? 2 : 0);
+    if (n_levels <= 0 || dirs == 0) return cudaSuccess;
+    (*launches)++;
+    return d.precision ? launch_sweeps<JVP, float>(d, L, cur, n_levels, dirs, fuse, s)
+                       : launch_sweeps<JVP, double>(d, L, cur, n_levels, dirs, fuse, s);
+}
+
+// Clouds whose lists fit the packed layout use the gathered form in every
+// shape (sweep_lanes 2, 4, 8 and 32 differ in who forms the framed points'
+// Jacobians); a list of more than 32 lower or upper neighbours needs the
+// per-slot form, one launch per level.
 template <int JVP>
 cudaError_t enqueue_sweeps(const Dev &d, const Launch &L, int cur, int n_levels, const int32_t *lvl_beg,
                            const int32_t *lvl_act_end, cudaStream_t s, int *launches, bool fwd, bool bwd)
 {
+    if (d.pk_pt[0]) return enqueue_sweeps_packed<JVP>(d, L, cur, n_levels, s, launches, fwd, bwd);
     switch (L.sweep_lanes) {
     case 2: enqueue_sweeps_g<JVP, 2>(d, cur, n_levels, lvl_beg, lvl_act_end, s, launches, fwd, bwd); break;
     case 4: enqueue_sweeps_g<JVP, 4>(d, cur, n_levels, lvl_beg, lvl_act_end, s, launches, fwd, bwd); break;
     case 8: enqueue_sweeps_g<JVP, 8>(d, cur, n_levels, lvl_beg, lvl_act_end, s, launches, fwd, bwd); break;
-    case 32:
-        if (!d.pk_pt[0] || !L.pk_lw[0] || !L.lp_lg[0] || !(d.precision ? (void *)d.jcf : (void *)d.jc))
-            return cudaErrorInvalidValue;
-        if (JVP == 0 && !(d.precision ? (void *)d.pk_jmf[0] : (void *)d.pk_jm[0])) return cudaErrorInvalidValue;
-        enqueue_sweeps_packed<JVP>(d, L, cur, n_levels, s, launches, fwd, bwd);
-        break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -1795,8 +2241,12 @@ cudaError_t enqueue_phase(const Dev &d, const Launch &L, int cur, int ph, int n_
             }
             return cudaGetLastError();
         }
-        if (d.jvp == 0) return enqueue_sweeps<0>(d, L, cur, n_levels, lvl_beg, lvl_act_end, s, launches, ph == 3, ph == 4);
-        return enqueue_sweeps<1>(d, L, cur, n_levels, lvl_beg, lvl_act_end, s, launches, ph == 3, ph == 4);
+        {
+            // a captured iteration enqueues both sweeps in phase 3
+            const bool both = L.side != nullptr, fwd = ph == 3, bwd = both ? ph == 3 : ph == 4;
+            if (d.jvp == 0) return enqueue_sweeps<0>(d, L, cur, n_levels, lvl_beg, lvl_act_end, s, launches, fwd, bwd);
+            return enqueue_sweeps<1>(d, L, cur, n_levels, lvl_beg, lvl_act_end, s, launches, fwd, bwd);
+        }
     case 5:
         k_update<<<(d.n + 255) / 256, 256, 0, s>>>(d, cur, true, true);
         (*launches)++;
