@@ -220,10 +220,25 @@ struct FxSum {
     int64_t hh, l, r;
 };
 
+// The two signed parts of a word that was biased by 2^31: high 2^32 + low.
+LSKUM_HD void split_word(uint64_t biased, int32_t &high, int32_t &low)
+{
+#ifdef __CUDA_ARCH__
+    // (opaque: from a shift the compiler forms some of the products with the
+    // high part as 64x64-bit ones)
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(low), "=r"(high) : "l"(biased));
+#else
+    low = (int32_t)(uint32_t)biased;
+    high = (int32_t)(uint32_t)(biased >> 32);
+#endif
+    low ^= (int32_t)0x80000000;
+}
+
 LSKUM_HD void fx_add(FxSum &s, int32_t wh, int32_t wl, uint64_t Gi, uint64_t G0)
 {
     const uint64_t D = Gi - G0 + 0x80000000ull;  // |Gi - G0| < 2^62.4
-    const int32_t dh = (int32_t)(uint32_t)(D >> 32), dl = (int32_t)((uint32_t)D ^ 0x80000000u);
+    int32_t dh, dl;
+    split_word(D, dh, dl);
     s.hh += (int64_t)wh * dh;
     s.l += (int64_t)wh * dl;
     s.r += (int64_t)wl * dh;

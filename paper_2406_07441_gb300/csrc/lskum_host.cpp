@@ -2,6 +2,7 @@
 // LU-SGS sweep order (Alg. 5), the internal point order and neighbour layout,
 // per-slot least-squares weights, device memory, one CUDA graph per
 // iteration parity, and the C-ABI of include/lskum.h.
+#include "lskum_fixgrad.cuh"
 #include "lskum_internal.h"
 #include "lskum_mlp_internal.h"
 
@@ -12,9 +13,12 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <numeric>
 #include <string>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "../../include/lskum.h"
@@ -217,8 +221,10 @@ struct HostPrep {
     std::vector<uint8_t> emb, fl_i;
     std::vector<uint4> ewq;       // residual weights, integers and remainders in units of G_WSC
     std::vector<double2> ehxy;    // half offsets
-    std::vector<double> egx, egy, geo_i, wnx, wny;
-    std::vector<double> exx, exy, eyx, eyy;  // wgx dx, wgx dy, wgy dx, wgy dy per slot
+    std::vector<double> geo_i, wnx, wny;
+    std::vector<uint4> ewg, ewj, wc;  // the q-derivatives' weights (Dev::wg, ...)
+    std::vector<short4> ge;
+    std::vector<short2> gb;
     // LU-SGS lower / upper slot lists (CSR, internal order) and level orders
     std::vector<int32_t> lo_off, lo_nbr, up_off, up_nbr, sw_fwd, sw_bwd;
     std::vector<uint8_t> lo_mb, up_mb;
@@ -238,13 +244,95 @@ struct HostPrep {
 };
 static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &hp);
 
+// f over ranges of 0..n - 1, in threads where there is enough to do (32,768
+// points each, at most 8: the slots' weights of 147,584 points take 0.12 s of
+// a create's 0.40 s in one).
+static void in_threads(int32_t n, const std::function<void(int32_t, int32_t)> &f)
+{
+    const int32_t parts = std::max(1, std::min({n / 32768, 8, (int32_t)std::thread::hardware_concurrency()}));
+    std::vector<std::thread> pool;
+    int32_t from = 0;
+    for (int32_t i = 1; i < parts; i++) {
+        const int32_t to = (int32_t)((int64_t)n * i / parts);
+        try {
+            pool.emplace_back(std::cref(f), from, to);
+        } catch (const std::system_error &) {
+            break;  // (no more threads: the rest here)
+        }
+        from = to;
+    }
+    f(from, n);
+    for (std::thread &t : pool) t.join();
+}
+
+// The nearest integer of |v| < 2^51 (llrint is a call unless errno is given up).
+static inline double nearest(double v)
+{
+    return (v + 0x1.8p52) - 0x1.8p52;
+}
+
 // A residual weight w in units of `unit` (a power of two, 0 where the point
 // has none): the nearest integer and the remainder in units of 2^-24.
 static uint2 split_weight(double w, double unit)
 {
     if (!(unit > 0.0)) return uint2{0, 0};
-    const double v = w / unit, r = std::nearbyint(v);
-    return uint2{(uint32_t)(int32_t)r, (uint32_t)(int32_t)std::nearbyint(std::ldexp(v - r, 24))};
+    const double v = w * (1.0 / unit);
+    const double r = nearest(v);
+    return uint2{(uint32_t)(int32_t)r, (uint32_t)(int32_t)nearest((v - r) * 0x1p24)};
+}
+
+// The smallest e with sum < 2^e (1 - 2^-16), so that up to 512 terms of that sum
+// of magnitudes, rounded to integers in units of 2^(e - 31), stay below 2^31.
+static int sum_exponent(double sum)
+{
+    int e = 0;
+    if (!std::isfinite(sum)) return kGradNoScale;
+    return std::frexp(sum, &e) < 1.0 - 0x1p-16 ? e : e + 1;
+}
+
+// 2^e.
+static double power(int e)
+{
+    if (e < -1000 || e > 1000) return std::ldexp(1.0, e);
+    const uint64_t bits = (uint64_t)(1023 + e) << 52;
+    double v;
+    std::memcpy(&v, &bits, sizeof v);
+    return v;
+}
+
+// The nearest integer of a scaled weight (0 where it has none, being not finite), and the rest.
+static int32_t weight_int(double &v)
+{
+    if (!(std::fabs(v) < 0x1p31)) return v = 0.0, 0;
+    const double r = nearest(v);
+    v -= r;
+    return (int32_t)(int64_t)r;
+}
+
+// The weights of the two derivatives of a point, v[2 m] and v[2 m + 1] of each
+// of n words scaled to units of their integers: the words, and the bits b of
+// their remainders, as many as let these, in units of 2^-b, add up to less
+// than 2^31 per derivative (up to 512 of them, each rounded).  `first`: word m
+// holds a weight of either derivative (w_x, w_y); else two of the derivative m
+// % 2.
+static int split_words(double *v, int n, bool first, uint4 *out)
+{
+    double sum[2] = {0.0, 0.0};
+    for (int m = 0; m < n; m++) {
+        out[m].x = (uint32_t)weight_int(v[2 * m]);
+        out[m].z = (uint32_t)weight_int(v[2 * m + 1]);
+        sum[first ? 0 : m & 1] += std::fabs(v[2 * m]);
+        sum[first ? 1 : m & 1] += std::fabs(v[2 * m + 1]);
+    }
+    int e = 0;
+    std::frexp(std::max(sum[0], sum[1]) + 0x1p-20, &e);
+    const int b = std::min(kMaxGradBits, 31 - e);
+    const double unit = power(b);
+    for (int m = 0; m < n; m++) {
+        out[m].y = (uint32_t)(int32_t)nearest(v[2 * m] * unit);
+        out[m].w = (uint32_t)(int32_t)nearest(v[2 * m + 1] * unit);
+    }
+    return b;
 }
 
 // Is point p (caller order of the union) an unknown of the iteration?  Outer
@@ -625,6 +713,7 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
     std::vector<uint8_t> &smb = hp.smb_caller;
     smb.assign(nnz, 0);
     std::vector<double> geo((size_t)G_NFIELDS * n, 0.0);
+    std::vector<int> gex(n), gey(n);  // powers of two of the q-derivatives (Dev::ge)
     for (int32_t p = 0; p < n; p++) {
         // frames: (t, n) at wall points (n into the fluid) and at outer points
         // of the kinetic far field (n out of the domain; their n- side is the
@@ -677,14 +766,15 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
         const double gdet = sxx * syy - sxy * sxy;
         if (deg < 2 || !(gdet > 1e-12 * sxx * syy))
             return fail(c, LSKUM_ERR_STENCIL, "degenerate least-squares stencil at point %d", p);
+        double gsx = 0.0, gsy = 0.0;
         for (int32_t e = off[p]; e < off[p + 1]; e++) {
             swgx[e] = (syy * sdx[e] - sxy * sdy[e]) / gdet;
             swgy[e] = (sxx * sdy[e] - sxy * sdx[e]) / gdet;
-            geo[G_SXX * n + p] += swgx[e] * sdx[e];
-            geo[G_SXY * n + p] += swgx[e] * sdy[e];
-            geo[G_SYX * n + p] += swgy[e] * sdx[e];
-            geo[G_SYY * n + p] += swgy[e] * sdy[e];
+            gsx += std::fabs(swgx[e]);
+            gsy += std::fabs(swgy[e]);
         }
+        gex[p] = sum_exponent(gsx);
+        gey[p] = sum_exponent(gsy);
         geo[G_IDMIN * n + p] = 1.0 / dmin;
         if (!swept(c, p)) continue;
         double det[4];
@@ -820,36 +910,83 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
     const size_t esz = std::max<int64_t>(ell, 1);
     std::vector<int32_t> &enb = hp.enb;
     std::vector<uint8_t> &emb = hp.emb;
-    std::vector<double> &egx = hp.egx, &egy = hp.egy;
     hp.ewq.assign(esz, uint4{0, 0, 0, 0});
     hp.ehxy.assign(esz, double2{0.0, 0.0});
     enb.assign(esz, 0);
     emb.assign(esz, 0);
-    for (auto *v : {&egx, &egy, &hp.exx, &hp.exy, &hp.eyx, &hp.eyy}) v->assign(esz, 0.0);
-    for (int32_t k = 0; k < n; k++) {
-        const int32_t p = c->perm[k];
-        deg[k] = off[p + 1] - off[p];
-        const int64_t base = slice_off[k / 32] + (k % 32);
-        const int32_t w = (slice_off[k / 32 + 1] - slice_off[k / 32]) / 32;
-        for (int32_t j = 0; j < w; j++) enb[base + 32 * j] = k;  // padding: self, never read
-        for (int32_t j = 0; j < deg[k]; j++) {
-            const int64_t e = off[p] + j, t = base + 32 * j;
-            enb[t] = c->inv[idx[e]];
-            emb[t] = smb[e];
-            // half offsets (exact): the residual's reconstruction steps
-            // q - (dx, dy)/2 . grad q
-            hp.ehxy[t] = double2{0.5 * sdx[e], 0.5 * sdy[e]};
-            const uint2 wa = split_weight(sw1[e], geo[(size_t)G_WSC * n + p]);
-            const uint2 wb = split_weight(sw2[e], geo[(size_t)G_WSC * n + p]);
-            hp.ewq[t] = uint4{wa.x, wa.y, wb.x, wb.y};
-            egx[t] = swgx[e];
-            egy[t] = swgy[e];
-            hp.exx[t] = swgx[e] * sdx[e];
-            hp.exy[t] = swgx[e] * sdy[e];
-            hp.eyx[t] = swgy[e] * sdx[e];
-            hp.eyy[t] = swgy[e] * sdy[e];
+    hp.ewg.assign(esz, uint4{0, 0, 0, 0});
+    hp.ewj.assign(2 * esz, uint4{0, 0, 0, 0});
+    hp.wc.assign(2 * (size_t)ld, uint4{0, 0, 0, 0});
+    hp.ge.assign(ld, short4{0, 0, 0, 0});
+    hp.gb.assign(ld, short2{0, 0});
+    auto pack = [&](int32_t from, int32_t to) {
+        double pv[4 * 256];  // a point's scaled weights (at most 255 slots and the centre) and their words
+        uint4 pw[2 * 256];
+        for (int32_t k = from; k < to; k++) {
+            const int32_t p = c->perm[k];
+            deg[k] = off[p + 1] - off[p];
+            const int64_t base = slice_off[k / 32] + (k % 32);
+            const int32_t w = (slice_off[k / 32 + 1] - slice_off[k / 32]) / 32;
+            for (int32_t j = 0; j < w; j++) enb[base + 32 * j] = k;  // padding: self, weights 0
+            for (int32_t j = 0; j < deg[k]; j++) {
+                const int64_t e = off[p] + j, t = base + 32 * j;
+                enb[t] = c->inv[idx[e]];
+                emb[t] = smb[e];
+                // half offsets (exact): the residual's reconstruction steps
+                // q - (dx, dy)/2 . grad q
+                hp.ehxy[t] = double2{0.5 * sdx[e], 0.5 * sdy[e]};
+                const uint2 wa = split_weight(sw1[e], geo[(size_t)G_WSC * n + p]);
+                const uint2 wb = split_weight(sw2[e], geo[(size_t)G_WSC * n + p]);
+                hp.ewq[t] = uint4{wa.x, wa.y, wb.x, wb.y};
+            }
+            // q-derivatives: the weights, the inner iterations' coefficients and the
+            // centre's (which add up, in magnitude, per derivative, to less than 2^p)
+            const int ex = gex[p], ey = gey[p], dg = deg[k];
+            const double ix = power(-ex), iy = power(-ey);
+            double cxx = 0, cxy = 0, cyx = 0, cyy = 0, sx = 0, sy = 0;
+            for (int32_t j = 0; j < dg; j++) {
+                const int64_t e = off[p] + j;
+                const double x = -0.5 * sdx[e], y = -0.5 * sdy[e], nx = power(gex[idx[e]]), ny = power(gey[idx[e]]);
+                double *v = &pv[4 * j];
+                cxx -= v[0] = swgx[e] * x;
+                cxy -= v[1] = swgx[e] * y;
+                cyx -= v[2] = swgy[e] * x;
+                cyy -= v[3] = swgy[e] * y;
+                v[0] *= nx * ix;
+                v[1] *= ny * ix;
+                v[2] *= nx * iy;
+                v[3] *= ny * iy;
+                sx += std::fabs(v[0]) + std::fabs(v[1]);
+                sy += std::fabs(v[2]) + std::fabs(v[3]);
+            }
+            double *v = &pv[4 * dg];
+            v[0] = cxx;
+            v[1] = cxy * (power(ey) * ix);
+            v[2] = cyx * (power(ex) * iy);
+            v[3] = cyy;
+            const int px = std::max(0, sum_exponent(sx + std::fabs(v[0]) + std::fabs(v[1])));
+            const int py = std::max(0, sum_exponent(sy + std::fabs(v[2]) + std::fabs(v[3])));
+            const double ux = power(31 - px), uy = power(31 - py);
+            for (int32_t j = 0; j <= dg; j++) {
+                pv[4 * j] *= ux;
+                pv[4 * j + 1] *= ux;
+                pv[4 * j + 2] *= uy;
+                pv[4 * j + 3] *= uy;
+            }
+            const int b2 = split_words(pv, 2 * (dg + 1), false, pw);
+            for (int32_t j = 0; j < dg; j++) std::copy_n(&pw[2 * j], 2, &hp.ewj[2 * (base + 32 * j)]);
+            std::copy_n(&pw[2 * dg], 2, &hp.wc[2 * (size_t)k]);
+            for (int32_t j = 0; j < dg; j++) {
+                pv[2 * j] = swgx[off[p] + j] * ix * 0x1p31;
+                pv[2 * j + 1] = swgy[off[p] + j] * iy * 0x1p31;
+            }
+            const int b1 = split_words(pv, dg, true, pw);
+            for (int32_t j = 0; j < dg; j++) hp.ewg[base + 32 * j] = pw[j];
+            hp.ge[k] = short4{(short)ex, (short)ey, (short)px, (short)py};
+            hp.gb[k] = short2{(short)b1, (short)b2};
         }
-    }
+    };
+    in_threads(n, pack);
     // LU-SGS lists: for each point its slots whose neighbour is earlier (lower)
     // or later (upper) in the sweep order; frozen neighbours (increment 0)
     // and slots in no split sub-stencil contribute nothing and are left out
@@ -1048,8 +1185,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     const int32_t n = c->n, ld = c->ld, nsl = ld / 32;
     std::vector<int32_t> &slice_off = hp.slice_off, &deg = hp.deg, &enb = hp.enb;
     std::vector<uint8_t> &emb = hp.emb, &fl_i = hp.fl_i;
-    std::vector<double> &egx = hp.egx, &egy = hp.egy;
-    const size_t esz = egx.size();
+    const size_t esz = enb.size();
     std::vector<double> &geo_i = hp.geo_i, &wnx = hp.wnx, &wny = hp.wny;
     // ---- device memory ----
     cudaError_t e = cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking);
@@ -1072,14 +1208,18 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     uint8_t *dmb = A.alloc<uint8_t>(emb.size());
     double2 *dhxy = A.alloc<double2>(esz);
     uint4 *dwq = A.alloc<uint4>(esz);
-    double *dgx = A.alloc<double>(esz), *dgy = A.alloc<double>(esz);
-    double *dxx = A.alloc<double>(esz), *dxy = A.alloc<double>(esz);
-    double *dyx = A.alloc<double>(esz), *dyy = A.alloc<double>(esz);
+    uint4 *dwg = A.alloc<uint4>(esz), *dwj = A.alloc<uint4>(2 * esz), *dwc = A.alloc<uint4>(2 * (size_t)ld);
+    short4 *dge = A.alloc<short4>(ld);
+    short2 *dgb = A.alloc<short2>(ld);
     for (int s = 0; s < 2; s++) {
         d.set[s].U = A.alloc<double>(4 * (size_t)ld);
         d.set[s].q = A.alloc<double>(4 * (size_t)ld);
         d.set[s].prim = A.alloc<double>((size_t)kPrimStride * ld);
+        d.set[s].qf = A.alloc<int64_t>(4 * (size_t)ld);
+    }
+    for (int s = 0; s < 3; s++) {
         d.gq[s] = A.alloc<double>(8 * (size_t)ld);
+        d.gf[s] = A.alloc<int4>(4 * (size_t)ld);
     }
     int32_t *dlo_off = A.alloc<int32_t>(n + 1), *dup_off = A.alloc<int32_t>(n + 1);
     int32_t *dlo_nbr = A.alloc<int32_t>(hp.lo_nbr.size()), *dup_nbr = A.alloc<int32_t>(hp.up_nbr.size());
@@ -1191,8 +1331,6 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
         d.fidx = A.alloc<int32_t>(ld);
         d.fpt = A.alloc<int32_t>(std::max<size_t>(h_fpt.size(), 1));
     }
-    d.g1x = A.alloc<double>(4 * (size_t)ld);
-    d.g1y = A.alloc<double>(4 * (size_t)ld);
     d.R = A.alloc<double>(4 * (size_t)ld);
     d.D = A.alloc<double>(ld);
     d.iD = A.alloc<double>(ld);
@@ -1242,12 +1380,11 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     d.memb = dmb;
     d.hxy = dhxy;
     d.wq = dwq;
-    d.wgx = dgx;
-    d.wgy = dgy;
-    d.gxx = dxx;
-    d.gxy = dxy;
-    d.gyx = dyx;
-    d.gyy = dyy;
+    d.wg = dwg;
+    d.wj = dwj;
+    d.wc = dwc;
+    d.ge = dge;
+    d.gb = dgb;
     d.ctrl = c->ctrl;
     d.case_state = c->case_state;
     d.blk_pos = dblk_pos;
@@ -1302,12 +1439,11 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     up(dmb, emb.data(), emb.size());
     up(dhxy, hp.ehxy.data(), esz * sizeof(double2));
     up(dwq, hp.ewq.data(), esz * sizeof(uint4));
-    up(dgx, egx.data(), egx.size() * sizeof(double));
-    up(dgy, egy.data(), egy.size() * sizeof(double));
-    up(dxx, hp.exx.data(), hp.exx.size() * sizeof(double));
-    up(dxy, hp.exy.data(), hp.exy.size() * sizeof(double));
-    up(dyx, hp.eyx.data(), hp.eyx.size() * sizeof(double));
-    up(dyy, hp.eyy.data(), hp.eyy.size() * sizeof(double));
+    up(dwg, hp.ewg.data(), esz * sizeof(uint4));
+    up(dwj, hp.ewj.data(), 2 * esz * sizeof(uint4));
+    up(dwc, hp.wc.data(), 2 * (size_t)ld * sizeof(uint4));
+    up(dge, hp.ge.data(), ld * sizeof(short4));
+    up(dgb, hp.gb.data(), ld * sizeof(short2));
     up(dlo_off, hp.lo_off.data(), hp.lo_off.size() * sizeof(int32_t));
     up(dup_off, hp.up_off.data(), hp.up_off.size() * sizeof(int32_t));
     up(dlo_nbr, hp.lo_nbr.data(), hp.lo_nbr.size() * sizeof(int32_t));
@@ -1379,8 +1515,12 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     }
     if (e != cudaSuccess) return cuda_fail(c, e, "cudaMemcpy");
     // zero intermediates; D = 1 at outer points (never written by the kernels)
-    for (double *p : {d.R, d.dUs, d.dU, d.gq[0], d.gq[0] + 4 * (size_t)ld, d.gq[1], d.gq[1] + 4 * (size_t)ld})
+    for (double *p : {d.R, d.dUs, d.dU})
         if (e == cudaSuccess) e = cudaMemset(p, 0, 4 * (size_t)ld * sizeof(double));
+    for (int s = 0; s < 3; s++) {
+        if (e == cudaSuccess) e = cudaMemset(d.gq[s], 0, 8 * (size_t)ld * sizeof(double));
+        if (e == cudaSuccess) e = cudaMemset(d.gf[s], 0, 4 * (size_t)ld * sizeof(int4));
+    }
     std::vector<double> ones(ld, 1.0);
     up(d.D, ones.data(), ld * sizeof(double));
     up(d.iD, ones.data(), ld * sizeof(double));
@@ -1772,7 +1912,7 @@ lskum_status lskum_get_field(lskum_ctx *c, int32_t field, double *out)
     if (!c || !out) return c ? fail(c, LSKUM_ERR_ARG, "NULL argument") : LSKUM_ERR_ARG;
     if (c->pending) return fail(c, LSKUM_ERR_ARG, "an enqueued run has not been waited for");
     const Dev &d = c->dev;
-    const int K = d.K & 1;
+    const int K = grad_buffer(d.K);
     const double *src = nullptr;
     int comps = 4, stride = 0;
     switch (field) {
@@ -1805,7 +1945,7 @@ lskum_status lskum_get_field_dev(lskum_ctx *c, int32_t field, double *out_dev, v
     if (!c || !out_dev) return c ? fail(c, LSKUM_ERR_ARG, "NULL argument") : LSKUM_ERR_ARG;
     if (c->pending) return fail(c, LSKUM_ERR_ARG, "an enqueued run has not been waited for");
     const Dev &d = c->dev;
-    const int K = d.K & 1;
+    const int K = grad_buffer(d.K);
     const double *src = nullptr;
     const float *srcf = nullptr;
     int comps = 4, stride = 0;
@@ -2029,7 +2169,7 @@ lskum_status lskum_autotune(lskum_ctx *c, int32_t trial_iters, int32_t *tpp, int
     // save the state set (device copies, so the restored state is bitwise
     // the same), the counters and the histories; every trial is restored
     const size_t ld = c->ld;
-    const size_t bytes_d = (8 * ld + (size_t)kPrimStride * ld) * sizeof(double);
+    const size_t bytes_d = (12 * ld + (size_t)kPrimStride * ld) * sizeof(double);
     const size_t bytes_f = c->dev.set[0].primf ? (size_t)kPrimStride * ld * sizeof(float) : 0;
     const size_t bytes_inc = 4 * ld * sizeof(double) + (c->dev.dUf ? 4 * ld * sizeof(float) : 0);
     char *save = nullptr;
@@ -2042,14 +2182,14 @@ lskum_status lskum_autotune(lskum_ctx *c, int32_t trial_iters, int32_t *tpp, int
     auto copy_set = [&](bool to_save) -> cudaError_t {
         const StateSet &st = c->dev.set[c->cur];
         // the state set and the last increments (the revised LU-SGS lags on them)
-        char *parts[6] = {(char *)st.U, (char *)st.q, (char *)st.prim, (char *)st.primf, (char *)c->dev.dU,
-                          (char *)c->dev.dUf};
-        const size_t sz[6] = {4 * ld * sizeof(double), 4 * ld * sizeof(double),
+        char *parts[7] = {(char *)st.U, (char *)st.q, (char *)st.prim, (char *)st.primf, (char *)c->dev.dU,
+                          (char *)c->dev.dUf, (char *)st.qf};
+        const size_t sz[7] = {4 * ld * sizeof(double), 4 * ld * sizeof(double),
                               (size_t)kPrimStride * ld * sizeof(double), bytes_f, 4 * ld * sizeof(double),
-                              c->dev.dUf ? 4 * ld * sizeof(float) : 0};
+                              c->dev.dUf ? 4 * ld * sizeof(float) : 0, 4 * ld * sizeof(int64_t)};
         size_t off = 0;
         cudaError_t ee = cudaSuccess;
-        for (int i = 0; i < 6 && ee == cudaSuccess; i++) {
+        for (int i = 0; i < 7 && ee == cudaSuccess; i++) {
             if (!sz[i]) continue;
             ee = to_save ? cudaMemcpyAsync(save + off, parts[i], sz[i], cudaMemcpyDeviceToDevice, c->stream)
                          : cudaMemcpyAsync(parts[i], save + off, sz[i], cudaMemcpyDeviceToDevice, c->stream);

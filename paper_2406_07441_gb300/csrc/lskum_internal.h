@@ -58,7 +58,6 @@ enum GeoField {
     G_ABS_0, G_ABS_1, G_ABS_2, G_ABS_3,  // sum_i |w_i| of each split sub-stencil
     G_IDMIN,                             // 1 / min_i |r_i - r_0|
     G_WSC,                               // unit of the residual's weights (a power of two)
-    G_SXX, G_SXY, G_SYX, G_SYY,          // sums over the stencil of wgx dx, wgx dy, wgy dx, wgy dy
     G_NFIELDS
 };
 
@@ -89,6 +88,7 @@ static_assert(P_NFIELDS <= kPrimStride, "prim record too small");
 struct StateSet {
     double *U;     // [4][ld] conserved variables
     double *q;     // [ld][4] q-variables (a neighbour's are one 32-byte gather)
+    int64_t *qf;   // [ld][4] q in fixed point (lskum_fixgrad.cuh)
     double *prim;  // [ld][kPrimStride]
     float *primf;  // [ld][kPrimStride] FP32 copy (mixed precision only, else null)
 };
@@ -110,13 +110,24 @@ struct Dev {
     // a point's magnitudes is below 2^30), y, w the remainders in units of
     // 2^-24 (int32)
     const uint4 *wq;
-    const double *wgx, *wgy;  // full-stencil LS weights of d/dx and d/dy (Eq. 10, 16)
-    const double *gxx, *gxy, *gyx, *gyy;  // wgx dx, wgx dy, wgy dx, wgy dy (inner iterations)
+    // full-stencil LS weights of d/dx and d/dy (Eq. 10, 16) in fixed point,
+    // each an integer (31 bits) and a remainder in units of 2^-b: per slot wg =
+    // w_x 2^-e_x, w_y 2^-e_y in units of 2^-31, and the inner iterations'
+    // coefficients wj = -w_x dx/2, -w_x dy/2, -w_y dx/2, -w_y dy/2
+    // over 2^e_x, 2^e_y of the point and times those of the neighbour, in
+    // units of 2^(p_x - 31), 2^(p_y - 31); wc per point: the centre's;
+    // ge = (e_x, e_y, p_x, p_y), gb = the b of wg and of the coefficients
+    const uint4 *wg, *wj, *wc;  // (wj, wc: two words per slot or point)
+    const short4 *ge;
+    const short2 *gb;
     // iteration buffers
     StateSet set[2];
-    double *gq[2];           // double-buffered q-derivatives, [ld][8]: point k's
-                             // (dq/dx 0..3, dq/dy 0..3) at 8k, one 64-byte record
-    double *g1x, *g1y;       // first-order LS derivatives (the fixed part of Eq. 16)
+    // q-derivatives, point k's (d/dx 0..3, d/dy 0..3) at 8k, one 64-byte record
+    // per buffer: [2] first order (the fixed part of Eq. 16), [0], [1] the
+    // inner iterations' in turn.  gf: in fixed point, over 2^e, per component
+    // (x low, x high, y low, y high: see split_g); gq: in FP64, of the last pass and at marked points
+    double *gq[3];
+    int4 *gf[3];
     double *R;               // [4][ld]
     double *D;               // [ld]
     double *iD;              // [ld] 1/D (explicit scheme: the local time step)
@@ -205,6 +216,12 @@ struct Dev {
 
 // Kernel launch wrappers (lskum_kernels.cu).  `cur` is the state set read by
 // this iteration; the update writes set 1 - cur.
+// The q-derivatives' buffer after K inner iterations.
+inline int grad_buffer(int K)
+{
+    return K == 0 ? 2 : 1 - (K & 1);
+}
+
 struct Launch {
     int tpp;          // threads per point of the gradient and residual kernels (1, 2, 4, 8)
     int sms;          // multiprocessors (the residual's persistent grid)

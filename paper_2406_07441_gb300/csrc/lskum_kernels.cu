@@ -33,7 +33,7 @@
 #include <cstdint>
 
 #include "lskum_fastmath.cuh"
-#include "lskum_fixflux.cuh"
+#include "lskum_fixgrad.cuh"
 #include "lskum_fluxtable.h"
 
 namespace lskum {
@@ -463,79 +463,265 @@ __device__ __forceinline__ void store4(float *p, const float v[4])
 // ---------------------------------------------------------------------------
 // An inner iteration's right-hand side sum_i w_i (Delta q_i - Delta r_i .
 // (grad q_i - grad q_0)/2) splits into the first-order term g1 = sum_i w_i
-// Delta q_i, fixed across iterations, and
+// Delta q_i, fixed across iterations, and -1/2 of
 //   sum_i (w_i dx_i) px_i + (w_i dy_i) py_i - px_0 sum_i w_i dx_i - py_0 sum_i w_i dy_i
-// with per-slot products w dx, w dy precomputed: 4 FMAs per component and
-// slot instead of 7 FP64 instructions.
-// The q-derivatives live in 64-byte records ([ld][8]), so a neighbour's
-// previous iterate is two 32-byte sectors instead of eight scattered ones.
-template <int TPP, bool CORR>
-__global__ void __launch_bounds__(256) k_grad(Dev d, const double *__restrict__ q, const double *__restrict__ pg,
-                                              double *__restrict__ g)
+// with the coefficients (-1/2 w dx, ...) precomputed per slot, and the
+// centre's as one more slot.
+//
+// Both passes run in 64-bit fixed point (lskum_fixgrad.cuh) on the integer
+// pipes.  Two lanes per slot, each two of the four components: their sums (16
+// 64-bit words) leave room for the loads in flight, and a pair reads one
+// neighbour's record.  147,584 points, three passes: 0.293 ms in FP64 (its
+// unit 92 % busy), 0.141 ms like this (0.033 first order, 0.047 per inner
+// iteration, which reads 130 MB: 0.019 ms); 41,194 points 0.137 -> 0.054 ms.
+// What is left is the gathers' latency with 20 warps per SM and the multiply
+// pipe, half busy.  Rings of cp.async stages in shared memory (0.182 ms) and
+// slots along a space-filling curve (the same) were no faster.
+
+// 32 bytes with one load (a pair's 64-byte record is one L1 tag instead of two).
+template <typename T>
+__device__ __forceinline__ void load32(const T *p, uint4 &a, uint4 &b)
 {
-    if (halted(d.ctrl)) return;
-    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const int k = gt / TPP, sub = gt % TPP;
-    const bool active = k < d.n;
-    const int kk = active ? k : d.n - 1;
-    const int ld = d.ld;
-    double q0[4], sx[4], sy[4];
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        if (!CORR) q0[c] = q[4 * (size_t)kk + c];
-        sx[c] = 0.0;
-        sy[c] = 0.0;
-    }
-    const int deg = d.deg[kk];
-    const int base = d.slice_off[kk >> 5] + (kk & 31);
-    for (int j = sub; j < deg; j += TPP) {
+    asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
+        : "l"(p));
+}
+
+// 2^e, |e| < 1023.
+__device__ __forceinline__ double pow2(int e)
+{
+    return __hiloint2double((1023 + e) << 20, 0);
+}
+
+// The value of a stored G (or of a mark's FP64 derivative) in units of q.
+__device__ __forceinline__ double g_value(int lo, int hi, const double *g, int ex, int c)
+{
+    return fix_marked(hi) ? scalbn(*g, -ex) : scalbn((double)join_g(hi, lo), -fix_unit(c));
+}
+
+// What k_grad forms, in FP64, for a point that meets a marked value or has no
+// fast scale: the lane's slots, its two components, v = x 0, x 1, y 0, y 1 in
+// units of q without the first-order term (the lanes of a group add them).
+template <int S, bool CORR>
+__device__ __noinline__ void grad_fp64(const Dev &d, const double *__restrict__ q, int from, int k, int sub, int c2,
+                                       double v[4])
+{
+    const int4 *__restrict__ gf = CORR ? d.gf[from] : nullptr;
+    const double *__restrict__ g = CORR ? d.gq[from] : nullptr;
+    const short4 ge = d.ge[k];
+    const double lsb = pow2(-(CORR ? d.gb[k].y : d.gb[k].x));
+    const int deg = d.deg[k];
+    const int base = d.slice_off[k >> 5] + (k & 31);
+    for (int c = 0; c < 4; c++) v[c] = 0.0;
+    // (the centre after the last slot of the first lane)
+    for (int j = sub, centre = 0; !centre && (j < deg || (CORR && sub == 0)); j += S) {
+        centre = j >= deg;
         const int e = base + 32 * j;
-        const int i = d.nbr[e];
+        const int i = centre ? k : d.nbr[e];
         if (!CORR) {
-            const double wx = d.wgx[e], wy = d.wgy[e];
-            double qi[4];
-            load4(q + 4 * (size_t)i, qi);
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const double dq = qi[c] - q0[c];
-                sx[c] = fma(wx, dq, sx[c]);
-                sy[c] = fma(wy, dq, sy[c]);
+            const uint4 w = d.wg[e];
+            const double wx = fma((double)(int)w.y, lsb, (double)(int)w.x);
+            const double wy = fma((double)(int)w.w, lsb, (double)(int)w.z);
+            for (int c = 0; c < 2; c++) {
+                const double dq = q[4 * (size_t)i + 2 * c2 + c] - q[4 * (size_t)k + 2 * c2 + c];
+                v[c] = fma(wx, dq, v[c]);
+                v[2 + c] = fma(wy, dq, v[2 + c]);
             }
         } else {
-            const double axx = d.gxx[e], axy = d.gxy[e], ayx = d.gyx[e], ayy = d.gyy[e];
-            const double2 *r = reinterpret_cast<const double2 *>(pg + 8 * (size_t)i);
-            const double2 a01 = r[0], a23 = r[1], b01 = r[2], b23 = r[3];
-            const double a[4] = {a01.x, a01.y, a23.x, a23.y}, b[4] = {b01.x, b01.y, b23.x, b23.y};
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                sx[c] = fma(axx, a[c], fma(axy, b[c], sx[c]));
-                sy[c] = fma(ayx, a[c], fma(ayy, b[c], sy[c]));
+            const uint4 *w = centre ? d.wc + 2 * (size_t)k : d.wj + 2 * (size_t)e;
+            const uint4 a = w[0], b = w[1];
+            const double axx = fma((double)(int)a.y, lsb, (double)(int)a.x);
+            const double axy = fma((double)(int)a.w, lsb, (double)(int)a.z);
+            const double ayx = fma((double)(int)b.y, lsb, (double)(int)b.x);
+            const double ayy = fma((double)(int)b.w, lsb, (double)(int)b.z);
+            const short4 gi = d.ge[i];
+            const int *f = reinterpret_cast<const int *>(gf + 4 * (size_t)i + 2 * c2);
+            for (int c = 0; c < 2; c++) {
+                const double *gx = g + 8 * (size_t)i + 2 * c2 + c;
+                const double x = g_value(f[4 * c], f[4 * c + 1], gx, gi.x, 2 * c2 + c);
+                const double y = g_value(f[4 * c + 2], f[4 * c + 3], gx + 4, gi.y, 2 * c2 + c);
+                v[c] = fma(axx, x, fma(axy, y, v[c]));
+                v[2 + c] = fma(ayx, x, fma(ayy, y, v[2 + c]));
             }
         }
     }
+    for (int c = 0; c < 4; c++) {
+        const int p = c < 2 ? ge.z : ge.w;
+        v[c] = p == kGradNoScale ? __longlong_as_double(0x7ff8000000000000ll) : scalbn(v[c], (CORR ? p : 0) - 31);
+    }
+}
+
+// Four slots' loads in flight per lane, the next four's neighbours with them:
+// a gather takes about 1000 cycles, a slot's 32 multiply-adds 150.
+// 128 threads and 96 registers, five blocks per SM.
+constexpr int kGradBlock = 128, kGradUnroll = 4;
+
+// Slot lanes per point of the q-derivatives for TPP lanes of the residual: a
+// warp's slots are short here, so splitting a point's list pays only in the
+// smallest clouds (40,621 points: one 0.054 ms, two 0.061; 10,240: equal).
+template <int TPP>
+constexpr int kGradLanes = TPP == 8 ? 2 : 1;
+
+// Pass `to` buffer: first order (CORR false, buffer 2) or an inner iteration
+// from buffer `from`; S slot lanes per point (2 S lanes in all).  The FP64
+// derivatives are stored by the last pass and, with a mark, wherever the
+// fixed-point form does not hold them.
+template <int S, bool CORR>
+__global__ void __launch_bounds__(kGradBlock, 5) k_grad(Dev d, StateSet st, int from, int to, bool last)
+{
+    if (halted(d.ctrl)) return;
+    constexpr int L = 2 * S;
+    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = gt / L, sub = (gt % L) >> 1, c2 = gt & 1;
+    const bool active = k < d.n;
+    const int kk = active ? k : d.n - 1;
+    const short4 ge = d.ge[kk];
+    bool bad = abs(ge.x) > kMaxGradExp || abs(ge.y) > kMaxGradExp || ge.z > kMaxGradShift || ge.w > kMaxGradShift;
+    const int bits = CORR ? d.gb[kk].y : d.gb[kk].x;
+    bad |= bits < kMinGradBits;
+    // every lane of a slice runs to the slice's width: a padding slot is the
+    // point itself with weights 0
+    const int beg = d.slice_off[kk >> 5], width = (d.slice_off[(kk >> 5) + 1] - beg) >> 5;
+    int e = beg + (kk & 31) + 32 * sub;
+    GradSum x[2] = {}, y[2] = {};
+    auto slots = [&](auto &&load, auto &&use) {
+        int i[kGradUnroll];
+        int j = sub;
+#pragma unroll
+        for (int u = 0; u < kGradUnroll; u++) i[u] = j + u * S < width ? d.nbr[e + 32 * S * u] : kk;
+        for (; j + (kGradUnroll - 1) * S < width; j += kGradUnroll * S) {
+            decltype(load(0, 0)) v[kGradUnroll];
+#pragma unroll
+            for (int u = 0; u < kGradUnroll; u++, e += 32 * S) v[u] = load(e, i[u]);
+#pragma unroll
+            for (int u = 0; u < kGradUnroll; u++) i[u] = j + (u + kGradUnroll) * S < width ? d.nbr[e + 32 * S * u] : kk;
+#pragma unroll
+            for (int u = 0; u < kGradUnroll; u++) use(v[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < kGradUnroll - 1; u++, j += S, e += 32 * S)
+            if (j < width) use(load(e, i[u]));
+    };
+    if (!CORR) {
+        struct Slot {
+            uint4 w;
+            longlong2 q;
+        };
+        const longlong2 *__restrict__ qf = reinterpret_cast<const longlong2 *>(st.qf) + c2;
+        const longlong2 q0 = qf[2 * (size_t)kk];
+        bad |= fix_marked((int)(q0.x >> 32)) || fix_marked((int)(q0.y >> 32));
+        const int64_t b0 = q0.x - 0x80000000ll, b1 = q0.y - 0x80000000ll;
+        slots([&](int e, int i) { return Slot{d.wg[e], qf[2 * (size_t)i]}; },
+              [&](const Slot &v) {
+                  const uint4 &w = v.w;
+                  bad |= fix_marked((int)(v.q.x >> 32)) || fix_marked((int)(v.q.y >> 32));
+                  int dh, dl;
+                  split_word(v.q.x - b0, dh, dl);
+                  grad_add(x[0], w.x, w.y, dh, dl);
+                  grad_add(y[0], w.z, w.w, dh, dl);
+                  split_word(v.q.y - b1, dh, dl);
+                  grad_add(x[1], w.x, w.y, dh, dl);
+                  grad_add(y[1], w.z, w.w, dh, dl);
+              });
+    } else {
+        struct Slot {
+            uint4 a, b, g0, g1;
+        };
+        const int4 *__restrict__ gf = d.gf[from] + 2 * c2;
+        auto load = [&](const uint4 *w, const int4 *g) {
+            Slot v;
+            load32(w, v.a, v.b);
+            load32(g, v.g0, v.g1);
+            return v;
+        };
+        auto use = [&](const Slot &v) {
+            const uint4 &a = v.a, &b = v.b, &g0 = v.g0, &g1 = v.g1;
+            bad |= fix_marked((int)g0.y);
+            grad_add(x[0], a.x, a.y, g0.y, g0.x);
+            grad_add(x[0], a.z, a.w, g0.w, g0.z);
+            grad_add(x[1], a.x, a.y, g1.y, g1.x);
+            grad_add(x[1], a.z, a.w, g1.w, g1.z);
+            grad_add(y[0], b.x, b.y, g0.y, g0.x);
+            grad_add(y[0], b.z, b.w, g0.w, g0.z);
+            grad_add(y[1], b.x, b.y, g1.y, g1.x);
+            grad_add(y[1], b.z, b.w, g1.w, g1.z);
+        };
+        if (sub == 0) use(load(d.wc + 2 * (size_t)kk, gf + 4 * (size_t)kk));
+        slots([&](int e, int i) { return load(d.wj + 2 * (size_t)e, gf + 4 * (size_t)i); }, use);
+    }
+    // the group's sums: every second lane holds the same components
+    int64_t hh[4], lo[4];
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+        hh[c] = x[c].hh, lo[c] = grad_low(x[c], bits);
+        hh[2 + c] = y[c].hh, lo[2 + c] = grad_low(y[c], bits);
+    }
+#pragma unroll
+    for (int o = S; o > 1; o >>= 1) {
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            hh[c] += __shfl_xor_sync(kFull, hh[c], o);
+            lo[c] += __shfl_xor_sync(kFull, lo[c], o);
+        }
+        bad |= __shfl_xor_sync(kFull, (int)bad, o) != 0;
+    }
+    int64_t v[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int c = 0; c < 4; c++) {
-        sx[c] = group_sum<TPP>(sx[c]);
-        sy[c] = group_sum<TPP>(sy[c]);
+        if (!bad) bad = !grad_value(hh[c], lo[c], bits, CORR ? (c < 2 ? ge.z : ge.w) : 0, v[c]);
     }
-    if (active && sub == 0) {
-        if (!CORR) {
+    double f[4] = {0.0, 0.0, 0.0, 0.0};  // a marked point's, in units of q
+    if (CORR && !bad) {
+        const int4 a = d.gf[2][4 * (size_t)kk + 2 * c2], b = d.gf[2][4 * (size_t)kk + 2 * c2 + 1];
+        bad |= fix_marked(a.y);
+        v[0] += join_g(a.y, a.x), v[2] += join_g(a.w, a.z);
+        v[1] += join_g(b.y, b.x), v[3] += join_g(b.w, b.z);
+    }
+#pragma unroll
+    for (int c = 0; c < 4; c++) bad |= !grad_in_range(v[c]);
+    if (__any_sync(kFull, bad)) {
+        double t[4] = {0.0, 0.0, 0.0, 0.0};
+        if (bad) grad_fp64<S, CORR>(d, st.q, from, kk, sub, c2, t);
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+#pragma unroll
+            for (int o = S; o > 1; o >>= 1) t[c] += __shfl_xor_sync(kFull, t[c], o);
+        }
+        if (bad) {
+            bool fits = true;
 #pragma unroll
             for (int c = 0; c < 4; c++) {
-                d.g1x[c * ld + k] = g[8 * (size_t)k + c] = sx[c];
-                d.g1y[c * ld + k] = g[8 * (size_t)k + 4 + c] = sy[c];
+                const int cc = 2 * c2 + (c & 1);
+                if (CORR) {
+                    const int *a = reinterpret_cast<const int *>(d.gf[2] + 4 * (size_t)kk + cc) + 2 * (c >> 1);
+                    t[c] += g_value(a[0], a[1], d.gq[2] + 8 * (size_t)kk + cc + 4 * (c >> 1), c < 2 ? ge.x : ge.y, cc);
+                }
+                fits = fits && fabs(t[c]) < (cc == 0 ? 7.5 : 3.75);
+                f[c] = t[c];
+                v[c] = fits ? __double2ll_rn(scalbn(t[c], fix_unit(cc))) : 0;
             }
+            bad = !fits || abs(ge.x) > kMaxGradExp || abs(ge.y) > kMaxGradExp;
+        }
+    }
+    if (!active || sub != 0) return;
+    int4 a, b;
+    split_g(v[0], a.y, a.x);
+    split_g(v[2], a.w, a.z);
+    split_g(v[1], b.y, b.x);
+    split_g(v[3], b.w, b.z);
+    if (bad) a = b = make_int4(0, INT32_MIN, 0, INT32_MIN);
+    int4 *gf = d.gf[to] + 4 * (size_t)k + 2 * c2;
+    gf[0] = a;
+    gf[1] = b;
+    if (last || bad) {
+        double2 *g = reinterpret_cast<double2 *>(d.gq[to] + 8 * (size_t)k) + c2;
+        if (bad) {
+            g[0] = make_double2(scalbn(f[0], ge.x), scalbn(f[1], ge.x));
+            g[2] = make_double2(scalbn(f[2], ge.y), scalbn(f[3], ge.y));
         } else {
-            const double cxx = d.geo[G_SXX * ld + k], cxy = d.geo[G_SXY * ld + k];
-            const double cyx = d.geo[G_SYX * ld + k], cyy = d.geo[G_SYY * ld + k];
-#pragma unroll
-            for (int c = 0; c < 4; c++) {
-                const double a0 = pg[8 * (size_t)k + c], b0 = pg[8 * (size_t)k + 4 + c];
-                const double rx = sx[c] - fma(cxx, a0, cxy * b0);
-                const double ry = sy[c] - fma(cyx, a0, cyy * b0);
-                g[8 * (size_t)k + c] = fma(-0.5, rx, d.g1x[c * ld + k]);
-                g[8 * (size_t)k + 4 + c] = fma(-0.5, ry, d.g1y[c * ld + k]);
-            }
+            const int u0 = fix_unit(2 * c2), u1 = fix_unit(1);
+            g[0] = make_double2((double)v[0] * pow2(ge.x - u0), (double)v[1] * pow2(ge.x - u1));
+            g[2] = make_double2((double)v[2] * pow2(ge.y - u0), (double)v[3] * pow2(ge.y - u1));
         }
     }
 }
@@ -740,8 +926,8 @@ constexpr int kResBlock = TPP == 1 ? 512 : 256;
 // into its frame, where every split flux is along an axis, and the sum's
 // momentum back out of it.  Measured on the 147,584-point cloud (1 lane per
 // point): 0.649 ms with the fluxes in FP64 and integer-pipe multiplies, 0.693
-// ms with compensated sums; 0.229 ms like this (41,194 points, four lanes:
-// 0.235 -> 0.097 ms).  The FMA-heavy pipe, which runs the 32-bit multiplies,
+// ms with compensated sums; 0.212 ms like this (41,194 points, four lanes:
+// 0.235 -> 0.092 ms).  The FMA-heavy pipe, which runs the 32-bit multiplies,
 // is about 60 % busy; four warps per scheduler (128 registers) do not hide
 // the rest of the chains' latency.  Staging the next slot's records in shared
 // memory, prefetching them, and a lane per state with more warps were slower.
@@ -1946,6 +2132,9 @@ __global__ void __launch_bounds__(256) k_update(Dev d, int cur, bool inc, bool p
     qn[2] = mul_i(twice(P.beta), P.v);
     qn[3] = signed_by(twice(P.beta), false);
     store4(dst.q + 4 * (size_t)k, qn);
+    longlong2 *qf = reinterpret_cast<longlong2 *>(dst.qf + 4 * (size_t)k);
+    qf[0] = make_longlong2(fix_q(qn[0], 0), fix_q(qn[1], 1));
+    qf[1] = make_longlong2(fix_q(qn[2], 2), fix_q(qn[3], 3));
     // the per-point record, assembled in registers and stored as 16-byte
     // vectors (and, in mixed precision, its FP32 copy from the same registers)
     double rec[P_NFIELDS];
@@ -2032,6 +2221,7 @@ __global__ void __launch_bounds__(256) k_repair(Dev d, int cur)
     for (int c = 0; c < 4; c++) {
         dst.U[c * ld + k] = src.U[c * ld + k];
         dst.q[4 * (size_t)k + c] = src.q[4 * (size_t)k + c];
+        dst.qf[4 * (size_t)k + c] = src.qf[4 * (size_t)k + c];
     }
     for (int f = 0; f < kPrimStride; f++) dst.prim[(size_t)k * kPrimStride + f] = src.prim[(size_t)k * kPrimStride + f];
     if (src.primf)
@@ -2062,13 +2252,13 @@ __global__ void k_prep_run(Ctrl *c, double target)
 template <int TPP>
 cudaError_t enqueue_grad(const Dev &d, int cur, cudaStream_t s, int *launches)
 {
-    const int gb = (d.n * TPP + 255) / 256;
+    constexpr int S = kGradLanes<TPP>;
+    const int gb = (int)(((int64_t)d.n * 2 * S + kGradBlock - 1) / kGradBlock);
     const StateSet st = d.set[cur];
-    k_grad<TPP, false><<<gb, 256, 0, s>>>(d, st.q, nullptr, d.gq[0]);
+    k_grad<S, false><<<gb, kGradBlock, 0, s>>>(d, st, 0, 2, d.K == 0);
     (*launches)++;
     for (int it = 1; it <= d.K; it++) {
-        const int a = (it - 1) & 1, b = it & 1;
-        k_grad<TPP, true><<<gb, 256, 0, s>>>(d, st.q, d.gq[a], d.gq[b]);
+        k_grad<S, true><<<gb, kGradBlock, 0, s>>>(d, st, it == 1 ? 2 : it & 1, 1 - (it & 1), it == d.K);
         (*launches)++;
     }
     return cudaGetLastError();
@@ -2077,10 +2267,9 @@ cudaError_t enqueue_grad(const Dev &d, int cur, cudaStream_t s, int *launches)
 template <int TPP>
 cudaError_t enqueue_res(const Dev &d, const Launch &L, int cur, cudaStream_t s, int *launches)
 {
-    const int fin = d.K & 1;
-    constexpr int block = kResBlock<TPP>;
+        constexpr int block = kResBlock<TPP>;
     const int want = (d.n * TPP + block - 1) / block, most = L.sms * (512 / block);
-    k_residual<TPP><<<want < most ? want : most, block, 0, s>>>(d, d.set[cur], d.gq[fin]);
+    k_residual<TPP><<<want < most ? want : most, block, 0, s>>>(d, d.set[cur], d.gq[grad_buffer(d.K)]);
     (*launches)++;
     return cudaGetLastError();
 }
