@@ -1,30 +1,23 @@
 // Learned warm start: the network of include/lskum_mlp.h on the Blackwell
 // tensor cores.
 //
-// Every matrix product D[M x N] = A[M x K] B[N x K]^T of training and
-// inference runs in k_gemm: one CTA of 4 warps owns a 128-row tile of D in
-// tensor memory (TMEM, FP32, one lane per row); K is staged through shared
-// memory in chunks of 64 (A: 128 x 64, B: N x 64 BF16) in the canonical
-// K-major, non-swizzled core-matrix layout (8 rows x 16 bytes per core
-// matrix, k-groups 128 B apart, 8-row groups 1024 B apart), and one elected
-// thread issues tcgen05.mma (kind::f16, BF16 x BF16 -> FP32, M = 128,
-// K = 16 per instruction) and commits to an mbarrier that all threads wait
-// on.  The epilogue reads the accumulator back with tcgen05.ld (32x32b: each
-// thread one row) and fuses what follows the product:
-//   kFwdHidden  Z + b -> GELU -> BF16 activations (row-major and transposed)
-//               and GELU'(Z) for the backward pass;
-//   kFwdOut     Z + b -> outputs (FP32);
-//   kBwdData    (G W) * GELU'(Z) -> BF16 gradients (row-major and transposed);
-//   kWgrad      split-K partial sums of G^T A for the weight gradients.
-// Inference (forward pass, prediction into a solver state) instead runs
-// k_mlp_fused: persistent CTAs keep all five layers' weights in shared memory
-// and carry each 128-point tile through the five products with the
-// activations staying on the SM (see the comment above that kernel).
-// Operand layouts: activations and gradients are kept both point-major
-// ([points][features], the A operand of forward and backward-data products)
-// and feature-major ([features][points], the operands of weight-gradient
-// products, where the points are the reduction dimension); the weights both
-// as W [out][in] (forward) and W^T [in][out] (backward data).
+// Training and inference each run in one persistent kernel whose CTAs carry
+// 128-point tiles through all five layers with the activations staying on the
+// SM: k_mlp_train (loss and gradients of a batch) and k_mlp_fused (forward
+// pass, prediction into a solver state).  Products are tcgen05.mma
+// (kind::f16, BF16 x BF16 -> FP32, M = 128, K = 16 per instruction), issued by
+// one elected thread that commits to an mbarrier all threads wait on; the
+// accumulators lie in tensor memory (TMEM, FP32, one lane per row) and are
+// read back with tcgen05.ld (32x32b: each thread one row).
+//
+// Operands lie in shared memory as BF16 core matrices (8 rows x 16 bytes, no
+// swizzle, k-groups of 8 columns 128 B apart).  A tile [points][features]
+// serves three products without a copy: as the K-major operand of the next
+// layer (or of the data gradient), and as the MN-major operand of the weight
+// gradients, where the points are the reduction dimension (there the stride
+// between core matrices along the points is the leading, the one along the
+// features the stride byte offset).  The weights W [out][in] serve the forward
+// products (K-major) and the data gradients (MN-major) in the same way.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -47,7 +40,6 @@ constexpr int kInTrue[kLayers] = {kIn, kWidth, kWidth, kWidth, kWidth};
 constexpr int kInP[kLayers] = {kInPad, kWidth, kWidth, kWidth, kWidth};
 constexpr int kOutTrue[kLayers] = {kWidth, kWidth, kWidth, kWidth, kOut};
 constexpr int kOutP[kLayers] = {kWidth, kWidth, kWidth, kWidth, kOutPad};
-constexpr int kSplitK = 128;  // points per CTA in weight-gradient products
 constexpr int kBatchAlign = 512;
 
 constexpr int n_params_total()
@@ -57,8 +49,7 @@ constexpr int n_params_total()
     return s;
 }
 constexpr int kNParams = n_params_total();  // 54,532
-
-enum Epi { kFwdHidden = 0, kFwdOut = 1, kBwdData = 2, kWgrad = 3 };
+static_assert(kNParams % 2 == 0, "a double follows the gradients");
 
 // ---------------------------------------------------------------------------
 // tcgen05 / mbarrier primitives (inline PTX)
@@ -136,7 +127,7 @@ __device__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity, uint64_t limit
 
 // Shared-memory matrix descriptor: start address, leading-dimension byte
 // offset (between core matrices along K), stride-dimension byte offset
-// (between 8-row groups), descriptor version 1, no swizzle.
+// (between core matrices along M or N), descriptor version 1, no swizzle.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo)
 {
     uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
@@ -146,11 +137,13 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
     return d;
 }
 
-// Instruction descriptor of kind::f16: D FP32, A and B BF16, both K-major, M = 128.
-template <int N>
+// Instruction descriptor of kind::f16: D FP32, A and B BF16, M = 128; A, B
+// K-major, or MN-major where kAT, kBT.
+template <int N, bool kAT = false, bool kBT = false>
 __host__ __device__ constexpr uint32_t idesc_bf16()
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)kAT << 15) | ((uint32_t)kBT << 16) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
@@ -184,6 +177,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v)
     for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
 
+// 32 columns.
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v)
+{
+    uint32_t r[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; i++) v[i] = __uint_as_float(r[i]);
+}
+
 __device__ __forceinline__ uint16_t bf16_bits(float x)
 {
     __nv_bfloat16 h = __float2bfloat16_rn(x);
@@ -206,167 +216,15 @@ __device__ __forceinline__ float gelu_grad(float z)
 }
 
 // ---------------------------------------------------------------------------
-// the product kernel
-// ---------------------------------------------------------------------------
-struct GemmArgs {
-    const uint16_t *A;  // [rows][lda] BF16, K contiguous; rows >= a_rows read as 0
-    int lda, a_rows;
-    const uint16_t *B;  // [N rows][ldb]; rows >= b_rows read as 0
-    int ldb, b_rows;
-    int K, k_split;     // K extent (multiple of 16); K per CTA along grid.y
-    int m_valid;        // rows of D that hold data; the tile's other rows get zeros
-    const float *bias;  // [N] (kFwdHidden, kFwdOut)
-    const float *gp_in; // [rows][128] GELU'(Z) of the product's output features (kBwdData)
-    float *gp_out;      // [rows][128] (kFwdHidden, may be null)
-    uint16_t *out;      // [rows][ldo] BF16
-    int ldo;
-    uint16_t *out_t;    // [N][ldt] BF16 transposed (may be null)
-    int ldt;
-    float *out_f;       // kFwdOut: [rows][4]; kWgrad: [split][m_valid][N]
-    int *err;
-    uint64_t wait_ns;   // time limit of each wait for the tensor core
-    int skip_products;  // failure-path test: issue neither products nor commit
-};
-
-// 24 KB of dynamic shared memory is requested on top of the 32 KB of operand
-// buffers so that at most 4 CTAs share an SM: 4 x 128 TMEM columns = 512.
-constexpr int kPadSmem = 24 * 1024;
-
-template <int EPI, int N>
-__global__ void __launch_bounds__(128) k_gemm(GemmArgs g)
-{
-    static_assert(N % 16 == 0 && N >= 16 && N <= 128, "N");
-    constexpr uint32_t kCols = N <= 32 ? 32 : (N <= 64 ? 64 : 128);
-    constexpr uint32_t kIdesc = idesc_bf16<N>();
-    __shared__ __align__(1024) uint8_t sA[128 * 64 * 2];
-    __shared__ __align__(1024) uint8_t sB[128 * 64 * 2];
-    __shared__ __align__(8) uint64_t bar;
-    __shared__ uint32_t tslot;
-    extern __shared__ uint8_t pad_smem[];
-    (void)pad_smem;
-
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * 128;
-    const int kb = blockIdx.y * g.k_split;
-    const int ke = min(g.K, kb + g.k_split);
-    if (warp == 0) tmem_alloc(&tslot, kCols);
-    if (tid == 0) mbar_init(&bar, 1);
-    fence_before_sync();
-    __syncthreads();
-    fence_after_sync();
-    const uint32_t tmem = tslot;
-
-    uint32_t parity = 0;
-    int ok = 1;
-    const bool any = ke > kb;
-    for (int kc = kb; kc < ke && ok; kc += 64) {
-        const int kw = min(64, ke - kc);  // a multiple of 16
-        const int kg = kw >> 3;           // 16-byte k-groups in this chunk
-        for (int v = tid; v < 128 * kg; v += 128) {
-            const int r = v / kg, j = v - r * kg;
-            const int row = m0 + r;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (row < g.a_rows) val = *reinterpret_cast<const uint4 *>(g.A + (size_t)row * g.lda + kc + 8 * j);
-            *reinterpret_cast<uint4 *>(sA + ((r >> 3) * 8 + j) * 128 + (r & 7) * 16) = val;
-        }
-        for (int v = tid; v < N * kg; v += 128) {
-            const int r = v / kg, j = v - r * kg;
-            uint4 val = make_uint4(0u, 0u, 0u, 0u);
-            if (r < g.b_rows) val = *reinterpret_cast<const uint4 *>(g.B + (size_t)r * g.ldb + kc + 8 * j);
-            *reinterpret_cast<uint4 *>(sB + ((r >> 3) * 8 + j) * 128 + (r & 7) * 16) = val;
-        }
-        fence_smem_to_async();
-        __syncthreads();
-        if (tid == 0 && !g.skip_products) {
-            fence_after_sync();
-            const uint32_t a0 = smem_u32(sA), b0 = smem_u32(sB);
-            for (int s = 0; s < (kw >> 4); s++)
-                mma_bf16(tmem, smem_desc(a0 + 256u * s, 128u, 1024u), smem_desc(b0 + 256u * s, 128u, 1024u), kIdesc,
-                         (kc > kb || s > 0) ? 1u : 0u);
-            mma_commit(&bar);
-        }
-        ok = __syncthreads_and(mbar_wait_bounded(&bar, parity, g.wait_ns) ? 1 : 0);
-        parity ^= 1u;
-    }
-    fence_after_sync();
-
-    const int r = warp * 32 + lane;
-    const int row = m0 + r;
-    const bool live = row < g.m_valid;
-    const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16);
-    if (ok) {
-#pragma unroll 1
-        for (int c0 = 0; c0 < N; c0 += 16) {
-            float v[16];
-            if (any) tmem_ld16(taddr + (uint32_t)c0, v);
-            else
-#pragma unroll
-                for (int i = 0; i < 16; i++) v[i] = 0.f;
-            if (EPI == kWgrad) {
-                if (live) {
-                    float *o = g.out_f + ((size_t)blockIdx.y * g.m_valid + row) * N + c0;
-#pragma unroll
-                    for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4 *>(o + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                }
-                continue;
-            }
-            if (EPI == kFwdOut) {
-                if (live && c0 == 0)
-#pragma unroll
-                    for (int i = 0; i < kOut; i++) g.out_f[(size_t)row * kOut + i] = v[i] + g.bias[i];
-                continue;
-            }
-            uint16_t h[16];
-            float gp[16];
-#pragma unroll
-            for (int i = 0; i < 16; i++) {
-                float y = 0.f;
-                gp[i] = 0.f;
-                if (live) {
-                    if (EPI == kFwdHidden) {
-                        const float z = v[i] + g.bias[c0 + i];
-                        y = gelu(z);
-                        gp[i] = gelu_grad(z);
-                    } else {  // kBwdData
-                        y = v[i] * g.gp_in[(size_t)row * kWidth + c0 + i];
-                    }
-                }
-                h[i] = bf16_bits(y);
-            }
-            uint4 *dst = reinterpret_cast<uint4 *>(g.out + (size_t)row * g.ldo + c0);
-            dst[0] = make_uint4(h[0] | (uint32_t)h[1] << 16, h[2] | (uint32_t)h[3] << 16, h[4] | (uint32_t)h[5] << 16,
-                                h[6] | (uint32_t)h[7] << 16);
-            dst[1] = make_uint4(h[8] | (uint32_t)h[9] << 16, h[10] | (uint32_t)h[11] << 16,
-                                h[12] | (uint32_t)h[13] << 16, h[14] | (uint32_t)h[15] << 16);
-            if (g.out_t)
-#pragma unroll
-                for (int i = 0; i < 16; i++) g.out_t[(size_t)(c0 + i) * g.ldt + row] = h[i];
-            if (EPI == kFwdHidden && g.gp_out) {
-                float *o = g.gp_out + (size_t)row * kWidth + c0;
-#pragma unroll
-                for (int i = 0; i < 16; i += 4) *reinterpret_cast<float4 *>(o + i) = make_float4(gp[i], gp[i + 1], gp[i + 2], gp[i + 3]);
-            }
-        }
-    } else if (tid == 0) {
-        atomicExch(g.err, 1);
-    }
-    fence_before_sync();
-    __syncthreads();
-    if (warp == 0) tmem_dealloc(tmem, kCols);
-}
-
-// ---------------------------------------------------------------------------
 // small kernels
 // ---------------------------------------------------------------------------
-// Network inputs of one point (x, y, wall distance, M, AoA deg) into X row i
-// (BF16, 48 columns) and column i of Xt.
-__device__ __forceinline__ void write_features(const float *B, float x, float y, float d, float mach, float aoa,
-                                               uint16_t *X, uint16_t *Xt, int i, int ldt)
+// Network inputs (BF16, 48 columns, 34 used) of one point (x, y, wall distance, M, AoA deg).
+__device__ __forceinline__ void point_features(const float *B, float x, float y, float d, float mach, float aoa,
+                                               uint16_t h[kInPad])
 {
     const float X0 = x - 0.5f;
     const float r = sqrtf(X0 * X0 + y * y);
     const float z0 = X0 / (1.f + r), z1 = y / (1.f + r), z2 = d / (1.f + d);
-    uint16_t h[kInPad];
 #pragma unroll
     for (int f = 0; f < kFreq; f++) {
         const float t = B[3 * f] * z0 + B[3 * f + 1] * z1 + B[3 * f + 2] * z2;
@@ -379,48 +237,30 @@ __device__ __forceinline__ void write_features(const float *B, float x, float y,
     h[2 * kFreq + 1] = bf16_bits(aoa * 0.1f);
 #pragma unroll
     for (int f = kIn; f < kInPad; f++) h[f] = 0;
+}
+
+// The inputs of points [0, n) of in5 as rows of X.
+__global__ void k_features(const float *in5, int n, const float *B, uint16_t *X)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float *s = in5 + (size_t)i * 5;
+    uint16_t h[kInPad];
+    point_features(B, s[0], s[1], s[2], s[3], s[4], h);
     uint4 *dst = reinterpret_cast<uint4 *>(X + (size_t)i * kInPad);
 #pragma unroll
     for (int q = 0; q < kInPad / 8; q++)
         dst[q] = make_uint4(h[8 * q] | (uint32_t)h[8 * q + 1] << 16, h[8 * q + 2] | (uint32_t)h[8 * q + 3] << 16,
                             h[8 * q + 4] | (uint32_t)h[8 * q + 5] << 16, h[8 * q + 6] | (uint32_t)h[8 * q + 7] << 16);
-    if (Xt)
-#pragma unroll
-        for (int f = 0; f < kInPad; f++) Xt[(size_t)f * ldt + i] = h[f];
 }
 
-__device__ __forceinline__ void zero_features(uint16_t *X, uint16_t *Xt, int i, int ldt)
-{
-    uint4 *dst = reinterpret_cast<uint4 *>(X + (size_t)i * kInPad);
-    for (int q = 0; q < kInPad / 8; q++) dst[q] = make_uint4(0u, 0u, 0u, 0u);
-    if (Xt)
-        for (int f = 0; f < kInPad; f++) Xt[(size_t)f * ldt + i] = 0;
-}
-
-// Rows [0, rows): sample idx[i] (or i without idx) of in5 for i < n, zeros after.
-__global__ void k_features(const float *in5, const int32_t *idx, int n, int rows, const float *B, uint16_t *X,
-                           uint16_t *Xt, int ldt)
+// Given inputs X [n][34] (FP32) -> BF16 X rows, zeros up to rows.
+__global__ void k_inputs_from_f32(const float *Xf, int n, int rows, uint16_t *X)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows) return;
-    if (i >= n) {
-        zero_features(X, Xt, i, ldt);
-        return;
-    }
-    const float *s = in5 + (size_t)(idx ? idx[i] : i) * 5;
-    write_features(B, s[0], s[1], s[2], s[3], s[4], X, Xt, i, ldt);
-}
-
-// Given inputs X [n][34] (FP32) -> BF16 X rows and Xt columns, zeros up to rows.
-__global__ void k_inputs_from_f32(const float *Xf, int n, int rows, uint16_t *X, uint16_t *Xt, int ldt)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= rows) return;
-    for (int f = 0; f < kInPad; f++) {
-        const uint16_t h = (i < n && f < kIn) ? bf16_bits(Xf[(size_t)i * kIn + f]) : (uint16_t)0;
-        X[(size_t)i * kInPad + f] = h;
-        if (Xt) Xt[(size_t)f * ldt + i] = h;
-    }
+    for (int f = 0; f < kInPad; f++)
+        X[(size_t)i * kInPad + f] = (i < n && f < kIn) ? bf16_bits(Xf[(size_t)i * kIn + f]) : (uint16_t)0;
 }
 
 // BF16 X rows back to FP32 [n][34].
@@ -429,65 +269,6 @@ __global__ void k_inputs_to_f32(const uint16_t *X, int n, float *Xf)
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     for (int f = 0; f < kIn; f++) Xf[(size_t)i * kIn + f] = bf16_val(X[(size_t)i * kInPad + f]);
-}
-
-// Loss and output gradient: E = O - T, loss += sum E^2 / (4 n), G = 2 E / (4 n)
-// (BF16, G [rows][16] and Gt [16][ldt]); rows >= n get zeros.
-__global__ void __launch_bounds__(256) k_loss(const float *O, const float *T, const int32_t *idx, int n, int rows,
-                                              uint16_t *G, uint16_t *Gt, int ldt, double *loss)
-{
-    __shared__ double red[8];
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double e2 = 0.0;
-    if (i < rows) {
-        const float sc = 2.f / (4.f * (float)n);
-        for (int c = 0; c < kOut; c++) {
-            uint16_t h = 0;
-            if (i < n) {
-                const float e = O[(size_t)i * kOut + c] - T[(size_t)(idx ? idx[i] : i) * kOut + c];
-                e2 += (double)e * e;
-                h = bf16_bits(sc * e);
-            }
-            G[(size_t)i * kOutPad + c] = h;
-            Gt[(size_t)c * ldt + i] = h;
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) e2 += __shfl_xor_sync(0xffffffffu, e2, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e2;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < 8; w++) s += red[w];
-        atomicAdd(loss, s / (4.0 * n));
-    }
-}
-
-// Bias gradient: db[o] = sum over points of Gt[o][p] (fixed order).
-__global__ void __launch_bounds__(256) k_colsum(const uint16_t *Gt, int ldt, int cols, float *db)
-{
-    __shared__ float red[8];
-    const int o = blockIdx.x;
-    float s = 0.f;
-    for (int p = threadIdx.x; p < cols; p += 256) s += bf16_val(Gt[(size_t)o * ldt + p]);
-    for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int w = 0; w < 8; w++) t += red[w];
-        db[o] = t;
-    }
-}
-
-// Weight gradient: dW[o][i] = sum over splits of partial[s][o][i] (i < in_true).
-__global__ void k_reduce_wgrad(const float *part, int splits, int m_valid, int N, int in_true, float *dW)
-{
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= m_valid * in_true) return;
-    const int o = t / in_true, i = t - o * in_true;
-    float s = 0.f;
-    for (int q = 0; q < splits; q++) s += part[((size_t)q * m_valid + o) * N + i];
-    dW[t] = s;
 }
 
 __global__ void k_adam(float *p, float *m, float *v, const float *g, int n, float lr, float bc1, float bc2)
@@ -504,11 +285,11 @@ __global__ void k_adam(float *p, float *m, float *v, const float *g, int n, floa
 
 struct PackArgs {
     const float *params;
-    uint16_t *W[kLayers], *Wt[kLayers];
+    uint16_t *W[kLayers];
     int off[kLayers], in_true[kLayers], in_pad[kLayers], out_true[kLayers], out_pad[kLayers];
 };
 
-// BF16 copies of the weights: W [out_pad][in_pad] and W^T [in_pad][out_pad], zero padded.
+// BF16 copies of the weights: W [out_pad][in_pad], zero padded.
 __global__ void k_pack(PackArgs a)
 {
     const int l = blockIdx.y;
@@ -517,9 +298,7 @@ __global__ void k_pack(PackArgs a)
     if (t >= ip * op) return;
     const int o = t / ip, i = t - o * ip;
     const float w = (o < a.out_true[l] && i < a.in_true[l]) ? a.params[a.off[l] + o * a.in_true[l] + i] : 0.f;
-    const uint16_t h = bf16_bits(w);
-    a.W[l][(size_t)o * ip + i] = h;
-    a.Wt[l][(size_t)i * op + o] = h;
+    a.W[l][(size_t)o * ip + i] = bf16_bits(w);
 }
 
 // ---------------------------------------------------------------------------
@@ -569,7 +348,7 @@ __device__ __forceinline__ void store_row_chunk(uint8_t *tile, int kg_stride, in
 template <int SRC>
 __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(FusedArgs a)
 {
-    extern __shared__ __align__(1024) uint8_t sm[];
+    extern __shared__ __align__(128) uint8_t sm[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t tslot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -622,21 +401,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(FusedArgs a)
                 } else {
                     const int k = a.k0 + i;
                     const int b = a.v.case_of[k];
-                    const float X0 = a.v.x[k] - 0.5f, y = a.v.y[k], d = a.v.dwall[k];
-                    const float r = sqrtf(X0 * X0 + y * y);
-                    const float z0 = X0 / (1.f + r), z1 = y / (1.f + r), z2 = d / (1.f + d);
-#pragma unroll
-                    for (int f = 0; f < kFreq; f++) {
-                        const float tt = a.fourier[3 * f] * z0 + a.fourier[3 * f + 1] * z1 + a.fourier[3 * f + 2] * z2;
-                        float sn, cs;
-                        sincospif(2.f * tt, &sn, &cs);
-                        h[f] = bf16_bits(sn);
-                        h[kFreq + f] = bf16_bits(cs);
-                    }
-                    h[2 * kFreq] = bf16_bits(a.v.case_mach[b]);
-                    h[2 * kFreq + 1] = bf16_bits(a.v.case_aoa[b] * 0.1f);
-#pragma unroll
-                    for (int f = kIn; f < kInPad; f++) h[f] = 0;
+                    point_features(a.fourier, a.v.x[k], a.v.y[k], a.v.dwall[k], a.v.case_mach[b], a.v.case_aoa[b], h);
                 }
             } else {
 #pragma unroll
@@ -730,6 +495,436 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_mlp_fused(FusedArgs a)
     if (warp == 0) tmem_dealloc(tmem, 128);
 }
 
+// ---------------------------------------------------------------------------
+// loss and gradients of a batch: forward and backward of a 128-point tile in
+// one CTA, the weight gradients accumulating in TMEM over its tiles
+// ---------------------------------------------------------------------------
+// Shared memory (226 KB): the weights (layer 3's apart), the input tile and
+// the four hidden tiles; going back, the gradient of a layer's
+// pre-activations takes the place of the layer's activations once its weight
+// gradient has used them.  Layer 3's weights pass through the tile that its
+// output (forward) or the gradient of its input (backward) will fill.
+// TMEM (all 512 columns): 64 for the products of a layer, taken in two halves
+// of N = 64 so that the tensor core forms one half while the threads work on
+// the other, and 448 for the weight gradients of all layers.
+// GELU' of a tile (FP32) waits in a scratch of the CTA, 16 bytes per thread
+// and access: 256 KB per CTA, 39 MB in all, which stays in L2.
+// Bias gradients: of layer 0 as the input column 34 of ones (the weights'
+// columns beyond 33 are 0), of layers 1 to 3 by each thread over one core
+// matrix of every tile, of the output layer by warp sums.
+// Bound by the error functions and exponentials of 512 activations per point
+// (61 instructions per activation in all: 45 % of the issue slots) and by the
+// latency of a tile's 17 dependent products.  512 threads: with 256 a
+// scheduler has two warps, 0.195 ms instead of 0.137.  65,536 points: 0.137 ms
+// and 0.015 ms for the reduction below; as one kernel per product, with
+// transposed copies of all operands and 512 partial sums per weight, 1.15 ms
+// (a call with its copies 1.22 -> 0.265 ms; 1,000 points 0.397 -> 0.100).
+constexpr int kTrainThreads = 512;
+constexpr int kTW0 = 0, kTW1 = kTW0 + kSmemW1, kTW2 = kTW1 + kSmemW, kTW4 = kTW2 + kSmemW, kTX = kTW4 + kSmemW5,
+              kTH = kTX + kSmemX, kTG = kTH + 4 * kSmemH, kTBias = kTG + 128 * kOutPad * 2,
+              kTrainSmem = kTBias + kBiasFloats * 4;
+constexpr uint32_t kColW0 = 64, kColW4 = kColW0 + kInPad, kColW1 = kColW4 + kOutPad;  // TMEM columns
+static_assert(kColW1 + 3 * kWidth == 512, "TMEM columns");
+constexpr int kPartTiles = (512 - 64) / 4;                        // float4 columns of the weight gradients
+constexpr int kPartFloats = kPartTiles * 4 * 128 + 3 * kWidth + kOut;
+constexpr size_t kGeluFloats = 4 * 128 * 128;  // GELU' of one tile
+
+struct TrainArgs {
+    const uint16_t *W[kLayers];  // global BF16 weights [out_pad][in_pad]
+    const float *params;
+    int off[kLayers];
+    int n;                       // points of the batch
+    const float *X;              // FP32 inputs [n][34], or null:
+    const float *in5, *fourier;  // samples of 5 floats and the Fourier matrix
+    const int32_t *idx;          // sample of each point, null: point i's is i
+    const float *T;              // targets [sample][4]
+    float *gelu;                 // [CTA][kGeluFloats]
+    float *part;                 // [CTA][kPartFloats]
+    double *loss;                // [CTA]
+    int *err;
+    uint64_t wait_ns;
+    int skip_products;
+};
+
+// Copy 128 rows of W (128 columns) into core matrices, asynchronously.
+__device__ __forceinline__ void load_w_async(uint8_t *dst, const uint16_t *W)
+{
+    for (int v = threadIdx.x; v < 128 * 16; v += kTrainThreads) {
+        const int r = v >> 4, j = v & 15;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + ((r >> 3) * 16 + j) * 128 + (r & 7) * 16)),
+                     "l"(W + r * kWidth + 8 * j)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+__device__ __forceinline__ void load_w_wait()
+{
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// One product over `steps` K-steps of 16: A and B at a0, b0, advancing by da,
+// db bytes per step, with their descriptors' offsets.
+struct Operand {
+    uint32_t at, step, lbo, sbo;
+};
+// K-major tile of kg k-groups; MN-major (reduced over its rows) tile of kg groups.
+__device__ __forceinline__ Operand k_major(uint32_t at, int kg)
+{
+    return {at, 256u, 128u, 128u * kg};
+}
+__device__ __forceinline__ Operand mn_major(uint32_t at, int kg)
+{
+    return {at, 256u * kg, 128u * kg, 128u};
+}
+__device__ __forceinline__ void product(uint32_t d, const Operand &a, const Operand &b, uint32_t idesc, int steps,
+                                        bool accumulate)
+{
+    for (int s = 0; s < steps; s++)
+        mma_bf16(d, smem_desc(a.at + a.step * s, a.lbo, a.sbo), smem_desc(b.at + b.step * s, b.lbo, b.sbo), idesc,
+                 (accumulate || s > 0) ? 1u : 0u);
+}
+
+__global__ void __launch_bounds__(kTrainThreads, 1) k_mlp_train(TrainArgs a)
+{
+    extern __shared__ __align__(128) uint8_t sm[];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t tslot;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    float *sbias = reinterpret_cast<float *>(sm + kTBias);
+    for (int l = 0; l < kLayers; l++) {
+        if (l == 3) continue;
+        const int ip = l == 0 ? kInPad : kWidth, op = l == 4 ? kOutPad : kWidth, kg = ip / 8;
+        uint8_t *dst = sm + (l == 0 ? kTW0 : (l == 1 ? kTW1 : (l == 2 ? kTW2 : kTW4)));
+        for (int v = tid; v < op * kg; v += kTrainThreads) {
+            const int r = v / kg, j = v - r * kg;
+            *reinterpret_cast<uint4 *>(dst + ((r >> 3) * kg + j) * 128 + (r & 7) * 16) =
+                *reinterpret_cast<const uint4 *>(a.W[l] + (size_t)r * ip + 8 * j);
+        }
+    }
+    for (int i = tid; i < kBiasFloats; i += kTrainThreads) {
+        const int l = i / kWidth, c = i - l * kWidth;
+        sbias[i] = (l < 4) ? a.params[a.off[l] + kWidth * (l == 0 ? kIn : kWidth) + c]
+                           : (c < kOut ? a.params[a.off[4] + kOut * kWidth + c] : 0.f);
+    }
+    if (warp == 0) tmem_alloc(&tslot, 512);
+    if (tid == 0) mbar_init(&bar, 1);
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    const uint32_t tmem = tslot;
+    const uint32_t smb = smem_u32(sm);
+    const uint32_t sX = smb + kTX, sG = smb + kTG;
+    auto sH = [&](int l) { return smb + kTH + l * kSmemH; };
+    const int row = 32 * (warp & 3) + lane, c_half = 16 * (warp >> 2);  // this thread's row and columns of a half
+    const uint32_t taddr = tmem + ((uint32_t)(32 * (warp & 3)) << 16);
+    float4 *gelu_at = reinterpret_cast<float4 *>(a.gelu + blockIdx.x * kGeluFloats) + tid;
+    const bool issuer = tid == 0 && !a.skip_products;
+    uint32_t parity = 0;
+    bool ok = true;  // (a thread that gave up waits no more; the tile's end makes it the block's)
+    auto wait = [&]() {
+        ok = ok && mbar_wait_bounded(&bar, parity, a.wait_ns);
+        parity ^= 1u;
+        fence_after_sync();
+    };
+    // after the threads' shared-memory writes and TMEM reads, before products that follow them
+    auto publish = [&]() {
+        fence_before_sync();
+        fence_smem_to_async();
+        __syncthreads();
+        fence_after_sync();
+    };
+    // both halves of a layer's products: issue(q) forms half q in columns 0..63,
+    // use(q, v, out) turns this thread's 16 accumulators into packed BF16, and
+    // the two halves are stored in `tile` when the products have read it
+    auto layer = [&](auto &&issue, auto &&use, uint8_t *tile) {
+        uint32_t pk[2][8];
+        if (issuer && ok) {
+            issue(0);
+            mma_commit(&bar);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            float v[16];
+            wait();
+            tmem_ld16(taddr + c_half, v);
+            if (q == 0) {
+                fence_before_sync();
+                __syncthreads();
+                if (issuer && ok) {
+                    fence_after_sync();
+                    issue(1);
+                    mma_commit(&bar);
+                }
+            }
+            use(q, v, pk[q]);
+        }
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+#pragma unroll
+            for (int j = 0; j < 2; j++)
+                *reinterpret_cast<uint4 *>(tile + ((row >> 3) * 16 + 8 * q + c_half / 8 + j) * 128 + (row & 7) * 16) =
+                    make_uint4(pk[q][4 * j], pk[q][4 * j + 1], pk[q][4 * j + 2], pk[q][4 * j + 3]);
+        publish();
+    };
+    auto pack2 = [](float x, float y) { return bf16_bits(x) | (uint32_t)bf16_bits(y) << 16; };
+    // column sums of a gradient tile: this thread's 8 features (tid % 16) over
+    // half of a core matrix's points
+    float db[3][8] = {};
+    auto add_columns = [&](const uint8_t *tile, float *s) {
+        const uint8_t *core = tile + (((tid >> 4) & 15) * 16 + (tid & 15)) * 128;
+#pragma unroll
+        for (int i = 0; i < 4; i++) {  // (the rows in turn by lane: no bank conflicts)
+            const uint4 u = *reinterpret_cast<const uint4 *>(core + ((i + 4 * (tid >> 8) + tid) & 7) * 16);
+            const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                s[2 * c] += __uint_as_float(w[c] << 16);
+                s[2 * c + 1] += __uint_as_float(w[c] & 0xFFFF0000u);
+            }
+        }
+    };
+    double e2 = 0.0;
+    float db4[kOut] = {};
+    const float sc = 2.f / (4.f * (float)a.n);
+    const int n_tiles = (a.n + 127) / 128;
+    bool first = true;  // the weight gradients start with this tile
+    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x, first = false) {
+        const int p0 = t * 128;
+        load_w_async(sm + kTH + 3 * kSmemH, a.W[3]);
+        if (a.X) {
+#pragma unroll
+            for (int v = tid; v < 128 * kInPad; v += kTrainThreads) {
+                const int r = v / kInPad, f = v - r * kInPad, i = p0 + r;
+                uint16_t h = 0;
+                if (i < a.n) h = f < kIn ? bf16_bits(a.X[(size_t)i * kIn + f]) : (uint16_t)(f == kIn ? 0x3F80 : 0);
+                *reinterpret_cast<uint16_t *>(sm + kTX + ((r >> 3) * (kInPad / 8) + (f >> 3)) * 128 + (r & 7) * 16 + (f & 7) * 2) = h;
+            }
+        } else if (tid < 128) {
+            const int i = p0 + tid;
+            uint16_t h[kInPad] = {};
+            if (i < a.n) {
+                const float *s = a.in5 + (size_t)(a.idx ? a.idx[i] : i) * 5;
+                point_features(a.fourier, s[0], s[1], s[2], s[3], s[4], h);
+                h[kIn] = 0x3F80;  // 1
+            }
+#pragma unroll
+            for (int j = 0; j < kInPad / 8; j++) store_row_chunk(sm + kTX, kInPad / 8, tid, j, h + 8 * j);
+        }
+        load_w_wait();
+        publish();
+        // forward: the four hidden layers
+#pragma unroll 1
+        for (int l = 0; l < 4; l++) {
+            const int kg = l == 0 ? kInPad / 8 : 16;
+            const uint32_t in = l == 0 ? sX : sH(l - 1);
+            const uint32_t w = l == 0 ? smb + kTW0 : (l == 1 ? smb + kTW1 : (l == 2 ? smb + kTW2 : sH(3)));
+            layer(
+                [&](int q) {
+                    product(tmem, k_major(in, kg), k_major(w + q * 1024u * kg, kg), idesc_bf16<64>(), kg / 2, false);
+                },
+                [&](int q, const float *v, uint32_t *out) {
+                    const float *b = sbias + l * kWidth + 64 * q + c_half;
+                    float4 *gp = gelu_at + (l * 8 + q * 4) * kTrainThreads;
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        float y[4], g[4];
+#pragma unroll
+                        for (int i = 0; i < 4; i++) {
+                            const float z = v[4 * j + i] + b[4 * j + i];
+                            y[i] = gelu(z);
+                            g[i] = gelu_grad(z);
+                        }
+                        gp[j * kTrainThreads] = make_float4(g[0], g[1], g[2], g[3]);
+                        out[2 * j] = pack2(y[0], y[1]);
+                        out[2 * j + 1] = pack2(y[2], y[3]);
+                    }
+                },
+                sm + kTH + l * kSmemH);
+        }
+        // the output layer: loss and its gradient
+        if (issuer && ok) {
+            product(tmem, k_major(sH(3), 16), k_major(smb + kTW4, 16), idesc_bf16<16>(), 8, false);
+            mma_commit(&bar);
+        }
+        wait();
+        if (warp < 4) {
+            float v[16];
+            tmem_ld16(taddr, v);
+            const int i = p0 + row;
+            uint16_t h[kOutPad] = {};
+            if (i < a.n) {
+                const float *T = a.T + (size_t)(a.idx ? a.idx[i] : i) * kOut;
+#pragma unroll
+                for (int c = 0; c < kOut; c++) {
+                    const float e = v[c] + sbias[4 * kWidth + c] - T[c];
+                    e2 += (double)e * e;
+                    h[c] = bf16_bits(sc * e);
+                    db4[c] += bf16_val(h[c]);
+                }
+            }
+            store_row_chunk(sm + kTG, kOutPad / 8, row, 0, h);
+            store_row_chunk(sm + kTG, kOutPad / 8, row, 1, h + 8);
+        }
+        publish();
+        // backward: the weight gradient of layer l, then the gradient of its input
+#pragma unroll 1
+        for (int l = 4; l >= 1; l--) {
+            const uint32_t g = l == 4 ? sG : sH(l), in = sH(l - 1);
+            const int kg = l == 4 ? kOutPad / 8 : 16;  // k-groups of g
+            auto weights = [&]() {
+                if (l == 4)  // (transposed: [in][out])
+                    product(tmem + kColW4, mn_major(in, 16), mn_major(g, kg), idesc_bf16<kOutPad, true, true>(), 8, !first);
+                else
+                    product(tmem + kColW1 + (l - 1) * kWidth, mn_major(g, 16), mn_major(in, 16),
+                            idesc_bf16<kWidth, true, true>(), 8, !first);
+            };
+            if (l == 3) {  // its weights take the place of its input
+                if (issuer && ok) {
+                    weights();
+                    mma_commit(&bar);
+                }
+                add_columns(sm + kTH + 3 * kSmemH, db[2]);
+                wait();
+                load_w_async(sm + kTH + 2 * kSmemH, a.W[3]);
+                load_w_wait();
+                publish();
+            }
+            const uint32_t w = l == 4 ? smb + kTW4 : (l == 3 ? in : (l == 2 ? smb + kTW2 : smb + kTW1));
+            float4 gp[8];
+#pragma unroll
+            for (int j = 0; j < 8; j++) gp[j] = gelu_at[((l - 1) * 8 + j) * kTrainThreads];
+            layer(
+                [&](int q) {
+                    if (q == 0 && l != 3) weights();
+                    product(tmem, k_major(g, kg), {w + q * 1024u, 4096u, 2048u, 128u}, idesc_bf16<64, false, true>(),
+                            kg / 2, false);
+                },
+                [&](int q, const float *v, uint32_t *out) {
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const float4 g4 = gp[4 * q + j];
+                        out[2 * j] = pack2(v[4 * j] * g4.x, v[4 * j + 1] * g4.y);
+                        out[2 * j + 1] = pack2(v[4 * j + 2] * g4.z, v[4 * j + 3] * g4.w);
+                    }
+                    if (q == 0) {
+                        if (l == 2) add_columns(sm + kTH + 2 * kSmemH, db[1]);
+                        if (l == 1) add_columns(sm + kTH + kSmemH, db[0]);
+                    }
+                },
+                sm + kTH + (l - 1) * kSmemH);
+        }
+        if (issuer && ok) {
+            product(tmem + kColW0, mn_major(sH(0), 16), mn_major(sX, kInPad / 8), idesc_bf16<kInPad, true, true>(), 8, !first);
+            mma_commit(&bar);
+        }
+        wait();
+        ok = __syncthreads_and(ok);
+        if (!ok) break;
+    }
+    if (ok) {
+        // this CTA's sums: the weight gradients as [column / 4][row] float4, then the biases'
+        float *part = a.part + (size_t)blockIdx.x * kPartFloats;
+        float4 *pw = reinterpret_cast<float4 *>(part);
+#pragma unroll 1
+        for (int c = 64 + 32 * (warp >> 2); c < 512; c += 128) {
+            float v[32];
+            tmem_ld32(taddr + c, v);
+#pragma unroll
+            for (int j = 0; j < 8; j++)
+                pw[((c - 64) / 4 + j) * 128 + row] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        }
+        float *red = reinterpret_cast<float *>(sm + kTH);  // [warp][3][128]: sums over the warps' points
+#pragma unroll
+        for (int l = 0; l < 3; l++)
+#pragma unroll
+            for (int c = 0; c < 8; c++) {
+                const float s = db[l][c] + __shfl_xor_sync(0xffffffffu, db[l][c], 16);
+                if (lane < 16) red[(warp * 3 + l) * kWidth + 8 * lane + c] = s;
+            }
+        float *red4 = red + 16 * 3 * kWidth;  // [warp][4]
+        double *rede = reinterpret_cast<double *>(red4 + 4 * kOut);
+        for (int o = 16; o > 0; o >>= 1) {
+            e2 += __shfl_xor_sync(0xffffffffu, e2, o);
+            for (int c = 0; c < kOut; c++) db4[c] += __shfl_xor_sync(0xffffffffu, db4[c], o);
+        }
+        if (lane == 0 && warp < 4) {
+            rede[warp] = e2;
+            for (int c = 0; c < kOut; c++) red4[warp * kOut + c] = db4[c];
+        }
+        __syncthreads();
+        float *pb = part + kPartTiles * 4 * 128;
+        for (int i = tid; i < 3 * kWidth; i += kTrainThreads) {
+            float s = 0.f;
+            for (int w = 0; w < 16; w++) s += red[w * 3 * kWidth + i];
+            pb[i] = s;
+        }
+        if (tid < kOut) pb[3 * kWidth + tid] = red4[tid] + red4[kOut + tid] + red4[2 * kOut + tid] + red4[3 * kOut + tid];
+        if (tid == 0) a.loss[blockIdx.x] = rede[0] + rede[1] + rede[2] + rede[3];
+    } else if (tid == 0) {
+        atomicExch(a.err, 1);
+    }
+    fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 512);
+}
+
+// Gradients and loss from the CTAs' sums: a block per 64 float4 of them, its
+// eight groups of 64 threads each every eighth CTA (fixed order).
+struct ReduceArgs {
+    const float *part;
+    const double *lossp;
+    int ctas, n;
+    int off[kLayers];
+    float *grads;
+    double *loss;
+    int add;       // add to the loss (the batches of an epoch)
+};
+__global__ void __launch_bounds__(512) k_train_reduce(ReduceArgs a)
+{
+    __shared__ float4 sum[7][64];
+    const int at = blockIdx.x * 64 + (threadIdx.x & 63), grp = threadIdx.x >> 6;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (at < kPartFloats / 4)
+#pragma unroll 10
+        for (int b = grp; b < a.ctas; b += 8) {
+            const float4 v = *reinterpret_cast<const float4 *>(a.part + (size_t)b * kPartFloats + 4 * at);
+            s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+        }
+    if (grp) sum[grp - 1][threadIdx.x & 63] = s;
+    __syncthreads();
+    if (grp || at >= kPartFloats / 4) return;
+    for (int q = 0; q < 7; q++) {
+        const float4 v = sum[q][threadIdx.x];
+        s.x += v.x, s.y += v.y, s.z += v.z, s.w += v.w;
+    }
+    const float v[4] = {s.x, s.y, s.z, s.w};
+    for (int j = 0; j < 4; j++) {
+        int to = -1;
+        if (at < kPartTiles * 128) {
+            const int c = 64 + 4 * (at >> 7) + j, r = at & 127;
+            if (c < (int)kColW4) {
+                const int i = c - (int)kColW0;
+                if (i <= kIn) to = a.off[0] + (i < kIn ? r * kIn + i : kWidth * kIn + r);
+            } else if (c < (int)kColW1) {
+                if (c - (int)kColW4 < kOut) to = a.off[4] + (c - (int)kColW4) * kWidth + r;
+            } else {
+                const int l = 1 + (c - (int)kColW1) / kWidth;
+                to = a.off[l] + r * kWidth + (c - (int)kColW1) % kWidth;
+            }
+        } else {
+            const int i = 4 * (at - kPartTiles * 128) + j;
+            to = i < 3 * kWidth ? a.off[1 + i / kWidth] + kWidth * kWidth + i % kWidth
+                                : a.off[4] + kOut * kWidth + i - 3 * kWidth;
+        }
+        if (to >= 0) a.grads[to] = v[j];
+    }
+    if (at == 0) {
+        double l = 0.0;
+        for (int b = 0; b < a.ctas; b++) l += a.lossp[b];
+        *a.loss = (a.add ? *a.loss : 0.0) + l / (4.0 * a.n);
+    }
+}
+
 // Free stream of each point's case (all points of [0, n)).
 __global__ void k_free_stream(lskum::MlpView v, const uint8_t *keep)
 {
@@ -799,19 +994,6 @@ double uniform01(uint64_t &s)
     return (double)(splitmix64(s) >> 11) * (1.0 / 9007199254740992.0);
 }
 
-template <int EPI, int N>
-cudaError_t gemm(const GemmArgs &g, int grid_x, int grid_y, cudaStream_t s)
-{
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm<EPI, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPadSmem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    k_gemm<EPI, N><<<dim3(grid_x, grid_y), 128, kPadSmem, s>>>(g);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
 struct lskum_mlp {
@@ -820,12 +1002,14 @@ struct lskum_mlp {
     int32_t P = 0;  // batch capacity (multiple of kBatchAlign)
     std::vector<void *> allocs;
     float *params = nullptr, *m = nullptr, *v = nullptr, *grads = nullptr, *fourier = nullptr;
-    uint16_t *W[kLayers] = {}, *Wt[kLayers] = {};
+    uint16_t *W[kLayers] = {};
     int off[kLayers] = {};
-    uint16_t *X = nullptr, *Xt = nullptr, *H[4] = {}, *Ht[4] = {}, *G5 = nullptr, *G5t = nullptr, *G[4] = {},
-             *Gt[4] = {};
-    float *GP[4] = {}, *O = nullptr, *part = nullptr, *Xf = nullptr, *Tf = nullptr;
-    double *loss = nullptr;
+    uint16_t *X = nullptr;
+    float *O = nullptr, *Xf = nullptr, *Tf = nullptr;
+    int ctas = 1;  // of the training kernel: one per SM, or per tile of the largest batch
+    float *gelu = nullptr, *part = nullptr;  // its scratch and sums
+    double *lossp = nullptr, *loss = nullptr;
+    float *h_out = nullptr;  // pinned: gradients, loss, error flag
     int *err = nullptr;
     uint64_t wait_ns = 1000000000ull;  // time limit of the tensor-core waits
     int skip_products = 0;             // failure-path test switch (lskum_mlp_set_wait_test)
@@ -871,7 +1055,6 @@ cudaError_t pack(lskum_mlp *m)
     a.params = m->params;
     for (int l = 0; l < kLayers; l++) {
         a.W[l] = m->W[l];
-        a.Wt[l] = m->Wt[l];
         a.off[l] = m->off[l];
         a.in_true[l] = kInTrue[l];
         a.in_pad[l] = kInP[l];
@@ -882,108 +1065,13 @@ cudaError_t pack(lskum_mlp *m)
     return cudaGetLastError();
 }
 
-// Forward pass of rows [0, rows) already in m->X (BF16); n valid rows.
-// train: also the transposed activations and GELU'(Z).
-cudaError_t forward(lskum_mlp *m, int n, int rows, bool train)
+// The error flag was set: clear it.
+lskum_status wait_error(lskum_mlp *m)
 {
-    const int P = m->P;
-    const int gx = rows / 128;
-    cudaError_t e = cudaSuccess;
-    for (int l = 0; l < 4 && e == cudaSuccess; l++) {
-        GemmArgs g{};
-        g.A = l == 0 ? m->X : m->H[l - 1];
-        g.lda = l == 0 ? kInPad : kWidth;
-        g.a_rows = n;
-        g.B = m->W[l];
-        g.ldb = kInP[l];
-        g.b_rows = kWidth;
-        g.K = kInP[l];
-        g.k_split = g.K;
-        g.m_valid = n;
-        g.bias = m->params + m->off[l] + kOutTrue[l] * kInTrue[l];
-        g.gp_out = train ? m->GP[l] : nullptr;
-        g.out = m->H[l];
-        g.ldo = kWidth;
-        g.out_t = train ? m->Ht[l] : nullptr;
-        g.ldt = P;
-        g.err = m->err;
-        g.wait_ns = m->wait_ns;
-        g.skip_products = m->skip_products;
-        e = gemm<kFwdHidden, 128>(g, gx, 1, m->stream);
-    }
-    if (e != cudaSuccess) return e;
-    GemmArgs g{};
-    g.A = m->H[3];
-    g.lda = kWidth;
-    g.a_rows = n;
-    g.B = m->W[4];
-    g.ldb = kWidth;
-    g.b_rows = kOutPad;
-    g.K = kWidth;
-    g.k_split = kWidth;
-    g.m_valid = n;
-    g.bias = m->params + m->off[4] + kOut * kWidth;
-    g.out_f = m->O;
-    g.err = m->err;
-    g.wait_ns = m->wait_ns;
-    g.skip_products = m->skip_products;
-    return gemm<kFwdOut, 16>(g, gx, 1, m->stream);
-}
-
-// Backward pass after forward(train) and k_loss: gradients into m->grads.
-cudaError_t backward(lskum_mlp *m, int n, int rows)
-{
-    const int P = m->P;
-    const int gx = rows / 128;
-    const int splits = rows / kSplitK;
-    cudaError_t e = cudaSuccess;
-    for (int l = 4; l >= 0 && e == cudaSuccess; l--) {
-        // weight gradient of layer l: (G_l)^T A_{l-1}, points as the reduction
-        GemmArgs w{};
-        w.A = l == 4 ? m->G5t : m->Gt[l];
-        w.lda = P;
-        w.a_rows = l == 4 ? kOutPad : kWidth;
-        w.B = l == 0 ? m->Xt : m->Ht[l - 1];
-        w.ldb = P;
-        w.b_rows = kInP[l];
-        w.K = rows;
-        w.k_split = kSplitK;
-        w.m_valid = kOutTrue[l];
-        w.out_f = m->part;
-        w.err = m->err;
-        w.wait_ns = m->wait_ns;
-        w.skip_products = m->skip_products;
-        e = l == 0 ? gemm<kWgrad, kInPad>(w, 1, splits, m->stream) : gemm<kWgrad, 128>(w, 1, splits, m->stream);
-        if (e != cudaSuccess) break;
-        const int nw = kOutTrue[l] * kInTrue[l];
-        k_reduce_wgrad<<<(nw + 255) / 256, 256, 0, m->stream>>>(m->part, splits, kOutTrue[l], kInP[l], kInTrue[l],
-                                                                 m->grads + m->off[l]);
-        k_colsum<<<kOutTrue[l], 256, 0, m->stream>>>(l == 4 ? m->G5t : m->Gt[l], P, rows,
-                                                     m->grads + m->off[l] + nw);
-        if (l == 0) break;
-        // data gradient into layer l's input: (G_l W_l) * GELU'(Z_{l-1})
-        GemmArgs d{};
-        d.A = l == 4 ? m->G5 : m->G[l];
-        d.lda = l == 4 ? kOutPad : kWidth;
-        d.a_rows = n;
-        d.B = m->Wt[l];
-        d.ldb = kOutP[l];
-        d.b_rows = kWidth;
-        d.K = kOutP[l];
-        d.k_split = d.K;
-        d.m_valid = n;
-        d.gp_in = m->GP[l - 1];
-        d.out = m->G[l - 1];
-        d.ldo = kWidth;
-        d.out_t = m->Gt[l - 1];
-        d.ldt = P;
-        d.err = m->err;
-        d.wait_ns = m->wait_ns;
-        d.skip_products = m->skip_products;
-        e = gemm<kBwdData, 128>(d, gx, 1, m->stream);
-    }
-    if (e == cudaSuccess) e = cudaGetLastError();
-    return e;
+    cudaMemsetAsync(m->err, 0, sizeof(int), m->stream);
+    char buf[96];
+    snprintf(buf, sizeof(buf), "tensor-core product did not complete within %.3g s", (double)m->wait_ns * 1e-9);
+    return mfail(m, LSKUM_ERR_TIMEOUT, buf);
 }
 
 lskum_status check_err(lskum_mlp *m)
@@ -992,13 +1080,7 @@ lskum_status check_err(lskum_mlp *m)
     cudaError_t e = cudaMemcpyAsync(&h, m->err, sizeof(int), cudaMemcpyDeviceToHost, m->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return mcuda(m, e, "network kernels");
-    if (h) {
-        cudaMemsetAsync(m->err, 0, sizeof(int), m->stream);
-        char buf[96];
-        snprintf(buf, sizeof(buf), "tensor-core product did not complete within %.3g s", (double)m->wait_ns * 1e-9);
-        return mfail(m, LSKUM_ERR_TIMEOUT, buf);
-    }
-    return LSKUM_OK;
+    return h ? wait_error(m) : LSKUM_OK;
 }
 
 int round_rows(int n)
@@ -1006,17 +1088,47 @@ int round_rows(int n)
     return std::max(kBatchAlign, (n + kBatchAlign - 1) / kBatchAlign * kBatchAlign);
 }
 
-// One training step on rows [0, n) of X/Xt (already filled), targets T via idx.
-cudaError_t train_step(lskum_mlp *m, int n, const float *T, const int32_t *idx)
+// Loss and gradients of a batch of n points: inputs X, or the samples idx of
+// in5 where X is null (their losses add up in m->loss); targets T.
+cudaError_t train_step(lskum_mlp *m, int n, const float *X, const float *in5, const float *T, const int32_t *idx)
 {
-    const int rows = round_rows(n);
-    cudaError_t e = forward(m, n, rows, true);
-    if (e == cudaSuccess) {
-        k_loss<<<(rows + 255) / 256, 256, 0, m->stream>>>(m->O, T, idx, n, rows, m->G5, m->G5t, m->P, m->loss);
-        e = cudaGetLastError();
+    static bool attr = false;
+    if (!attr) {
+        cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, kTrainSmem);
+        if (e != cudaSuccess) return e;
+        attr = true;
     }
-    if (e == cudaSuccess) e = backward(m, n, rows);
-    return e;
+    TrainArgs a{};
+    ReduceArgs r{};
+    for (int l = 0; l < kLayers; l++) {
+        a.W[l] = m->W[l];
+        a.off[l] = r.off[l] = m->off[l];
+    }
+    a.params = m->params;
+    a.n = r.n = n;
+    a.X = X;
+    a.in5 = in5;
+    a.fourier = m->fourier;
+    a.idx = idx;
+    a.T = T;
+    a.gelu = m->gelu;
+    a.part = m->part;
+    a.loss = m->lossp;
+    a.err = m->err;
+    a.wait_ns = m->wait_ns;
+    a.skip_products = m->skip_products;
+    const int ctas = std::min((n + 127) / 128, m->ctas);
+    k_mlp_train<<<ctas, kTrainThreads, kTrainSmem, m->stream>>>(a);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    r.part = m->part;
+    r.lossp = m->lossp;
+    r.ctas = ctas;
+    r.grads = m->grads;
+    r.loss = m->loss;
+    r.add = X == nullptr;
+    k_train_reduce<<<(kPartFloats / 4 + 63) / 64, 512, 0, m->stream>>>(r);
+    return cudaGetLastError();
 }
 
 cudaError_t adam(lskum_mlp *m, float lr)
@@ -1028,6 +1140,14 @@ cudaError_t adam(lskum_mlp *m, float lr)
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = pack(m);
     return e;
+}
+
+int num_sms()
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(sms, 1);
 }
 
 int g_num_sms = 0;
@@ -1044,12 +1164,7 @@ cudaError_t fused_forward(lskum_mlp *m, int n, const uint16_t *X, float *O, cons
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    if (!g_num_sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev);
-        if (g_num_sms <= 0) g_num_sms = 1;
-    }
+    if (!g_num_sms) g_num_sms = num_sms();
     FusedArgs a{};
     for (int l = 0; l < kLayers; l++) {
         a.W[l] = m->W[l];
@@ -1102,6 +1217,7 @@ void lskum_mlp_destroy(lskum_mlp *m)
     for (void *p : m->allocs) cudaFree(p);
     if (m->s_in) cudaFree(m->s_in);
     if (m->s_tgt) cudaFree(m->s_tgt);
+    if (m->h_out) cudaFreeHost(m->h_out);
     if (m->stream) cudaStreamDestroy(m->stream);
     delete m;
 }
@@ -1141,30 +1257,22 @@ lskum_status lskum_mlp_create(uint64_t seed, int32_t max_batch, void *cuda_strea
     A(&m->params, kNParams);
     A(&m->m, kNParams);
     A(&m->v, kNParams);
-    A(&m->grads, kNParams);
+    // gradients, loss and error flag in one piece: one copy brings all three
+    A(&m->grads, kNParams + 4);
+    m->loss = reinterpret_cast<double *>(m->grads + kNParams);
+    m->err = reinterpret_cast<int *>(m->loss + 1);
     A(&m->fourier, 3 * kFreq);
-    for (int l = 0; l < kLayers; l++) {
-        A(&m->W[l], (size_t)kOutP[l] * kInP[l]);
-        A(&m->Wt[l], (size_t)kOutP[l] * kInP[l]);
-    }
+    for (int l = 0; l < kLayers; l++) A(&m->W[l], (size_t)kOutP[l] * kInP[l]);
     A(&m->X, P * kInPad);
-    A(&m->Xt, P * kInPad);
-    for (int l = 0; l < 4; l++) {
-        A(&m->H[l], P * kWidth);
-        A(&m->Ht[l], P * kWidth);
-        A(&m->G[l], P * kWidth);
-        A(&m->Gt[l], P * kWidth);
-        A(&m->GP[l], P * kWidth);
-    }
-    A(&m->G5, P * kOutPad);
-    A(&m->G5t, P * kOutPad);
+    m->ctas = std::min((int)(P / 128), num_sms());
+    A(&m->gelu, m->ctas * kGeluFloats);
+    A(&m->part, m->ctas * (size_t)kPartFloats);
+    A(&m->lossp, m->ctas);
     A(&m->O, P * kOut);
-    A(&m->part, (P / kSplitK) * (size_t)kWidth * kWidth);
     A(&m->Xf, P * kIn);
     A(&m->Tf, P * kOut);
-    A(&m->loss, 1);
-    A(&m->err, 1);
     A(&m->idx, P);
+    if (e == cudaSuccess) e = cudaMallocHost(reinterpret_cast<void **>(&m->h_out), (kNParams + 4) * sizeof(float));
     if (e != cudaSuccess) {
         lskum_mlp_destroy(m);
         return mcuda(nullptr, e, "cudaMalloc");
@@ -1228,7 +1336,7 @@ lskum_status lskum_mlp_features(lskum_mlp *m, const float *in5, int32_t n, float
         cudaError_t e = cudaMemcpyAsync(m->Xf, in5 + (size_t)k0 * 5, (size_t)nb * 5 * sizeof(float),
                                         cudaMemcpyHostToDevice, m->stream);  // Xf holds >= 5 floats per row
         if (e == cudaSuccess) {
-            k_features<<<(nb + 255) / 256, 256, 0, m->stream>>>(m->Xf, nullptr, nb, nb, m->fourier, m->X, nullptr, 0);
+            k_features<<<(nb + 255) / 256, 256, 0, m->stream>>>(m->Xf, nb, m->fourier, m->X);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) {
@@ -1253,7 +1361,7 @@ lskum_status lskum_mlp_forward(lskum_mlp *m, const float *X, int32_t n, float *o
         cudaError_t e = cudaMemcpyAsync(m->Xf, X + (size_t)k0 * kIn, (size_t)nb * kIn * sizeof(float),
                                         cudaMemcpyHostToDevice, m->stream);
         if (e == cudaSuccess) {
-            k_inputs_from_f32<<<(rows + 255) / 256, 256, 0, m->stream>>>(m->Xf, nb, rows, m->X, nullptr, 0);
+            k_inputs_from_f32<<<(rows + 255) / 256, 256, 0, m->stream>>>(m->Xf, nb, rows, m->X);
             e = cudaGetLastError();
         }
         if (e == cudaSuccess) e = fused_forward<kSrcBuffer>(m, nb, m->X, m->O, nullptr, 0);
@@ -1270,24 +1378,26 @@ lskum_status lskum_mlp_forward(lskum_mlp *m, const float *X, int32_t n, float *o
 lskum_status lskum_mlp_loss_grads(lskum_mlp *m, const float *X, const float *T, int32_t n, float *loss, float *grads)
 {
     if (!m || n < 1 || n > m->P || !X || !T) return m ? mfail(m, LSKUM_ERR_ARG, "bad argument") : LSKUM_ERR_ARG;
-    const int rows = round_rows(n);
     cudaError_t e = cudaMemcpyAsync(m->Xf, X, (size_t)n * kIn * sizeof(float), cudaMemcpyHostToDevice, m->stream);
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(m->Tf, T, (size_t)n * kOut * sizeof(float), cudaMemcpyHostToDevice, m->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(m->loss, 0, sizeof(double), m->stream);
-    if (e == cudaSuccess) {
-        k_inputs_from_f32<<<(rows + 255) / 256, 256, 0, m->stream>>>(m->Xf, n, rows, m->X, m->Xt, m->P);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = train_step(m, n, m->Tf, nullptr);
-    double l = 0.0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&l, m->loss, sizeof(double), cudaMemcpyDeviceToHost, m->stream);
-    if (grads && e == cudaSuccess)
-        e = cudaMemcpyAsync(grads, m->grads, kNParams * sizeof(float), cudaMemcpyDeviceToHost, m->stream);
+    if (e == cudaSuccess) e = train_step(m, n, m->Xf, nullptr, m->Tf, nullptr);
+    // one copy into pinned memory (14 us) instead of three to pageable memory (17 us each)
+    const size_t first = grads ? 0 : kNParams;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(m->h_out + first, m->grads + first, (kNParams + 4 - first) * sizeof(float),
+                            cudaMemcpyDeviceToHost, m->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(m->stream);
     if (e != cudaSuccess) return mcuda(m, e, "loss and gradients");
-    lskum_status s = check_err(m);
-    if (s != LSKUM_OK) return s;
-    if (loss) *loss = (float)l;
+    int err;
+    std::memcpy(&err, m->h_out + kNParams + 2, sizeof err);
+    if (err) return wait_error(m);
+    if (grads) std::memcpy(grads, m->h_out, kNParams * sizeof(float));
+    if (loss) {
+        double l;
+        std::memcpy(&l, m->h_out + kNParams, sizeof l);
+        *loss = (float)l;
+    }
     return LSKUM_OK;
 }
 
@@ -1423,11 +1533,7 @@ lskum_status lskum_mlp_train(lskum_mlp *m, int32_t epochs, int32_t batch, float 
         int steps = 0;
         for (int32_t b0 = 0; b0 < S && e == cudaSuccess; b0 += batch, steps++) {
             const int nb = std::min(batch, S - b0);
-            const int rows = round_rows(nb);
-            k_features<<<(rows + 255) / 256, 256, 0, m->stream>>>(m->s_in, dperm + b0, nb, rows, m->fourier, m->X,
-                                                                  m->Xt, m->P);
-            e = cudaGetLastError();
-            if (e == cudaSuccess) e = train_step(m, nb, m->s_tgt, dperm + b0);
+            e = train_step(m, nb, nullptr, m->s_in, m->s_tgt, dperm + b0);
             if (e == cudaSuccess) e = adam(m, lr);
         }
         double l = 0.0;
