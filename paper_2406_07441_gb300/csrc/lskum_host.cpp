@@ -1363,6 +1363,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     c->case_hist0 = A.alloc<double>(c->n_cases);
     c->case_err = A.alloc<int32_t>(c->n_cases);
     c->case_bad = A.alloc<int32_t>(c->n_cases);
+    d.suspect = A.alloc<int32_t>(c->n_cases);
     c->hist_cap = 4096;
     c->hist = A.alloc<double>((size_t)c->n_cases * c->hist_cap);
     c->hist4 = A.alloc<double>((size_t)c->n_cases * c->hist_cap * 4);
@@ -1501,6 +1502,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     if (e == cudaSuccess && d.jc) e = cudaMemset(d.jc, 0, 16 * (size_t)ld * sizeof(double));
     if (e == cudaSuccess && d.jcf) e = cudaMemset(d.jcf, 0, 16 * (size_t)ld * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(c->case_state, 0, c->n_cases * sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMemset(d.suspect, 0, c->n_cases * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(c->case_it, 0, c->n_cases * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(c->case_hist0, 0, c->n_cases * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(c->case_err, 0, c->n_cases * sizeof(int32_t));

@@ -38,6 +38,7 @@ struct Ctrl {
     int32_t it_start;    // it when the current run was enqueued
     int32_t hist_cap;    // capacity of each case's history
     int32_t n_cases;
+    int32_t live;        // set by k_begin: this iteration runs
     uint32_t sweep_bar;  // arrivals at the sweeps' level boundaries; 0 between launches
     double target;       // drop target of the current run (<= 0: none)
     int32_t *case_state; // [n_cases] CaseState; kReachedTarget finishes the
@@ -202,6 +203,7 @@ struct Dev {
     const int32_t *case_of;  // [ld] internal index -> case
     int32_t n_blk, n_cases;
     Ctrl *ctrl;
+    int32_t *suspect;        // [n_cases] 1: a residual that can make the norm non-finite
     const int32_t *case_state;  // = ctrl->case_state (read per point)
     // options
     double cfl, ramp, u_inf[4];
