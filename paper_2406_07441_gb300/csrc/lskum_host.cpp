@@ -1305,6 +1305,14 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
         d.pk_jmf[dir] = nullptr;
         d.pk_lanes[dir] = 0;
     }
+    d.g0 = d.pk_g0[0] = d.pk_g0[1] = nullptr;
+    if (c->pk_ok && c->opts.jvp == LSKUM_JVP_INCREMENT) {
+        d.g0 = A.alloc<double>(16 * (size_t)ld);
+        for (int dir = 0; dir < 2; dir++) {
+            d.pk_lanes[dir] = (int32_t)hp.pk_pt[dir].size();
+            d.pk_g0[dir] = A.alloc<double>(8 * hp.pk_pt[dir].size());
+        }
+    }
     d.fj = nullptr;
     d.fjf = nullptr;
     d.fidx = d.fpt = nullptr;

@@ -193,6 +193,11 @@ struct Dev {
     float *pk_jmf[2], *fjf;
     const int32_t *fidx, *fpt;  // fpt[f] = internal index of framed point f
     int32_t pk_lanes[2], nf;
+    // packed form, increment products: the axis split fluxes of every point at
+    // the state of the iteration, [ld][4 products][4], and of every packed
+    // slot's neighbour along the two directions of the point's frame, [2][4]
+    // per slot lane (null: exact products, or lists too long for the form)
+    double *g0, *pk_g0[2];
     // per-case residual norm: stage 1 sums R_rho^2 over blocks of up to 256
     // points of one case (caller order), stage 2 adds each case's blocks
     double *blk;             // [n_blk][4] partial sums of the four components

@@ -225,6 +225,29 @@ __device__ __forceinline__ PrimU prim_from_cons(const double U[4])
     return P;
 }
 
+// The same for the increment products, by the shortest chain: with Q = 2 rho p
+// = 0.8 (rho E - |m|^2/2) everything needs one reciprocal square root, beside
+// the one division, instead of three divisions and a square root in a row.
+// (Only what flux_prim reads.)
+__device__ __forceinline__ PrimU prim_short(const double U[4])
+{
+    PrimU P;
+    P.rho = U[0];
+    P.irho = 1.0 / U[0];
+    const double hm = 0.5 * fma(U[1], U[1], __dmul_rn(U[2], U[2]));
+    const double Q = 0.8 * fma(U[0], U[3], -hm);
+    const double r = rsqrt(Q);
+    P.sb = __dmul_rn(fabs(U[0]), r);
+    P.u = __dmul_rn(U[1], P.irho);
+    P.v = __dmul_rn(U[2], P.irho);
+    P.p = __dmul_rn(0.5 * Q, P.irho);
+    P.isb = __dmul_rn(__dmul_rn(Q, r), fabs(P.irho));
+    const double k = __dmul_rn(hm, P.irho);
+    P.e1 = fma(3.5, P.p, k);
+    P.e2 = fma(3.0, P.p, k);
+    return P;
+}
+
 template <typename T>
 __device__ __forceinline__ PrimT<T> load_prim(const T *__restrict__ pr, int i)
 {
@@ -411,23 +434,29 @@ __device__ __forceinline__ void euler_jvp(double rho, double u, double v, double
     out[3] = (dU[3] + dp) * ud + (E + p) * dud;
 }
 
+// (no contraction is left to the compiler: two evaluations of a state agree bit for bit)
+__device__ __forceinline__ void flux_prim(const MathTables &T, const PrimU &P, double dx, double dy, bool pos,
+                                          double G[4])
+{
+    const double ud = fma(P.u, dx, __dmul_rn(P.v, dy));
+    const double S = __dmul_rn(ud, P.sb);
+    double A, eS;
+    split_A(T, S, pos, A, eS);
+    const double B = __dmul_rn(__dmul_rn(eS, kInv2SqrtPi), P.isb);
+    const double sB = signed_by(B, pos);
+    const double M1 = fma(ud, A, sB);
+    const double rm = __dmul_rn(P.rho, M1);
+    const double pA = __dmul_rn(P.p, A);
+    G[0] = rm;
+    G[1] = fma(rm, P.u, __dmul_rn(pA, dx));
+    G[2] = fma(rm, P.v, __dmul_rn(pA, dy));
+    G[3] = fma(__dmul_rn(ud, P.e1), A, __dmul_rn(P.e2, sB));
+}
+
 __device__ __forceinline__ void flux_cons(const MathTables &T, const double U[4], double dx, double dy, bool pos,
                                           double G[4])
 {
-    const PrimU P = prim_from_cons(U);
-    const double ud = P.u * dx + P.v * dy;
-    const double S = ud * P.sb;
-    double A, eS;
-    split_A(T, S, pos, A, eS);
-    const double B = eS * kInv2SqrtPi * P.isb;
-    const double sB = signed_by(B, pos);
-    const double M1 = fma(ud, A, sB);
-    const double rm = P.rho * M1;
-    const double pA = P.p * A;
-    G[0] = rm;
-    G[1] = fma(rm, P.u, pA * dx);
-    G[2] = fma(rm, P.v, pA * dy);
-    G[3] = fma(ud * P.e1, A, P.e2 * sB);
+    flux_prim(T, prim_from_cons(U), dx, dy, pos, G);
 }
 
 template <int TPP, typename T>
@@ -1367,24 +1396,63 @@ __global__ void __launch_bounds__(256) k_sweep(Dev d, StateSet st, int lb, int l
 // formed by jvp_axis_sel from the point's record, or from the framed
 // points' precomputed Jacobians.)
 template <typename T>
-__device__ __forceinline__ void store_increment_product(const Dev &d, const StateSet &st, const MathTables &Tb,
-                                                        const SweepBufs<T> &sb, const T w[4], int k, int cb)
+__device__ __forceinline__ void store_increment_product(const MathTables &Tb, const SweepBufs<T> &sb, const PrimU &P,
+                                                        const double G0[4], int k, int cb)
 {
-    const bool pos = !(cb & 1);
-    const int ld = d.ld;
-    double Ui[4], Up[4], G1[4], G0[4];
-#pragma unroll
-    for (int c = 0; c < 4; c++) {
-        Ui[c] = st.U[c * ld + k];
-        Up[c] = Ui[c] + (double)w[c];
-    }
-    const double ddx = cb < 2 ? 1.0 : 0.0, ddy = cb < 2 ? 0.0 : 1.0;
-    flux_cons(Tb, Up, ddx, ddy, pos, G1);
-    flux_cons(Tb, Ui, ddx, ddy, pos, G0);
+    double G1[4];
+    flux_prim(Tb, P, cb < 2 ? 1.0 : 0.0, cb < 2 ? 0.0 : 1.0, !(cb & 1), G1);
     T J[4];
 #pragma unroll
     for (int c = 0; c < 4; c++) J[c] = (T)(G1[c] - G0[c]);
     store4(sb.jc + 16 * (size_t)k + 4 * cb, J);
+}
+
+// Split fluxes at the state of this iteration, which the increment products
+// subtract: of every point along the axes (g0), and of every framed slot's
+// neighbour in the point's frame (pk_g0).  They do not depend on the sweeps'
+// increments, so they are formed beside the q-derivatives and the residual,
+// whose integer work leaves the FP64 unit idle, instead of twice per point on
+// the sweeps' critical path (41,194 points, an iteration: 0.804 ms with them
+// there, 0.535 like this, 0.511 with prim_short's chain).
+__host__ __device__ inline int increment_base_items(const Dev &d)
+{
+    return 4 * d.n + 2 * (d.pk_lanes[0] + d.pk_lanes[1]);
+}
+__global__ void __launch_bounds__(256) k_increment_base(Dev d, StateSet st)
+{
+    __shared__ MathTables Tb;
+    if (halted(d.ctrl)) return;
+    load_math_tables(Tb);
+    __syncthreads();
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= increment_base_items(d)) return;
+    double dx, dy;
+    bool pos;
+    int i;
+    double *out;
+    if (t < 4 * d.n) {
+        i = t >> 2;
+        pos = !(t & 1);
+        dx = t & 2 ? 0.0 : 1.0;
+        dy = t & 2 ? 1.0 : 0.0;
+        out = d.g0 + 4 * (size_t)t;
+    } else {
+        t -= 4 * d.n;
+        const int dir = t >= 2 * d.pk_lanes[0];
+        t -= dir ? 2 * d.pk_lanes[0] : 0;
+        const int e = t >> 1, k = d.pk_k[dir][e], m = t & 1 ? d.pk_mb[dir][e] >> 2 : d.pk_mb[dir][e] & 3;
+        if (k < 0 || !m) return;
+        i = d.pk_nbr[dir][e];
+        pos = m & 1;
+        dx = d.geo[(t & 1 ? G_E2X : G_E1X) * d.ld + k];
+        dy = d.geo[(t & 1 ? G_E2Y : G_E1Y) * d.ld + k];
+        out = d.pk_g0[dir] + 4 * (size_t)t;
+    }
+    double U[4], G[4];
+#pragma unroll
+    for (int c = 0; c < 4; c++) U[c] = st.U[c * d.ld + i];
+    flux_prim(Tb, prim_short(U), dx, dy, pos, G);
+    store4(out, G);
 }
 
 // Jacobians of the framed points' products (exact products).  The split-flux
@@ -1583,10 +1651,11 @@ struct LanePre {
     PrimT<T> P;
     T Ap, Am, EK, B, BS, UE, iD;
     double R[2];
+    double U[4], G0[8];  // increment products: the state, the fluxes of the lane's products there
 };
 
 template <int JVP, int L, typename T>
-__device__ __forceinline__ void lane_load(const Dev &d, const SweepBufs<T> &sb, int dir, int g, int lane,
+__device__ __forceinline__ void lane_load(const Dev &d, const StateSet &st, const SweepBufs<T> &sb, int dir, int g, int lane,
                                           WarpStage<T> &ws, LanePre<T> &a)
 {
     const int p = lane / L, s = lane % L;
@@ -1622,6 +1691,12 @@ __device__ __forceinline__ void lane_load(const Dev &d, const SweepBufs<T> &sb, 
         a.B = rec[xdir ? P_BX : P_BY];
         a.BS = rec[xdir ? P_BSX : P_BSY];
         a.UE = rec[xdir ? P_UE1 : P_VE1];
+    }
+    if (JVP == 1) {
+#pragma unroll
+        for (int c = 0; c < 4; c++) a.U[c] = st.U[c * d.ld + kk];
+#pragma unroll
+        for (int c = 0; c < 4 / L; c++) load4(d.g0 + 16 * (size_t)kk + 4 * (4 / L * s + c), a.G0 + 4 * c);
     }
     a.iD = (T)d.iD[kk];
 #pragma unroll
@@ -1775,8 +1850,12 @@ __device__ __forceinline__ void sweep_interior(const Dev &d, const StateSet &st,
             store4(sb.jc + 16 * (size_t)k + 8 * s + 4, Jm);
         }
     } else {
-#pragma unroll 1
-        for (int c = 0; c < C; c++) store_increment_product<T>(d, st, g_math, sb, w, k, C * s + c);
+        double Up[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) Up[c] = a.U[c] + (double)w[c];
+        const PrimU P = prim_short(Up);
+#pragma unroll
+        for (int c = 0; c < C; c++) store_increment_product<T>(g_math, sb, P, a.G0 + 4 * c, k, C * s + c);
     }
 }
 
@@ -1944,8 +2023,23 @@ __device__ __noinline__ void sweep_framed(const Dev &d, const StateSet &st, cons
         } else {
             const T w1 = sizeof(T) == 4 ? (T)d.pk_w1f[dir][e] : (T)d.pk_w1[dir][e];
             const T w2 = sizeof(T) == 4 ? (T)d.pk_w2f[dir][e] : (T)d.pk_w2[dir][e];
-            sweep_slot<JVP, T>(d, st, g_math, dW, sb.prim, framed, e1x, e1y, e2x, e2y, d.pk_nbr[dir][e], mb, w1, w2,
-                               acc);
+            const int i = d.pk_nbr[dir][e];
+            T dl[4];
+            load4_l2(dW + 4 * (size_t)i, dl);
+            double Up[4];
+#pragma unroll
+            for (int c = 0; c < 4; c++) Up[c] = st.U[c * d.ld + i] + (double)dl[c];
+            const PrimU P = prim_short(Up);
+#pragma unroll
+            for (int s = 0; s < 2; s++) {
+                const int m = s == 0 ? (mb & 3) : (mb >> 2);
+                if (!m) continue;
+                double G1[4], G0[4];
+                load4(d.pk_g0[dir] + 8 * e + 4 * s, G0);
+                flux_prim(g_math, P, s == 0 ? e1x : e2x, s == 0 ? e1y : e2y, m & 1, G1);
+#pragma unroll
+                for (int c = 0; c < 4; c++) acc[c] = fma(s == 0 ? w1 : w2, (T)(G1[c] - G0[c]), acc[c]);
+            }
         }
     }
     // segmented suffix sum: lane l adds lane l + o when both hold the same
@@ -1988,7 +2082,14 @@ __device__ __noinline__ void sweep_framed(const Dev &d, const StateSet &st, cons
             store4(sb.jc + 16 * (size_t)k + 4 * cb, J);
         }
     } else {
-        for (int cb = r; cb < 4; cb += seg) store_increment_product<T>(d, st, g_math, sb, w, k, cb);
+        double Up[4], G0[4];
+#pragma unroll
+        for (int c = 0; c < 4; c++) Up[c] = st.U[c * d.ld + k] + (double)w[c];
+        const PrimU P = prim_short(Up);
+        for (int cb = r; cb < 4; cb += seg) {
+            load4(d.g0 + 16 * (size_t)k + 4 * cb, G0);
+            store_increment_product<T>(g_math, sb, P, G0, k, cb);
+        }
     }
 }
 
@@ -2043,10 +2144,10 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_sweeps(Dev d, StateSet st, i
                         sweep_framed<JVP, T>(d, st, sb, dir, wb + t, lane);
                     }
                 } else if (two) {
-                    if (!ready) lane_load<JVP, 2, T>(d, sb, dir, g0 + t - wf, lane, ws, pre);
+                    if (!ready) lane_load<JVP, 2, T>(d, st, sb, dir, g0 + t - wf, lane, ws, pre);
                     sweep_interior<JVP, 2, T>(d, st, sb, dir, lane, pre, ws);
                 } else {
-                    if (!ready) lane_load<JVP, 4, T>(d, sb, dir, g0 + t - wf, lane, ws, pre);
+                    if (!ready) lane_load<JVP, 4, T>(d, st, sb, dir, g0 + t - wf, lane, ws, pre);
                     sweep_interior<JVP, 4, T>(d, st, sb, dir, lane, pre, ws);
                 }
                 ready = false;
@@ -2065,8 +2166,8 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_sweeps(Dev d, StateSet st, i
                     ready = true;
                 }
             } else if (t0 < nt) {
-                if (d.lvl_lanes[l] == 2) lane_load<JVP, 2, T>(d, sb, dir, g0 + t0 - wf, lane, ws, pre);
-                else lane_load<JVP, 4, T>(d, sb, dir, g0 + t0 - wf, lane, ws, pre);
+                if (d.lvl_lanes[l] == 2) lane_load<JVP, 2, T>(d, st, sb, dir, g0 + t0 - wf, lane, ws, pre);
+                else lane_load<JVP, 4, T>(d, st, sb, dir, g0 + t0 - wf, lane, ws, pre);
                 ready = true;
             }
             target += gridDim.x;
@@ -2359,6 +2460,17 @@ void enqueue_framed_jac(const Dev &d, int cur, cudaStream_t s, int *launches)
     (*launches)++;
 }
 
+bool needs_increment_base(const Dev &d)
+{
+    return d.scheme == 0 && d.jvp == 1 && d.g0;
+}
+
+void enqueue_increment_base(const Dev &d, int cur, cudaStream_t s, int *launches)
+{
+    k_increment_base<<<(increment_base_items(d) + 255) / 256, 256, 0, s>>>(d, d.set[cur]);
+    (*launches)++;
+}
+
 void enqueue_diag(const Dev &d, int cur, cudaStream_t s, int *launches)
 {
     k_diag<<<(d.n + 255) / 256, 256, 0, s>>>(d, d.set[cur]);
@@ -2385,6 +2497,7 @@ cudaError_t enqueue_sweeps_packed(const Dev &d, const Launch &L, int cur, int n_
     // the framed points' Jacobians: by k_framed_jac in the packed shape
     // (beside the q-derivatives when captured), else by the sweeps' launch
     if (fwd && !L.side && needs_framed_jac(d, L)) enqueue_framed_jac(d, cur, s, launches);
+    if (fwd && !L.side && needs_increment_base(d)) enqueue_increment_base(d, cur, s, launches);
     const bool fuse = fwd && JVP == 0 && L.sweep_lanes != 32 && framed_jac_items(d) > 0;
     const int dirs = (fwd ? 1 : 0) + (bwd ? 2 : 0);
     if (n_levels <= 0 || dirs == 0) return cudaSuccess;
@@ -2425,7 +2538,7 @@ cudaError_t enqueue_norm(const Dev &d, cudaStream_t s, int *launches)
 cudaError_t enqueue_phase(const Dev &d, const Launch &L, int cur, int ph, int n_levels, const int32_t *lvl_beg,
                           const int32_t *lvl_act_end, const int32_t *lvl_end, cudaStream_t s, int *launches)
 {
-    const bool side = L.side && (needs_framed_jac(d, L) || L.tpp > 1);
+    const bool side = L.side && (needs_framed_jac(d, L) || needs_increment_base(d) || L.tpp > 1);
     switch (ph) {
     case 0:
         k_begin<<<1, 1, 0, s>>>(d.ctrl, d.suspect);
@@ -2438,6 +2551,7 @@ cudaError_t enqueue_phase(const Dev &d, const Launch &L, int cur, int ph, int n_
             if (e != cudaSuccess) return e;
             if (needs_framed_jac(d, L)) enqueue_framed_jac(d, cur, L.side, launches);
             if (L.tpp > 1) enqueue_diag(d, cur, L.side, launches);
+            if (needs_increment_base(d)) enqueue_increment_base(d, cur, L.side, launches);
             e = cudaEventRecord(L.join, L.side);
             if (e != cudaSuccess) return e;
         }
