@@ -30,6 +30,8 @@ namespace {
 
 thread_local std::string g_create_error = "no error";
 
+lskum_status write_ctrl(lskum_ctx *c, Ctrl &h);
+
 struct Arena {
     std::vector<void *> ptrs;
     cudaError_t err = cudaSuccess;
@@ -75,6 +77,7 @@ struct lskum_ctx {
     Dev dev{};
     Launch launch{};
     Ctrl *ctrl = nullptr;
+    Ctrl *h_ctrl = nullptr;  // pinned: where the control block is read to
     double *hist = nullptr, *hist4 = nullptr;
     int32_t hist_cap = 0;
     cudaStream_t stream = nullptr;      // internal, capture-capable
@@ -1366,6 +1369,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     int32_t *dcase_blk = A.alloc<int32_t>(hp.case_blk.size()), *dinv = A.alloc<int32_t>(n);
     int32_t *dcase_of = A.alloc<int32_t>(ld);
     c->ctrl = A.alloc<Ctrl>(1);
+    if (A.err == cudaSuccess) A.err = cudaMallocHost(reinterpret_cast<void **>(&c->h_ctrl), sizeof(Ctrl));
     c->case_state = A.alloc<int32_t>(c->n_cases);
     c->case_it = A.alloc<int32_t>(c->n_cases);
     c->case_hist0 = A.alloc<double>(c->n_cases);
@@ -1558,7 +1562,9 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
             vv[p] = vb;
         }
     }
-    lskum_status s = lskum_set_state(c, rho.data(), uu.data(), vv.data(), pp.data());
+    Ctrl h{};
+    lskum_status s = write_ctrl(c, h);
+    if (s == LSKUM_OK) s = lskum_set_state(c, rho.data(), uu.data(), vv.data(), pp.data());
     if (s != LSKUM_OK) return s;
 
     return build_graphs(c);
@@ -1604,6 +1610,7 @@ void lskum_destroy(lskum_ctx *c)
     for (auto &g : c->graph)
         if (g) cudaGraphExecDestroy(g);
     c->arena.release();
+    if (c->h_ctrl) cudaFreeHost(c->h_ctrl);
     if (c->ev) cudaEventDestroy(c->ev);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
@@ -1635,9 +1642,10 @@ cudaError_t release_user(lskum_ctx *c)
 
 lskum_status read_ctrl(lskum_ctx *c, Ctrl *h)
 {
-    cudaError_t e = cudaMemcpyAsync(h, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream);
+    cudaError_t e = cudaMemcpyAsync(c->h_ctrl, c->ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "reading the control block");
+    *h = *c->h_ctrl;
     return LSKUM_OK;
 }
 
@@ -1661,31 +1669,20 @@ lskum_status write_ctrl(lskum_ctx *c, Ctrl &h)
     return LSKUM_OK;
 }
 
-// Per-case counters.  A new state (`fresh`) clears everything: every case
-// runs again, failures are forgotten and, with `history`, the histories are
-// cleared.  Otherwise stopped cases run again and failed cases stay failed.
-lskum_status reset_cases(lskum_ctx *c, bool history, bool fresh)
+// Per-case counters after a step of its own kind (a new state's are reset on
+// the device, launch_accept_state): stopped cases run again and failed cases
+// stay failed.
+lskum_status reset_cases(lskum_ctx *c)
 {
-    cudaError_t e = cudaSuccess;
-    if (fresh) {
-        e = cudaMemsetAsync(c->case_state, 0, c->n_cases * sizeof(int32_t), c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->case_err, 0, c->n_cases * sizeof(int32_t), c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->case_bad, 0x7f, c->n_cases * sizeof(int32_t), c->stream);
-    } else {
-        std::vector<int32_t> st(c->n_cases);
-        e = cudaMemcpyAsync(st.data(), c->case_state, c->n_cases * sizeof(int32_t), cudaMemcpyDeviceToHost,
-                            c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        for (auto &x : st) x = (x == kFailed || x == kFailedNow) ? (int32_t)kFailed : (int32_t)kRunning;
-        if (e == cudaSuccess)
-            e = cudaMemcpyAsync(c->case_state, st.data(), c->n_cases * sizeof(int32_t), cudaMemcpyHostToDevice,
-                                c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    }
-    if (history && e == cudaSuccess) e = cudaMemsetAsync(c->case_it, 0, c->n_cases * sizeof(int32_t), c->stream);
-    if (history && e == cudaSuccess) e = cudaMemsetAsync(c->case_hist0, 0, c->n_cases * sizeof(double), c->stream);
-    if (e != cudaSuccess) return cuda_fail(c, e, "resetting the cases");
-    return LSKUM_OK;
+    std::vector<int32_t> st(c->n_cases);
+    cudaError_t e = cudaMemcpyAsync(st.data(), c->case_state, c->n_cases * sizeof(int32_t), cudaMemcpyDeviceToHost,
+                                    c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    for (auto &x : st) x = (x == kFailed || x == kFailedNow) ? (int32_t)kFailed : (int32_t)kRunning;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(c->case_state, st.data(), c->n_cases * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    return e == cudaSuccess ? LSKUM_OK : cuda_fail(c, e, "resetting the cases");
 }
 
 lskum_status read_case_arrays(lskum_ctx *c, std::vector<int32_t> *state, std::vector<int32_t> *it)
@@ -1784,20 +1781,14 @@ lskum_status finish_state(lskum_ctx *c, bool reset_hist, bool project)
         e = cudaMemsetAsync(c->dev.dUf, 0, 4 * (size_t)c->ld * sizeof(float), c->stream);
     if (e == cudaSuccess) e = launch_reset_ctrl(c->ctrl, c->stream);
     if (e == cudaSuccess) e = launch_init_state(c->dev, c->cur, project, c->stream);
+    // (the counters on the device, behind the check: one wait for both)
+    if (e == cudaSuccess) e = launch_accept_state(c->ctrl, reset_hist, c->stream);
     Ctrl h{};
     if (e != cudaSuccess) return cuda_fail(c, e, "setting the state");
     lskum_status s = read_ctrl(c, &h);
     if (s != LSKUM_OK) return s;
     if (h.error) return fail(c, LSKUM_ERR_NONPOSITIVE, "non-physical state at point %d", c->perm[h.bad_point]);
-    if (reset_hist) {
-        h.it = 0;
-        c->hist_bound = 0;
-    }
-    h.stop = h.error = 0;
-    h.bad_point = 0x7fffffff;
-    s = reset_cases(c, reset_hist, true);
-    if (s == LSKUM_OK) s = write_ctrl(c, h);
-    if (s != LSKUM_OK) return s;
+    if (reset_hist) c->hist_bound = 0;
     e = release_user(c);
     if (e != cudaSuccess) return cuda_fail(c, e, "ordering the caller's stream");
     return LSKUM_OK;
@@ -2134,7 +2125,7 @@ lskum_status lskum_time_phases(lskum_ctx *c, int32_t reps, double *ms)
     c->hist_bound += reps;
     h.stop = h.error = 0;
     h.target = 0.0;
-    s = reset_cases(c, false, false);
+    s = reset_cases(c);
     if (s == LSKUM_OK) s = write_ctrl(c, h);
     if (s != LSKUM_OK) return s;
     cudaError_t e = cudaSuccess;
@@ -2458,17 +2449,11 @@ lskum_status ctx_state_written(lskum_ctx *c)
 // are cleared.  A norm that is not finite comes back as infinity.
 lskum_status ctx_case_norms(lskum_ctx *c, std::vector<double> &norms)
 {
-    Ctrl h{};
-    lskum_status s = read_ctrl(c, &h);
-    if (s == LSKUM_OK) s = reset_cases(c, true, true);
-    if (s != LSKUM_OK) return s;
-    h.it = 0;
-    h.stop = h.error = 0;
-    h.target = 0.0;
-    h.bad_point = 0x7fffffff;
-    s = write_ctrl(c, h);
-    if (s != LSKUM_OK) return s;
-    cudaError_t e = cudaSuccess;
+    auto clear = [&]() {
+        cudaError_t e = launch_reset_ctrl(c->ctrl, c->stream);
+        return e == cudaSuccess ? launch_accept_state(c->ctrl, true, c->stream) : e;
+    };
+    cudaError_t e = clear();
     for (int ph = 0; ph < 3 && e == cudaSuccess; ph++)
         e = launch_phase(c->dev, c->launch, c->cur, ph, c->n_levels, c->lvl_beg.data(), c->lvl_act_end.data(),
                          c->lvl_end.data(), c->stream);
@@ -2480,13 +2465,8 @@ lskum_status ctx_case_norms(lskum_ctx *c, std::vector<double> &norms)
     if (e != cudaSuccess) return cuda_fail(c, e, "residual norms");
     for (auto &x : norms)
         if (!std::isfinite(x)) x = INFINITY;
-    s = read_ctrl(c, &h);
-    if (s == LSKUM_OK) s = reset_cases(c, true, true);
-    if (s != LSKUM_OK) return s;
-    h.it = 0;
-    h.stop = h.error = 0;
-    h.bad_point = 0x7fffffff;
-    return write_ctrl(c, h);
+    e = clear();
+    return e == cudaSuccess ? LSKUM_OK : cuda_fail(c, e, "residual norms");
 }
 
 }  // namespace lskum

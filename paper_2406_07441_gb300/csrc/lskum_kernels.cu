@@ -2360,6 +2360,26 @@ __global__ void k_reset_ctrl(Ctrl *c)
     c->sweep_bar = 0;
 }
 
+// After the update that checked a new state: if it is a state, every case runs
+// again and failures are forgotten, with `history` as if newly created.
+__global__ void k_accept_state(Ctrl *c, bool history)
+{
+    if (c->error) return;
+    for (int b = threadIdx.x; b < c->n_cases; b += blockDim.x) {
+        c->case_state[b] = kRunning;
+        c->case_err[b] = 0;
+        c->case_bad[b] = 0x7f7f7f7f;
+        if (history) {
+            c->case_it[b] = 0;
+            c->case_hist0[b] = 0.0;
+        }
+    }
+    if (history && threadIdx.x == 0) {
+        c->it = 0;
+        c->target = 0.0;
+    }
+}
+
 __global__ void k_prep_run(Ctrl *c, double target)
 {
     c->stop = 0;
@@ -2717,6 +2737,12 @@ cudaError_t launch_init_math(cudaStream_t s)
 cudaError_t launch_prep_run(Ctrl *c, double target, cudaStream_t s)
 {
     k_prep_run<<<1, 1, 0, s>>>(c, target);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_accept_state(Ctrl *ctrl, bool history, cudaStream_t s)
+{
+    k_accept_state<<<1, 64, 0, s>>>(ctrl, history);
     return cudaGetLastError();
 }
 
