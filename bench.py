@@ -79,38 +79,32 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 # construction (the count depends on the mix of slots joining one or two
 # sub-stencils)
 RES_FLOPS_PER_SLOT = {MID_WORKLOAD: 336.07, SUPER_WORKLOAD: 336.07, PROF_WORKLOAD: 334.668, WORKLOAD: 334.668}
-# The current kernel runs exp and erfcx in fixed point and the split fluxes'
-# multiplications as correctly rounded integer multiplies on the integer
-# pipes, beside the FP64 unit; the FP64 flops it still executes on the FP64
-# unit per slot (ncu, the same counting; profiles/)
-RES_FP64_UNIT_FLOPS_PER_SLOT = {MID_WORKLOAD: 154.72, SUPER_WORKLOAD: 154.72, PROF_WORKLOAD: 154.67,
-                                WORKLOAD: 154.67}
+# The current kernel evaluates the split fluxes and their sums in 64-bit fixed
+# point on the integer pipes; the FP64 flops it still executes on the FP64
+# unit per slot (ncu, the same counting; profiles/): the reconstruction's 16
+# FMAs and what a point costs besides
+RES_FP64_UNIT_FLOPS_PER_SLOT = {MID_WORKLOAD: 36.74, SUPER_WORKLOAD: 36.74, PROF_WORKLOAD: 36.74, WORKLOAD: 36.74}
 START = 50  # first-order start-up iterations before warm-up and timing
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one residual
 # launch, from one ncu capture of the current kernel (profiles/), per
 # workload and threads per point; reported only for that launch shape and FP64
-RES_TRAFFIC = {MID_WORKLOAD: {1: 163.482624e6}, PROF_WORKLOAD: {1: 3.407065856e9},
-               WORKLOAD: {1: 14.584e9}}  # the last from a one-pass capture of the full-size launch
-# Unit utilisation of that launch (fraction of peak sustained, ncu): the FP64
-# pipe is the binding unit; the integer pipes (ALU, FMA-heavy: IMAD) carry
-# the fixed-point functions and the integer multiplies
-RES_UNITS_NCU = {MID_WORKLOAD: {"fp64_pipe": 0.8058, "alu_pipe": 0.3980, "fmaheavy_pipe": 0.3469, "issue": 0.4153},
-                 PROF_WORKLOAD: {"fp64_pipe": 0.8342, "alu_pipe": 0.4119, "fmaheavy_pipe": 0.3591,
-                                 "issue": 0.4282}}
+RES_TRAFFIC = {MID_WORKLOAD: {1: 178.356736e6}}
+# Unit utilisation of that launch (fraction of peak sustained, ncu): the
+# FMA-heavy pipe (32-bit multiplies into 64 bits) is the busiest unit, with
+# the latency of the integer chains at four warps per scheduler
+RES_UNITS_NCU = {MID_WORKLOAD: {"fp64_pipe": 0.4894, "alu_pipe": 0.3991, "fmaheavy_pipe": 0.6389, "issue": 0.4965}}
 RES_UNITS_NCU[SUPER_WORKLOAD] = RES_UNITS_NCU[MID_WORKLOAD]
-RES_UNITS_NCU[WORKLOAD] = RES_UNITS_NCU[PROF_WORKLOAD]
 ROOFLINE_NOTE = ("achieved counts the method's FP64 arithmetic as the all-FP64 form executes it "
-                 "(flops_per_active_slot); frac can exceed 1 because exp and erfcx run in 64-bit fixed point "
-                 "and the split fluxes' multiplications as correctly rounded integer multiplies on the integer "
-                 "pipes, beside the FP64 unit; fp64_unit gives the FP64 unit's own share and utilisation")
+                 "(flops_per_active_slot); frac exceeds 1 because the split fluxes and their sums run in 64-bit "
+                 "fixed point on the integer pipes; fp64_unit gives the FP64 unit's own share and utilisation")
 
 
 def _sweep_form(lanes):
     """What the library's sweep launch-shape value means."""
-    if lanes == 32:
-        return ("packed: each point's axis Jacobian products formed once and gathered, 4 lanes per "
-                "interior point, one lane per slot for wall points")
-    return f"{lanes} lanes per point, products per slot"
+    return ("both sweeps in one launch, each point's axis products formed once and gathered, 2 or 4 lanes per "
+            "interior point, one lane per slot for framed points, their Jacobians formed "
+            + ("beside the q-derivatives" if lanes == 32 else "by that launch")
+            + "; lists above 32 neighbours: one launch per level, products per slot")
 
 
 def _env_int(k, d):
@@ -866,8 +860,8 @@ def _memberships(cloud, kinetic=False):
 
 def _working_set_bytes(cloud):
     n, nnz = cloud.n, cloud.nnz
-    per_slot = 4 + 1 + 6 * 8
-    per_point = 8 * (2 * (4 + 4 + 20) + 4 * 4 + 4 + 1 + 4 + 4 + 13)
+    per_slot = 4 + 1 + 16 + 16 + 16 + 32
+    per_point = 8 * (2 * (4 + 4 + 4 + 24) + 3 * (8 + 8) + 16 + 4 + 2 + 4 + 4 + 14 + 6)
     return nnz * per_slot + n * per_point
 
 

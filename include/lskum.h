@@ -40,7 +40,8 @@ typedef enum {
     LSKUM_ERR_NONPOSITIVE = -3, /* an update produced rho <= 0, p <= 0 or a non-finite value */
     LSKUM_ERR_DIVERGED = -4,    /* the residual norm became non-finite */
     LSKUM_ERR_CUDA = -5,        /* a CUDA runtime call failed */
-    LSKUM_ERR_TIMEOUT = -6,     /* a bounded device wait gave up */
+    LSKUM_ERR_TIMEOUT = -6,     /* a bounded device wait gave up (the sweeps' level
+                                   boundaries, the network's products) */
     LSKUM_ERR_OOM = -7          /* device or host allocation failed */
 } lskum_status;
 
@@ -103,8 +104,8 @@ typedef struct {
  *                    q-derivatives (Eq. 16)
  *   jvp              LSKUM_JVP_EXACT or LSKUM_JVP_INCREMENT
  *   precision        0 = FP64 everywhere; 1 = mixed: the LU-SGS sweeps and
- *                    their Jacobian products in FP32, the residual (with
- *                    compensated neighbour sums), norm and update in FP64
+ *                    their Jacobian products in FP32, the residual (whose
+ *                    neighbour sums are exact), norm and update in FP64
  *   first_order_iters  iterations n <= first_order_iters (counted since the
  *                    last set_state / create) use the first-order residual
  *                    (q~ = q: no defect correction); a start-up aid, >= 0
@@ -329,19 +330,19 @@ lskum_status lskum_time_phases(lskum_ctx *ctx, int32_t reps, double *ms);
 /* Autotune the launch shape (no counterpart in the paper; the kernels'
  * results do not depend on it beyond the order of floating-point sums): for
  * every threads-per-point count {1,2,4,8} of the q-derivative and residual
- * kernels and lanes-per-point count {2,4,8} of the sweep kernels, plus the
- * packed sweep form (sweep_lanes = 32: each point forms the axis Jacobian
- * products of its new increment once and interior points gather their
- * neighbours' products, four lanes per interior point; wall points, and
- * outer points under the kinetic far field, form their products per slot in
- * their own frame, one lane per list slot with whole points packed into
- * warps; available when no point has more than 32 lower or upper
- * neighbours), re-capture
+ * kernels and every sweep form, re-capture
  * the iteration graphs, run one warm-up iteration and time `trial_iters`
  * iterations between CUDA events on the context's stream; keep the fastest
  * shape.  The state, the per-case counters, stop flags and histories are
  * saved before and restored after every trial, so the caller sees the
- * context as before, only faster.  Outputs (each may be NULL): the chosen
+ * context as before, only faster.  Sweep forms: where no point has more than
+ * 32 lower or upper neighbours, the packed form (both sweeps in one launch;
+ * each point forms the axis Jacobian products of its new increment once and
+ * interior points gather their neighbours' products; wall points, and outer
+ * points under the kinetic far field, take one lane per list slot in their own
+ * frame), with the framed points' Jacobians formed beside the q-derivatives
+ * (sweep_lanes = 32) or by the sweeps' launch (4); elsewhere one launch per
+ * level with 2, 4 or 8 lanes per point.  Outputs (each may be NULL): the chosen
  * threads per point, lanes per point and its mean device time per iteration
  * in ms.  Errors as lskum_run (the launch shape is then left unchanged). */
 lskum_status lskum_autotune(lskum_ctx *ctx, int32_t trial_iters, int32_t *tpp, int32_t *sweep_lanes,
@@ -349,9 +350,9 @@ lskum_status lskum_autotune(lskum_ctx *ctx, int32_t trial_iters, int32_t *tpp, i
 
 /* Set the launch shape directly (e.g. one found by lskum_autotune for the
  * same cloud earlier): tpp in {1, 2, 4, 8} threads per point of the
- * q-derivative and residual kernels, sweep_lanes in {2, 4, 8} lanes per point
- * of the sweep kernels or 32 for the packed form.  The iteration graphs are
- * re-captured.  Errors: LSKUM_ERR_ARG (other values, the packed form where
+ * residual kernel (the q-derivatives derive theirs from it), sweep_lanes as
+ * above (2, 4 and 8 are the same form where the packed form is available).
+ * The iteration graphs are re-captured.  Errors: LSKUM_ERR_ARG (other values, the packed form where
  * it is not available, or a run not waited for), LSKUM_ERR_CUDA. */
 lskum_status lskum_set_launch_shape(lskum_ctx *ctx, int32_t tpp, int32_t sweep_lanes);
 

@@ -6,9 +6,10 @@
 // it.  Constants: lskum_mathconst.h (gen_mathconst.py documents the methods
 // and their accuracy).  The tables are read per thread at diverging
 // indices, which would serialise constant-cache reads, so they live in
-// memory: the kernels that evaluate them at every point (the residual and
-// the update) stage a copy in shared memory; the sweeps, which need them
-// only at wall and outer points, read one global copy (g_math).
+// memory: the kernels that evaluate them at every point (the update, the
+// framed points' Jacobians, the increment products' base fluxes) stage a copy
+// in shared memory; the sweeps and the residual's FP64 fallback, which need
+// them at few points, read one global copy (g_math).
 #pragma once
 #include "lskum_fixmath.cuh"
 #include "lskum_intmul.cuh"
@@ -33,10 +34,8 @@ __device__ __forceinline__ void load_math_tables(MathTables &T)
 
 // exp(x) in fixed point on the integer pipes (lskum_fixmath.cuh): within
 // 0.51 ulp for |x| <= 100, 1 ulp up to 708, the library's exp beyond.  A
-// real call, not inlined: each of its call sites in the residual's slot
-// loop would otherwise carry ~80 instructions into a loop that already
-// strains the instruction cache (measured 2% faster out of line; erfcx and
-// split_E out of line measured slower).
+// real call, not inlined: each of its call sites would otherwise carry ~80
+// instructions into loops that already strain the instruction cache.
 __device__ __noinline__ double exp_t(const MathTables &T, double x)
 {
     return exp_fx<kExpShift>((const uint64_t *)T.exp2j, kExpFxC, kExpFxL, x);

@@ -3,31 +3,32 @@
 //   k_residual  defect-corrected kinetic split-flux residual (Eq. 11-15), local time
 //               step and scalar LU-SGS diagonal (Eq. 26, 33-34), density-norm partials
 //   k_norm_*    per-case residual norms, histories and stopping tests
-//   k_sweep     one colour level of the forward or backward LU-SGS sweep (Eq. 27) with
-//               exact (forward-mode AD) or increment (Eq. 28) Jacobian-vector products;
-//               k_sweep_packed: the same level with each point's axis products formed
-//               once and gathered by its neighbours
+//   k_sweeps    all levels of the forward and the backward LU-SGS sweep (Eq. 27) in
+//               one cooperative launch, with exact (forward-mode AD) or increment
+//               (Eq. 28) Jacobian-vector products, each point's axis products formed
+//               once and gathered by its neighbours; k_sweep: one level with the
+//               products formed per slot, where lists are too long for the packed form
 //   k_update    U += dU, wall projection, q-variables and the per-point primal
 //               quantities the next iteration's sweeps need
 //
-// GB300 has 62x more FP32 than FP64 throughput (1.2 FP64 TFLOP/s measured), so
-// the FP64 path is bound by FP64 instruction issue, not HBM.  The kernels are
-// shaped to issue as few FP64 instructions as possible: every geometric
-// quantity (LS weights, frames, stencil membership) is precomputed per
-// neighbour slot; the inverse of Eq. 14 uses beta^(-5/2) instead of a log;
-// the sweeps' Jacobian products reuse erf/exp of each point's own state,
-// computed once per iteration by k_update, so an exact product has no
-// transcendental call at all, and a neighbour's product along an axis is
-// formed once and gathered; exp and A = (1 + s erf S)/2 are the kernels' own
-// (lskum_fastmath.cuh), which share exp(-S^2) and keep index work off the
-// FP64 pipe, as are signs and multiplications by 2 and 1/2 (integer steps).
-// exp and erfcx run in fixed point on the integer pipes (lskum_fixmath.cuh),
-// and the multiplications of the split fluxes and of the update on the
-// integer pipes too (mul_i, lskum_intmul.cuh: correctly rounded, the same
-// bits), which leaves the FP64 unit the fused multiply-adds, the additions
-// and the multiplications on the residual's critical path (q to primitives);
-// the sweeps, bound by the latency of their dependent chains rather than by
-// FP64 issue, keep the FP64 multiply.
+// GB300 has 62x more FP32 than FP64 throughput (1.2 FP64 TFLOP/s measured),
+// and an SM's FP64 unit takes one warp instruction in 19 cycles, its integer
+// pipes one in 1 or 2 (a 32-bit multiply-add into 64 bits in 4.5).  So the
+// kernels that evaluate formulas per neighbour slot, the q-derivatives and the
+// residual, run in 64-bit fixed point on the integer pipes (lskum_fixgrad.cuh,
+// lskum_fixflux.cuh), with sums that are exact integers, and fall back to FP64
+// where a state leaves the fixed-point ranges.  The sweeps, whose increments
+// have no fixed range, stay in FP64 (or FP32) and issue few FP64
+// instructions: every geometric quantity is precomputed per slot; the exact
+// Jacobian products reuse erf and exp of each point's own state, computed once
+// per iteration by k_update, so they have no transcendental call at all, and a
+// neighbour's product along an axis is formed once and gathered.  Where FP64
+// evaluates the split fluxes (the fallback, the update, the framed
+// Jacobians, the increment products), exp and A = (1 + s erf S)/2 are the
+// kernels' own (lskum_fastmath.cuh: fixed point, exp(-S^2) shared), as are
+// signs and multiplications by 2 and 1/2 (integer steps) and, off the critical
+// paths, multiplications (mul_i, lskum_intmul.cuh: correctly rounded, the same
+// bits).
 #include "lskum_internal.h"
 
 #include <cstdint>
