@@ -6,10 +6,10 @@
 // it.  Constants: lskum_mathconst.h (gen_mathconst.py documents the methods
 // and their accuracy).  The tables are read per thread at diverging
 // indices, which would serialise constant-cache reads, so they live in
-// memory: the kernels that evaluate them at every point (the update, the
+// memory: kernels with several evaluations per thread's point and item (the
 // framed points' Jacobians, the increment products' base fluxes) stage a copy
-// in shared memory; the sweeps and the residual's FP64 fallback, which need
-// them at few points, read one global copy (g_math).
+// in shared memory; the update, the sweeps and the residual's FP64 fallback
+// read one global copy (g_math).
 #pragma once
 #include "lskum_fixmath.cuh"
 #include "lskum_intmul.cuh"
