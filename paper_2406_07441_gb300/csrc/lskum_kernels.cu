@@ -480,16 +480,35 @@ __device__ __forceinline__ void load4(const float *__restrict__ p, float v[4])
     v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
 }
 
-// The same from L2: values that other blocks write within the launch.
+// The same, and single values, of what other blocks write within the launch:
+// ordinary coherent loads from L2, kept behind the level boundary whose
+// acquire orders them (volatile, with a memory clobber: the compiler moves
+// none of them across it, and takes none of them for read-only data).
 __device__ __forceinline__ void load4_l2(const double *p, double v[4])
 {
-    const double2 a = __ldcg(reinterpret_cast<const double2 *>(p)), b = __ldcg(reinterpret_cast<const double2 *>(p) + 1);
-    v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+    asm volatile("ld.global.cg.v4.f64 {%0, %1, %2, %3}, [%4];"
+                 : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3])
+                 : "l"(p)
+                 : "memory");
 }
 __device__ __forceinline__ void load4_l2(const float *p, float v[4])
 {
-    const float4 a = __ldcg(reinterpret_cast<const float4 *>(p));
-    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                 : "l"(p)
+                 : "memory");
+}
+__device__ __forceinline__ double load_l2(const double *p)
+{
+    double v;
+    asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float load_l2(const float *p)
+{
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
 }
 
 __device__ __forceinline__ void store4(double *p, const double v[4])
@@ -1344,7 +1363,7 @@ __device__ __forceinline__ void sweep_point(bool FWD, const Dev &d, const StateS
         for (int c = 0; c < 4; c++) w[c] = -((T)rhs[c] + acc[c]) * iD;
     } else {
 #pragma unroll
-        for (int c = 0; c < 4; c++) w[c] = fma(-acc[c], iD, __ldcg(sb.dUs + 4 * k + c));
+        for (int c = 0; c < 4; c++) w[c] = fma(-acc[c], iD, load_l2(sb.dUs + 4 * (size_t)k + c));
     }
     if (wall) {
         const T nx = (T)d.wnx[k], ny = (T)d.wny[k];
@@ -1555,9 +1574,11 @@ constexpr int kErrTimeout = -6;  // LSKUM_ERR_TIMEOUT
 // blocks are resident).  The arrivals are counted in ctrl->sweep_bar; the
 // launch's last one (number `limit`) wraps it to 0 for the next launch.  The
 // block's last warp arrives and polls for it.  The arrival releases the
-// block's stores to L2; there is no acquiring fence, which would empty L1 of
-// what was loaded ahead: values that other blocks write are read from L2
-// (load4_l2, cp_async16), never from L1.
+// block's stores (the barrier before it orders them all before the one
+// thread's release).  The poll is relaxed; the load that follows it acquires
+// what the arrivals released, and the barrier behind it hands that on to the
+// block's other threads.  The acquire empties L1; what was loaded ahead for a
+// warp's first task of the level lies in registers and shared memory.
 __device__ __forceinline__ void boundary_arrive(Ctrl *c, uint32_t limit)
 {
     __syncthreads();
@@ -1576,7 +1597,11 @@ __device__ __forceinline__ bool boundary_wait(Ctrl *c, uint32_t target, uint32_t
         int ok = 1;
         for (uint32_t tries = 1;; tries++) {
             const uint32_t v = *bar;
-            if (target == limit ? v == 0 : v >= target) break;
+            if (target == limit ? v == 0 : v >= target) {
+                uint32_t seen;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&c->sweep_bar) : "memory");
+                break;
+            }
             if ((tries & 1023) == 0) {
                 uint64_t now;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
@@ -1776,7 +1801,7 @@ __device__ __forceinline__ void sweep_interior(const Dev &d, const StateSet &st,
     }
     if (live && !fwd)
 #pragma unroll
-        for (int c = 0; c < C; c++) dus[c] = __ldcg(sb.dUs + 4 * (size_t)k + C * s + c);
+        for (int c = 0; c < C; c++) dus[c] = load_l2(sb.dUs + 4 * (size_t)k + C * s + c);
 #pragma unroll
     for (int r = 0; r < kRows; r++) {
         if (r >= a.rows) break;
@@ -1893,7 +1918,7 @@ __device__ __forceinline__ void framed_load(const Dev &d, int dir, int fw, int l
     a.steps = d.pk_steps[dir][fw];
     const T *M = (sizeof(T) == 4 ? (const T *)d.pk_jmf[dir] : (const T *)d.pk_jm[dir]) + 16 * e;
 #pragma unroll
-    for (int c = 0; c < 4; c++) load4(M + 4 * c, a.M + 4 * c);
+    for (int c = 0; c < 4; c++) load4_l2(M + 4 * c, a.M + 4 * c);
     const unsigned m = __match_any_sync(kFull, a.k);
     a.head = __ffs(m) - 1;
     a.seg = __popc(m);
@@ -1906,7 +1931,7 @@ __device__ __forceinline__ void framed_load(const Dev &d, int dir, int fw, int l
     if (a.r < 4) {
         const T *F = axis_jacobians<T>(d, a.f) + 16 * a.r;
 #pragma unroll
-        for (int c = 0; c < 4; c++) load4(F + 4 * c, a.F + 4 * c);
+        for (int c = 0; c < 4; c++) load4_l2(F + 4 * c, a.F + 4 * c);
     }
     if (a.r == 0) {
         a.iD = (T)d.iD[k];
@@ -1984,7 +2009,7 @@ __device__ __forceinline__ void framed_run(const Dev &d, const SweepBufs<T> &sb,
         const T *F = axis_jacobians<T>(d, a.f) + 16 * cb;
         T Fc[16];
 #pragma unroll
-        for (int c = 0; c < 4; c++) load4(F + 4 * c, Fc + 4 * c);
+        for (int c = 0; c < 4; c++) load4_l2(F + 4 * c, Fc + 4 * c);
         mat_vec(Fc, w, J);
         store4(sb.jc + 16 * (size_t)k + 4 * cb, J);
     }
@@ -2017,7 +2042,7 @@ __device__ __noinline__ void sweep_framed(const Dev &d, const StateSet &st, cons
 #pragma unroll
             for (int c = 0; c < 4; c++) {
                 T Mc[4];
-                load4(M + 4 * c, Mc);
+                load4_l2(M + 4 * c, Mc);
 #pragma unroll
                 for (int j = 0; j < 4; j++) acc[c] = fma(Mc[j], dl[j], acc[c]);
             }
@@ -2075,7 +2100,7 @@ __device__ __noinline__ void sweep_framed(const Dev &d, const StateSet &st, cons
 #pragma unroll
             for (int c = 0; c < 4; c++) {
                 T Fc[4];
-                load4(F + 16 * cb + 4 * c, Fc);
+                load4_l2(F + 16 * cb + 4 * c, Fc);
                 J[c] = Fc[0] * w[0];
 #pragma unroll
                 for (int j = 1; j < 4; j++) J[c] = fma(Fc[j], w[j], J[c]);
