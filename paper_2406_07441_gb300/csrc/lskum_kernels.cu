@@ -2534,7 +2534,10 @@ cudaError_t launch_sweeps(const Dev &d, const Launch &L, int cur, int n_levels, 
     void *args[] = {&dd, &st, &n_levels, &dirs, &fuse};
     const size_t smem = (size_t)(L.sw_threads / 32) * sizeof(WarpStage<T>);
     const void *kernel = (const void *)k_sweeps<JVP, T>;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (the kernel's limit is the process's: always the largest block's, so that
+    // contexts of other sizes in other threads set the same)
+    constexpr int most = kSweepBlock / 32 * (int)sizeof(WarpStage<T>);
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return e;
     return cudaLaunchCooperativeKernel(kernel, dim3(L.sw_blocks), dim3(L.sw_threads), args, smem, s);
 }
