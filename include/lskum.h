@@ -283,7 +283,9 @@ lskum_status lskum_set_conserved(lskum_ctx *ctx, const double *U);
  * iterations.  iters_done (may be NULL) receives the number of iterations run.
  * Errors: LSKUM_ERR_NONPOSITIVE (an update produced a non-physical state; the
  * state of the last good iteration is kept), LSKUM_ERR_DIVERGED,
- * LSKUM_ERR_ARG, LSKUM_ERR_CUDA.
+ * LSKUM_ERR_TIMEOUT (the state of the last complete iteration is kept, the
+ * increments are zero as after lskum_set_conserved, and the iteration and its
+ * norm are not counted), LSKUM_ERR_ARG, LSKUM_ERR_CUDA.
  */
 lskum_status lskum_run(lskum_ctx *ctx, int32_t max_iters, double target_drop, int32_t *iters_done);
 
@@ -355,6 +357,15 @@ lskum_status lskum_autotune(lskum_ctx *ctx, int32_t trial_iters, int32_t *tpp, i
  * The iteration graphs are re-captured.  Errors: LSKUM_ERR_ARG (other values, the packed form where
  * it is not available, or a run not waited for), LSKUM_ERR_CUDA. */
 lskum_status lskum_set_launch_shape(lskum_ctx *ctx, int32_t tpp, int32_t sweep_lanes);
+
+/* Failure-path test of the bounded wait at the sweeps' level boundaries: with
+ * skip_arrival = 1 the first block of the sweeps' launch does not arrive, so
+ * a run reports LSKUM_ERR_TIMEOUT after the limit; 0 restores the normal
+ * launch.  wait_limit_s in [1e-4, 10] (2 in a new context) is the limit of
+ * each wait.  (Lists too long for the packed form: no such wait.)  The
+ * iteration graphs are re-captured.  Errors: LSKUM_ERR_ARG (other values, or
+ * a run not waited for), LSKUM_ERR_CUDA. */
+lskum_status lskum_set_wait_test(lskum_ctx *ctx, int32_t skip_arrival, double wait_limit_s);
 
 /* Number of points, of colours and of kernel launches one iteration makes. */
 lskum_status lskum_get_info(lskum_ctx *ctx, int32_t *n_points, int32_t *n_colours, int32_t *launches_per_iter);

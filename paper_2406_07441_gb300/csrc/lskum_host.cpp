@@ -1400,6 +1400,8 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     d.gb = dgb;
     d.ctrl = c->ctrl;
     d.case_state = c->case_state;
+    d.sweep_wait_ns = 2000000000ull;
+    d.sweep_skip = 0;
     d.blk_pos = dblk_pos;
     d.blk_case = dblk_case;
     d.case_blk = dcase_blk;
@@ -1685,6 +1687,19 @@ lskum_status reset_cases(lskum_ctx *c)
     return e == cudaSuccess ? LSKUM_OK : cuda_fail(c, e, "resetting the cases");
 }
 
+// After sweeps that gave up waiting (LSKUM_ERR_TIMEOUT): the increments, partly
+// written, restart from zero as for a new state, and the iteration that did
+// not happen is not counted.
+lskum_status forget_iteration(lskum_ctx *c, Ctrl &h)
+{
+    cudaError_t e = cudaMemsetAsync(c->dev.dU, 0, 4 * (size_t)c->ld * sizeof(double), c->stream);
+    if (e == cudaSuccess && c->dev.dUf)
+        e = cudaMemsetAsync(c->dev.dUf, 0, 4 * (size_t)c->ld * sizeof(float), c->stream);
+    if (e != cudaSuccess) return cuda_fail(c, e, "clearing the increments");
+    h.it -= 1;
+    return write_ctrl(c, h);
+}
+
 lskum_status read_case_arrays(lskum_ctx *c, std::vector<int32_t> *state, std::vector<int32_t> *it)
 {
     cudaError_t e = cudaSuccess;
@@ -1864,8 +1879,12 @@ lskum_status lskum_wait(lskum_ctx *c, int32_t *iters_done)
     if (h.error == LSKUM_ERR_DIVERGED)
         return fail(c, LSKUM_ERR_DIVERGED, "residual norm of case %d not finite in iteration %d", -1 - h.bad_point,
                     h.it);
-    if (h.error == LSKUM_ERR_TIMEOUT)
-        return fail(c, LSKUM_ERR_TIMEOUT, "the sweeps' blocks did not meet within their time limit in iteration %d", h.it);
+    if (h.error == LSKUM_ERR_TIMEOUT) {
+        const int32_t it = h.it;
+        s = forget_iteration(c, h);
+        if (s != LSKUM_OK) return s;
+        return fail(c, LSKUM_ERR_TIMEOUT, "the sweeps' blocks did not meet within their time limit in iteration %d", it);
+    }
     if (h.error) return fail(c, LSKUM_ERR_CUDA, "device error %d", h.error);
     return LSKUM_OK;
 }
@@ -2135,10 +2154,9 @@ lskum_status lskum_time_phases(lskum_ctx *c, int32_t reps, double *ms)
     double acc[6] = {0, 0, 0, 0, 0, 0};
     const Dev &d = c->dev;
     for (int32_t r = 0; r < reps && e == cudaSuccess; r++) {
-        const int cur = c->cur;
         for (int ph = 0; ph < 6 && e == cudaSuccess; ph++) {
             e = cudaEventRecord(ev[ph], c->stream);
-            if (e == cudaSuccess) e = launch_phase(d, c->launch, cur, ph, c->n_levels, c->lvl_beg.data(),
+            if (e == cudaSuccess) e = launch_phase(d, c->launch, (c->cur + r) & 1, ph, c->n_levels, c->lvl_beg.data(),
                                                    c->lvl_act_end.data(), c->lvl_end.data(), c->stream);
         }
         if (e == cudaSuccess) e = cudaEventRecord(ev[6], c->stream);
@@ -2148,17 +2166,27 @@ lskum_status lskum_time_phases(lskum_ctx *c, int32_t reps, double *ms)
             e = cudaEventElapsedTime(&t, ev[ph], ev[ph + 1]);
             acc[ph] += t;
         }
-        c->cur ^= 1;
     }
     for (auto &x : ev) cudaEventDestroy(x);
     if (e != cudaSuccess) return cuda_fail(c, e, "timing phases");
     Ctrl h2{};
     s = read_ctrl(c, &h2);
     if (s != LSKUM_OK) return s;
-    if (h2.error) {
-        c->cur ^= 1;
-        return fail(c, (lskum_status)h2.error, "iteration failed while timing phases");
+    // (iterations started; of a failed one the update was not applied, and the
+    // rest did nothing)
+    const int32_t done = h2.it - h.it - (h2.error ? 1 : 0);
+    c->cur = (c->cur + done) & 1;
+    if (h2.error == LSKUM_ERR_TIMEOUT) {  // (here the norm came before the sweeps)
+        std::vector<int32_t> now;
+        s = read_case_arrays(c, nullptr, &now);
+        for (int32_t b = 0; b < c->n_cases && s == LSKUM_OK; b++) now[b] = std::min(now[b], its[b] + done);
+        if (s == LSKUM_OK) {
+            e = cudaMemcpyAsync(c->case_it, now.data(), c->n_cases * sizeof(int32_t), cudaMemcpyHostToDevice, c->stream);
+            s = e == cudaSuccess ? forget_iteration(c, h2) : cuda_fail(c, e, "timing phases");
+        }
+        if (s != LSKUM_OK) return s;
     }
+    if (h2.error) return fail(c, (lskum_status)h2.error, "iteration failed while timing phases");
     for (int ph = 0; ph < 6; ph++) ms[ph] = acc[ph] / reps;
     return LSKUM_OK;
 }
@@ -2310,6 +2338,17 @@ lskum_status lskum_set_host_io(lskum_ctx *c, int32_t direct)
         return fail(c, LSKUM_ERR_ARG, "the device cannot access pageable host memory directly");
     c->host_direct = direct == 1;
     return LSKUM_OK;
+}
+
+lskum_status lskum_set_wait_test(lskum_ctx *c, int32_t skip_arrival, double wait_limit_s)
+{
+    if (!c) return LSKUM_ERR_ARG;
+    if ((skip_arrival != 0 && skip_arrival != 1) || !(wait_limit_s >= 1e-4 && wait_limit_s <= 10.0))
+        return fail(c, LSKUM_ERR_ARG, "skip_arrival must be 0 or 1, wait_limit_s in [1e-4, 10]");
+    if (c->pending) return fail(c, LSKUM_ERR_ARG, "an enqueued run has not been waited for");
+    c->dev.sweep_skip = skip_arrival;
+    c->dev.sweep_wait_ns = (uint64_t)(wait_limit_s * 1e9);
+    return build_graphs(c);
 }
 
 lskum_status lskum_get_host_io(lskum_ctx *c, int32_t *direct, int32_t *supported)

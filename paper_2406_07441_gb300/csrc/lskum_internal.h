@@ -210,6 +210,10 @@ struct Dev {
     Ctrl *ctrl;
     int32_t *suspect;        // [n_cases] 1: a residual that can make the norm non-finite
     const int32_t *case_state;  // = ctrl->case_state (read per point)
+    // the sweeps' launch: time limit of the wait at a level boundary, and 1 to
+    // leave out the first block's arrivals (lskum_set_wait_test)
+    uint64_t sweep_wait_ns;
+    int32_t sweep_skip;
     // options
     double cfl, ramp, u_inf[4];
     int32_t K, jvp;

@@ -46,6 +46,8 @@ constexpr double kInv2SqrtPi = 0.28209479177387814347;    // 1 / (2 sqrt(pi))
 constexpr double kInvSqrtPi = 0.56418958354775628695;     // 1 / sqrt(pi)
 constexpr unsigned kFull = 0xffffffffu;
 
+constexpr int kErrTimeout = -6;  // LSKUM_ERR_TIMEOUT: the sweeps' wait at a level boundary
+
 // Every kernel returns at once after a stop or a failure (the norm goes by
 // what k_begin found: it records the iteration that fails).  When a case
 // reaches its drop target, k_norm marks it kReachedTarget, so the sweeps and
@@ -58,6 +60,14 @@ __device__ __forceinline__ bool halted(const Ctrl *c)
 {
     const volatile Ctrl *v = c;
     return (v->stop | v->error) != 0;
+}
+
+// Does this iteration's norm count?  (Not if the sweeps before it gave up
+// waiting for one another: the iteration did not happen.)
+__device__ __forceinline__ bool counted(const Ctrl *c)
+{
+    const volatile Ctrl *v = c;
+    return v->live && v->error != kErrTimeout;
 }
 
 // Is point k's case stopped?  (Only batches have cases that stop while
@@ -1135,7 +1145,7 @@ __global__ void __launch_bounds__(kResBlock<TPP>, 512 / kResBlock<TPP>)
 __global__ void __launch_bounds__(256) k_norm_partials(Dev d)
 {
     __shared__ double red[4][8];
-    if (!((const volatile Ctrl *)d.ctrl)->live) return;
+    if (!counted(d.ctrl)) return;
     const int j = blockIdx.x;
     const int p = d.blk_pos[j] + threadIdx.x;
     double t[4] = {0.0, 0.0, 0.0, 0.0};
@@ -1170,7 +1180,7 @@ __global__ void __launch_bounds__(256) k_norm_partials(Dev d)
 __global__ void __launch_bounds__(256) k_norm_cases(Dev d)
 {
     __shared__ double red[4][8];
-    if (!((const volatile Ctrl *)d.ctrl)->live) return;
+    if (!counted(d.ctrl)) return;
     const int b = blockIdx.x;
     Ctrl *c = d.ctrl;
     if (frozen_state(((volatile int32_t *)c->case_state)[b])) return;  // block-uniform
@@ -1564,10 +1574,6 @@ __global__ void __launch_bounds__(256) k_framed_jac(Dev d, StateSet st)
 // the FP64 unit busy, and 255 registers hold what is loaded ahead.
 constexpr int kSweepBlock = 256;
 
-// Time limit of the wait at a level boundary, and the status reported past it.
-constexpr uint64_t kSweepWaitNs = 2000000000ull;
-constexpr int kErrTimeout = -6;  // LSKUM_ERR_TIMEOUT
-
 // A level boundary in two halves: every thread of a block arrives, then (after
 // work that needs nothing of the other blocks) waits until all blocks of the
 // launch have arrived with their stores visible (cooperative launch: all
@@ -1579,16 +1585,16 @@ constexpr int kErrTimeout = -6;  // LSKUM_ERR_TIMEOUT
 // what the arrivals released, and the barrier behind it hands that on to the
 // block's other threads.  The acquire empties L1; what was loaded ahead for a
 // warp's first task of the level lies in registers and shared memory.
-__device__ __forceinline__ void boundary_arrive(Ctrl *c, uint32_t limit)
+__device__ __forceinline__ void boundary_arrive(Ctrl *c, uint32_t limit, bool skip)
 {
     __syncthreads();
-    if (threadIdx.x == blockDim.x - 32) {
+    if (threadIdx.x == blockDim.x - 32 && !skip) {
         asm volatile("red.release.gpu.global.inc.u32 [%0], %1;" ::"l"(&c->sweep_bar), "r"(limit - 1) : "memory");
     }
 }
 
 // False past the time limit.
-__device__ __forceinline__ bool boundary_wait(Ctrl *c, uint32_t target, uint32_t limit)
+__device__ __forceinline__ bool boundary_wait(Ctrl *c, uint32_t target, uint32_t limit, uint64_t wait_ns)
 {
     __shared__ int reached;
     if (threadIdx.x == blockDim.x - 32) {
@@ -1606,7 +1612,7 @@ __device__ __forceinline__ bool boundary_wait(Ctrl *c, uint32_t target, uint32_t
                 uint64_t now;
                 asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
                 if (t0 == 0) t0 = now;
-                if (now - t0 > kSweepWaitNs) {
+                if (now - t0 > wait_ns) {
                     atomicExch(&c->error, kErrTimeout);
                     ok = 0;
                     break;
@@ -2180,7 +2186,7 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_sweeps(Dev d, StateSet st, i
             }
         }
         if (step + 1 < steps) {
-            boundary_arrive(d.ctrl, limit);
+            boundary_arrive(d.ctrl, limit, d.sweep_skip && blockIdx.x == 0);
             const int dir = dirs == 3 ? (step + 1 < n_levels ? 0 : 1) : dirs - 1;
             const int l = dir == 0 ? step + 1 : steps - 2 - step;
             const int wb = d.lvl_fw[dir][l], wf = d.lvl_fw[dir][l + 1] - wb;
@@ -2197,7 +2203,10 @@ __global__ void __launch_bounds__(kSweepBlock, 1) k_sweeps(Dev d, StateSet st, i
                 ready = true;
             }
             target += gridDim.x;
-            if (!boundary_wait(d.ctrl, target, limit)) return;
+            if (!boundary_wait(d.ctrl, target, limit, d.sweep_wait_ns)) {
+                cp_async_wait<0>();  // what was loaded ahead
+                return;
+            }
         }
     }
 }

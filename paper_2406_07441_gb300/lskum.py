@@ -86,6 +86,7 @@ def load():
     L.lskum_get_host_io.argtypes = [vp, vp, vp]
     L.lskum_set_start_iters.argtypes = [vp, i32]
     L.lskum_set_launch_shape.argtypes = [vp, i32, i32]
+    L.lskum_set_wait_test.argtypes = [vp, i32, d]
     u64 = C.c_uint64
     L.lskum_mlp_n_params.argtypes = []
     L.lskum_mlp_n_params.restype = i32
@@ -115,7 +116,7 @@ def load():
               "lskum_get_info", "lskum_time_phases", "lskum_density_norm_noalloc", "lskum_selftest_fpint",
               "lskum_batch_create",
               "lskum_get_case_residuals", "lskum_get_case_residuals4", "lskum_get_case_forces", "lskum_get_case_info", "lskum_autotune",
-              "lskum_get_wall_distance", "lskum_validate", "lskum_set_start_iters", "lskum_get_field_dev", "lskum_set_conserved_dev", "lskum_set_launch_shape",
+              "lskum_get_wall_distance", "lskum_validate", "lskum_set_start_iters", "lskum_get_field_dev", "lskum_set_conserved_dev", "lskum_set_launch_shape", "lskum_set_wait_test",
               "lskum_set_host_io", "lskum_get_host_io", "lskum_mlp_create", "lskum_mlp_get_params",
               "lskum_mlp_set_params", "lskum_mlp_features", "lskum_mlp_forward", "lskum_mlp_loss_grads",
               "lskum_mlp_adam", "lskum_mlp_add_samples", "lskum_mlp_time_forward", "lskum_mlp_n_samples", "lskum_mlp_train",
@@ -354,6 +355,10 @@ class Solver:
 
     def set_launch_shape(self, tpp, sweep_lanes):
         self._check(load().lskum_set_launch_shape(self._h, int(tpp), int(sweep_lanes)))
+
+    def set_wait_test(self, skip_arrival, wait_limit_s=2.0):
+        """Failure-path test of the sweeps' bounded wait (see lskum_set_wait_test)."""
+        self._check(load().lskum_set_wait_test(self._h, int(skip_arrival), float(wait_limit_s)))
 
     def set_host_io(self, direct):
         """1: host arrays straight to / from the device's reorder kernels
