@@ -1031,6 +1031,8 @@ __global__ void __launch_bounds__(kResBlock<TPP>, 512 / kResBlock<TPP>)
         const bool framed = fl != kInterior;  // (t, n) frame: wall and kinetic outer points
         FxSum acc[4] = {};
         uint32_t bad = 0;
+        const double *pr = st.prim + (size_t)kk * kPrimStride;
+        const uint32_t sh = fx_shift((uint32_t)__double2hiint(pr[P_RHO]), (uint32_t)__double2hiint(pr[P_ISB]));
         if (work) {
             double q0[4], gx0[4], gy0[4];
             load4(q + 4 * (size_t)kk, q0);
@@ -1071,8 +1073,8 @@ __global__ void __launch_bounds__(kResBlock<TPP>, 512 / kResBlock<TPP>)
                     q0t[2] = fma(b, e2x, q0t[2] * e2y);
                 }
                 FxState si, s0;
-                fx_state(T, qi[0], qi[1], qi[2], qi[3], si, bad);
-                fx_state(T, q0t[0], q0t[1], q0t[2], q0t[3], s0, bad);
+                fx_state(T, qi[0], qi[1], qi[2], qi[3], si, bad, sh);
+                fx_state(T, q0t[0], q0t[1], q0t[2], q0t[3], s0, bad, sh);
                 if (m & 3) {
                     const bool pos = m & 1;
                     FxFlux Gi, G0;
@@ -1106,7 +1108,7 @@ __global__ void __launch_bounds__(kResBlock<TPP>, 512 / kResBlock<TPP>)
             acc[c].l = group_sum<TPP>(acc[c].l);
             acc[c].r = group_sum<TPP>(acc[c].r);
         }
-        const double wsc = d.geo[G_WSC * ld + kk];
+        const double wsc = d.geo[G_WSC * ld + kk] * pow2(-(int)sh);
         R[0] = fx_total(acc[0]) * (wsc * 0x1p-27);
         R[3] = fx_total(acc[3]) * (wsc * 0x1p-23);
         const double Ra = fx_total(acc[1]) * (wsc * 0x1p-25), Ro = fx_total(acc[2]) * (wsc * 0x1p-25);
