@@ -105,7 +105,8 @@ typedef struct {
  *   jvp              LSKUM_JVP_EXACT or LSKUM_JVP_INCREMENT
  *   precision        0 = FP64 everywhere; 1 = mixed: the LU-SGS sweeps and
  *                    their Jacobian products in FP32, the residual (whose
- *                    neighbour sums are exact), norm and update in FP64
+ *                    neighbour sums are exact, or compensated at points
+ *                    outside the fixed-point ranges), norm and update in FP64
  *   first_order_iters  iterations n <= first_order_iters (counted since the
  *                    last set_state / create) use the first-order residual
  *                    (q~ = q: no defect correction); a start-up aid, >= 0

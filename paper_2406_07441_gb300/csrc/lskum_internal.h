@@ -218,7 +218,7 @@ struct Dev {
     double cfl, ramp, u_inf[4];
     int32_t K, jvp;
     int32_t first_order;  // iterations n <= first_order use q~ = q
-    int32_t precision;    // 0 FP64; 1 FP32 sweeps, compensated FP64 residual sums
+    int32_t precision;    // 0 FP64; 1 FP32 sweeps (residual sums exact, compensated where FP64 forms them)
     int32_t scheme;       // 0 implicit LU-SGS; 1 explicit (forward Euler, no sweeps)
     int32_t lusgs;        // 0 Anandhanarayanan's diagonal; 1 the revised form of Manish et al.
     int32_t farfield;     // 0 outer points frozen at the free stream; 1 the kinetic far field

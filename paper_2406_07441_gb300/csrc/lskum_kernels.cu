@@ -835,9 +835,21 @@ __device__ __forceinline__ void reconstruct(const double q[4], const double x[4]
     }
 }
 
+// R += y with Kahan's compensated summation (W. Kahan, "Further remarks on
+// reducing truncation errors", CACM 8(1), 1965): c carries the negated
+// rounding error of the running sum into the next term.
+__device__ __forceinline__ void comp_add(double &R, double &c, double y)
+{
+    const double t = R + y;
+    c = (t - R) - y;  // what the addition lost (negated)
+    R = t;
+}
+
 // The slots sub, sub + TPP, ... of point k in FP64, for points of which a
 // state lies outside the fixed-point ranges (hypersonic, very hot or very
-// dense states, non-finite ones); the group's lanes add their sums.
+// dense states, non-finite ones); the group's lanes add their sums.  In mixed
+// precision the sums are compensated: the terms of a group of four slots, by
+// FMAs, less the error carried so far, enter R by one compensated addition.
 template <int TPP>
 __device__ __noinline__ void residual_fp64(const Dev &d, const double *__restrict__ q, const double *__restrict__ g,
                                            int k, int sub, bool second, double R[4])
@@ -852,10 +864,12 @@ __device__ __noinline__ void residual_fp64(const Dev &d, const double *__restric
     load4(q + 4 * (size_t)k, q0);
     load4(g + 8 * (size_t)k, gx0);
     load4(g + 8 * (size_t)k + 4, gy0);
+    double y[4] = {0.0, 0.0, 0.0, 0.0}, carry[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
     for (int c = 0; c < 4; c++) R[c] = 0.0;
     const int deg = d.deg[k];
     const int base = d.slice_off[k >> 5] + (k & 31);
+    int ng = 0;  // slots in the current group
     for (int j = sub; j < deg; j += TPP) {
         const int e = base + 32 * j;
         const int mb = d.memb[e];
@@ -881,8 +895,21 @@ __device__ __noinline__ void residual_fp64(const Dev &d, const double *__restric
             split_flux(T, Pi, framed, xdir, dx, dy, pos, Gi);
             split_flux(T, P0, framed, xdir, dx, dy, pos, G0);
 #pragma unroll
-            for (int c = 0; c < 4; c++) R[c] = fma(w, Gi[c] - G0[c], R[c]);
+            for (int c = 0; c < 4; c++) y[c] = fma(w, Gi[c] - G0[c], y[c]);
         }
+        if (d.precision && ++ng == 4) {
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                comp_add(R[c], carry[c], y[c]);
+                y[c] = -carry[c];
+            }
+            ng = 0;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+        if (d.precision && ng > 0) comp_add(R[c], carry[c], y[c]);
+        R[c] = d.precision ? R[c] - carry[c] : y[c];
     }
 }
 
