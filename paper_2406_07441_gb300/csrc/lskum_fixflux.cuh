@@ -119,6 +119,14 @@ LSKUM_HD uint32_t fx_shift(uint32_t rho, uint32_t isb)
     return e >= -1 ? 0u : (e < -25 ? 24u : (uint32_t)(-1 - e));
 }
 
+// Do q-variables with these high words lie outside fx_state's ranges?
+// (-4 < z3 < -0.5 (1 + 2^-10); |z1|, |z2| < 4; |z0| < 16)
+LSKUM_HD bool fx_outside(uint32_t h0, uint32_t h1, uint32_t h2, uint32_t h3)
+{
+    return !(h3 - 0xbfe00400u < 0xc0100000u - 0xbfe00400u) | ((h1 & 0x7fffffffu) >= 0x40100000u) |
+           ((h2 & 0x7fffffffu) >= 0x40100000u) | ((h0 & 0x7fffffffu) >= 0x40300000u);
+}
+
 // The state of q-variables z (Eq. 14 inverted) with z[1], z[2] along the
 // frame's axes.  bad: bit 31 set when the state leaves the ranges above (the
 // values are then meaningless but every table index stays in range).
@@ -127,10 +135,7 @@ LSKUM_HD void fx_state(const uint64_t *tab, double z0, double z1, double z2, dou
 {
     const uint32_t h0 = (uint32_t)(f64_bits(z0) >> 32), h1 = (uint32_t)(f64_bits(z1) >> 32);
     const uint32_t h2 = (uint32_t)(f64_bits(z2) >> 32), h3 = (uint32_t)(f64_bits(z3) >> 32);
-    // -4 < z3 < -0.5 (1 + 2^-10); |z1|, |z2| < 4; |z0| < 16
-    const bool out = !(h3 - 0xbfe00400u < 0xc0100000u - 0xbfe00400u) | ((h1 & 0x7fffffffu) >= 0x40100000u) |
-                     ((h2 & 0x7fffffffu) >= 0x40100000u) | ((h0 & 0x7fffffffu) >= 0x40300000u);
-    uint32_t b = out ? 0x80000000u : 0u;
+    uint32_t b = fx_outside(h0, h1, h2, h3) ? 0x80000000u : 0u;
     s.su = (int32_t)h1 >> 31;
     s.sv = (int32_t)h2 >> 31;
     const uint64_t beta = fix_mag(z3, 62);  // 2 beta in 2^-62 = beta in 2^-63

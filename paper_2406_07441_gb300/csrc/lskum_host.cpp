@@ -129,6 +129,15 @@ void host_free_stream(const lskum_ctx *c, int32_t b, double *u, double *v)
     *v = c->case_mach[b] * std::sin(alb);
 }
 
+// q-variables of the free stream (rho = 1, p = 1/1.4: beta = 0.7).
+void free_stream_q(double u, double v, double q[4])
+{
+    q[0] = 2.5 * std::log(0.7) - 0.7 * (u * u + v * v);
+    q[1] = 1.4 * u;
+    q[2] = 1.4 * v;
+    q[3] = -1.4;
+}
+
 lskum_status fail(lskum_ctx *c, lskum_status s, const char *fmt, ...)
 {
     char buf[512];
@@ -1433,14 +1442,24 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     d.lusgs = c->opts.lusgs;
     d.farfield = c->opts.farfield;
     double *dcase_uinf = A.alloc<double>(4 * (size_t)c->n_cases);
+    uint8_t *dcase_fp64 = A.alloc<uint8_t>(c->n_cases);
     if (A.err != cudaSuccess) return cuda_fail(c, A.err, "cudaMalloc");
     d.case_uinf = dcase_uinf;
+    d.case_fp64 = dcase_fp64;
     std::vector<double> cuinf(4 * (size_t)c->n_cases);
+    std::vector<uint8_t> fp64(c->n_cases);
     for (int32_t b = 0; b < c->n_cases; b++) {
         double ub, vb;
         host_free_stream(c, b, &ub, &vb);
         host_prim_to_cons(1.0, ub, vb, 1.0 / 1.4, &cuinf[4 * b]);  // as the start state below
+        double q[4];
+        free_stream_q(ub, vb, q);
+        uint32_t h[4];
+        for (int k = 0; k < 4; k++) h[k] = (uint32_t)(f64_bits(q[k]) >> 32);
+        fp64[b] = fx_outside(h[0], h[1], h[2], h[3]);
     }
+    const int32_t n_fp64 = (int32_t)std::count(fp64.begin(), fp64.end(), (uint8_t)1);
+    d.fp64_cases = n_fp64 == 0 ? 0 : (n_fp64 == c->n_cases ? 1 : 2);
     auto up = [&](void *dst, const void *src, size_t bytes) {
         if (e == cudaSuccess && bytes) e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
     };
@@ -1477,6 +1496,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     up(dinv, c->inv.data(), n * sizeof(int32_t));
     up(dcase_of, hp.case_of_i.data(), ld * sizeof(int32_t));
     up(dcase_uinf, cuinf.data(), cuinf.size() * sizeof(double));
+    up(dcase_fp64, fp64.data(), fp64.size());
     if (d.lvl_lanes) up((void *)d.lvl_lanes, c->lvl_lanes.data(), c->lvl_lanes.size() * sizeof(int32_t));
     for (int dir = 0; dir < 2; dir++) {
         if (!d.pk_pt[dir]) continue;

@@ -223,6 +223,10 @@ struct Dev {
     int32_t lusgs;        // 0 Anandhanarayanan's diagonal; 1 the revised form of Manish et al.
     int32_t farfield;     // 0 outer points frozen at the free stream; 1 the kinetic far field
     const double *case_uinf;  // [n_cases][4] free-stream conserved state of each case
+    // [n_cases] 1: the residual in FP64 throughout (a free stream outside the
+    // fixed-point ranges); fp64_cases: 0 no case, 1 all, 2 some
+    const uint8_t *case_fp64;
+    int32_t fp64_cases;
 };
 
 // Kernel launch wrappers (lskum_kernels.cu).  `cur` is the state set read by

@@ -845,16 +845,15 @@ __device__ __forceinline__ void comp_add(double &R, double &c, double y)
     R = t;
 }
 
-// The slots sub, sub + TPP, ... of point k in FP64, for points of which a
-// state lies outside the fixed-point ranges (hypersonic, very hot or very
-// dense states, non-finite ones); the group's lanes add their sums.  In mixed
-// precision the sums are compensated: the terms of a group of four slots, by
-// FMAs, less the error carried so far, enter R by one compensated addition.
+// The slots sub, sub + TPP, ... of point k in FP64, for states outside the
+// fixed-point ranges (hypersonic, very hot or very dense, non-finite ones);
+// the group's lanes add their sums.  In mixed precision the sums are
+// compensated: the terms of a group of four slots, by FMAs, less the error
+// carried so far, enter R by one compensated addition.
 template <int TPP>
-__device__ __noinline__ void residual_fp64(const Dev &d, const double *__restrict__ q, const double *__restrict__ g,
-                                           int k, int sub, bool second, double R[4])
+__device__ __forceinline__ void residual_slots(const Dev &d, const MathTables &T, const double *__restrict__ q,
+                                               const double *__restrict__ g, int k, int sub, bool second, double R[4])
 {
-    const MathTables &T = g_math;
     const int ld = d.ld;
     const bool framed = d.flag[k] != kInterior;
     const double e1x = d.geo[G_E1X * ld + k], e1y = d.geo[G_E1Y * ld + k];
@@ -911,6 +910,20 @@ __device__ __noinline__ void residual_fp64(const Dev &d, const double *__restric
         if (d.precision && ng > 0) comp_add(R[c], carry[c], y[c]);
         R[c] = d.precision ? R[c] - carry[c] : y[c];
     }
+}
+
+// The same for a point among points inside the ranges.
+template <int TPP>
+__device__ __noinline__ void residual_fp64(const Dev &d, const double *__restrict__ q, const double *__restrict__ g,
+                                           int k, int sub, bool second, double R[4])
+{
+    residual_slots<TPP>(d, g_math, q, g, k, sub, second, R);
+}
+
+// Is point k's residual formed in FP64 throughout (by k_residual_fp64)?
+__device__ __forceinline__ bool hypersonic(const Dev &d, int k)
+{
+    return d.fp64_cases == 2 && d.case_fp64[d.case_of[k]] != 0;
 }
 
 // The ghost term of a kinetic outer point: the n- side is free-stream ghosts
@@ -990,6 +1003,20 @@ __device__ __forceinline__ double cfl_now(const Dev &d, int n1)
     return (d.ramp > 0.0 && (double)n1 < d.ramp) ? d.cfl * ((double)n1 / d.ramp) : d.cfl;
 }
 
+// Point k's residual from its sums: the ghost term, the store, and the diagonal
+// (by k_diag with several lanes per point).
+template <int TPP>
+__device__ __forceinline__ void finish_residual(const Dev &d, const StateSet &st, int k, int fl, int n1, double e1x,
+                                                double e1y, double e2x, double e2y, double R[4])
+{
+    if (fl == kOuter) add_ghosts(d, st.U, k, e2x, e2y, R);
+#pragma unroll
+    for (int c = 0; c < 4; c++) d.R[c * d.ld + k] = R[c];
+    // (a norm of smaller values is finite)
+    if (!(fabs(R[0]) < 1e140)) d.suspect[d.case_of[k]] = 1;
+    if (TPP == 1) diag_point(d, st, k, cfl_now(d, n1), e1x, e1y, e2x, e2y);
+}
+
 // Diagonals of all swept points, a thread per point, for the launch shapes
 // with several lanes per point in the residual: there a warp holds few
 // points, and its FP64 sequence per point (about 45 instructions) would cost
@@ -1014,6 +1041,7 @@ __global__ void __launch_bounds__(256) k_diag(Dev d, StateSet st)
 // (10,240 points, two lanes: 0.032 ms against 0.038).
 template <int TPP>
 constexpr int kResBlock = TPP == 1 ? 512 : 256;
+constexpr int kRes64Block = 128;
 
 // Flux residual, local time step and scalar diagonal; TPP lanes per point
 // over its slots, persistent blocks (a warp takes every W-th group of 32/TPP
@@ -1054,7 +1082,7 @@ __global__ void __launch_bounds__(kResBlock<TPP>, 512 / kResBlock<TPP>)
         const bool active = k < d.n;
         const int kk = active ? k : d.n - 1;
         const int fl = d.flag[kk];
-        const bool work = active && (fl != kOuter || d.farfield == 1) && !frozen(d, kk);
+        const bool work = active && (fl != kOuter || d.farfield == 1) && !frozen(d, kk) && !hypersonic(d, kk);
         const bool framed = fl != kInterior;  // (t, n) frame: wall and kinetic outer points
         FxSum acc[4] = {};
         uint32_t bad = 0;
@@ -1154,14 +1182,39 @@ __global__ void __launch_bounds__(kResBlock<TPP>, 512 / kResBlock<TPP>)
                 if (slow) R[c] = Rs[c];
             }
         }
-        if (work && sub == 0) {
-            if (fl == kOuter) add_ghosts(d, st.U, k, e2x, e2y, R);
+        if (work && sub == 0) finish_residual<TPP>(d, st, k, fl, n1, e1x, e1y, e2x, e2y, R);
+    }
+}
+
+// The residual of cases whose free stream is itself outside the fixed-point
+// ranges (from M 2.86 on along an axis; decided per case at create): FP64
+// throughout, the tables in shared memory.  Beside the fixed-point form every
+// one of its points would be formed twice: 147,584 points at M 3.5 and 6
+// 0.74 ms like this, 0.92 ms there (at M 2.5 the fixed-point form takes
+// 0.22 ms).  128 threads, four blocks per SM (128 registers).
+template <int TPP>
+__global__ void __launch_bounds__(kRes64Block, 4) k_residual_fp64(Dev d, StateSet st, const double *__restrict__ g)
+{
+    __shared__ MathTables T;
+    if (halted(d.ctrl)) return;
+    load_math_tables(T);
+    __syncthreads();
+    const int n1 = ((const volatile Ctrl *)d.ctrl)->it;
+    const int gt = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = gt / TPP, sub = gt % TPP;
+    const bool active = k < d.n;
+    const int kk = active ? k : d.n - 1;
+    const int fl = d.flag[kk];
+    const bool work = active && (fl != kOuter || d.farfield == 1) && !frozen(d, kk) &&
+                      (d.fp64_cases == 1 || hypersonic(d, kk));
+    double R[4] = {0.0, 0.0, 0.0, 0.0};
+    if (work) residual_slots<TPP>(d, T, st.q, g, kk, sub, n1 > d.first_order, R);
 #pragma unroll
-            for (int c = 0; c < 4; c++) d.R[c * ld + k] = R[c];
-            // (a norm of smaller values is finite)
-            if (!(fabs(R[0]) < 1e140)) d.suspect[d.case_of[k]] = 1;
-            if (TPP == 1) diag_point(d, st, k, cfl_now(d, n1), e1x, e1y, e2x, e2y);  // else k_diag
-        }
+    for (int c = 0; c < 4; c++) R[c] = group_sum<TPP>(R[c]);
+    if (work && sub == 0) {
+        double e1x, e1y, e2x, e2y;
+        point_frame(d, kk, fl != kInterior, e1x, e1y, e2x, e2y);
+        finish_residual<TPP>(d, st, k, fl, n1, e1x, e1y, e2x, e2y, R);
     }
 }
 
@@ -2477,10 +2530,17 @@ cudaError_t enqueue_grad(const Dev &d, int cur, cudaStream_t s, int *launches)
 template <int TPP>
 cudaError_t enqueue_res(const Dev &d, const Launch &L, int cur, cudaStream_t s, int *launches)
 {
-        constexpr int block = kResBlock<TPP>;
+    constexpr int block = kResBlock<TPP>;
     const int want = (d.n * TPP + block - 1) / block, most = L.sms * (512 / block);
-    k_residual<TPP><<<want < most ? want : most, block, 0, s>>>(d, d.set[cur], d.gq[grad_buffer(d.K)]);
-    (*launches)++;
+    const double *g = d.gq[grad_buffer(d.K)];
+    if (d.fp64_cases != 1) {
+        k_residual<TPP><<<want < most ? want : most, block, 0, s>>>(d, d.set[cur], g);
+        (*launches)++;
+    }
+    if (d.fp64_cases) {
+        k_residual_fp64<TPP><<<(d.n * TPP + kRes64Block - 1) / kRes64Block, kRes64Block, 0, s>>>(d, d.set[cur], g);
+        (*launches)++;
+    }
     return cudaGetLastError();
 }
 
