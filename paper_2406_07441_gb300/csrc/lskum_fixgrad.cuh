@@ -11,7 +11,10 @@
 // of two such that the weights times X add up to less than 1, so |G_x| is at
 // most the largest difference of q over the stencil (the same for y, with its
 // own power, whatever the stencil's aspect ratio), and q and G share a unit:
-// 2^-59 for the first component (|q| < 8), 2^-60 for the others (|q| < 4).
+// 2^-59 for the first component (|q| < 8), 2^-60 for the others (|q| < 4), times
+// a power of two for the first three components of a case whose free stream
+// comes near those bounds (fix_shift: from M 2.14 on; FP64's unit in the last
+// place of such a value is 2^-51 or more).
 // The inner iterations' coefficients absorb the ratios of their points'
 // powers.  A value out of range (or not finite) is stored as a mark, with its
 // FP64 value beside; points that meet a mark are evaluated in FP64.
@@ -30,19 +33,32 @@ constexpr int kMaxGradShift = 10;    // largest power of two of a fast inner ite
 constexpr int kMaxGradExp = 900;     // largest |exponent| of X or Y of a fast point
 constexpr int kGradNoScale = 32000;  // weights without a scale (not finite): the result is NaN
 
-// -log2 of component c's unit.
-LSKUM_HD int fix_unit(int c)
+// A case's powers of two, from its free stream's q: bits 0 to 7 of the first
+// component (to three quarters of its bound or less), 8 up of the second and
+// third (the fourth is -1.4 in every free stream).
+constexpr int kMaxFixShift = 20;
+inline int fix_shift(const double q[4])
 {
-    return c == 0 ? 59 : 60;
+    int s0 = 0, s1 = 0;
+    while (s0 < kMaxFixShift && !(std::fabs(q[0]) <= 6.0 * (1 << s0))) s0++;
+    while (s1 < kMaxFixShift && !(std::fabs(q[1]) <= 3.0 * (1 << s1) && std::fabs(q[2]) <= 3.0 * (1 << s1))) s1++;
+    return s0 | s1 << 8;
+}
+
+// -log2 of component c's unit in a case with these powers.
+LSKUM_HD int fix_unit(int c, int shift = 0)
+{
+    return c == 0 ? 59 - (shift & 255) : (c < 3 ? 60 - (shift >> 8) : 60);
 }
 
 // Component c of q, to the nearest unit, or the mark.
-LSKUM_HD int64_t fix_q(double q, int c)
+LSKUM_HD int64_t fix_q(double q, int c, int shift = 0)
 {
     const int32_t h = (int32_t)(f64_bits(q) >> 32);
-    if ((h & 0x7fffffff) >= (c == 0 ? 0x401fffff : 0x400fffff)) return kFixMark;
-    if ((h & 0x7fffffff) < (1022 - fix_unit(c)) << 20) return 0;  // less than half a unit
-    return (int64_t)neg_if((fix_mag(q, fix_unit(c) + 1) + 1) >> 1, h >> 31);
+    const int unit = fix_unit(c, shift);
+    if ((h & 0x7fffffff) >= ((c == 0 ? 0x401fffff + (59 << 20) : 0x400fffff + (60 << 20)) - (unit << 20))) return kFixMark;
+    if ((h & 0x7fffffff) < (1022 - unit) << 20) return 0;  // less than half a unit
+    return (int64_t)neg_if((fix_mag(q, unit + 1) + 1) >> 1, h >> 31);
 }
 
 // The mark of a value's high word (a split or a plain word).

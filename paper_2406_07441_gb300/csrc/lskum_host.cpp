@@ -129,9 +129,11 @@ void host_free_stream(const lskum_ctx *c, int32_t b, double *u, double *v)
     *v = c->case_mach[b] * std::sin(alb);
 }
 
-// q-variables of the free stream (rho = 1, p = 1/1.4: beta = 0.7).
-void free_stream_q(double u, double v, double q[4])
+// q-variables of case b's free stream (rho = 1, p = 1/1.4: beta = 0.7).
+void free_stream_q(const lskum_ctx *c, int32_t b, double q[4])
 {
+    double u, v;
+    host_free_stream(c, b, &u, &v);
     q[0] = 2.5 * std::log(0.7) - 0.7 * (u * u + v * v);
     q[1] = 1.4 * u;
     q[2] = 1.4 * v;
@@ -237,6 +239,7 @@ struct HostPrep {
     std::vector<uint4> ewg, ewj, wc;  // the q-derivatives' weights (Dev::wg, ...)
     std::vector<short4> ge;
     std::vector<short2> gb;
+    std::vector<int32_t> case_shift;  // fix_shift of each case
     // LU-SGS lower / upper slot lists (CSR, internal order) and level orders
     std::vector<int32_t> lo_off, lo_nbr, up_off, up_nbr, sw_fwd, sw_bwd;
     std::vector<uint8_t> lo_mb, up_mb;
@@ -931,6 +934,11 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
     hp.wc.assign(2 * (size_t)ld, uint4{0, 0, 0, 0});
     hp.ge.assign(ld, short4{0, 0, 0, 0});
     hp.gb.assign(ld, short2{0, 0});
+    for (int32_t b = 0; b < c->n_cases; b++) {
+        double q[4];
+        free_stream_q(c, b, q);
+        hp.case_shift.push_back(fix_shift(q));
+    }
     auto pack = [&](int32_t from, int32_t to) {
         double pv[4 * 256];  // a point's scaled weights (at most 255 slots and the centre) and their words
         uint4 pw[2 * 256];
@@ -995,7 +1003,8 @@ static lskum_status prepare_host(lskum_ctx *c, const lskum_cloud *cl, HostPrep &
             const int b1 = split_words(pv, dg, true, pw);
             for (int32_t j = 0; j < dg; j++) hp.ewg[base + 32 * j] = pw[j];
             hp.ge[k] = short4{(short)ex, (short)ey, (short)px, (short)py};
-            hp.gb[k] = short2{(short)b1, (short)b2};
+            const int shift = hp.case_shift[c->case_of_caller[p]];
+            hp.gb[k] = short2{(short)(b1 | (shift & 255) << 8), (short)(b2 | (shift >> 8) << 8)};
         }
     };
     in_threads(n, pack);
@@ -1443,6 +1452,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     d.farfield = c->opts.farfield;
     double *dcase_uinf = A.alloc<double>(4 * (size_t)c->n_cases);
     uint8_t *dcase_fp64 = A.alloc<uint8_t>(c->n_cases);
+    int32_t *dcase_shift = A.alloc<int32_t>(c->n_cases);
     if (A.err != cudaSuccess) return cuda_fail(c, A.err, "cudaMalloc");
     d.case_uinf = dcase_uinf;
     d.case_fp64 = dcase_fp64;
@@ -1453,7 +1463,7 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
         host_free_stream(c, b, &ub, &vb);
         host_prim_to_cons(1.0, ub, vb, 1.0 / 1.4, &cuinf[4 * b]);  // as the start state below
         double q[4];
-        free_stream_q(ub, vb, q);
+        free_stream_q(c, b, q);
         uint32_t h[4];
         for (int k = 0; k < 4; k++) h[k] = (uint32_t)(f64_bits(q[k]) >> 32);
         fp64[b] = fx_outside(h[0], h[1], h[2], h[3]);
@@ -1497,6 +1507,9 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     up(dcase_of, hp.case_of_i.data(), ld * sizeof(int32_t));
     up(dcase_uinf, cuinf.data(), cuinf.size() * sizeof(double));
     up(dcase_fp64, fp64.data(), fp64.size());
+    up(dcase_shift, hp.case_shift.data(), hp.case_shift.size() * sizeof(int32_t));
+    d.case_shift = dcase_shift;
+    d.shift = hp.case_shift[0];
     if (d.lvl_lanes) up((void *)d.lvl_lanes, c->lvl_lanes.data(), c->lvl_lanes.size() * sizeof(int32_t));
     for (int dir = 0; dir < 2; dir++) {
         if (!d.pk_pt[dir]) continue;

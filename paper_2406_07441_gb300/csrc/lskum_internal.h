@@ -117,7 +117,8 @@ struct Dev {
     // coefficients wj = -w_x dx/2, -w_x dy/2, -w_y dx/2, -w_y dy/2
     // over 2^e_x, 2^e_y of the point and times those of the neighbour, in
     // units of 2^(p_x - 31), 2^(p_y - 31); wc per point: the centre's;
-    // ge = (e_x, e_y, p_x, p_y), gb = the b of wg and of the coefficients
+    // ge = (e_x, e_y, p_x, p_y), gb = the b of wg and of the coefficients in
+    // the low bytes, the powers of two of the case's units above (fix_shift)
     const uint4 *wg, *wj, *wc;  // (wj, wc: two words per slot or point)
     const short4 *ge;
     const short2 *gb;
@@ -227,6 +228,8 @@ struct Dev {
     // fixed-point ranges); fp64_cases: 0 no case, 1 all, 2 some
     const uint8_t *case_fp64;
     int32_t fp64_cases;
+    const int32_t *case_shift;  // [n_cases] powers of two of the units of q (fix_shift)
+    int32_t shift;              // of the first case
 };
 
 // Kernel launch wrappers (lskum_kernels.cu).  `cur` is the state set read by

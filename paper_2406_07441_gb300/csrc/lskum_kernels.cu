@@ -567,9 +567,20 @@ __device__ __forceinline__ double pow2(int e)
 }
 
 // The value of a stored G (or of a mark's FP64 derivative) in units of q.
-__device__ __forceinline__ double g_value(int lo, int hi, const double *g, int ex, int c)
+__device__ __forceinline__ double g_value(int lo, int hi, const double *g, int ex, int unit)
 {
-    return fix_marked(hi) ? scalbn(*g, -ex) : scalbn((double)join_g(hi, lo), -fix_unit(c));
+    return fix_marked(hi) ? scalbn(*g, -ex) : scalbn((double)join_g(hi, lo), -unit);
+}
+
+// A point's word gb: the bits of its weights' remainders, and the powers of two
+// of its case's units (fix_shift).
+__device__ __forceinline__ int grad_bits(short2 gb, bool corr)
+{
+    return (corr ? gb.y : gb.x) & 255;
+}
+__device__ __forceinline__ int grad_shift(short2 gb)
+{
+    return gb.x >> 8 | (gb.y >> 8) << 8;
 }
 
 // What k_grad forms, in FP64, for a point that meets a marked value or has no
@@ -582,7 +593,8 @@ __device__ __noinline__ void grad_fp64(const Dev &d, const double *__restrict__ 
     const int4 *__restrict__ gf = CORR ? d.gf[from] : nullptr;
     const double *__restrict__ g = CORR ? d.gq[from] : nullptr;
     const short4 ge = d.ge[k];
-    const double lsb = pow2(-(CORR ? d.gb[k].y : d.gb[k].x));
+    const double lsb = pow2(-grad_bits(d.gb[k], CORR));
+    const int shift = grad_shift(d.gb[k]);
     const int deg = d.deg[k];
     const int base = d.slice_off[k >> 5] + (k & 31);
     for (int c = 0; c < 4; c++) v[c] = 0.0;
@@ -611,8 +623,9 @@ __device__ __noinline__ void grad_fp64(const Dev &d, const double *__restrict__ 
             const int *f = reinterpret_cast<const int *>(gf + 4 * (size_t)i + 2 * c2);
             for (int c = 0; c < 2; c++) {
                 const double *gx = g + 8 * (size_t)i + 2 * c2 + c;
-                const double x = g_value(f[4 * c], f[4 * c + 1], gx, gi.x, 2 * c2 + c);
-                const double y = g_value(f[4 * c + 2], f[4 * c + 3], gx + 4, gi.y, 2 * c2 + c);
+                const int unit = fix_unit(2 * c2 + c, shift);
+                const double x = g_value(f[4 * c], f[4 * c + 1], gx, gi.x, unit);
+                const double y = g_value(f[4 * c + 2], f[4 * c + 3], gx + 4, gi.y, unit);
                 v[c] = fma(axx, x, fma(axy, y, v[c]));
                 v[2 + c] = fma(ayx, x, fma(ayy, y, v[2 + c]));
             }
@@ -650,7 +663,7 @@ __global__ void __launch_bounds__(kGradBlock, 5) k_grad(Dev d, StateSet st, int 
     const int kk = active ? k : d.n - 1;
     const short4 ge = d.ge[kk];
     bool bad = abs(ge.x) > kMaxGradExp || abs(ge.y) > kMaxGradExp || ge.z > kMaxGradShift || ge.w > kMaxGradShift;
-    const int bits = CORR ? d.gb[kk].y : d.gb[kk].x;
+    const int bits = grad_bits(d.gb[kk], CORR);
     bad |= bits < kMinGradBits;
     // every lane of a slice runs to the slice's width: a padding slot is the
     // point itself with weights 0
@@ -762,16 +775,17 @@ __global__ void __launch_bounds__(kGradBlock, 5) k_grad(Dev d, StateSet st, int 
         }
         if (bad) {
             bool fits = true;
+            const int shift = grad_shift(d.gb[kk]);
 #pragma unroll
             for (int c = 0; c < 4; c++) {
-                const int cc = 2 * c2 + (c & 1);
+                const int cc = 2 * c2 + (c & 1), unit = fix_unit(cc, shift);
                 if (CORR) {
                     const int *a = reinterpret_cast<const int *>(d.gf[2] + 4 * (size_t)kk + cc) + 2 * (c >> 1);
-                    t[c] += g_value(a[0], a[1], d.gq[2] + 8 * (size_t)kk + cc + 4 * (c >> 1), c < 2 ? ge.x : ge.y, cc);
+                    t[c] += g_value(a[0], a[1], d.gq[2] + 8 * (size_t)kk + cc + 4 * (c >> 1), c < 2 ? ge.x : ge.y, unit);
                 }
-                fits = fits && fabs(t[c]) < (cc == 0 ? 7.5 : 3.75);
+                fits = fits && fabs(t[c]) < scalbn(3.75, 60 - unit);
                 f[c] = t[c];
-                v[c] = fits ? __double2ll_rn(scalbn(t[c], fix_unit(cc))) : 0;
+                v[c] = fits ? __double2ll_rn(scalbn(t[c], unit)) : 0;
             }
             bad = !fits || abs(ge.x) > kMaxGradExp || abs(ge.y) > kMaxGradExp;
         }
@@ -792,7 +806,7 @@ __global__ void __launch_bounds__(kGradBlock, 5) k_grad(Dev d, StateSet st, int 
             g[0] = make_double2(scalbn(f[0], ge.x), scalbn(f[1], ge.x));
             g[2] = make_double2(scalbn(f[2], ge.y), scalbn(f[3], ge.y));
         } else {
-            const int u0 = fix_unit(2 * c2), u1 = fix_unit(1);
+            const int shift = grad_shift(d.gb[kk]), u0 = fix_unit(2 * c2, shift), u1 = fix_unit(2 * c2 + 1, shift);
             g[0] = make_double2((double)v[0] * pow2(ge.x - u0), (double)v[1] * pow2(ge.x - u1));
             g[2] = make_double2((double)v[2] * pow2(ge.y - u0), (double)v[3] * pow2(ge.y - u1));
         }
@@ -2376,8 +2390,9 @@ __global__ void __launch_bounds__(kUpdateBlock) k_update(Dev d, int cur, bool in
     qn[3] = signed_by(twice(P.beta), false);
     store4(dst.q + 4 * (size_t)k, qn);
     longlong2 *qf = reinterpret_cast<longlong2 *>(dst.qf + 4 * (size_t)k);
-    qf[0] = make_longlong2(fix_q(qn[0], 0), fix_q(qn[1], 1));
-    qf[1] = make_longlong2(fix_q(qn[2], 2), fix_q(qn[3], 3));
+    const int shift = d.n_cases > 1 ? d.case_shift[d.case_of[k]] : d.shift;
+    qf[0] = make_longlong2(fix_q(qn[0], 0, shift), fix_q(qn[1], 1, shift));
+    qf[1] = make_longlong2(fix_q(qn[2], 2, shift), fix_q(qn[3], 3, shift));
     // the per-point record, assembled in registers and stored as 16-byte
     // vectors (and, in mixed precision, its FP32 copy from the same registers)
     double rec[P_NFIELDS];
