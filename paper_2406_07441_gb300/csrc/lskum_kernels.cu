@@ -1026,8 +1026,8 @@ __device__ __forceinline__ void finish_residual(const Dev &d, const StateSet &st
     if (fl == kOuter) add_ghosts(d, st.U, k, e2x, e2y, R);
 #pragma unroll
     for (int c = 0; c < 4; c++) d.R[c * d.ld + k] = R[c];
-    // (a norm of smaller values is finite)
-    if (!(fabs(R[0]) < 1e140)) d.suspect[d.case_of[k]] = 1;
+    // (the sum of 2^28 squares of smaller values is finite)
+    if (!(fabs(R[0]) < 8e149)) d.suspect[d.case_of[k]] = 1;
     if (TPP == 1) diag_point(d, st, k, cfl_now(d, n1), e1x, e1y, e2x, e2y);
 }
 
