@@ -239,14 +239,23 @@ __device__ __forceinline__ PrimU prim_from_cons(const double U[4])
 // The same for the increment products, by the shortest chain: with Q = 2 rho p
 // = 0.8 (rho E - |m|^2/2) everything needs one reciprocal square root, beside
 // the one division, instead of three divisions and a square root in a row.
-// (Only what flux_prim reads.)
+// (Only what flux_prim reads.)  Q is a product of two such values: where it
+// leaves 2^-960 .. 2^1000 (or is not positive) the other form takes over.
+__device__ __noinline__ void prim_by_division(const double U[4], PrimU &P)
+{
+    P = prim_from_cons(U);
+}
 __device__ __forceinline__ PrimU prim_short(const double U[4])
 {
     PrimU P;
-    P.rho = U[0];
-    P.irho = 1.0 / U[0];
     const double hm = 0.5 * fma(U[1], U[1], __dmul_rn(U[2], U[2]));
     const double Q = 0.8 * fma(U[0], U[3], -hm);
+    if ((unsigned)__double2hiint(Q) - (63u << 20) > (1960u << 20)) {
+        prim_by_division(U, P);
+        return P;
+    }
+    P.rho = U[0];
+    P.irho = 1.0 / U[0];
     const double r = rsqrt(Q);
     P.sb = __dmul_rn(fabs(U[0]), r);
     P.u = __dmul_rn(U[1], P.irho);

@@ -35,3 +35,12 @@ def test_a_dense_state_whose_norm_is_finite_does_not_diverge(opts):
     U, hist = _run(480, **opts)
     assert np.all(np.isfinite(hist)) and hist[0] > 1e140
     assert np.max(np.abs(U - ref)) <= TOL
+
+
+@pytest.mark.parametrize("opts", [dict(jvp=1), dict(jvp=1, lusgs=1), dict()])
+@pytest.mark.parametrize("power", [-520, -500])
+def test_a_state_of_which_products_underflow(power, opts):
+    """(The norm's squares underflow too: only the state is compared.)"""
+    ref, _ = _run(0, **opts)
+    U, _ = _run(power, **opts)
+    assert np.max(np.abs(U - ref)) <= TOL
