@@ -19,6 +19,7 @@
 #include <string>
 #include <system_error>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/lskum.h"
@@ -1247,11 +1248,26 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
         d.gq[s] = A.alloc<double>(8 * (size_t)ld);
         d.gf[s] = A.alloc<int4>(4 * (size_t)ld);
     }
-    int32_t *dlo_off = A.alloc<int32_t>(n + 1), *dup_off = A.alloc<int32_t>(n + 1);
-    int32_t *dlo_nbr = A.alloc<int32_t>(hp.lo_nbr.size()), *dup_nbr = A.alloc<int32_t>(hp.up_nbr.size());
-    uint8_t *dlo_mb = A.alloc<uint8_t>(hp.lo_mb.size()), *dup_mb = A.alloc<uint8_t>(hp.up_mb.size());
-    double *dlo_w1 = A.alloc<double>(hp.lo_w1.size()), *dlo_w2 = A.alloc<double>(hp.lo_w2.size());
-    double *dup_w1 = A.alloc<double>(hp.up_w1.size()), *dup_w2 = A.alloc<double>(hp.up_w2.size());
+    // the lower and upper lists by point, which only the form with one launch
+    // per level reads (lists too long for the packed one)
+    const bool lists = !c->pk_ok;
+    auto list = [&](auto &v, auto *&dev) {
+        dev = nullptr;
+        if (lists) dev = A.alloc<std::remove_reference_t<decltype(*dev)>>(v.size());
+    };
+    int32_t *dlo_off, *dup_off, *dlo_nbr, *dup_nbr;
+    uint8_t *dlo_mb, *dup_mb;
+    double *dlo_w1, *dlo_w2, *dup_w1, *dup_w2;
+    list(hp.lo_off, dlo_off);
+    list(hp.up_off, dup_off);
+    list(hp.lo_nbr, dlo_nbr);
+    list(hp.up_nbr, dup_nbr);
+    list(hp.lo_mb, dlo_mb);
+    list(hp.up_mb, dup_mb);
+    list(hp.lo_w1, dlo_w1);
+    list(hp.lo_w2, dlo_w2);
+    list(hp.up_w1, dup_w1);
+    list(hp.up_w2, dup_w2);
     int32_t *dsw_fwd = A.alloc<int32_t>(hp.sw_fwd.size()), *dsw_bwd = A.alloc<int32_t>(hp.sw_bwd.size());
     // mixed precision: FP32 increments, primal records and weights
     const bool mixed = c->opts.precision == 1;
@@ -1262,11 +1278,11 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     if (mixed) {
         for (auto pr : {std::make_pair(&hp.lo_w1, &flo_w1), std::make_pair(&hp.lo_w2, &flo_w2),
                         std::make_pair(&hp.up_w1, &fup_w1), std::make_pair(&hp.up_w2, &fup_w2)})
-            pr.second->assign(pr.first->begin(), pr.first->end());
-        dlo_w1f = A.alloc<float>(flo_w1.size());
-        dlo_w2f = A.alloc<float>(flo_w2.size());
-        dup_w1f = A.alloc<float>(fup_w1.size());
-        dup_w2f = A.alloc<float>(fup_w2.size());
+            if (lists) pr.second->assign(pr.first->begin(), pr.first->end());
+        list(flo_w1, dlo_w1f);
+        list(flo_w2, dlo_w2f);
+        list(fup_w1, dup_w1f);
+        list(fup_w2, dup_w2f);
         d.dUsf = A.alloc<float>(4 * (size_t)ld);
         d.dUf = A.alloc<float>(4 * (size_t)ld);
         for (int s = 0; s < 2; s++) d.set[s].primf = A.alloc<float>((size_t)kPrimStride * ld);
@@ -1493,16 +1509,18 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     up(dwc, hp.wc.data(), 2 * (size_t)ld * sizeof(uint4));
     up(dge, hp.ge.data(), ld * sizeof(short4));
     up(dgb, hp.gb.data(), ld * sizeof(short2));
-    up(dlo_off, hp.lo_off.data(), hp.lo_off.size() * sizeof(int32_t));
-    up(dup_off, hp.up_off.data(), hp.up_off.size() * sizeof(int32_t));
-    up(dlo_nbr, hp.lo_nbr.data(), hp.lo_nbr.size() * sizeof(int32_t));
-    up(dup_nbr, hp.up_nbr.data(), hp.up_nbr.size() * sizeof(int32_t));
-    up(dlo_mb, hp.lo_mb.data(), hp.lo_mb.size());
-    up(dup_mb, hp.up_mb.data(), hp.up_mb.size());
-    up(dlo_w1, hp.lo_w1.data(), hp.lo_w1.size() * sizeof(double));
-    up(dlo_w2, hp.lo_w2.data(), hp.lo_w2.size() * sizeof(double));
-    up(dup_w1, hp.up_w1.data(), hp.up_w1.size() * sizeof(double));
-    up(dup_w2, hp.up_w2.data(), hp.up_w2.size() * sizeof(double));
+    if (lists) {
+        up(dlo_off, hp.lo_off.data(), hp.lo_off.size() * sizeof(int32_t));
+        up(dup_off, hp.up_off.data(), hp.up_off.size() * sizeof(int32_t));
+        up(dlo_nbr, hp.lo_nbr.data(), hp.lo_nbr.size() * sizeof(int32_t));
+        up(dup_nbr, hp.up_nbr.data(), hp.up_nbr.size() * sizeof(int32_t));
+        up(dlo_mb, hp.lo_mb.data(), hp.lo_mb.size());
+        up(dup_mb, hp.up_mb.data(), hp.up_mb.size());
+        up(dlo_w1, hp.lo_w1.data(), hp.lo_w1.size() * sizeof(double));
+        up(dlo_w2, hp.lo_w2.data(), hp.lo_w2.size() * sizeof(double));
+        up(dup_w1, hp.up_w1.data(), hp.up_w1.size() * sizeof(double));
+        up(dup_w2, hp.up_w2.data(), hp.up_w2.size() * sizeof(double));
+    }
     up(dsw_fwd, hp.sw_fwd.data(), hp.sw_fwd.size() * sizeof(int32_t));
     up(dsw_bwd, hp.sw_bwd.data(), hp.sw_bwd.size() * sizeof(int32_t));
     up(dblk_pos, hp.blk_pos.data(), hp.blk_pos.size() * sizeof(int32_t));
@@ -1559,11 +1577,13 @@ static lskum_status upload(lskum_ctx *c, HostPrep &hp)
     if (e == cudaSuccess) e = cudaMemset(c->case_hist0, 0, c->n_cases * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(c->case_err, 0, c->n_cases * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMemset(c->case_bad, 0x7f, c->n_cases * sizeof(int32_t));
-    if (mixed) {
+    if (mixed && lists) {
         up(dlo_w1f, flo_w1.data(), flo_w1.size() * sizeof(float));
         up(dlo_w2f, flo_w2.data(), flo_w2.size() * sizeof(float));
         up(dup_w1f, fup_w1.data(), fup_w1.size() * sizeof(float));
         up(dup_w2f, fup_w2.data(), fup_w2.size() * sizeof(float));
+    }
+    if (mixed) {
         if (e == cudaSuccess) e = cudaMemset(d.dUsf, 0, 4 * (size_t)ld * sizeof(float));
         if (e == cudaSuccess) e = cudaMemset(d.dUf, 0, 4 * (size_t)ld * sizeof(float));
     }
