@@ -1648,7 +1648,7 @@ static lskum_status build_graphs(lskum_ctx *c)
         L.fork = c->ev_fork;
         L.join = c->ev_join;
         cudaError_t le = launch_iteration(c->dev, L, par, c->n_levels, c->lvl_beg.data(),
-                                          c->lvl_act_end.data(), c->lvl_end.data(), c->stream, &launches);
+                                          c->lvl_act_end.data(), c->stream, &launches);
         e = cudaStreamEndCapture(c->stream, &g);
         if (le != cudaSuccess) {
             if (g) cudaGraphDestroy(g);
@@ -2215,7 +2215,7 @@ lskum_status lskum_time_phases(lskum_ctx *c, int32_t reps, double *ms)
         for (int ph = 0; ph < 6 && e == cudaSuccess; ph++) {
             e = cudaEventRecord(ev[ph], c->stream);
             if (e == cudaSuccess) e = launch_phase(d, c->launch, (c->cur + r) & 1, ph, c->n_levels, c->lvl_beg.data(),
-                                                   c->lvl_act_end.data(), c->lvl_end.data(), c->stream);
+                                                   c->lvl_act_end.data(), c->stream);
         }
         if (e == cudaSuccess) e = cudaEventRecord(ev[6], c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(ev[6]);
@@ -2553,7 +2553,7 @@ lskum_status ctx_case_norms(lskum_ctx *c, std::vector<double> &norms)
     cudaError_t e = clear();
     for (int ph = 0; ph < 3 && e == cudaSuccess; ph++)
         e = launch_phase(c->dev, c->launch, c->cur, ph, c->n_levels, c->lvl_beg.data(), c->lvl_act_end.data(),
-                         c->lvl_end.data(), c->stream);
+                         c->stream);
     norms.assign(c->n_cases, 0.0);
     if (e == cudaSuccess)
         e = cudaMemcpy2DAsync(norms.data(), sizeof(double), c->hist, c->hist_cap * sizeof(double), sizeof(double),

@@ -256,12 +256,12 @@ struct Launch {
 };
 
 cudaError_t launch_iteration(const Dev &d, const Launch &L, int cur, int n_levels, const int32_t *lvl_beg,
-                             const int32_t *lvl_act_end, const int32_t *lvl_end, cudaStream_t s,
+                             const int32_t *lvl_act_end, cudaStream_t s,
                              int *launches);
 // One phase of an iteration (0 q-derivatives, 1 residual, 2 norm, 3 forward
 // sweep, 4 backward sweep, 5 update), launched directly on s.
 cudaError_t launch_phase(const Dev &d, const Launch &L, int cur, int phase, int n_levels, const int32_t *lvl_beg,
-                         const int32_t *lvl_act_end, const int32_t *lvl_end, cudaStream_t s);
+                         const int32_t *lvl_act_end, cudaStream_t s);
 // Derive q and the per-point records of a new state in set cur (with the
 // wall projection of the state when project).
 cudaError_t launch_init_state(const Dev &d, int cur, bool project, cudaStream_t s);

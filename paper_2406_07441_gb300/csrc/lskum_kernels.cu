@@ -493,11 +493,6 @@ __device__ __forceinline__ void load4(const double *__restrict__ p, double v[4])
     const double2 a = reinterpret_cast<const double2 *>(p)[0], b = reinterpret_cast<const double2 *>(p)[1];
     v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
 }
-__device__ __forceinline__ void load4(const float *__restrict__ p, float v[4])
-{
-    const float4 a = *reinterpret_cast<const float4 *>(p);
-    v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
-}
 
 // The same, and single values, of what other blocks write within the launch:
 // ordinary coherent loads from L2, kept behind the level boundary whose
@@ -1089,6 +1084,7 @@ __global__ void __launch_bounds__(kResBlock<TPP>, 512 / kResBlock<TPP>)
     __shared__ __align__(16) uint64_t T[kFluxTableWords];
     if (halted(d.ctrl)) return;
     static_assert(kFluxTableR == kFluxRows && kFluxTableExp == kFluxExpRows && kFluxTableWords % 2 == 0, "tables");
+    static_assert(kLn2Fx == kFluxLn2 && kInvLn2Fx == kFluxInvLn2, "the table's constants");
     for (int i = threadIdx.x; i < kFluxTableWords / 2; i += kResBlock<TPP>)
         reinterpret_cast<ulonglong2 *>(T)[i] = reinterpret_cast<const ulonglong2 *>(kFluxTable)[i];
     __syncthreads();
@@ -1707,10 +1703,9 @@ __device__ __forceinline__ bool boundary_wait(Ctrl *c, uint32_t target, uint32_t
         uint64_t t0 = 0;
         int ok = 1;
         for (uint32_t tries = 1;; tries++) {
-            const uint32_t v = *bar;
+            uint32_t v = *bar;
             if (target == limit ? v == 0 : v >= target) {
-                uint32_t seen;
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&c->sweep_bar) : "memory");
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&c->sweep_bar) : "memory");
                 break;
             }
             if ((tries & 1023) == 0) {
@@ -2710,7 +2705,7 @@ cudaError_t enqueue_norm(const Dev &d, cudaStream_t s, int *launches)
 }
 
 cudaError_t enqueue_phase(const Dev &d, const Launch &L, int cur, int ph, int n_levels, const int32_t *lvl_beg,
-                          const int32_t *lvl_act_end, const int32_t *lvl_end, cudaStream_t s, int *launches)
+                          const int32_t *lvl_act_end, cudaStream_t s, int *launches)
 {
     const bool side = L.side && (needs_framed_jac(d, L) || needs_increment_base(d) || L.tpp > 1);
     switch (ph) {
@@ -2779,22 +2774,22 @@ cudaError_t enqueue_phase(const Dev &d, const Launch &L, int cur, int ph, int n_
 }  // namespace
 
 cudaError_t launch_iteration(const Dev &d, const Launch &L, int cur, int n_levels, const int32_t *lvl_beg,
-                             const int32_t *lvl_act_end, const int32_t *lvl_end, cudaStream_t s, int *launches)
+                             const int32_t *lvl_act_end, cudaStream_t s, int *launches)
 {
     for (int ph = 0; ph < 6; ph++) {
-        cudaError_t e = enqueue_phase(d, L, cur, ph, n_levels, lvl_beg, lvl_act_end, lvl_end, s, launches);
+        cudaError_t e = enqueue_phase(d, L, cur, ph, n_levels, lvl_beg, lvl_act_end, s, launches);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
 }
 
 cudaError_t launch_phase(const Dev &d, const Launch &L, int cur, int phase, int n_levels, const int32_t *lvl_beg,
-                         const int32_t *lvl_act_end, const int32_t *lvl_end, cudaStream_t s)
+                         const int32_t *lvl_act_end, cudaStream_t s)
 {
     int launches = 0;
     Launch Li = L;  // one phase at a time: the framed Jacobians inline, in the forward sweep's phase
     Li.side = nullptr;
-    return enqueue_phase(d, Li, cur, phase, n_levels, lvl_beg, lvl_act_end, lvl_end, s, &launches);
+    return enqueue_phase(d, Li, cur, phase, n_levels, lvl_beg, lvl_act_end, s, &launches);
 }
 
 cudaError_t launch_init_state(const Dev &d, int cur, bool project, cudaStream_t s)
