@@ -48,6 +48,7 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 WORKLOAD = "naca0012_2560x2048_jit"      # default: 5,242,880 points
+BATCH_WORKLOAD = "naca0012_batch64"
 MID_WORKLOAD = "naca0012_640x256_jit"    # 147,584 points
 PROF_WORKLOAD = "naca0012_1280x1024_jit"  # 1,310,720 points, the default's construction (profiling)
 SUPER_WORKLOAD = "naca0012_640x256_jit_m1.2"
@@ -78,25 +79,49 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
 # + 477,404,332), which stand for the 5,242,880-point cloud of the same
 # construction (the count depends on the mix of slots joining one or two
 # sub-stencils)
-RES_FLOPS_PER_SLOT = {MID_WORKLOAD: 336.07, SUPER_WORKLOAD: 336.07, PROF_WORKLOAD: 334.668, WORKLOAD: 334.668}
-# The current kernel evaluates the split fluxes and their sums in 64-bit fixed
-# point on the integer pipes; the FP64 flops it still executes on the FP64
-# unit per slot (ncu, the same counting; profiles/): the reconstruction's 16
-# FMAs and what a point costs besides
-RES_FP64_UNIT_FLOPS_PER_SLOT = {MID_WORKLOAD: 36.74, SUPER_WORKLOAD: 36.74, PROF_WORKLOAD: 36.74, WORKLOAD: 36.74}
+RES_FLOPS_PER_SLOT = {MID_WORKLOAD: 336.07, SUPER_WORKLOAD: 336.07, BATCH_WORKLOAD: 336.07, PROF_WORKLOAD: 334.668,
+                      WORKLOAD: 334.668}
+# The kernel's busiest unit is the pipe of the 32-bit multiplies into 64 bits
+# (the split fluxes and their sums run in 64-bit fixed point): cycles that an
+# SM's pipe is busy per active slot, from ncu on the 147,584-point cloud at 1
+# thread per point (69.7 % of 399,642 cycles on 152 SMs, 2,926,611 slots;
+# profiles/), which stand for the other clouds
+RES_MULT_CYCLES_PER_SLOT = 14.47
+MULT_PEAK = 152 * 2.070e9  # SM-cycles per second
+# FP64 flops that the kernel still executes on the FP64 unit per slot (the same
+# capture: 2 x 52,472,824 DFMA + 2,718,920 DMUL): the reconstruction's 16 FMAs
+# and what a point costs besides; given only for the cloud it was counted on
+RES_FP64_UNIT_FLOPS_PER_SLOT = {MID_WORKLOAD: 36.79}
 START = 50  # first-order start-up iterations before warm-up and timing
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one residual
 # launch, from one ncu capture of the current kernel (profiles/), per
 # workload and threads per point; reported only for that launch shape and FP64
-RES_TRAFFIC = {MID_WORKLOAD: {1: 178.356736e6}}
-# Unit utilisation of that launch (fraction of peak sustained, ncu): the
-# FMA-heavy pipe (32-bit multiplies into 64 bits) is the busiest unit, with
-# the latency of the integer chains at four warps per scheduler
-RES_UNITS_NCU = {MID_WORKLOAD: {"fp64_pipe": 0.4894, "alu_pipe": 0.3991, "fmaheavy_pipe": 0.6389, "issue": 0.4965}}
-RES_UNITS_NCU[SUPER_WORKLOAD] = RES_UNITS_NCU[MID_WORKLOAD]
-ROOFLINE_NOTE = ("achieved counts the method's FP64 arithmetic as the all-FP64 form executes it "
-                 "(flops_per_active_slot); frac exceeds 1 because the split fluxes and their sums run in 64-bit "
-                 "fixed point on the integer pipes; fp64_unit gives the FP64 unit's own share and utilisation")
+RES_TRAFFIC = {MID_WORKLOAD: {1: 189.634048e6}}
+# Unit utilisation of that launch (fraction of peak sustained, ncu)
+RES_UNITS_NCU = {MID_WORKLOAD: {"fp64_pipe": 0.4869, "alu_pipe": 0.3963, "fmaheavy_pipe": 0.6972, "issue": 0.4957}}
+ROOFLINE_NOTE = ("bound: the pipe of the 32-bit multiplies, the kernel's busiest unit, by its busy cycles per active "
+                 "slot (counted once on the 147,584-point cloud); fp64_equivalent: the method's FP64 arithmetic as "
+                 "an all-FP64 form executes it against the FP64 unit, which the kernel leaves behind (frac above 1); "
+                 "fp64_unit: what the kernel still runs there")
+
+
+def _residual_roofline(wl, nslots, res_ms):
+    """The residual kernel's rates from its event-timed duration."""
+    per_s = nslots / (res_ms / 1e3)
+    flops = RES_FLOPS_PER_SLOT.get(wl)
+    unit = RES_FP64_UNIT_FLOPS_PER_SLOT.get(wl)
+
+    def fp64(f):
+        return None if f is None else {"flops_per_active_slot": f, "achieved": f * per_s / 1e12,
+                                       "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+                                       "frac": f * per_s / 1e12 / FP64_PEAK_TFLOPS}
+
+    mult = RES_MULT_CYCLES_PER_SLOT * per_s
+    return {"bound": "alu", "kernel": "k_residual", "achieved": mult / 1e9, "peak": MULT_PEAK / 1e9,
+            "unit": "G SM-cycles/s of the 32-bit multiply pipe", "frac": mult / MULT_PEAK,
+            "cycles_per_active_slot": RES_MULT_CYCLES_PER_SLOT, "active_slots": nslots,
+            "peak_source": "derived: 152 SMs x 2070 MHz", "note": ROOFLINE_NOTE,
+            "fp64_equivalent": fp64(flops), "fp64_unit": fp64(unit)}
 
 
 def _sweep_form(lanes):
@@ -316,10 +341,6 @@ def run_ours(args, rank, world, local_rank):
     # live per-phase timing (CUDA events on the library stream) for the roofline
     phases = s.time_phases(5)
     res_ms = phases["residual"]
-    flops_slot = RES_FLOPS_PER_SLOT.get(wl)
-    achieved = flops_slot * nslots / (res_ms / 1e3) / 1e12 if flops_slot else None
-    unit_slot = RES_FP64_UNIT_FLOPS_PER_SLOT.get(wl)
-    unit_tf = unit_slot * nslots / (res_ms / 1e3) / 1e12 if unit_slot else None
 
     # end to end through the C-ABI with host buffers: state in (H2D), one
     # iteration, state out (D2H) every step
@@ -390,17 +411,11 @@ def run_ours(args, rank, world, local_rank):
                                     "by": "given" if args.launch_shape else "autotune"},
                    "parallelism": "replicas" if world > 1 else "single",
                    "l2": f"inputs larger than L2: device working set {ws / 2**20:.0f} MiB > 129 MiB L2"},
-        "roofline": {"bound": "alu", "kernel": "k_residual", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                     "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS if achieved else None,
+        "roofline": {**_residual_roofline(wl, nslots, res_ms),
                      "traffic": traffic, "traffic_unit": "bytes per launch (ncu)",
                      "algorithmic_bytes_per_launch": int(cloud.nnz) * 37 + n * 360,
                      "algorithmic_bytes_rule": "37 B per neighbour slot (index, membership, dx, dy, 2 weights) "
                                                "+ 360 B per point (q, grad q, frame, geometry, state, R, D)",
-                     "flops_per_active_slot": flops_slot, "active_slots": nslots,
-                     "peak_source": "derived: 152 SMs x 4 FP64 flop/clk x 2070 MHz (the FP64 unit)",
-                     "note": ROOFLINE_NOTE,
-                     "fp64_unit": {"flops_per_active_slot": unit_slot, "achieved": unit_tf,
-                                   "frac": unit_tf / FP64_PEAK_TFLOPS if unit_tf else None},
                      "units_active_ncu": RES_UNITS_NCU.get(wl) if args.precision == 0 else None,
                      "launch_ms": res_ms, "phase_ms": phases},
         "cpu_baseline": cpu,
@@ -520,9 +535,6 @@ def solve_block(args, torch):
     }
 
 
-BATCH_WORKLOAD = "naca0012_batch64"
-
-
 def combine_over_ranks(dist, ms, counts, device):
     """The job's time is the slowest rank's, its work the sum of the ranks'
     (dist = torch.distributed or None for one process)."""
@@ -619,7 +631,6 @@ def run_batch(args, rank, world, local_rank):
 
     phases = s.time_phases(5)
     res_ms = phases["residual"]
-    achieved = RES_FLOPS_PER_SLOT[MID_WORKLOAD] * nslots / (res_ms / 1e3) / 1e12
 
     e2e_steps = min(args.steps, 10)
     U = s.field(lskum.FIELD_U)
@@ -687,11 +698,7 @@ def run_batch(args, rank, world, local_rank):
                    "parallelism": f"cases sharded over {world} ranks" if world > 1 else "single",
                    "residual_drop_min_max": [min(drops), max(drops)] if drops else None,
                    "l2": "inputs larger than L2"},
-        "roofline": {"bound": "alu", "kernel": "k_residual", "achieved": achieved, "peak": FP64_PEAK_TFLOPS,
-                     "unit": "TFLOP/s", "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None,
-                     "flops_per_active_slot": RES_FLOPS_PER_SLOT[MID_WORKLOAD],
-                     "peak_source": "derived: 152 SMs x 4 FP64 flop/clk x 2070 MHz (the FP64 unit)",
-                     "note": ROOFLINE_NOTE,
+        "roofline": {**_residual_roofline(BATCH_WORKLOAD, nslots, res_ms), "traffic": None,
                      "launch_ms": res_ms, "phase_ms": phases},
         "cpu_baseline": cpu,
         "e2e": e2e,

@@ -1,7 +1,9 @@
 // Kinetic split fluxes of reconstructed states in 64-bit fixed point.
 //
-// GB300 issues an FP64 instruction in 64 cycles per warp and sub-partition
-// (measured), a 32x32-bit multiply-add in 4 and an integer add or shift in 2.
+// An SM's FP64 unit takes a warp instruction in 19 cycles, so each of its four
+// schedulers, all asking, issues one in 76 (64, the latency, when it asks
+// alone); a 32x32-bit multiply-add takes a scheduler 4.5, an integer add or
+// shift 2 (measured).
 // A flux evaluated in FP64, or in FP64 with single operations moved to the
 // integer pipes, is bound by that unit (or by unpacking, normalising and
 // packing each result: about 80 cycles for a correctly rounded multiply).

@@ -1072,9 +1072,9 @@ constexpr int kRes64Block = 128;
 // into its frame, where every split flux is along an axis, and the sum's
 // momentum back out of it.  Measured on the 147,584-point cloud (1 lane per
 // point): 0.649 ms with the fluxes in FP64 and integer-pipe multiplies, 0.693
-// ms with compensated sums; 0.212 ms like this (41,194 points, four lanes:
-// 0.235 -> 0.092 ms).  The FMA-heavy pipe, which runs the 32-bit multiplies,
-// is about 60 % busy; four warps per scheduler (128 registers) do not hide
+// ms with compensated sums; 0.216 ms like this (41,194 points, four lanes:
+// 0.235 -> 0.091 ms).  The FMA-heavy pipe, which runs the 32-bit multiplies,
+// is about 70 % busy; four warps per scheduler (128 registers) do not hide
 // the rest of the chains' latency.  Staging the next slot's records in shared
 // memory, prefetching them, and a lane per state with more warps were slower.
 template <int TPP>
@@ -1544,7 +1544,7 @@ __device__ __forceinline__ void store_increment_product(const MathTables &Tb, co
 // increments, so they are formed beside the q-derivatives and the residual,
 // whose integer work leaves the FP64 unit idle, instead of twice per point on
 // the sweeps' critical path (41,194 points, an iteration: 0.804 ms with them
-// there, 0.535 like this, 0.511 with prim_short's chain).
+// there, 0.519 like this and with prim_short's chain).
 __host__ __device__ inline int increment_base_items(const Dev &d)
 {
     return 4 * d.n + 2 * (d.pk_lanes[0] + d.pk_lanes[1]);
